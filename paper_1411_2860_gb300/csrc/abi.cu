@@ -387,8 +387,7 @@ static pj_status gemm_validate(const void* A, int64_t lda, const void* B, int64_
 // Tile height of the E4M3 product of a single call (the quantiser lays the A_c
 // scale blocks out per tile, so both stages must agree): waves over the SMs.
 static int mx_single_bn(const GemmGeom& g, int sms) {
-  return single_launch_bn(g.M, ceil_div(g.N, 128), (g.Kq_pad / 128) * (g.qsplit == 1 ? 1 : 3), sms, 16,
-                          kMxTileRows);
+  return mx_single_rows(g.M, ceil_div(g.N, 128), g.Kq_pad / 128, g.qsplit != 1, sms);
 }
 
 static pj_status gemm_project_impl(const void* A, int64_t lda, const void* B, int64_t ldb, int32_t in_dtype,

@@ -413,8 +413,18 @@ struct GemmInst {  // 128-byte aligned through its tensor maps
   int tma_cols;
   int bn;   // rows of A_c per tile (MMA N): a multiple of 32, at most 256
   int mnQ, mnP;   // MN-major operands (see GemmTcArgs)
-  int ilv;        // three equal segments walked stage by stage (stage kk: segment kk % 3, chunk kk / 3)
+  // The plain hi/lo split (three equal segments): the K stages are counted as
+  // segments x chunks, but the kernels load the hi and the lo tiles of a chunk once,
+  // into two ring slots, and form its three products from them.  A range [k0, k1)
+  // of stages stands for the chunks [share_chunk(k0), share_chunk(k1)), so ranges
+  // that partition the stages partition the chunks.
+  int share;
 };
+constexpr
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+int share_chunk(int k) { return (k + 2) / 3; }
 // One tile of a grouped launch: instance, tile row / column, the range
 // [k0, k1) of K stages it multiplies (all kc * nseg stages unless the
 // instance's reduced dimension is split), and red = 1 when its partial product
@@ -494,11 +504,13 @@ struct MxInst {  // 128-byte aligned through its tensor maps
   int tma_cols;   // as GemmInst::tma_cols
   int bn;   // rows of A_c per tile (MMA N): a multiple of 16, at most 240
   int accum;      // every tile adds its product into Y
+  int share;      // two terms: hi and lo tiles of a chunk loaded once (as GemmInst::share)
   int conv_mode;  // as MxGemmArgs
   int64_t conv_stride, conv_limit;
 };
 bool build_mx_inst(const MxGemmArgs& a, MxInst* I);
 cudaError_t launch_gemm_mx(const MxGemmArgs& a, int* err, int num_sms, cudaStream_t st);
+int mx_single_rows(int64_t rows, int64_t tiles_n, int64_t chunks, bool split, int sms);   // a.bn of a single product
 cudaError_t launch_gemm_mx_grouped(const MxInst* insts, const GemmTile* tiles, const int* cta_off, int ctas,
                                    int* err, cudaStream_t st);
 

@@ -124,7 +124,9 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
         const int half = I->bn / 2;
         const uint32_t stage_bytes = kCStageP + static_cast<uint32_t>(half) * CK * 2;
         const int prow = pc * 2 * CM + static_cast<int>(rank) * CM;
-        for (int kk = 0; kk < I->kc; ++kk, ++issued) {
+        const bool share = I->share != 0;   // hi and lo tiles in alternate slots (GemmInst::share)
+        const int fills = share ? I->kc / 3 * 2 : I->kc;
+        for (int kk = 0; kk < fills; ++kk, ++issued) {
           if (issued == p.stall) {
             ok = false;
             break;
@@ -133,28 +135,31 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             ok = false;
             break;
           }
-          int seg = 0, kin = kk;
-          if (I->ilv) {
-            seg = kk % 3;
-            kin = kk / 3;
+          int sp = 0, sq = 0, kin = kk;
+          if (share) {
+            kin = kk >> 1;
+            sp = kk & 1;
+            sq = 2 * (kk & 1);
           } else {
-            while (seg + 1 < I->nseg && kin >= I->segKc[seg]) kin -= I->segKc[seg++];
+            while (sp + 1 < I->nseg && kin >= I->segKc[sp]) kin -= I->segKc[sp++];
+            sq = sp;
           }
+          const int px = I->segP[sp] + kin * CK, qx = I->segQ[sq] + kin * CK;
           if (leader) mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
           const uint32_t bar = full_leader + stage * 8;
           if (kMN && I->mnP) {
-            tma_load_2d_cg2(sP + stage * kCStageP, &I->mapP, bar, prow, I->segP[seg] + kin * CK);
-            tma_load_2d_cg2(sP + stage * kCStageP + 8192, &I->mapP, bar, prow + 64, I->segP[seg] + kin * CK);
+            tma_load_2d_cg2(sP + stage * kCStageP, &I->mapP, bar, prow, px);
+            tma_load_2d_cg2(sP + stage * kCStageP + 8192, &I->mapP, bar, prow + 64, px);
           } else {
-            tma_load_2d_cg2(sP + stage * kCStageP, &I->mapP, bar, I->segP[seg] + kin * CK, prow);
+            tma_load_2d_cg2(sP + stage * kCStageP, &I->mapP, bar, px, prow);
           }
           if (kMN && I->mnQ) {
             const int hc = half / 64;
             for (int c = 0; c < hc; ++c)
               tma_load_2d_cg2(sQ + stage * kCStageQ + c * 8192, &I->mapQ, bar,
-                              ti * I->bn + static_cast<int>(rank) * half + 64 * c, I->segQ[seg] + kin * CK);
+                              ti * I->bn + static_cast<int>(rank) * half + 64 * c, qx);
           } else {
-            tma_load_2d_cg2(sQ + stage * kCStageQ, &I->mapQ, bar, I->segQ[seg] + kin * CK,
+            tma_load_2d_cg2(sQ + stage * kCStageQ, &I->mapQ, bar, qx,
                             ti * I->bn + static_cast<int>(rank) * half);
           }
           used[stage] = true;
@@ -190,21 +195,42 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
         if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * CN;
-        for (int kk = 0; kk < I->kc; ++kk) {
+        // One 64-component product of the P tiles in slot sp and the Q tiles in slot sq.
+        auto products = [&](int sp, int sq, bool first) {
+          const uint32_t aP = smem_u32(sP + sp * kCStageP);
+          const uint32_t aQ = smem_u32(sQ + sq * kCStageQ);
+#pragma unroll
+          for (int k = 0; k < CK / 16; ++k) {
+            const uint64_t dp = mnP ? sdesc_sw128_mn(aP + k * 2048, 8192) : sdesc_sw128(aP + k * 32, 0);
+            const uint64_t dq = mnQ ? sdesc_sw128_mn(aQ + k * 2048, 8192) : sdesc_sw128(aQ + k * 32, 0);
+            umma_f16_cg2(d, dp, dq, idesc, !first || (k != 0));
+          }
+        };
+        const bool share = I->share != 0;
+        const int chunks = share ? I->kc / 3 : I->kc;
+        for (int kk = 0; kk < chunks; ++kk) {
           if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t aP = smem_u32(sP + stage * kCStageP);
-          const uint32_t aQ = smem_u32(sQ + stage * kCStageQ);
-#pragma unroll
-          for (int k = 0; k < CK / 16; ++k) {
-            const uint64_t dp = mnP ? sdesc_sw128_mn(aP + k * 2048, 8192) : sdesc_sw128(aP + k * 32, 0);
-            const uint64_t dq = mnQ ? sdesc_sw128_mn(aQ + k * 2048, 8192) : sdesc_sw128(aQ + k * 32, 0);
-            umma_f16_cg2(d, dp, dq, idesc, (kk != 0) || (k != 0));
-          }
+          products(stage, stage, kk == 0);
           issued_any = true;
+          if (share) {
+            const int hi = stage;
+            if (++stage == CSTAGES) {
+              stage = 0;
+              phase ^= 1u;
+            }
+            if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            products(stage, hi, false);
+            products(hi, stage, false);
+            umma_commit_cg2_mc(&empty[hi], 0x3);
+          }
           umma_commit_cg2_mc(&empty[stage], 0x3);
           if (++stage == CSTAGES) {
             stage = 0;

@@ -14,6 +14,9 @@
 // kernels (x to 2^-16 relative), so one projection code path serves both
 // precisions.
 //
+// With two terms, the hi and lo tiles of a K chunk take two ring slots and serve
+// the three products from there (four tile loads per chunk instead of six).
+//
 // GEMM (gemm_mx_kernel): tile 128 output columns (rows of B_d, MMA M) x 240
 // output rows (rows of A_c, MMA N), 128 components per stage (one 128-byte
 // swizzle row of E4M3, four MMAs of K = 32).  Each stage brings its operand
@@ -53,17 +56,27 @@ namespace {
 constexpr int XBM = 128;  // output columns per tile (MMA M)
 constexpr int XBN = 240;  // output rows per tile (MMA N)
 constexpr int XBK = 128;  // components per stage
-constexpr int XSTAGES = 4;
+// The ring takes as many slots of (128 + tile height) operand rows and their scale
+// blocks as its memory holds: four at 240 rows, five at 176, eight at most.
+constexpr int kXMaxStages = 8;
 constexpr int kXThreads = 192;
 constexpr uint32_t kXStageP = XBM * XBK;
-constexpr uint32_t kXStageQ = XBN * XBK;
 constexpr uint32_t kXStageSF = 512 + 1024;
 constexpr int kXEpiRows = 16;
 constexpr uint32_t kXStageOut = kXEpiRows * XBM * 4;
-constexpr size_t kXSmemBytes = 1024 + XSTAGES * (kXStageP + kXStageQ + kXStageSF) + kXStageOut + 256;
+constexpr uint32_t kXBars = 256;
+constexpr size_t kXSmemBytes = 232448;                                 // all of a block's shared memory
+constexpr uint32_t kXRing = 232448 - 1024 - kXStageOut - kXBars;       // operand slots, then their scale blocks
 constexpr uint32_t kSlot0 = 240, kSlot1 = 496;
-static_assert(kXStageQ % 1024 == 0 && kXStageP % 1024 == 0, "swizzled stages stay 1024-byte aligned");
-static_assert(kXSmemBytes <= 232448, "shared memory per block");
+static_assert((2 * kXMaxStages + 5) * 8 + 16 + 8 * 4 <= kXBars, "barriers, TMEM slot and votes");
+
+// Ring slots at a tile height of bn rows (a multiple of 16: slots of whole 2 KB).
+__host__ __device__ constexpr int mx_ring_slots(int bn) {
+  const uint32_t slot = kXStageP + static_cast<uint32_t>(bn) * XBK + kXStageSF;
+  const int n = static_cast<int>(kXRing / slot);
+  return n < kXMaxStages ? n : kXMaxStages;
+}
+static_assert(mx_ring_slots(XBN) >= 4, "at least two K chunks of a split product");
 
 struct MxParams {
   MxInst single;
@@ -72,6 +85,7 @@ struct MxParams {
   const int* cta_off;       // grouped launch: tiles of CTA c are [cta_off[c], cta_off[c+1])
   int num_tiles;            // single instance: tiles, walked with a grid stride
   int streamk;              // single instance: CTAs share the K stages of all tiles evenly
+  int slot_rows;            // tile height the ring slots are sized for (the instance's, or 240 when grouped)
   int* err;
 };
 
@@ -98,10 +112,11 @@ __device__ __forceinline__ const MxInst* mx_tile_of(const MxParams& p, int n, Ge
     t = p.tiles[k];
     return p.insts + t.inst;
   }
-  const int S = p.single.kc * p.single.nseg;
+  const int unit = p.single.share ? 3 : 1;   // a split K chunk is three stages, never cut
+  const int S = p.single.kc * p.single.nseg / unit;
   if (p.streamk) {
-    // Stream-K: CTA b owns the K stages [U b / G, U (b+1) / G) of the U = tiles * S
-    // stages of the whole product, tile by tile; a tile cut between CTAs adds its
+    // Stream-K: CTA b owns the K chunks [U b / G, U (b+1) / G) of the U = tiles * S
+    // chunks of the whole product, tile by tile; a tile cut between CTAs adds its
     // partial products into the (zeroed) output.
     const int64_t U = static_cast<int64_t>(p.num_tiles) * S;
     const int64_t u0 = U * blockIdx.x / gridDim.x, u1 = U * (blockIdx.x + 1) / gridDim.x;
@@ -111,9 +126,9 @@ __device__ __forceinline__ const MxInst* mx_tile_of(const MxParams& p, int n, Ge
     const int64_t end = u1 < static_cast<int64_t>(tile + 1) * S ? u1 : static_cast<int64_t>(tile + 1) * S;
     t.tj = tile % p.single.tiles_n;
     t.ti = tile / p.single.tiles_n;
-    t.k0 = static_cast<int>(start - static_cast<int64_t>(tile) * S);
-    t.k1 = static_cast<int>(end - static_cast<int64_t>(tile) * S);
-    t.red = (t.k0 != 0 || t.k1 != S || p.single.accum) ? 1 : 0;
+    t.k0 = unit * static_cast<int>(start - static_cast<int64_t>(tile) * S);
+    t.k1 = unit * static_cast<int>(end - static_cast<int64_t>(tile) * S);
+    t.red = (t.k0 != 0 || t.k1 != unit * S || p.single.accum) ? 1 : 0;
     t.pad0 = 0;
     return &p.single;
   }
@@ -122,7 +137,7 @@ __device__ __forceinline__ const MxInst* mx_tile_of(const MxParams& p, int n, Ge
   t.tj = tile % p.single.tiles_n;
   t.ti = tile / p.single.tiles_n;
   t.k0 = 0;
-  t.k1 = S;
+  t.k1 = unit * S;
   t.red = p.single.accum;
   t.pad0 = 0;
   return &p.single;
@@ -137,14 +152,14 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  uint8_t* sP = sm;
-  uint8_t* sQ = sP + XSTAGES * kXStageP;
-  uint8_t* sSF = sQ + XSTAGES * kXStageQ;
-  uint8_t* stage_out = sSF + XSTAGES * kXStageSF;
+  const int nst = mx_ring_slots(p.slot_rows);
+  const uint32_t slot_bytes = kXStageP + static_cast<uint32_t>(p.slot_rows) * XBK;   // P rows, then Q rows
+  uint8_t* sSF = sm + nst * slot_bytes;
+  uint8_t* stage_out = sm + kXRing;
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + kXStageOut);
   uint64_t* full = bars;
-  uint64_t* empty = bars + XSTAGES;
-  uint64_t* acc_full = bars + 2 * XSTAGES;
+  uint64_t* empty = bars + kXMaxStages;
+  uint64_t* acc_full = bars + 2 * kXMaxStages;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
@@ -153,7 +168,7 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int rank = kPair ? static_cast<int>(cluster_ctarank()) : 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < XSTAGES; ++s) {
+    for (int s = 0; s < nst; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kPair ? 2 : 1);
     }
@@ -179,9 +194,7 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
       // ---------------- producer: operand tiles by TMA, scale blocks by bulk copy
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t last_phase[XSTAGES];
-      bool used[XSTAGES];
-      for (int s = 0; s < XSTAGES; ++s) used[s] = false;
+      uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
       bool ok = true;
       GemmTile T{};
       for (int n = 0; ok; ++n) {
@@ -191,43 +204,49 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         tma_prefetch(&I->mapP);
         tma_prefetch(&I->mapQ);
         const uint32_t stage_bytes = kXStageP + static_cast<uint32_t>(I->bn) * XBK + kXStageSF;
-        for (int kk = T.k0; kk < T.k1; ++kk) {
+        // A split product's hi and lo tiles take alternate slots (see MxInst::share).
+        const bool share = I->share != 0;
+        const int f0 = share ? 2 * share_chunk(T.k0) : T.k0, f1 = share ? 2 * share_chunk(T.k1) : T.k1;
+        for (int kk = f0; kk < f1; ++kk) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
-          const int seg = kk / I->kc, kin = kk - seg * I->kc;
-          const int xp = I->segP[seg] + kin * XBK, xq = I->segQ[seg] + kin * XBK;
+          const int lo = share ? kk & 1 : 0, kin = share ? kk >> 1 : kk;
+          const int xp = (lo ? I->segP[2] : 0) + kin * XBK, xq = (lo ? I->segQ[1] : 0) + kin * XBK;
+          uint8_t* const sP = sm + stage * slot_bytes;
+          uint8_t* const sQ = sP + kXStageP;
           const uint8_t* sfp = I->sfP + (static_cast<int64_t>(tj) * I->sf_stages + xp / XBK) * 512;
           const uint8_t* sfq = I->sfQ + (static_cast<int64_t>(ti) * I->sf_stages + xq / XBK) * 1024;
           mbar_arrive_expect_tx(&full[stage], stage_bytes);
-          tma_load_2d(sP + stage * kXStageP, &I->mapP, &full[stage], xp, tj * XBM);
+          tma_load_2d(sP, &I->mapP, &full[stage], xp, tj * XBM);
 #if PJ_CTA_PAIRS
           if (kPair) {  // this CTA's half of the Q tile, for both CTAs of the pair
             const int half = I->bn / 2;
-            tma_load_2d_mc(sQ + stage * kXStageQ + rank * half * XBK, &I->mapQ, &full[stage], xq,
+            tma_load_2d_mc(sQ + rank * half * XBK, &I->mapQ, &full[stage], xq,
                            ti * I->bn + rank * half, 0x3);
           } else
 #endif
           {
             // (lowered correlation: stage kk of output rows r reads Q rows r + kk)
             if (I->conv_mode)
-              tma_load_2d(sQ + stage * kXStageQ, &I->mapQ, &full[stage], 0, ti * I->bn + kk);
+              tma_load_2d(sQ, &I->mapQ, &full[stage], 0, ti * I->bn + kk);
             else
-              tma_load_2d(sQ + stage * kXStageQ, &I->mapQ, &full[stage], xq, ti * I->bn);
+              tma_load_2d(sQ, &I->mapQ, &full[stage], xq, ti * I->bn);
           }
           bulk_load(sSF + stage * kXStageSF, sfp, 512, &full[stage]);
           bulk_load(sSF + stage * kXStageSF + 512, sfq, 1024, &full[stage]);
-          used[stage] = true;
-          last_phase[stage] = phase;
-          if (++stage == XSTAGES) {
+          used |= 1u << stage;
+          last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
       }
-      for (int s = 0; s < XSTAGES; ++s)
-        if (used[s] && !mbar_wait_drain(&full[s], last_phase[s])) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+      for (int s = 0; s < nst; ++s)
+        if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
+          atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -247,31 +266,62 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * 256;
-        for (int kk = T.k0; kk < T.k1; ++kk) {
+        // The scales of ring slot sl into TMEM (two sets of columns, used in turn).
+        auto scales = [&](int sl) {
+          const uint32_t cols = tmem + ((nslot++ & 1u) ? kSlot1 : kSlot0);
+          const uint32_t aSF = smem_u32(sSF + sl * kXStageSF);
+          tmem_cp_32x128b_warpx4(cols, sdesc_rows16(aSF));
+          tmem_cp_32x128b_warpx4(cols + 4, sdesc_rows16(aSF + 512));
+          tmem_cp_32x128b_warpx4(cols + 8, sdesc_rows16(aSF + 1024));
+          return cols;
+        };
+        // One 128-component product of the P tile in slot sp (scales at columns cp) and
+        // the Q tile in slot sq (scales at cq).
+        auto products = [&](int sp, uint32_t cp, int sq, uint32_t cq, bool first) {
+          const uint32_t aP = smem_u32(sm + sp * slot_bytes);
+          const uint32_t aQ = smem_u32(sm + sq * slot_bytes + kXStageP);
+#pragma unroll
+          for (int k = 0; k < XBK / 32; ++k)
+            umma_mx(d, sdesc_sw128(aP + k * 32, 0), sdesc_sw128(aQ + k * 32, 0), idesc_mx_e4m3(XBM, I->bn, k, k), cp,
+                    cq + 4, !first || (k != 0));
+        };
+        auto release = [&](int sl) {
+#if PJ_CTA_PAIRS
+          if (kPair)
+            umma_commit_mc(&empty[sl], 0x3);
+          else
+#endif
+            umma_commit(&empty[sl]);
+        };
+        const bool share = I->share != 0;
+        const int c0 = share ? share_chunk(T.k0) : T.k0, c1 = share ? share_chunk(T.k1) : T.k1;
+        for (int kk = c0; kk < c1; ++kk) {
           if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t slot = tmem + ((nslot++ & 1u) ? kSlot1 : kSlot0);
-          const uint32_t aSF = smem_u32(sSF + stage * kXStageSF);
-          tmem_cp_32x128b_warpx4(slot, sdesc_rows16(aSF));
-          tmem_cp_32x128b_warpx4(slot + 4, sdesc_rows16(aSF + 512));
-          tmem_cp_32x128b_warpx4(slot + 8, sdesc_rows16(aSF + 1024));
-          const uint32_t aP = smem_u32(sP + stage * kXStageP);
-          const uint32_t aQ = smem_u32(sQ + stage * kXStageQ);
-#pragma unroll
-          for (int k = 0; k < XBK / 32; ++k)
-            umma_mx(d, sdesc_sw128(aP + k * 32, 0), sdesc_sw128(aQ + k * 32, 0), idesc_mx_e4m3(XBM, I->bn, k, k),
-                    slot, slot + 4, (kk != T.k0) || (k != 0));
+          const uint32_t ch = scales(stage);
+          products(stage, ch, stage, ch, kk == c0);
           issued_any = true;
-#if PJ_CTA_PAIRS
-          if (kPair)
-            umma_commit_mc(&empty[stage], 0x3);
-          else
-#endif
-            umma_commit(&empty[stage]);
-          if (++stage == XSTAGES) {
+          if (share) {  // hi*hi issued; then hi(P)*lo(Q) and lo(P)*hi(Q) from the same four tiles
+            const int hi = stage;
+            if (++stage == nst) {
+              stage = 0;
+              phase ^= 1u;
+            }
+            if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t cl = scales(stage);
+            products(hi, ch, stage, cl, false);
+            products(stage, cl, hi, ch, false);
+            release(hi);
+          }
+          release(stage);
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
@@ -571,6 +621,7 @@ bool build_mx_inst(const MxGemmArgs& a, MxInst* I) {
   I->segP[0] = 0; I->segQ[0] = 0;
   I->segP[1] = 0; I->segQ[1] = static_cast<int>(a.Kq_pad);
   I->segP[2] = static_cast<int>(a.Kq_pad); I->segQ[2] = 0;
+  I->share = I->nseg == 3;
   I->tiles_n = static_cast<int>(ceil_div(a.rowsP, XBM));
   I->tiles_m = static_cast<int>(ceil_div(a.rowsQ, a.bn));
   const size_t es = I->out_bf16 ? 2 : 4;
@@ -588,6 +639,31 @@ bool build_mx_inst(const MxGemmArgs& a, MxInst* I) {
   return true;
 }
 
+// Tile height of a single product of `rows` x (tiles_n x 128) outputs over `chunks` K
+// chunks of 128: whole waves of tiles over the SMs, each ring slot costed (in ns) as
+// the longest of its loads from L2 (128 B_d rows and half of the pair's bn A_c rows at
+// the ~82 bytes per ns a SM draws when all of them load), its MMAs (a slot of a split
+// product serves 1.5 products) and the ~1.6 us a load takes shared by the slots in
+// flight; plus 1 us a tile.  (1500 x 2048 over 81 split chunks: 176 rows, one wave.)
+int mx_single_rows(int64_t rows, int64_t tiles_n, int64_t chunks, bool split, int sms) {
+  int best = XBN;
+  double best_t = 0;
+  for (int bn = XBN; bn >= 64; bn -= 16) {
+    const int64_t tiles = (rows + bn - 1) / bn * tiles_n;
+    const int64_t waves = (tiles + sms - 1) / sms;
+    const double load = 1.56 * (128 + (tiles_n % 2 ? bn : bn / 2)), mma = bn * (split ? 1.5 : 1.0);
+    double slot = load > mma ? load : mma;
+    const double flight = 1600.0 / mx_ring_slots(bn);
+    if (flight > slot) slot = flight;
+    const double t = static_cast<double>(waves) * (static_cast<double>(chunks) * (split ? 2 : 1) * slot + 1000.0);
+    if (bn == XBN || t < best_t * 0.99) {
+      best = bn;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
 cudaError_t launch_gemm_mx(const MxGemmArgs& a_in, int* err, int num_sms, cudaStream_t st) {
   if (a_in.rowsQ == 0 || a_in.rowsP == 0) return cudaSuccess;
   // The tile height is fixed by the scale-block layout the quantiser wrote (a.bn).
@@ -603,6 +679,7 @@ cudaError_t launch_gemm_mx(const MxGemmArgs& a_in, int* err, int num_sms, cudaSt
   p.tiles = nullptr;
   p.cta_off = nullptr;
   p.num_tiles = p.single.tiles_n * p.single.tiles_m;
+  p.slot_rows = a.bn;
   p.err = err;
   cudaError_t e = set_mx_smem_attr();
   if (e != cudaSuccess) return e;
@@ -647,6 +724,7 @@ cudaError_t launch_gemm_mx_grouped(const MxInst* insts, const GemmTile* tiles, c
   p.cta_off = cta_off;
   p.num_tiles = 0;
   p.streamk = 0;
+  p.slot_rows = XBN;   // instances of any height share the ring
   p.err = err;
   cudaError_t e = set_mx_smem_attr();
   if (e != cudaSuccess) return e;

@@ -18,8 +18,9 @@
 // rate that is more than the SMs can draw from L2, so K-major products run in
 // clusters of two CTAs on neighbouring tile columns of one tile row: each CTA
 // loads half of the shared A_c rows and multicasts them to both (kPair).
-// With the hi/lo split, the three segments are walked stage by stage, so the
-// hi tiles of a K chunk are read again while they are still in L2.
+// With the hi/lo split, the hi and lo tiles of a K chunk take two ring slots and
+// serve all three products (hi*hi, lo*hi, hi*lo) from there: four tile loads per
+// chunk instead of six, and the same shared memory covers 1.5x the MMA time.
 //
 // A grouped launch walks a per-CTA tile list planned on the host; a tile may
 // cover only a range of the K stages of its instance (a split reduced
@@ -85,10 +86,11 @@ __device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, G
     t = p.tiles[k];
     return p.insts + t.inst;
   }
-  const int S = p.single.kc;
+  const int unit = p.single.share ? 3 : 1;   // a shared-tile chunk is three stages, never cut
+  const int S = p.single.kc / unit;
   if (p.streamk) {
-    // Stream-K: CTA b owns the K stages [U b / G, U (b+1) / G) of the U = tiles * S
-    // stages of the whole product, tile by tile; a tile cut between CTAs adds its
+    // Stream-K: CTA b owns the K chunks [U b / G, U (b+1) / G) of the U = tiles * S
+    // chunks of the whole product, tile by tile; a tile cut between CTAs adds its
     // partial products into the (zeroed) output.
     const int64_t U = static_cast<int64_t>(p.num_tiles) * S;
     const int64_t u0 = U * blockIdx.x / gridDim.x, u1 = U * (blockIdx.x + 1) / gridDim.x;
@@ -98,9 +100,9 @@ __device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, G
     const int64_t end = u1 < static_cast<int64_t>(tile + 1) * S ? u1 : static_cast<int64_t>(tile + 1) * S;
     t.tj = tile % p.single.tiles_n;
     t.ti = tile / p.single.tiles_n;
-    t.k0 = static_cast<int>(start - static_cast<int64_t>(tile) * S);
-    t.k1 = static_cast<int>(end - static_cast<int64_t>(tile) * S);
-    t.red = (t.k0 != 0 || t.k1 != S) ? 1 : 0;
+    t.k0 = unit * static_cast<int>(start - static_cast<int64_t>(tile) * S);
+    t.k1 = unit * static_cast<int>(end - static_cast<int64_t>(tile) * S);
+    t.red = (t.k0 != 0 || t.k1 != p.single.kc) ? 1 : 0;
     t.pad0 = 0;
     return &p.single;
   }
@@ -109,7 +111,7 @@ __device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, G
   t.tj = tile % p.single.tiles_n;
   t.ti = tile / p.single.tiles_n;
   t.k0 = 0;
-  t.k1 = S;
+  t.k1 = p.single.kc;
   t.red = 0;
   t.pad0 = 0;  // no pair flags: the epilogue's stores (and its barriers) run in every warp
   return &p.single;
@@ -181,7 +183,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         tma_prefetch(&I->mapQ);
         const uint32_t stage_bytes = kStageP + static_cast<uint32_t>(I->bn) * BK * 2;
         const int qchunks = I->bn / 64;
-        for (int kk = T.k0; kk < T.k1; ++kk, ++issued) {
+        // Shared tiles: K chunk c is ring slots 2c (hi P, hi Q) and 2c + 1 (lo P, lo Q).
+        const bool share = I->share != 0;
+        const int f0 = share ? 2 * share_chunk(T.k0) : T.k0, f1 = share ? 2 * share_chunk(T.k1) : T.k1;
+        for (int kk = f0; kk < f1; ++kk, ++issued) {
           if (issued == p.stall) {  // self-test only: the consumers' bounded waits must run out
             ok = false;
             break;
@@ -190,37 +195,38 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             ok = false;
             break;
           }
-          int seg = 0, kin = kk;
-          if (I->ilv) {  // three equal segments taken stage by stage: a K chunk's hi tiles are reused at once
-            seg = kk % 3;
-            kin = kk / 3;
+          int sp = 0, sq = 0, kin = kk;   // segments whose P and Q offsets this slot takes
+          if (share) {
+            kin = kk >> 1;
+            sp = kk & 1;
+            sq = 2 * (kk & 1);
           } else {
-            while (seg + 1 < I->nseg && kin >= I->segKc[seg]) kin -= I->segKc[seg++];
+            while (sp + 1 < I->nseg && kin >= I->segKc[sp]) kin -= I->segKc[sp++];
+            sq = sp;
           }
+          const int px = I->segP[sp] + kin * BK;
           // Row-split mode: Q row r, K chunk k lives at row r + k/2, column 64 (k mod 2) of
           // a 128-wide view (the signal segments of a lowered correlation); there a
           // segment's Q offset counts rows (the split residual rows follow the hi rows).
-          const int qx = I->conv_mode ? (kin & 1) * BK : I->segQ[seg] + kin * BK;
-          const int qy = I->conv_mode ? ti * I->bn + (kin >> 1) + I->segQ[seg] : ti * I->bn;
+          const int qx = I->conv_mode ? (kin & 1) * BK : I->segQ[sq] + kin * BK;
+          const int qy = I->conv_mode ? ti * I->bn + (kin >> 1) + I->segQ[sq] : ti * I->bn;
           mbar_arrive_expect_tx(&full[stage], stage_bytes);
           if (kMN && I->mnP) {  // 64-wide MN chunks of 64 K rows (8 KB each)
-            tma_load_2d(sP + stage * kStageP, &I->mapP, &full[stage], tj * BM, I->segP[seg] + kin * BK);
-            tma_load_2d(sP + stage * kStageP + 8192, &I->mapP, &full[stage], tj * BM + 64, I->segP[seg] + kin * BK);
+            tma_load_2d(sP + stage * kStageP, &I->mapP, &full[stage], tj * BM, px);
+            tma_load_2d(sP + stage * kStageP + 8192, &I->mapP, &full[stage], tj * BM + 64, px);
           } else {
-            tma_load_2d(sP + stage * kStageP, &I->mapP, &full[stage], I->segP[seg] + kin * BK, tj * BM);
+            tma_load_2d(sP + stage * kStageP, &I->mapP, &full[stage], px, tj * BM);
           }
           if (kMN && I->mnQ) {
 #if PJ_CTA_PAIRS
             if (kPair) {  // this CTA's half of the Q chunks, for both CTAs of the pair
               const int hc = qchunks / 2;
               for (int c = rank * hc; c < (rank + 1) * hc; ++c)
-                tma_load_2d_mc(sQ + stage * kStageQ + c * 8192, &I->mapQ, &full[stage], ti * I->bn + 64 * c,
-                               I->segQ[seg] + kin * BK, 0x3);
+                tma_load_2d_mc(sQ + stage * kStageQ + c * 8192, &I->mapQ, &full[stage], ti * I->bn + 64 * c, qx, 0x3);
             } else
 #endif
             for (int c = 0; c < qchunks; ++c)
-              tma_load_2d(sQ + stage * kStageQ + c * 8192, &I->mapQ, &full[stage], ti * I->bn + 64 * c,
-                          I->segQ[seg] + kin * BK);
+              tma_load_2d(sQ + stage * kStageQ + c * 8192, &I->mapQ, &full[stage], ti * I->bn + 64 * c, qx);
 #if PJ_CTA_PAIRS
           } else if (kPair && !(T.pad0 & 1)) {
             // this CTA's half of the Q tile, for both CTAs of the pair
@@ -268,27 +274,51 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * BN;
-        for (int kk = T.k0; kk < T.k1; ++kk) {
+        // One 64-component product of the P tile in slot sp and the Q tile in slot sq.
+        auto products = [&](int sp, int sq, bool first) {
+          const uint32_t aP = smem_u32(sP + sp * kStageP);
+          const uint32_t aQ = smem_u32(sQ + sq * kStageQ);
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k) {
+            const uint64_t dp = mnP ? sdesc_sw128_mn(aP + k * 2048, 8192) : sdesc_sw128(aP + k * 32, 0);
+            const uint64_t dq = mnQ ? sdesc_sw128_mn(aQ + k * 2048, 8192) : sdesc_sw128(aQ + k * 32, 0);
+            umma_f16(d, dp, dq, idesc, !first || (k != 0));
+          }
+        };
+        auto release = [&](int sl) {
+#if PJ_CTA_PAIRS
+          if (kPair)
+            umma_commit_mc(&empty[sl], 0x3);
+          else
+#endif
+            umma_commit(&empty[sl]);
+        };
+        const bool share = I->share != 0;
+        const int c0 = share ? share_chunk(T.k0) : T.k0, c1 = share ? share_chunk(T.k1) : T.k1;
+        for (int kk = c0; kk < c1; ++kk) {
           if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t aP = smem_u32(sP + stage * kStageP);
-          const uint32_t aQ = smem_u32(sQ + stage * kStageQ);
-#pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t dp = mnP ? sdesc_sw128_mn(aP + k * 2048, 8192) : sdesc_sw128(aP + k * 32, 0);
-            const uint64_t dq = mnQ ? sdesc_sw128_mn(aQ + k * 2048, 8192) : sdesc_sw128(aQ + k * 32, 0);
-            umma_f16(d, dp, dq, idesc, (kk != T.k0) || (k != 0));
-          }
+          products(stage, stage, kk == c0);
           issued_any = true;
-#if PJ_CTA_PAIRS
-          if (kPair)
-            umma_commit_mc(&empty[stage], 0x3);
-          else
-#endif
-            umma_commit(&empty[stage]);
+          if (share) {  // hi*hi issued; then lo(P)*hi(Q) and hi(P)*lo(Q) from the same four tiles
+            const int hi = stage;
+            if (++stage == STAGES) {
+              stage = 0;
+              phase ^= 1u;
+            }
+            if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            products(stage, hi, false);
+            products(hi, stage, false);
+            release(hi);
+          }
+          release(stage);
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1u;
@@ -468,9 +498,10 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
     I->segKc[s] = s < a.nseg ? static_cast<int>(ceil_div(a.segK[s] ? a.segK[s] : a.kdim, BK)) : 0;
     I->kc += I->segKc[s];
   }
-  // The plain split's three segments (hi*hi, hi*lo, lo*hi) share their hi tiles:
-  // interleaved, each K chunk's hi tiles are read again while still in L2.
-  I->ilv = (a.nseg == 3 && !a.conv_mode && I->segKc[0] == I->segKc[1] && I->segKc[1] == I->segKc[2]) ? 1 : 0;
+  // The plain split's three segments (hi*hi, lo(P)*hi(Q), hi(P)*lo(Q)) share their
+  // tiles: four loads per K chunk instead of six (see GemmInst::share).
+  I->share = a.nseg == 3 && I->segKc[0] == I->segKc[1] && I->segKc[1] == I->segKc[2] && I->segP[0] == I->segP[2] &&
+             I->segQ[0] == I->segQ[1];
   I->tiles_n = static_cast<int>(ceil_div(a.rowsP, BM));
   I->conv_mode = a.conv_mode;
   I->conv_stride = a.conv_stride;
