@@ -200,42 +200,47 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
       for (int n = 0; ok; ++n) {
         const MxInst* I = mx_tile_of<kPair>(p, n, T, rank);
         if (!I) break;
-        const int ti = T.ti, tj = T.tj;
-        tma_prefetch(&I->mapP);
-        tma_prefetch(&I->mapQ);
-        const uint32_t stage_bytes = kXStageP + static_cast<uint32_t>(I->bn) * XBK + kXStageSF;
+        // read once (see gemm_tc.cu: a value read through I would be read again after every copy)
+        const CUtensorMap* const mapP = &I->mapP;
+        const CUtensorMap* const mapQ = &I->mapQ;
+        tma_prefetch(mapP);
+        tma_prefetch(mapQ);
+        const int bn = I->bn, half = bn / 2, y0 = T.ti * bn, p0 = T.tj * XBM;
+        const bool conv = I->conv_mode != 0;
+        const uint32_t stage_bytes = kXStageP + static_cast<uint32_t>(bn) * XBK + kXStageSF;
         // A split product's hi and lo tiles take alternate slots (see MxInst::share).
         const bool share = I->share != 0;
         const int f0 = share ? 2 * share_chunk(T.k0) : T.k0, f1 = share ? 2 * share_chunk(T.k1) : T.k1;
+        const int loP = I->segP[2], loQ = I->segQ[1];
+        const uint8_t* const sfP = I->sfP + static_cast<int64_t>(T.tj) * I->sf_stages * 512;
+        const uint8_t* const sfQ = I->sfQ + static_cast<int64_t>(T.ti) * I->sf_stages * 1024;
         for (int kk = f0; kk < f1; ++kk) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
           const int lo = share ? kk & 1 : 0, kin = share ? kk >> 1 : kk;
-          const int xp = (lo ? I->segP[2] : 0) + kin * XBK, xq = (lo ? I->segQ[1] : 0) + kin * XBK;
+          const int xp = (lo ? loP : 0) + kin * XBK, xq = (lo ? loQ : 0) + kin * XBK;
           uint8_t* const sP = sm + stage * slot_bytes;
           uint8_t* const sQ = sP + kXStageP;
-          const uint8_t* sfp = I->sfP + (static_cast<int64_t>(tj) * I->sf_stages + xp / XBK) * 512;
-          const uint8_t* sfq = I->sfQ + (static_cast<int64_t>(ti) * I->sf_stages + xq / XBK) * 1024;
-          mbar_arrive_expect_tx(&full[stage], stage_bytes);
-          tma_load_2d(sP, &I->mapP, &full[stage], xp, tj * XBM);
+          uint8_t* const sf = sSF + stage * kXStageSF;
+          uint64_t* const bar = &full[stage];
+          mbar_arrive_expect_tx(bar, stage_bytes);
+          tma_load_2d(sP, mapP, bar, xp, p0);
 #if PJ_CTA_PAIRS
           if (kPair) {  // this CTA's half of the Q tile, for both CTAs of the pair
-            const int half = I->bn / 2;
-            tma_load_2d_mc(sQ + rank * half * XBK, &I->mapQ, &full[stage], xq,
-                           ti * I->bn + rank * half, 0x3);
+            tma_load_2d_mc(sQ + rank * half * XBK, mapQ, bar, xq, y0 + rank * half, 0x3);
           } else
 #endif
           {
             // (lowered correlation: stage kk of output rows r reads Q rows r + kk)
-            if (I->conv_mode)
-              tma_load_2d(sQ, &I->mapQ, &full[stage], 0, ti * I->bn + kk);
+            if (conv)
+              tma_load_2d(sQ, mapQ, bar, 0, y0 + kk);
             else
-              tma_load_2d(sQ, &I->mapQ, &full[stage], xq, ti * I->bn);
+              tma_load_2d(sQ, mapQ, bar, xq, y0);
           }
-          bulk_load(sSF + stage * kXStageSF, sfp, 512, &full[stage]);
-          bulk_load(sSF + stage * kXStageSF + 512, sfq, 1024, &full[stage]);
+          bulk_load(sf, sfP + static_cast<int64_t>(xp / XBK) * 512, 512, bar);
+          bulk_load(sf + 512, sfQ + static_cast<int64_t>(xq / XBK) * 1024, 1024, bar);
           used |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == nst) {
@@ -251,6 +256,8 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
   } else if (warp == 1) {
     if (lane == 0) {
       // ---------------- MMA issuer
+      const uint64_t b0 = sdesc_sw128(smem_u32(sm), 0), bS = sdesc_rows16(smem_u32(sSF));
+      const uint32_t slot_units = slot_bytes / 16;
       int stage = 0;
       uint32_t phase = 0;
       int it = 0;
@@ -266,24 +273,24 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * 256;
+        const uint32_t idesc = idesc_mx_e4m3(XBM, I->bn, 0, 0);
         // The scales of ring slot sl into TMEM (two sets of columns, used in turn).
         auto scales = [&](int sl) {
           const uint32_t cols = tmem + ((nslot++ & 1u) ? kSlot1 : kSlot0);
-          const uint32_t aSF = smem_u32(sSF + sl * kXStageSF);
-          tmem_cp_32x128b_warpx4(cols, sdesc_rows16(aSF));
-          tmem_cp_32x128b_warpx4(cols + 4, sdesc_rows16(aSF + 512));
-          tmem_cp_32x128b_warpx4(cols + 8, sdesc_rows16(aSF + 1024));
+          const uint64_t ds = sdesc_advance(bS, sl * (kXStageSF / 16));
+          tmem_cp_32x128b_warpx4(cols, ds);
+          tmem_cp_32x128b_warpx4(cols + 4, sdesc_advance(ds, 512 / 16));
+          tmem_cp_32x128b_warpx4(cols + 8, sdesc_advance(ds, 1024 / 16));
           return cols;
         };
         // One 128-component product of the P tile in slot sp (scales at columns cp) and
         // the Q tile in slot sq (scales at cq).
         auto products = [&](int sp, uint32_t cp, int sq, uint32_t cq, bool first) {
-          const uint32_t aP = smem_u32(sm + sp * slot_bytes);
-          const uint32_t aQ = smem_u32(sm + sq * slot_bytes + kXStageP);
+          const uint64_t dp = sdesc_advance(b0, sp * slot_units), dq = sdesc_advance(b0, sq * slot_units + kXStageP / 16);
 #pragma unroll
           for (int k = 0; k < XBK / 32; ++k)
-            umma_mx(d, sdesc_sw128(aP + k * 32, 0), sdesc_sw128(aQ + k * 32, 0), idesc_mx_e4m3(XBM, I->bn, k, k), cp,
-                    cq + 4, !first || (k != 0));
+            umma_mx(d, sdesc_advance(dp, 2 * k), sdesc_advance(dq, 2 * k), idesc | idesc_mx_block(k), cp, cq + 4,
+                    !first || (k != 0));
         };
         auto release = [&](int sl) {
 #if PJ_CTA_PAIRS

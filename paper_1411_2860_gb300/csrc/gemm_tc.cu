@@ -169,23 +169,31 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       // ---------------- TMA producer
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t last_phase[STAGES];
-      bool used[STAGES];
-      for (int s = 0; s < STAGES; ++s) used[s] = false;
+      uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
       bool ok = true;
       int issued = 0;
       GemmTile T{};
       for (int n = 0; ok; ++n) {
         const GemmInst* I = tile_of<kPair>(p, n, T, rank);
         if (!I) break;
-        const int ti = T.ti, tj = T.tj;
-        tma_prefetch(&I->mapP);
-        tma_prefetch(&I->mapQ);
-        const uint32_t stage_bytes = kStageP + static_cast<uint32_t>(I->bn) * BK * 2;
-        const int qchunks = I->bn / 64;
+        // Everything the loop needs, read once: the copies are asm volatile with a memory
+        // clobber, so a value read through I would be read again for every one of them,
+        // and this thread's chain of loads would set the pace of the whole CTA.
+        const CUtensorMap* const mapP = &I->mapP;
+        const CUtensorMap* const mapQ = &I->mapQ;
+        tma_prefetch(mapP);
+        tma_prefetch(mapQ);
+        const int tj = T.tj, bn = I->bn, half = bn / 2;
+        const int y0 = T.ti * bn;
+        const bool conv = I->conv_mode != 0, mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
+        const uint32_t stage_bytes = kStageP + static_cast<uint32_t>(bn) * BK * 2;
+        const int qchunks = bn / 64;
         // Shared tiles: K chunk c is ring slots 2c (hi P, hi Q) and 2c + 1 (lo P, lo Q).
         const bool share = I->share != 0;
         const int f0 = share ? 2 * share_chunk(T.k0) : T.k0, f1 = share ? 2 * share_chunk(T.k1) : T.k1;
+        const int sP0 = I->segP[0], sP1 = I->segP[1], sP2 = I->segP[2];
+        const int sQ0 = I->segQ[0], sQ1 = I->segQ[1], sQ2 = I->segQ[2];
+        const int e0 = I->nseg > 1 ? I->segKc[0] : 0x7fffffff, e1 = I->nseg > 2 ? e0 + I->segKc[1] : 0x7fffffff;
         for (int kk = f0; kk < f1; ++kk, ++issued) {
           if (issued == p.stall) {  // self-test only: the consumers' bounded waits must run out
             ok = false;
@@ -195,55 +203,55 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             ok = false;
             break;
           }
-          int sp = 0, sq = 0, kin = kk;   // segments whose P and Q offsets this slot takes
+          int kin, oP, oQ;   // chunk, and the segments' offsets in P and Q
           if (share) {
             kin = kk >> 1;
-            sp = kk & 1;
-            sq = 2 * (kk & 1);
+            oP = (kk & 1) ? sP1 : sP0;
+            oQ = (kk & 1) ? sQ2 : sQ0;
           } else {
-            while (sp + 1 < I->nseg && kin >= I->segKc[sp]) kin -= I->segKc[sp++];
-            sq = sp;
+            kin = kk < e0 ? kk : (kk < e1 ? kk - e0 : kk - e1);
+            oP = kk < e0 ? sP0 : (kk < e1 ? sP1 : sP2);
+            oQ = kk < e0 ? sQ0 : (kk < e1 ? sQ1 : sQ2);
           }
-          const int px = I->segP[sp] + kin * BK;
+          const int px = oP + kin * BK;
           // Row-split mode: Q row r, K chunk k lives at row r + k/2, column 64 (k mod 2) of
           // a 128-wide view (the signal segments of a lowered correlation); there a
           // segment's Q offset counts rows (the split residual rows follow the hi rows).
-          const int qx = I->conv_mode ? (kin & 1) * BK : I->segQ[sq] + kin * BK;
-          const int qy = I->conv_mode ? ti * I->bn + (kin >> 1) + I->segQ[sq] : ti * I->bn;
-          mbar_arrive_expect_tx(&full[stage], stage_bytes);
-          if (kMN && I->mnP) {  // 64-wide MN chunks of 64 K rows (8 KB each)
-            tma_load_2d(sP + stage * kStageP, &I->mapP, &full[stage], tj * BM, px);
-            tma_load_2d(sP + stage * kStageP + 8192, &I->mapP, &full[stage], tj * BM + 64, px);
+          const int qx = conv ? (kin & 1) * BK : oQ + kin * BK;
+          const int qy = conv ? y0 + (kin >> 1) + oQ : y0;
+          uint64_t* const bar = &full[stage];
+          uint8_t* const dP = sP + stage * kStageP;
+          uint8_t* const dQ = sQ + stage * kStageQ;
+          mbar_arrive_expect_tx(bar, stage_bytes);
+          if (mnP) {  // 64-wide MN chunks of 64 K rows (8 KB each)
+            tma_load_2d(dP, mapP, bar, tj * BM, px);
+            tma_load_2d(dP + 8192, mapP, bar, tj * BM + 64, px);
           } else {
-            tma_load_2d(sP + stage * kStageP, &I->mapP, &full[stage], px, tj * BM);
+            tma_load_2d(dP, mapP, bar, px, tj * BM);
           }
-          if (kMN && I->mnQ) {
+          if (mnQ) {
 #if PJ_CTA_PAIRS
             if (kPair) {  // this CTA's half of the Q chunks, for both CTAs of the pair
               const int hc = qchunks / 2;
               for (int c = rank * hc; c < (rank + 1) * hc; ++c)
-                tma_load_2d_mc(sQ + stage * kStageQ + c * 8192, &I->mapQ, &full[stage], ti * I->bn + 64 * c, qx, 0x3);
+                tma_load_2d_mc(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx, 0x3);
             } else
 #endif
-            for (int c = 0; c < qchunks; ++c)
-              tma_load_2d(sQ + stage * kStageQ + c * 8192, &I->mapQ, &full[stage], ti * I->bn + 64 * c, qx);
+            for (int c = 0; c < qchunks; ++c) tma_load_2d(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx);
 #if PJ_CTA_PAIRS
           } else if (kPair && !(T.pad0 & 1)) {
             // this CTA's half of the Q tile, for both CTAs of the pair
-            const int half = I->bn / 2;
-            tma_load_2d_mc(sQ + stage * kStageQ + rank * half * (BK * 2), &I->mapQ, &full[stage], qx,
-                           qy + rank * half, 0x3);
+            tma_load_2d_mc(dQ + rank * half * (BK * 2), mapQ, bar, qx, qy + rank * half, 0x3);
 #endif
           } else if (kPair) {
             // a tile of its own (grouped launch): both halves for this CTA only
-            const int half = I->bn / 2;
-            tma_load_2d(sQ + stage * kStageQ, &I->mapQ, &full[stage], qx, qy);
-            tma_load_2d(sQ + stage * kStageQ + half * (BK * 2), &I->mapQ, &full[stage], qx, qy + half);
+            tma_load_2d(dQ, mapQ, bar, qx, qy);
+            tma_load_2d(dQ + half * (BK * 2), mapQ, bar, qx, qy + half);
           } else {
-            tma_load_2d(sQ + stage * kStageQ, &I->mapQ, &full[stage], qx, qy);
+            tma_load_2d(dQ, mapQ, bar, qx, qy);
           }
-          used[stage] = true;
-          last_phase[stage] = phase;
+          used |= 1u << stage;
+          last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1u;
@@ -252,7 +260,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       }
       // Every issued copy must land before the CTA may exit.
       for (int s = 0; s < STAGES; ++s)
-        if (used[s] && !mbar_wait_drain(&full[s], last_phase[s])) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+        if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
+          atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -275,15 +284,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         // One 64-component product of the P tile in slot sp and the Q tile in slot sq.
+        // (A K step of 16 moves a K-major start by 32 bytes, an MN-major one by 2048.)
+        const uint64_t bP = mnP ? sdesc_sw128_mn(smem_u32(sP), 8192) : sdesc_sw128(smem_u32(sP), 0);
+        const uint64_t bQ = mnQ ? sdesc_sw128_mn(smem_u32(sQ), 8192) : sdesc_sw128(smem_u32(sQ), 0);
+        const uint32_t kP = mnP ? 128 : 2, kQ = mnQ ? 128 : 2;
         auto products = [&](int sp, int sq, bool first) {
-          const uint32_t aP = smem_u32(sP + sp * kStageP);
-          const uint32_t aQ = smem_u32(sQ + sq * kStageQ);
+          const uint64_t dp = sdesc_advance(bP, sp * (kStageP / 16)), dq = sdesc_advance(bQ, sq * (kStageQ / 16));
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t dp = mnP ? sdesc_sw128_mn(aP + k * 2048, 8192) : sdesc_sw128(aP + k * 32, 0);
-            const uint64_t dq = mnQ ? sdesc_sw128_mn(aQ + k * 2048, 8192) : sdesc_sw128(aQ + k * 32, 0);
-            umma_f16(d, dp, dq, idesc, !first || (k != 0));
-          }
+          for (int k = 0; k < BK / 16; ++k)
+            umma_f16(d, sdesc_advance(dp, k * kP), sdesc_advance(dq, k * kQ), idesc, !first || (k != 0));
         };
         auto release = [&](int sl) {
 #if PJ_CTA_PAIRS

@@ -343,6 +343,10 @@ __device__ __forceinline__ uint64_t sdesc_sw128_mn(uint32_t saddr, uint32_t chun
   return d;
 }
 
+// The start address of a descriptor moved by `units` 16-byte units (the address
+// field is the descriptor's low bits, and shared memory ends below its range).
+__device__ __forceinline__ uint64_t sdesc_advance(uint64_t d, uint32_t units) { return d + units; }
+
 // Descriptor of a contiguous 32-row x 16-byte block (no swizzle; 8-row core
 // matrices 128 bytes apart), the source of tmem_cp_32x128b_warpx4.
 __device__ __forceinline__ uint64_t sdesc_rows16(uint32_t saddr) {
@@ -359,6 +363,12 @@ __device__ __forceinline__ uint64_t sdesc_rows16(uint32_t saddr) {
 __host__ __device__ constexpr uint32_t idesc_mx_e4m3(int M, int N, int asf, int bsf) {
   return (static_cast<uint32_t>(bsf & 3) << 4) | (static_cast<uint32_t>(N >> 3) << 17) | (1u << 23) |
          (static_cast<uint32_t>(M >> 4) << 24) | (static_cast<uint32_t>(asf & 3) << 29);
+}
+
+// The scale-byte fields of K block k (0..3) for both operands, to be or-ed into
+// idesc_mx_e4m3(M, N, 0, 0).
+__host__ __device__ constexpr uint32_t idesc_mx_block(int k) {
+  return (static_cast<uint32_t>(k & 3) << 4) | (static_cast<uint32_t>(k & 3) << 29);
 }
 
 // Instruction descriptor, kind::f16: BF16 x BF16 -> FP32, both operands K-major.
