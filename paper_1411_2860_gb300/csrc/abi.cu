@@ -227,12 +227,12 @@ pj_status check_gemm_dtypes(int in_dtype, int out_dtype, const pj_precision* pre
   return PJ_OK;
 }
 
-pj_status stage_basis(const pj_basis* basis, int lp1, void* ws, cudaStream_t st, void* area, int p0) {
+pj_status stage_basis(const pj_basis* basis, int lp1, void* ws, cudaStream_t st, void* area, int p0, bool clear) {
   BasisDev b = basis_area(area ? area : ws);
   if (basis->kind == PJ_BASIS_USER)
     PJ_CUDA_TRY(cudaMemcpyAsync(b.U64, basis->user_C, sizeof(double) * basis->L * basis->L, cudaMemcpyHostToDevice,
                                 st));
-  PJ_CUDA_TRY(launch_basis_build(basis->kind, basis->L, lp1, b, error_word(ws), st, p0));
+  PJ_CUDA_TRY(launch_basis_build(basis->kind, basis->L, lp1, b, error_word(ws), st, p0, clear));
   return PJ_OK;
 }
 
@@ -348,8 +348,8 @@ pj_status pj_basis_build(const pj_basis* basis, int32_t lp1, double* C_out, doub
   PJ_TRY(check_ws(workspace, ws_bytes, align_up(kHeaderBytes + kBasisBytes)));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int sms = 0;
-  PJ_TRY(begin_call(workspace, st, &sms));
-  PJ_TRY(stage_basis(basis, lp1, workspace, st));
+  PJ_TRY(device_sms(&sms));
+  PJ_TRY(stage_basis(basis, lp1, workspace, st, nullptr, 0, true));
   BasisDev b = basis_area(workspace);
   const size_t bytes = sizeof(double) * basis->L * lp1;
   PJ_CUDA_TRY(cudaMemcpyAsync(C_out, b.Cs64, bytes, cudaMemcpyDeviceToDevice, st));
@@ -393,11 +393,21 @@ static int mx_single_bn(const GemmGeom& g, int sms) {
 static pj_status gemm_project_impl(const void* A, int64_t lda, const void* B, int64_t ldb, int32_t in_dtype,
                                    const pj_basis* basis, const pj_precision* prec, void* ws, const GemmGeom& g,
                                    const GemmWs& w, int sms, cudaStream_t st) {
-  PJ_TRY(stage_basis(basis, g.lp1, ws, st));
+  // The call's first kernel clears the error word: the basis kernel, or with a built-in
+  // basis of groups of 8 (whose vectors are kernel arguments) the projection itself.
+  Coef8 c8v;
+  const Coef8* c8 = prec->compute != PJ_F64 && coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
+  bool clear = false;
+  if (c8) {
+    clear = A || B;
+    if (!clear) PJ_CUDA_TRY(cudaMemsetAsync(ws, 0, sizeof(int), st));
+  } else {
+    PJ_TRY(stage_basis(basis, g.lp1, ws, st, nullptr, 0, true));
+  }
   BasisDev b = basis_area(ws);
   if (prec->compute == PJ_F64) {
-    if (A) PJ_CUDA_TRY(launch_project_rows_f64(static_cast<const double*>(A), lda, g, b.Cs64, at<double>(ws, w.off_ac), st));
-    if (B) PJ_CUDA_TRY(launch_project_cols_f64(static_cast<const double*>(B), ldb, g, b.Ds64, at<double>(ws, w.off_bd), st));
+    PJ_CUDA_TRY(launch_project_pair_f64(static_cast<const double*>(A), lda, static_cast<const double*>(B), ldb, g, b.Cs64,
+                                        b.Ds64, at<double>(ws, w.off_ac), at<double>(ws, w.off_bd), st));
   } else {
     if (prec->compute == PJ_E4M3) {
       const MxQuantSide qa = make_mx_side(at<uint16_t>(ws, w.off_ac), g.Kp_pad, g.M, at<uint8_t>(ws, w.off_aq),
@@ -407,18 +417,20 @@ static pj_status gemm_project_impl(const void* A, int64_t lda, const void* B, in
       // E4M3 components straight from the projection where it can write them; the
       // other sides go through BF16 hi + lo and the quantiser pass.
       bool a_done = false, b_done = false;
-      PJ_CUDA_TRY(launch_project_pair_mx(A, lda, B, ldb, in_dtype, g, b.Cs32, b.Ds32, A ? &qa : nullptr,
-                                         B ? &qb : nullptr, error_word(ws), sms, st, &a_done, &b_done));
+      PJ_CUDA_TRY(launch_project_pair_mx(A, lda, B, ldb, in_dtype, g, b.Cs32, b.Ds32, c8, A ? &qa : nullptr,
+                                         B ? &qb : nullptr, error_word(ws), clear, sms, st, &a_done, &b_done));
+      if (a_done || b_done) clear = false;
       const void* A2 = a_done ? nullptr : A;
       const void* B2 = b_done ? nullptr : B;
       if (A2 || B2) {
-        PJ_CUDA_TRY(launch_project_pair_bf16(A2, lda, B2, ldb, in_dtype, g, b.Cs32, b.Ds32, at<uint16_t>(ws, w.off_ac),
-                                             at<uint16_t>(ws, w.off_bd), error_word(ws), sms, st));
+        PJ_CUDA_TRY(launch_project_pair_bf16(A2, lda, B2, ldb, in_dtype, g, b.Cs32, b.Ds32, c8,
+                                             at<uint16_t>(ws, w.off_ac), at<uint16_t>(ws, w.off_bd), error_word(ws),
+                                             clear, sms, st));
         PJ_CUDA_TRY(launch_quantize_mx(A2 ? &qa : nullptr, B2 ? &qb : nullptr, st));
       }
     } else {
-      PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g, b.Cs32, b.Ds32, at<uint16_t>(ws, w.off_ac),
-                                           at<uint16_t>(ws, w.off_bd), error_word(ws), sms, st));
+      PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g, b.Cs32, b.Ds32, c8, at<uint16_t>(ws, w.off_ac),
+                                           at<uint16_t>(ws, w.off_bd), error_word(ws), clear, sms, st));
     }
   }
   if (g.tier > 0) {
@@ -427,10 +439,12 @@ static pj_status gemm_project_impl(const void* A, int64_t lda, const void* B, in
     void* sub = at<char>(ws, w.off_tier);
     const GemmGeom gt = tier_geom(g);
     const GemmWs wt = gemm_ws_layout(gt, PJ_E4M3);
-    PJ_TRY(stage_basis(basis, gt.lp1, ws, st, sub, g.lp1));
+    Coef8 t8v;
+    const Coef8* t8 = coef8(basis, gt.lp1, g.lp1, &t8v) ? &t8v : nullptr;
+    if (!t8) PJ_TRY(stage_basis(basis, gt.lp1, ws, st, sub, g.lp1));
     BasisDev bt = basis_area(sub);
-    PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, gt, bt.Cs32, bt.Ds32, at<uint16_t>(sub, wt.off_ac),
-                                         at<uint16_t>(sub, wt.off_bd), error_word(ws), sms, st));
+    PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, gt, bt.Cs32, bt.Ds32, t8, at<uint16_t>(sub, wt.off_ac),
+                                         at<uint16_t>(sub, wt.off_bd), error_word(ws), false, sms, st));
     const MxQuantSide qa = make_mx_side(at<uint16_t>(sub, wt.off_ac), gt.Kp_pad, gt.M, at<uint8_t>(sub, wt.off_aq),
                                         gt.Kq_pad, 1, at<uint8_t>(sub, wt.off_sfq), 1, mx_single_bn(gt, sms));
     const MxQuantSide qb = make_mx_side(at<uint16_t>(sub, wt.off_bd), gt.Kp_pad, gt.N, at<uint8_t>(sub, wt.off_bq),
@@ -509,8 +523,11 @@ pj_status proj_gemm(const void* A, int64_t lda, const void* B, int64_t ldb, void
   if (M == 0 || N == 0) return PJ_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int sms = 0;
-  PJ_TRY(begin_call(workspace, st, &sms));
-  if (K == 0) return zero_output(Y, ldy, M, N, out_dtype, st);
+  if (K == 0) {
+    PJ_TRY(begin_call(workspace, st, &sms));
+    return zero_output(Y, ldy, M, N, out_dtype, st);
+  }
+  PJ_TRY(device_sms(&sms));
   PJ_TRY(gemm_project_impl(A, lda, B, ldb, in_dtype, basis, prec, workspace, g, w, sms, st));
   return gemm_multiply_impl(Y, ldy, out_dtype, prec, workspace, g, w, sms, st);
 }
@@ -523,8 +540,8 @@ pj_status proj_gemm_project(const void* A, int64_t lda, const void* B, int64_t l
   PJ_TRY(gemm_validate(A, lda, B, ldb, M, N, K, in_dtype, block_k, R, basis, prec, workspace, ws_bytes, &g, &w));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int sms = 0;
-  PJ_TRY(begin_call(workspace, st, &sms));
-  if (K == 0) return PJ_OK;
+  if (K == 0) return begin_call(workspace, st, &sms);
+  PJ_TRY(device_sms(&sms));
   return gemm_project_impl(M > 0 ? A : nullptr, lda, N > 0 ? B : nullptr, ldb, in_dtype, basis, prec, workspace, g,
                            w, sms, st);
 }
@@ -620,13 +637,23 @@ size_t proj_gemm_backward_workspace_size(int64_t M, int64_t N, int64_t K, int64_
   return bwd_ws_layout(g, prec->compute).total;
 }
 
+// With L = 8 and l+1 a power of two, each product's epilogue maps its components
+// back to samples (expand_C for dA, expand_D for dB) and writes the gradient itself;
+// otherwise the FP32 reduced gradients go through the expansion kernels.
+static bool bwd_fused(const GemmGeom& g, int compute, int64_t ldda, int64_t lddb, int32_t out_dtype) {
+  const size_t oes = out_dtype == PJ_BF16 ? 2 : 4;
+  return compute != PJ_F64 && g.L == 8 && (g.lp1 == 1 || g.lp1 == 2 || g.lp1 == 4 || g.lp1 == 8) &&
+         (ldda * oes) % 16 == 0 && (lddb * oes) % 16 == 0;
+}
+
 // The two gradient products and their expansion, from projected operands Ac
 // (M x pitch) and Bd (N x pitch) -- computed by the backward itself or saved by
-// the forward -- and dY (dy_dtype).  The basis is staged in `workspace`.
+// the forward -- and dY (dy_dtype).  The basis is staged in `workspace`, or given as c8
+// (fused products only).
 static pj_status backward_products(const void* Ac_v, const void* Bd_v, const void* dY, int64_t lddy, int32_t dy_dtype,
                                    void* dA, int64_t ldda, void* dB, int64_t lddb, int32_t out_dtype,
-                                   const GemmGeom& g, int compute, const BwdWs& w, void* workspace, int sms,
-                                   cudaStream_t st) {
+                                   const GemmGeom& g, int compute, const BwdWs& w, const Coef8* c8, void* workspace,
+                                   int sms, cudaStream_t st) {
   BasisDev b = basis_area(workspace);
   if (compute == PJ_F64) {
     const double* Ac = static_cast<const double*>(Ac_v);
@@ -654,12 +681,7 @@ static pj_status backward_products(const void* Ac_v, const void* Bd_v, const voi
   if (!dy_direct) PJ_CUDA_TRY(launch_convert_bf16(dY, dy_dtype, lddy, g.M, g.N, dYb, w.ldn, st));
   const uint16_t* dYq = dy_direct ? static_cast<const uint16_t*>(dY) : dYb;
   const int64_t lddq = dy_direct ? lddy : w.ldn;
-  // With L = 8 and l+1 a power of two, each product's epilogue maps its components
-  // back to samples (expand_C for dA, expand_D for dB) and writes the gradient
-  // itself; otherwise the FP32 reduced gradients go through the expansion kernels.
-  const size_t oes = out_dtype == PJ_BF16 ? 2 : 4;
-  const bool fuse = g.L == 8 && (g.lp1 == 1 || g.lp1 == 2 || g.lp1 == 4 || g.lp1 == 8) &&
-                    (ldda * oes) % 16 == 0 && (lddb * oes) % 16 == 0;
+  const bool fuse = bwd_fused(g, compute, ldda, lddb, out_dtype);
   GemmTcArgs a1{};  // dA_c[i][k'] = sum_j dY[i][j] B_d[k'][j]: B_d read MN-major (N rows of components)
   a1.Q = dYq;
   a1.ldq = lddq;
@@ -674,7 +696,8 @@ static pj_status backward_products(const void* Ac_v, const void* Bd_v, const voi
     a1.ex.K = g.K;
     a1.ex.out = dA;
     a1.ex.ld = ldda;
-    a1.ex.coef = b.Cs32;
+    a1.ex.coef = c8 ? nullptr : b.Cs32;
+    a1.ex_c8 = c8;
   }
   // dB_d[k'][j] = sum_i A_c[i][k'] dY[i][j]: both operands are read MN-major
   // (A_c and dY as stored, reduced over their rows), so nothing is transposed.
@@ -688,7 +711,8 @@ static pj_status backward_products(const void* Ac_v, const void* Bd_v, const voi
     a2.ex.mode = 2;
     a2.ex.out = dB;
     a2.ex.ld = lddb;
-    a2.ex.coef = b.Ds32;
+    a2.ex.coef = c8 ? nullptr : b.Ds32;
+    a2.ex_c8 = c8;
   }
   // (One launch over both products' tiles measured slower: 0.18 against 0.158 ms
   // for the 8192 x 4096 x 4096 layer, the two operand streams sharing L2.)
@@ -746,26 +770,34 @@ pj_status proj_gemm_backward(const void* A, int64_t lda, const void* B, int64_t 
   if (K == 0) return PJ_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int sms = 0;
-  PJ_TRY(begin_call(workspace, st, &sms));
-  if (M == 0 || N == 0) return backward_zero(dA, ldda, dB, lddb, g, out_dtype, st);
-  PJ_TRY(stage_basis(basis, g.lp1, workspace, st));
+  if (M == 0 || N == 0) {
+    PJ_TRY(begin_call(workspace, st, &sms));
+    return backward_zero(dA, ldda, dB, lddb, g, out_dtype, st);
+  }
+  PJ_TRY(device_sms(&sms));
+  // the first kernel clears the error word (as in gemm_project_impl); the expansion
+  // kernels read the staged tables
+  Coef8 c8v;
+  const Coef8* c8 =
+      bwd_fused(g, prec->compute, ldda, lddb, out_dtype) && coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
+  if (!c8) PJ_TRY(stage_basis(basis, g.lp1, workspace, st, nullptr, 0, true));
   BasisDev b = basis_area(workspace);
   if (prec->compute == PJ_F64) {
     double* Ac = at<double>(workspace, w.ac);
     double* Bd = at<double>(workspace, w.bd);
-    PJ_CUDA_TRY(launch_project_rows_f64(static_cast<const double*>(A), lda, g, b.Cs64, Ac, st));
-    PJ_CUDA_TRY(launch_project_cols_f64(static_cast<const double*>(B), ldb, g, b.Ds64, Bd, st));
-    return backward_products(Ac, Bd, dY, lddy, PJ_F64, dA, ldda, dB, lddb, out_dtype, g, PJ_F64, w, workspace, sms,
-                             st);
+    PJ_CUDA_TRY(launch_project_pair_f64(static_cast<const double*>(A), lda, static_cast<const double*>(B), ldb, g, b.Cs64,
+                                        b.Ds64, Ac, Bd, st));
+    return backward_products(Ac, Bd, dY, lddy, PJ_F64, dA, ldda, dB, lddb, out_dtype, g, PJ_F64, w, nullptr, workspace,
+                             sms, st);
   }
   uint16_t* Ac = at<uint16_t>(workspace, w.ac);
   uint16_t* Bd = at<uint16_t>(workspace, w.bd);
   GemmGeom g1 = g;
   g1.nsplit = 1;
   // A_c (M x Kp_pad) and B_d (N x Kp_pad) exactly as the forward projects them, in one launch
-  PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g1, b.Cs32, b.Ds32, Ac, Bd, error_word(workspace),
-                                       sms, st));
-  return backward_products(Ac, Bd, dY, lddy, in_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, workspace,
+  PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g1, b.Cs32, b.Ds32, c8, Ac, Bd, error_word(workspace),
+                                       c8 != nullptr, sms, st));
+  return backward_products(Ac, Bd, dY, lddy, in_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace,
                            sms, st);
 }
 
@@ -790,12 +822,22 @@ pj_status proj_gemm_backward_saved(const void* fwd_workspace, size_t fwd_ws_byte
   if (K == 0) return PJ_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int sms = 0;
-  PJ_TRY(begin_call(workspace, st, &sms));
-  if (M == 0 || N == 0) return backward_zero(dA, ldda, dB, lddb, g, out_dtype, st);
-  PJ_TRY(stage_basis(basis, g.lp1, workspace, st));
+  if (M == 0 || N == 0) {
+    PJ_TRY(begin_call(workspace, st, &sms));
+    return backward_zero(dA, ldda, dB, lddb, g, out_dtype, st);
+  }
+  Coef8 c8v;
+  const Coef8* c8 =
+      bwd_fused(g, prec->compute, ldda, lddb, out_dtype) && coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
+  if (c8) {   // no kernel runs before the products, whose waits read the error word
+    PJ_TRY(begin_call(workspace, st, &sms));
+  } else {
+    PJ_TRY(device_sms(&sms));
+    PJ_TRY(stage_basis(basis, g.lp1, workspace, st, nullptr, 0, true));
+  }
   const void* fws = fwd_workspace;
   return backward_products(static_cast<const char*>(fws) + fw.off_ac, static_cast<const char*>(fws) + fw.off_bd, dY,
-                           lddy, dy_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, workspace, sms, st);
+                           lddy, dy_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace, sms, st);
 }
 
 // ------------------------------------------------------------------ CONV --
@@ -861,13 +903,15 @@ pj_status proj_conv_project(const void* signal, int64_t S, const void* templates
                                     error_word(workspace), st));
     return PJ_OK;
   }
-  // General basis: the kept columns of C (signal) and rows of D (templates) first.
-  PJ_CUDA_TRY(cudaMemsetAsync(workspace, 0, sizeof(int), st));
-  PJ_TRY(stage_basis(basis, g.lp1, workspace, st));
+  // General basis: the kept columns of C (signal) and rows of D (templates), as
+  // arguments or staged first.
+  Coef8 c8v;
+  const Coef8* c8 = coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
+  if (!c8) PJ_TRY(stage_basis(basis, g.lp1, workspace, st, nullptr, 0, true));
   BasisDev b = basis_area(workspace);
   PJ_CUDA_TRY(launch_conv_project(static_cast<const float*>(signal), static_cast<const float*>(templates), g,
                                   at<uint16_t>(workspace, w.off_g), at<uint16_t>(workspace, w.off_tp),
-                                  error_word(workspace), st, b.Cs32, b.Ds32));
+                                  error_word(workspace), st, b.Cs32, b.Ds32, c8));
   return PJ_OK;
 }
 

@@ -4,6 +4,7 @@
 // next ones for an FP8 tier of truncated projections) in FP64 and FP32 for the
 // projection kernels.
 #include "common.hpp"
+#include "pdl.cuh"
 #include "tc.cuh"
 
 namespace pj {
@@ -24,13 +25,17 @@ __device__ double haar_raw(int L, int i, int j) {
 }
 
 __global__ void __launch_bounds__(kBasisThreads) basis_kernel(int kind, int L, int lp1, int p0, BasisDev b,
-                                                               int* err) {
+                                                               int* err, int clear) {
   __shared__ int s_fail;
   __shared__ int s_piv;
   const int tid = threadIdx.x, nth = blockDim.x;
   double* C = b.C64;
   double* D = b.D64;
-  if (tid == 0) s_fail = 0;
+  pdl_begin();
+  if (tid == 0) {
+    s_fail = 0;
+    if (clear) *err = 0;
+  }
   if (kind == PJ_BASIS_DCT2 || kind == PJ_BASIS_HAAR) {
     // Unit-length columns: the truncated product does not depend on column
     // scaling, and with orthogonal columns it makes D = C^T.  The squared
@@ -133,9 +138,37 @@ __global__ void __launch_bounds__(kBasisThreads) basis_kernel(int kind, int L, i
 
 }  // namespace
 
-cudaError_t launch_basis_build(int kind, int L, int lp1, BasisDev b, int* err, cudaStream_t st, int p0) {
-  basis_kernel<<<1, kBasisThreads, 0, st>>>(kind, L, lp1, p0, b, err);
-  return cudaGetLastError();
+cudaError_t launch_basis_build(int kind, int L, int lp1, BasisDev b, int* err, cudaStream_t st, int p0,
+                               bool clear) {
+  return launch_plain(basis_kernel, dim3(1), kBasisThreads, 0, st, kind, L, lp1, p0, b, err, clear ? 1 : 0);
+}
+
+bool coef8(const pj_basis* basis, int lp1, int p0, Coef8* out) {
+  if (basis->L != 8 || basis->kind == PJ_BASIS_USER) return false;
+  // cos(k pi / 16), k = 0 .. 8; cos(m pi / 16) follows from the cosine's symmetries.
+  static const double kCos[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                                 0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                                 0.19509032201612826785, 0.0};
+  const double r8 = 0.5 * kCos[4];   // 1 / sqrt(8)
+  for (int q = 0; q < 8; ++q)
+    for (int i = 0; i < 8; ++i) {
+      const int j = p0 + q;
+      double v = 0.0;
+      if (q < lp1 && j < 8) {
+        if (basis->kind == PJ_BASIS_DCT2) {   // cos(pi (2 i + 1) j / 16), columns of unit length
+          int m = (2 * i + 1) * j % 32;
+          if (m > 16) m = 32 - m;
+          v = (m <= 8 ? kCos[m] : -kCos[16 - m]) * (j == 0 ? r8 : 0.5);
+        } else {   // Haar: +-1 on a support of 8 >> level samples, columns of unit length
+          const int level = j == 0 ? 0 : (j >= 4 ? 2 : (j >= 2 ? 1 : 0));
+          const int width = 8 >> level, start = j == 0 ? 0 : (j - (1 << level)) * width;
+          const double h = level == 0 ? r8 : (level == 1 ? 0.5 : kCos[4]);
+          if (i >= start && i < start + width) v = (j == 0 || i < start + width / 2) ? h : -h;
+        }
+      }
+      out->c[q * 8 + i] = static_cast<float>(v);
+    }
+  return true;
 }
 
 }  // namespace pj

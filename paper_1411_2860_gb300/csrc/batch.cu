@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "common.hpp"
+#include "pdl.cuh"
 #include "mx.cuh"
 #include "tc.cuh"
 
@@ -66,6 +67,7 @@ __device__ __forceinline__ float from_bf16(uint16_t b) { return __uint_as_float(
 // with the split, Qlo[u] = bf16(b - Q[u]).
 __global__ void __launch_bounds__(256) batch_signal_kernel(const SigJob* __restrict__ jobs,
                                                            const int* __restrict__ job_of) {
+  pdl_begin();
   const SigJob& J = jobs[job_of[blockIdx.x]];
   const int64_t u = (static_cast<int64_t>(blockIdx.x) - J.block0) * blockDim.x + threadIdx.x;
   if (u >= J.n) return;
@@ -84,6 +86,7 @@ __global__ void __launch_bounds__(256) batch_signal_kernel(const SigJob* __restr
 // with the split, Kt[p][Kpad + j] = bf16(kb[j - p] - Kt[p][j]).
 __global__ void __launch_bounds__(256) batch_toeplitz_kernel(const TplJob* __restrict__ jobs,
                                                              const int* __restrict__ job_of) {
+  pdl_begin();
   const TplJob& J = jobs[job_of[blockIdx.x]];
   const int64_t e = (static_cast<int64_t>(blockIdx.x) - J.block0) * blockDim.x + threadIdx.x;
   if (e >= 128 * J.Kpad) return;
@@ -123,6 +126,7 @@ struct SfExpJob {
 
 __global__ void __launch_bounds__(256) batch_sigquant_kernel(const SigQJob* __restrict__ jobs,
                                                              const int* __restrict__ job_of) {
+  pdl_begin();
   const SigQJob& J = jobs[job_of[blockIdx.x]];
   const int64_t blk = (static_cast<int64_t>(blockIdx.x) - J.block0) * blockDim.x + threadIdx.x;
   if (blk >= J.nblk) return;
@@ -156,6 +160,7 @@ __global__ void __launch_bounds__(256) batch_sigquant_kernel(const SigQJob* __re
 
 __global__ void __launch_bounds__(256) batch_sfexpand_kernel(const SfExpJob* __restrict__ jobs,
                                                              const int* __restrict__ job_of) {
+  pdl_begin();
   const SfExpJob& J = jobs[job_of[blockIdx.x]];
   const int64_t e = (static_cast<int64_t>(blockIdx.x) - J.block0) * blockDim.x + threadIdx.x;
   if (e >= J.total) return;
@@ -177,6 +182,7 @@ struct ZeroJob {
 
 __global__ void __launch_bounds__(256) batch_zero_kernel(const ZeroJob* __restrict__ jobs,
                                                          const int* __restrict__ job_of) {
+  pdl_begin();
   const ZeroJob& J = jobs[job_of[blockIdx.x]];
   const int64_t r0 = (static_cast<int64_t>(blockIdx.x) - J.block0) * 4;
   for (int64_t r = r0; r < r0 + 4 && r < J.rows; ++r)
@@ -1086,26 +1092,21 @@ pj_status proj_batch_run(const pj_batch_plan* plan, void* stream) {
     PJ_CUDA_TRY(launch_project_cols_jobs(cls, plan->d_cols[cls], plan->cols_of[cls], plan->cols_blocks[cls], st));
   }
   if (plan->sig_blocks > 0) {
-    batch_signal_kernel<<<static_cast<unsigned>(plan->sig_blocks), 256, 0, st>>>(plan->d_sig, plan->sig_of);
-    PJ_CUDA_TRY(cudaGetLastError());
+    PJ_CUDA_TRY(launch_plain(batch_signal_kernel, dim3(static_cast<unsigned>(plan->sig_blocks)), 256, 0, st, plan->d_sig, plan->sig_of));
   }
   if (plan->tpl_blocks > 0) {
-    batch_toeplitz_kernel<<<static_cast<unsigned>(plan->tpl_blocks), 256, 0, st>>>(plan->d_tpl, plan->tpl_of);
-    PJ_CUDA_TRY(cudaGetLastError());
+    PJ_CUDA_TRY(launch_plain(batch_toeplitz_kernel, dim3(static_cast<unsigned>(plan->tpl_blocks)), 256, 0, st, plan->d_tpl, plan->tpl_of));
   }
   if (plan->sigq_blocks > 0) {   // after the signal kernel: its hi + lo sequences
-    batch_sigquant_kernel<<<static_cast<unsigned>(plan->sigq_blocks), 256, 0, st>>>(plan->d_sigq, plan->sigq_of);
-    PJ_CUDA_TRY(cudaGetLastError());
+    PJ_CUDA_TRY(launch_plain(batch_sigquant_kernel, dim3(static_cast<unsigned>(plan->sigq_blocks)), 256, 0, st, plan->d_sigq, plan->sigq_of));
   }
   if (plan->sfx_blocks > 0) {    // after the block scales
-    batch_sfexpand_kernel<<<static_cast<unsigned>(plan->sfx_blocks), 256, 0, st>>>(plan->d_sfx, plan->sfx_of);
-    PJ_CUDA_TRY(cudaGetLastError());
+    PJ_CUDA_TRY(launch_plain(batch_sfexpand_kernel, dim3(static_cast<unsigned>(plan->sfx_blocks)), 256, 0, st, plan->d_sfx, plan->sfx_of));
   }
   if (plan->qsides_blocks > 0)
     PJ_CUDA_TRY(launch_quantize_mx_jobs(plan->d_qsides, plan->qsides_of, plan->qsides_blocks, st));
   if (plan->zero_blocks > 0) {
-    batch_zero_kernel<<<static_cast<unsigned>(plan->zero_blocks), 256, 0, st>>>(plan->d_zero, plan->zero_of);
-    PJ_CUDA_TRY(cudaGetLastError());
+    PJ_CUDA_TRY(launch_plain(batch_zero_kernel, dim3(static_cast<unsigned>(plan->zero_blocks)), 256, 0, st, plan->d_zero, plan->zero_of));
   }
   PJ_CUDA_TRY(launch_gemm_tc_grouped(plan->d_insts, plan->d_tiles, plan->d_cta_off, plan->ctas, plan->paired,
                                      error_word(plan->ws), st));

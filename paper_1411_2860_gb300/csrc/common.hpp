@@ -48,7 +48,16 @@ pj_status begin_call(void* ws, cudaStream_t st, int* sms);
 // The basis tables for l+1 = lp1 built into the workspace's basis area on `st`
 // (`area`: the basis area of a sub-workspace starting there, NULL = ws; p0: the
 // first projection kept).
-pj_status stage_basis(const pj_basis* basis, int lp1, void* ws, cudaStream_t st, void* area = nullptr, int p0 = 0);
+// clear: the basis kernel also clears the workspace's error word (in place of begin_call).
+pj_status stage_basis(const pj_basis* basis, int lp1, void* ws, cudaStream_t st, void* area = nullptr, int p0 = 0,
+                      bool clear = false);
+// The kept vectors of a built-in basis with groups of L = 8, passed to the kernels as
+// arguments: c[q * 8 + t] is element t of projection p0 + q (both sides: the columns
+// are orthonormal, so D = C^T).  False for other bases, which go through stage_basis.
+struct Coef8 {
+  float c[64];
+};
+bool coef8(const pj_basis* basis, int lp1, int p0, Coef8* out);
 pj_status gemm_geom(int64_t M, int64_t N, int64_t K, int64_t block_k, int64_t R, const pj_basis* basis,
                     const pj_precision* prec, GemmGeom* g);
 pj_status conv_geom(int64_t S, int64_t T, int64_t nt, int64_t block, int64_t R, const pj_basis* basis,
@@ -97,7 +106,9 @@ inline int* error_word(void* ws) { return static_cast<int*>(ws); }
 
 // basis.cu: build C, D (FP64) and the kept tables of the lp1 projections from p0
 // on into `b` (for PJ_BASIS_USER the matrix must already sit in b.U64).
-cudaError_t launch_basis_build(int kind, int L, int lp1, BasisDev b, int* err, cudaStream_t st, int p0 = 0);
+// clear: *err is cleared first.
+cudaError_t launch_basis_build(int kind, int L, int lp1, BasisDev b, int* err, cudaStream_t st, int p0 = 0,
+                               bool clear = false);
 
 // project.cu ------------------------------------------------------------
 // Rows of A (M x K, pitch lda, dtype in) -> A_c (M x pitch BF16) and columns
@@ -129,18 +140,17 @@ inline int64_t gemm_pitch(const GemmGeom& g) {
 // Projections of A's rows and B's columns to BF16 (either operand may be
 // NULL): one TMA-staged persistent launch (project_tma.cu) for the operands
 // whose layout suits TMA when L = 8, the per-group kernels of project.cu
-// otherwise.
+// otherwise.  c8 (NULL: the tables Cs and Ds): the kept vectors as arguments.
+// clear: the first kernel launched clears *err (its waits do not read it, and no
+// kernel of the call runs before it), so a call with a built-in basis starts with
+// its projection: no memset and no basis launch before it.
 cudaError_t launch_project_pair_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
-                                     const GemmGeom& g, const float* Cs, const float* Ds, uint16_t* Ac,
-                                     uint16_t* Bd, int* err, int sms, cudaStream_t st);
-cudaError_t launch_project_rows_bf16(const void* A, int64_t lda, int in_dtype, const GemmGeom& g, const float* Cs,
-                                     uint16_t* Ac, int* err, int sms, cudaStream_t st);
-cudaError_t launch_project_cols_bf16(const void* B, int64_t ldb, int in_dtype, const GemmGeom& g, const float* Ds,
-                                     uint16_t* Bd, int* err, int sms, cudaStream_t st);
-cudaError_t launch_project_rows_simt(const void* A, int64_t lda, int in_dtype, const GemmGeom& g, const float* Cs,
-                                     uint16_t* Ac, cudaStream_t st);
-cudaError_t launch_project_cols_simt(const void* B, int64_t ldb, int in_dtype, const GemmGeom& g, const float* Ds,
-                                     uint16_t* Bd, cudaStream_t st);
+                                     const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
+                                     uint16_t* Ac, uint16_t* Bd, int* err, bool clear, int sms, cudaStream_t st);
+// The per-group kernels (either operand may be NULL).
+cudaError_t launch_project_pair_simt(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
+                                     const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
+                                     uint16_t* Ac, uint16_t* Bd, int* clear_err, cudaStream_t st);
 
 // Where one operand's E4M3 components and block scales go (gemm_mx.cu, mx.cuh).
 struct MxQuantSide {
@@ -287,11 +297,10 @@ constexpr int kProjectionClasses = 4;
 // job_of[b] = the job of block b (blocks of job j are [block0_j, block0_{j+1})).
 cudaError_t launch_project_rows_jobs(int cls, const RowsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st);
 cudaError_t launch_project_cols_jobs(int cls, const ColsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st);
-// FP64 path: A_c (M x Kp, pitch Kp) and B_d (Kp x N, pitch N), both double.
-cudaError_t launch_project_rows_f64(const double* A, int64_t lda, const GemmGeom& g, const double* Cs, double* Ac,
-                                    cudaStream_t st);
-cudaError_t launch_project_cols_f64(const double* B, int64_t ldb, const GemmGeom& g, const double* Ds, double* Bd,
-                                    cudaStream_t st);
+// FP64 path: A_c (M x Kp, pitch Kp) and B_d (Kp x N, pitch N), both double, in one
+// launch (A or B may be NULL).
+cudaError_t launch_project_pair_f64(const double* A, int64_t lda, const double* B, int64_t ldb, const GemmGeom& g,
+                                    const double* Cs, const double* Ds, double* Ac, double* Bd, cudaStream_t st);
 
 // gemm_f64.cu: Y = Ac (M x Kp) * Bd (Kp x N) in double.
 cudaError_t launch_gemm_f64(const double* Ac, const double* Bd, double* Y, int64_t ldy, int64_t M, int64_t N,
@@ -316,11 +325,12 @@ struct ExpandArgs {
   int64_t K = 0;
   void* out = nullptr;
   int64_t ld = 0;
-  const float* coef = nullptr;
+  const float* coef = nullptr;   // NULL: the kept vectors are kernel arguments (GemmTcArgs::ex_c8)
 };
 
 struct GemmTcArgs {
   ExpandArgs ex;   // expansion in the epilogue (mode 0: Y is written as it is)
+  const Coef8* ex_c8 = nullptr;   // its vectors, when ex.coef is NULL
   const uint16_t* Q;
   int64_t ldq, rowsQ;
   const uint16_t* P;
@@ -463,9 +473,9 @@ cudaError_t launch_quantize_mx(const MxQuantSide* a, const MxQuantSide* b, cudaS
 // others to BF16 and quantises them (launch_quantize_mx).
 bool project_mx_fusable(const GemmGeom& g, int side);
 cudaError_t launch_project_pair_mx(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
-                                   const GemmGeom& g, const float* Cs, const float* Ds, const MxQuantSide* qa,
-                                   const MxQuantSide* qb, int* err, int sms, cudaStream_t st, bool* a_done,
-                                   bool* b_done);
+                                   const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
+                                   const MxQuantSide* qa, const MxQuantSide* qb, int* err, bool clear, int sms,
+                                   cudaStream_t st, bool* a_done, bool* b_done);
 // Batched: sides in device memory, job_of[block] = side of that block.
 int64_t mx_side_blocks(const MxQuantSide& a);
 cudaError_t launch_quantize_mx_jobs(const MxQuantSide* sides, const int* job_of, int64_t blocks, cudaStream_t st);
@@ -551,11 +561,12 @@ struct ConvGeom {
 };
 
 // Projected signal copies G and (k != NULL) template pairs TP in one launch.  The
-// box path also clears the error word *err; the general path reads the kept basis
-// tables Cs (L x lp1) and Ds (lp1 x L) and leaves *err alone (the caller clears it
-// before the basis is built).
+// box path also clears the error word *err, and so does the general path with c8 (the
+// kept vectors as arguments); without c8 it reads the kept basis tables Cs (L x lp1)
+// and Ds (lp1 x L) and leaves *err alone (the caller clears it when the basis is built).
 cudaError_t launch_conv_project(const float* s, const float* k, const ConvGeom& g, uint16_t* G, uint16_t* TP,
-                                int* err, cudaStream_t st, const float* Cs = nullptr, const float* Ds = nullptr);
+                                int* err, cudaStream_t st, const float* Cs = nullptr, const float* Ds = nullptr,
+                                const Coef8* c8 = nullptr);
 // pstep > 1: only the lags that are multiples of pstep (pstep divides Lb).
 cudaError_t launch_conv_tc(const uint16_t* G, const uint16_t* TP, float* out, const ConvGeom& g, int* err,
                            int num_sms, cudaStream_t st, int pstep = 1);

@@ -31,6 +31,7 @@
 // TMEM holds two 128 x 256 FP32 accumulators so the epilogue of one tile
 // overlaps the main loop of the next.
 #include "common.hpp"
+#include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
 
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_begin();
   const int nchunks = p.Kc + 1;
 
   if (warp == 0) {
@@ -431,10 +433,8 @@ cudaError_t launch_conv_tc(const uint16_t* G, const uint16_t* TP, float* out, co
   }
   const int grid = p.num_tiles < num_sms ? p.num_tiles : num_sms;
   if (nepi == 2)
-    conv_tc_kernel<2><<<grid, conv_threads<2>(), kSmemBytes, st>>>(p);
-  else
-    conv_tc_kernel<1><<<grid, conv_threads<1>(), kSmemBytes, st>>>(p);
-  return cudaGetLastError();
+    return launch_pdl(conv_tc_kernel<2>, dim3(static_cast<unsigned>(grid)), conv_threads<2>(), kSmemBytes, st, 1, p);
+  return launch_pdl(conv_tc_kernel<1>, dim3(static_cast<unsigned>(grid)), conv_threads<1>(), kSmemBytes, st, 1, p);
 }
 
 // Lags between computed ones (every step-th lag): linear interpolation of the
@@ -444,6 +444,7 @@ cudaError_t launch_conv_tc(const uint16_t* G, const uint16_t* TP, float* out, co
 // fills 32 / lpr missing lags.
 __global__ void __launch_bounds__(256) conv_interp_kernel(float* __restrict__ out, int64_t lags, int nt, int step,
                                                           int64_t rows, int lpr) {
+  pdl_begin();
   const int64_t gt = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t q = gt / lpr;
   const int lane = static_cast<int>(gt - q * lpr);
@@ -479,9 +480,8 @@ cudaError_t launch_conv_interp(float* out, const ConvGeom& g, int step, cudaStre
   const int64_t per_row = g.nt % 4 == 0 ? g.nt / 4 : g.nt;
   int lpr = 1;
   while (lpr < 32 && lpr < per_row) lpr *= 2;
-  conv_interp_kernel<<<static_cast<unsigned>(ceil_div(rows * lpr, 256)), 256, 0, st>>>(
-      out, g.lags, static_cast<int>(g.nt), step, rows, lpr);
-  return cudaGetLastError();
+  return launch_plain(conv_interp_kernel, dim3(static_cast<unsigned>(ceil_div(rows * lpr, 256))), 256, 0, st, out,
+                    g.lags, static_cast<int>(g.nt), step, rows, lpr);
 }
 
 }  // namespace pj

@@ -28,6 +28,7 @@
 
 #include "common.hpp"
 #include "gemm_epi.cuh"
+#include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
 #if PJ_CTA_PAIRS
@@ -58,6 +59,7 @@ static_assert(kCSmemBytes + 64 * sizeof(float) <= 232448, "shared memory per blo
 struct Cg2Params {
   GemmInst I;       // P map box {CK, CM} (MN-major: {64, CK}); Q map box {CK, bn/2} (MN-major: {64, CK})
   ExpandArgs ex;
+  Coef8 ex_c8;      // the expansion's vectors when ex.coef is null
   int npp;          // pair columns: P tile columns of 256
   int num_pairs;    // npp x Q tile rows
   int stall;        // failure-detection self-test: the producers stop after this many stages (-1: never)
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
   const uint32_t tmem = *tslot;
   const uint32_t full_leader = mapa_shared(smem_u32(full), 0);
   const uint32_t acc_empty_leader = mapa_shared(smem_u32(acc_empty), 0);
+  pdl_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -278,7 +281,8 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
     const int nbuf = static_cast<int>(kCStageOut / chunk_bytes);
     int sbuf = 0;
     if (ex.mode)
-      for (int e = threadIdx.x - 64; e < 8 * ex.lp1; e += 256) s_coef[e] = ex.coef[e];
+      for (int e = threadIdx.x - 64; e < 8 * ex.lp1; e += 256)
+        s_coef[e] = ex.coef ? ex.coef[e] : p.ex_c8.c[expand_c8_index(ex, e)];
     named_barrier(1, 256);
     for (int n = 0, it = 0;; ++n, ++it) {
       const int pi = static_cast<int>(blockIdx.x / 2) + n * static_cast<int>(gridDim.x / 2);
@@ -417,20 +421,9 @@ static cudaError_t launch_cg2(Cg2Params& p, bool mn, int num_sms, cudaStream_t s
   cudaError_t e = set_cg2_smem_attr();
   if (e != cudaSuccess) return e;
   const int slots = num_sms / 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(2 * (p.num_pairs < slots ? p.num_pairs : slots)));
-  cfg.blockDim = dim3(kCThreads);
-  cfg.dynamicSmemBytes = kCSmemBytes;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (mn) return cudaLaunchKernelEx(&cfg, gemm_cg2_kernel<true>, p);
-  return cudaLaunchKernelEx(&cfg, gemm_cg2_kernel<false>, p);
+  return launch_pdl(mn ? gemm_cg2_kernel<true> : gemm_cg2_kernel<false>,
+                    dim3(static_cast<unsigned>(2 * (p.num_pairs < slots ? p.num_pairs : slots))), kCThreads, kCSmemBytes,
+                    st, 2, p);
 }
 
 cudaError_t launch_gemm_cg2(const GemmTcArgs& a_in, int* err, int num_sms, cudaStream_t st) {
@@ -445,6 +438,7 @@ cudaError_t launch_gemm_cg2(const GemmTcArgs& a_in, int* err, int num_sms, cudaS
   p.stall = a.stall_stage;
   p.err = err;
   p.ex = a.ex;
+  if (a.ex_c8) p.ex_c8 = *a.ex_c8;
   return launch_cg2(p, a.mnP || a.mnQ, num_sms, st);
 }
 

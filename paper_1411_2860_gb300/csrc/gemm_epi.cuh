@@ -13,6 +13,12 @@
 namespace pj {
 namespace {
 
+// Where entry e of the expansion's coefficient table (Cs: t (l+1) + p for mode 1, Ds:
+// p 8 + t for mode 2) sits in a Coef8.
+__device__ __forceinline__ int expand_c8_index(const ExpandArgs& ex, int e) {
+  return ex.mode == 1 ? (e % ex.lp1) * 8 + e / ex.lp1 : e;
+}
+
 template <bool kBF16>
 __device__ __forceinline__ void store_run(void* out, int64_t off, const float (&y)[8], int n, int per) {
   if (kBF16) {

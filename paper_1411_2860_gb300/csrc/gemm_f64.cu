@@ -1,6 +1,7 @@
 // Reduced product in double precision on CUDA cores (the FP64 correctness
 // path): Y = A_c B_d with A_c M x Kp and B_d Kp x N, both row-major.
 #include "common.hpp"
+#include "pdl.cuh"
 
 namespace pj {
 namespace {
@@ -19,6 +20,7 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(const double* __restrict_
   __shared__ double sB[TILE][TILE + 1];
   const int tx = threadIdx.x % TILE, ty = threadIdx.x / TILE;
   const int64_t i0 = static_cast<int64_t>(blockIdx.y) * TILE, j0 = static_cast<int64_t>(blockIdx.x) * TILE;
+  pdl_begin();
   double acc[PER];
 #pragma unroll
   for (int r = 0; r < PER; ++r) acc[r] = 0.0;
@@ -54,12 +56,11 @@ cudaError_t launch_gemm_f64(const double* Ac, const double* Bd, double* Y, int64
   if (device_sms(&sms) != PJ_OK) sms = 152;
   if (ceil_div(M, 32) * ceil_div(N, 32) < 2 * sms) {
     dim3 grid(static_cast<unsigned>(ceil_div(N, 16)), static_cast<unsigned>(ceil_div(M, 16)));
-    gemm_f64_kernel<16><<<grid, 256, 0, st>>>(Ac, Bd, Y, ldy, M, N, Kp);
+    return launch_plain(gemm_f64_kernel<16>, grid, 256, 0, st, Ac, Bd, Y, ldy, M, N, Kp);
   } else {
     dim3 grid(static_cast<unsigned>(ceil_div(N, 32)), static_cast<unsigned>(ceil_div(M, 32)));
-    gemm_f64_kernel<32><<<grid, 256, 0, st>>>(Ac, Bd, Y, ldy, M, N, Kp);
+    return launch_plain(gemm_f64_kernel<32>, grid, 256, 0, st, Ac, Bd, Y, ldy, M, N, Kp);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace pj

@@ -44,6 +44,7 @@
 
 #include "common.hpp"
 #include "mx.cuh"
+#include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
 #if PJ_CTA_PAIRS
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
   if (kPair) cluster_sync_all();  // the peer's barriers exist before any copy or commit reaches them
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -513,6 +515,7 @@ __device__ __forceinline__ void quantize_unit(const MxQuantSide& a, int64_t u) {
 
 __global__ void __launch_bounds__(256) quantize_mx_kernel(const MxQuantSide s0, const MxQuantSide s1, int64_t n0,
                                                           int64_t total) {
+  pdl_begin();
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= total) return;
   if (t < n0)
@@ -524,6 +527,7 @@ __global__ void __launch_bounds__(256) quantize_mx_kernel(const MxQuantSide s0, 
 // Batched form: block b belongs to side job_of[b], whose units start at block block0.
 __global__ void __launch_bounds__(256) quantize_mx_jobs_kernel(const MxQuantSide* __restrict__ sides,
                                                                const int* __restrict__ job_of) {
+  pdl_begin();
   const MxQuantSide& a = sides[job_of[blockIdx.x]];
   const int64_t u = (static_cast<int64_t>(blockIdx.x) - a.block0) * blockDim.x + threadIdx.x;
   if (u < a.tiles * a.tile_rows * (a.Kq_pad / 32)) quantize_unit(a, u);
@@ -577,8 +581,7 @@ int64_t mx_side_blocks(const MxQuantSide& a) { return ceil_div(a.tiles * a.tile_
 
 cudaError_t launch_quantize_mx_jobs(const MxQuantSide* sides, const int* job_of, int64_t blocks, cudaStream_t st) {
   if (blocks == 0) return cudaSuccess;
-  quantize_mx_jobs_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(sides, job_of);
-  return cudaGetLastError();
+  return launch_plain(quantize_mx_jobs_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, st, sides, job_of);
 }
 
 cudaError_t launch_quantize_mx(const MxQuantSide* a, const MxQuantSide* b, cudaStream_t st) {
@@ -589,8 +592,8 @@ cudaError_t launch_quantize_mx(const MxQuantSide* a, const MxQuantSide* b, cudaS
   const int64_t n1 = (a && b) ? s1.tiles * s1.tile_rows * (s1.Kq_pad / 32) : 0;
   const int64_t total = n0 + n1;
   if (total == 0) return cudaSuccess;
-  quantize_mx_kernel<<<static_cast<unsigned>(ceil_div(total, 256)), 256, 0, st>>>(s0, s1, n0, total);
-  return cudaGetLastError();
+  return launch_plain(quantize_mx_kernel, dim3(static_cast<unsigned>(ceil_div(total, 256))), 256, 0, st, s0, s1, n0,
+                    total);
 }
 
 bool build_mx_inst(const MxGemmArgs& a, MxInst* I) {
@@ -702,23 +705,11 @@ cudaError_t launch_gemm_mx(const MxGemmArgs& a_in, int* err, int num_sms, cudaSt
 #if PJ_CTA_PAIRS
   if (a.pair) {
     const int pairs = p.num_tiles / 2, slots = num_sms / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs < slots ? pairs : slots)));
-    cfg.blockDim = dim3(kXThreads);
-    cfg.dynamicSmemBytes = kXSmemBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_mx_kernel<true>, p);
+    return launch_pdl(gemm_mx_kernel<true>, dim3(static_cast<unsigned>(2 * (pairs < slots ? pairs : slots))), kXThreads,
+                      kXSmemBytes, st, 2, p);
   }
 #endif
-  gemm_mx_kernel<false><<<grid, kXThreads, kXSmemBytes, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(gemm_mx_kernel<false>, dim3(static_cast<unsigned>(grid)), kXThreads, kXSmemBytes, st, 1, p);
 }
 
 cudaError_t launch_gemm_mx_grouped(const MxInst* insts, const GemmTile* tiles, const int* cta_off, int ctas,
@@ -735,8 +726,7 @@ cudaError_t launch_gemm_mx_grouped(const MxInst* insts, const GemmTile* tiles, c
   p.err = err;
   cudaError_t e = set_mx_smem_attr();
   if (e != cudaSuccess) return e;
-  gemm_mx_kernel<false><<<ctas, kXThreads, kXSmemBytes, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(gemm_mx_kernel<false>, dim3(static_cast<unsigned>(ctas)), kXThreads, kXSmemBytes, st, 1, p);
 }
 
 }  // namespace pj

@@ -31,6 +31,7 @@
 
 #include "common.hpp"
 #include "gemm_epi.cuh"
+#include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
 #if PJ_CTA_PAIRS
@@ -60,6 +61,7 @@ struct GemmParams {
   int stall;                 // failure-detection self-test: the producer stops after this many stages (-1: never)
   int* err;
   ExpandArgs ex;             // single instance: expansion to samples in the epilogue (mode 0: none)
+  Coef8 ex_c8;               // its vectors when ex.coef is null
 };
 
 // The n-th tile of this CTA: instance, coordinates and K-stage range; false past the last.
@@ -163,6 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   if (kPair) cluster_sync_all();  // the peer's barriers exist before any copy or commit reaches them
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -354,7 +357,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     const ExpandArgs ex = p.ex;
     if (ex.mode) {
       const int ncoef = 8 * ex.lp1;
-      for (int e = threadIdx.x - 64; e < ncoef; e += 128) s_coef[e] = ex.coef[e];
+      for (int e = threadIdx.x - 64; e < ncoef; e += 128)
+        s_coef[e] = ex.coef ? ex.coef[e] : p.ex_c8.c[expand_c8_index(ex, e)];
       named_barrier(1, 128);
     }
     int it = 0;
@@ -597,6 +601,7 @@ cudaError_t launch_gemm_tc_generic(const GemmTcArgs& a_in, int* err, int num_sms
   p.err = err;
   p.stall = a.stall_stage;
   p.ex = a.ex;
+  p.ex_c8 = a.ex_c8 ? *a.ex_c8 : Coef8{};
   cudaError_t e = set_smem_attr();
   if (e != cudaSuccess) return e;
   int grid = p.num_tiles < num_sms ? p.num_tiles : num_sms;
@@ -610,27 +615,12 @@ cudaError_t launch_gemm_tc_generic(const GemmTcArgs& a_in, int* err, int num_sms
 #if PJ_CTA_PAIRS
   if (a.pair) {
     const int pairs = p.num_tiles / 2, slots = num_sms / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs < slots ? pairs : slots)));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (a.mnQ || a.mnP) return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true, true>, p);
-    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<false, true>, p);
+    return launch_pdl(a.mnQ || a.mnP ? gemm_tc_kernel<true, true> : gemm_tc_kernel<false, true>,
+                      dim3(static_cast<unsigned>(2 * (pairs < slots ? pairs : slots))), kThreads, kSmemBytes, st, 2, p);
   }
 #endif
-  if (a.mnP || a.mnQ)
-    gemm_tc_kernel<true, false><<<grid, kThreads, kSmemBytes, st>>>(p);
-  else
-    gemm_tc_kernel<false, false><<<grid, kThreads, kSmemBytes, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(a.mnP || a.mnQ ? gemm_tc_kernel<true, false> : gemm_tc_kernel<false, false>,
+                    dim3(static_cast<unsigned>(grid)), kThreads, kSmemBytes, st, 1, p);
 }
 
 cudaError_t launch_gemm_tc_grouped(const GemmInst* insts, const GemmTile* tiles, const int* cta_off, int ctas,
@@ -646,29 +636,18 @@ cudaError_t launch_gemm_tc_grouped(const GemmInst* insts, const GemmTile* tiles,
   p.stall = -1;
   p.err = err;
   p.ex = ExpandArgs{};
+  p.ex_c8 = Coef8{};
   cudaError_t e = set_smem_attr();
   if (e != cudaSuccess) return e;
   if (pair) {  // CTAs 2c and 2c + 1 form a cluster; their tile lists are paired
 #if !PJ_CTA_PAIRS
     return cudaErrorNotSupported;   // a build without CTA pairs plans none
 #else
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(ctas));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<false, true>, p);
+    return launch_pdl(gemm_tc_kernel<false, true>, dim3(static_cast<unsigned>(ctas)), kThreads, kSmemBytes, st, 2, p);
 #endif
   }
-  gemm_tc_kernel<false, false><<<ctas, kThreads, kSmemBytes, st>>>(p);  // grouped instances are K-major
-  return cudaGetLastError();
+  // grouped instances are K-major
+  return launch_pdl(gemm_tc_kernel<false, false>, dim3(static_cast<unsigned>(ctas)), kThreads, kSmemBytes, st, 1, p);
 }
 
 cudaError_t launch_gemm_tc(const uint16_t* Ac, const uint16_t* Bd, void* Y, int64_t ldy, int out_dtype,

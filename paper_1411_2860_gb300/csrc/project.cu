@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 
 #include "common.hpp"
+#include "pdl.cuh"
 
 namespace pj {
 namespace {
@@ -166,7 +167,7 @@ __device__ __forceinline__ void stage_coef8(float* c, int lp1, At at) {
 // The thread of group 0 of a row also zeroes the row's padding columns.
 // Every thread of the block reaches the one __syncthreads.
 constexpr int kRowRun = 32;                         // groups per run (L = 8)
-constexpr int kRowUnits = 2;                        // runs per warp, loaded together
+constexpr int kRowUnits = 2;                        // runs per warp, loaded together (2 consecutive: <= 2 rows)
 constexpr int kRowBuf = 8 * kRowRun + 8;            // padded floats per run
 
 template <int LP1>
@@ -205,17 +206,24 @@ __device__ __forceinline__ void rows_span_odd(const RowsJob& J, const float (&x)
 
 // Warp units w0 .. w0 + kRowUnits - 1 (each a run of one row): all their loads are
 // issued before any arithmetic.
-template <typename InT>
+// kArg: the caller has staged the kept vectors in sC.
+template <typename InT, bool kArg>
 __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* sC, float* sX) {
   const int lane = threadIdx.x & 31;
   const int64_t nrun = (J.NG + kRowRun - 1) / kRowRun;
+  const int64_t units = J.M * nrun;
   const int lp1 = J.lp1;
+  // The row of the first run; the next run is the next one of the row or the first of
+  // the next row.  (A 64-bit division per run, twice, was more instructions than the
+  // projection itself.)
+  const int64_t i0 = units < (int64_t(1) << 32) ? static_cast<uint32_t>(w0) / static_cast<uint32_t>(nrun) : w0 / nrun;
+  const int64_t r0 = w0 - i0 * nrun;
+  auto row_of = [&](int v) { return i0 + (r0 + v >= nrun ? 1 : 0); };
   float* bufs = sX + (threadIdx.x >> 5) * (kRowUnits * kRowBuf);
 #pragma unroll
   for (int v = 0; v < kRowUnits; ++v) {
-    const int64_t w = w0 + v;
-    const bool live = w < J.M * nrun;
-    const int64_t i = live ? w / nrun : 0, run = live ? w - i * nrun : 0;
+    const bool live = w0 + v < units;
+    const int64_t i = live ? row_of(v) : 0, run = live ? w0 + v - i * nrun : 0;
     const InT* a = static_cast<const InT*>(J.A) + i * J.lda + run * (8 * kRowRun);
     const int64_t left = J.K - run * (8 * kRowRun);
     const int nk = static_cast<int>(left < 8 * kRowRun ? left : 8 * kRowRun);
@@ -226,14 +234,13 @@ __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* 
       buf[e + s] = live && e < nk ? load_as_float(a + e) : 0.0f;
     }
   }
-  stage_coef8(sC, lp1, [&](int t, int q) { return J.Cs[t * lp1 + q]; });
+  if (!kArg) stage_coef8(sC, lp1, [&](int t, int q) { return J.Cs[t * lp1 + q]; });
   __syncthreads();
   const bool odd_span = (lp1 == 3 || lp1 == 5 || lp1 == 6 || lp1 == 7) && !(J.nsplit > 1 && J.tl < lp1);
 #pragma unroll 1
   for (int v = 0; v < kRowUnits; ++v) {
-    const int64_t w = w0 + v;
-    if (w >= J.M * nrun) break;
-    const int64_t i = w / nrun, run = w - i * nrun;
+    if (w0 + v >= units) break;
+    const int64_t i = row_of(v), run = w0 + v - i * nrun;
     const int64_t gg = run * kRowRun + lane;
     if (odd_span) {   // the same for the whole warp
       float* fbuf = bufs + v * kRowBuf;
@@ -300,29 +307,45 @@ __device__ __forceinline__ void rows_body_any(const RowsJob& J, int64_t e, float
 
 // Thread t of block b handles unit b * 256 + t (LT = 0), or warp units
 // (b * 8 + t / 32) * kRowUnits onwards (LT = 8).
-template <typename InT, int LT>
+template <typename InT, int LT, bool kArg>
 __device__ __forceinline__ void rows_body(const RowsJob& J, int64_t b, float* sC, float* sX) {
   if (LT == 8)
-    rows_body8<InT>(J, (b * 8 + (threadIdx.x >> 5)) * kRowUnits, sC, sX);
+    rows_body8<InT, kArg>(J, (b * 8 + (threadIdx.x >> 5)) * kRowUnits, sC, sX);
   else
     rows_body_any<InT>(J, b * blockDim.x + threadIdx.x, sC);
 }
 
-template <typename InT, int LT>
-__global__ void __launch_bounds__(256) project_rows_kernel(const __grid_constant__ RowsJob J) {
-  __shared__ __align__(16) float sC[LT ? LT * LT : 64 * 64];
-  __shared__ float sX[LT == 8 ? 8 * kRowUnits * kRowBuf : 1];
-  rows_body<InT, LT>(J, blockIdx.x, sC, sX);
+// Arguments of a single operand's launch: the kept vectors (kArg; else they are in the
+// job's table) and the call's error word when this is the call's first kernel.
+struct SideArgs {
+  Coef8 c8;
+  int* clear;
+};
+
+template <bool kArg>
+__device__ __forceinline__ void side_begin(const SideArgs& a, float* sC) {
+  if (kArg && threadIdx.x < 64) sC[threadIdx.x] = a.c8.c[(threadIdx.x & 7) * 8 + (threadIdx.x >> 3)];   // [t * 8 + q]
+  pdl_begin();
+  if (a.clear && blockIdx.x == 0 && threadIdx.x == 0) *a.clear = 0;
 }
 
+template <typename InT, int LT, bool kArg>
+__global__ void __launch_bounds__(256) project_rows_kernel(const __grid_constant__ RowsJob J,
+                                                           const __grid_constant__ SideArgs a) {
+  __shared__ __align__(16) float sC[LT ? LT * LT : 64 * 64];
+  __shared__ float sX[LT == 8 ? 8 * kRowUnits * kRowBuf : 1];
+  side_begin<kArg>(a, sC);
+  rows_body<InT, LT, kArg>(J, blockIdx.x, sC, sX);
+}
 
 template <typename InT, int LT>
 __global__ void __launch_bounds__(256) project_rows_jobs_kernel(const RowsJob* __restrict__ jobs,
                                                                 const int* __restrict__ job_of) {
   __shared__ __align__(16) float sC[LT ? LT * LT : 64 * 64];
   __shared__ float sX[LT == 8 ? 8 * kRowUnits * kRowBuf : 1];
+  pdl_begin();
   const RowsJob& J = jobs[job_of[blockIdx.x]];
-  rows_body<InT, LT>(J, static_cast<int64_t>(blockIdx.x) - J.block0, sC, sX);
+  rows_body<InT, LT, false>(J, static_cast<int64_t>(blockIdx.x) - J.block0, sC, sX);
 }
 
 // ---- columns of B -> B_d stored transposed (N x pitch, K-major) -----------
@@ -411,7 +434,7 @@ __device__ __forceinline__ void col_group8(const ColsJob& J, uint16_t* row, int6
   if (J.nsplit > 1) store_split_part(row, gg, hi, lo, LP1, J.tl, J.Kp_pad, J.Kt_pad, StoreUpto8{});
 }
 
-template <typename InT, int LT>
+template <typename InT, int LT, bool kArg>
 __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t qd, float* sD, uint8_t* stage) {
   constexpr int LMAX = LT ? LT : 64;
   const int L = LT ? LT : J.L;
@@ -431,7 +454,8 @@ __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t q
       for (int t = 0; t < 8; ++t) xa[q * 8 + t] = t < n ? load_as_float(B + (k0 + t) * J.ldb + j) : 0.0f;
     }
   }
-  if (LT == 8)
+  if (kArg) {
+  } else if (LT == 8)
     stage_coef8(sD, lp1, [&](int t, int q) { return J.Ds[q * 8 + t]; });
   else
     for (int k = threadIdx.x; k < L * lp1; k += blockDim.x) sD[k] = J.Ds[k];
@@ -498,12 +522,14 @@ __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t q
   if (qd == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
 }
 
-template <typename InT, int LT>
-__global__ void __launch_bounds__(256, LT == 8 ? 3 : 2) project_cols_kernel(const __grid_constant__ ColsJob J) {
+template <typename InT, int LT, bool kArg>
+__global__ void __launch_bounds__(256, LT == 8 ? 3 : 2) project_cols_kernel(const __grid_constant__ ColsJob J,
+                                                                            const __grid_constant__ SideArgs a) {
   __shared__ __align__(16) float sD[LT ? LT * LT : 64 * 64];
   __shared__ __align__(16) uint8_t sStage[LT == 8 ? 8 * 4096 : 16];
-  const int64_t b = blockIdx.x;
-  cols_body<InT, LT>(J, (b % J.nbx) * blockDim.x + threadIdx.x, b / J.nbx, sD, sStage);
+  side_begin<kArg>(a, sD);
+  const uint32_t b = blockIdx.x, nbx = static_cast<uint32_t>(J.nbx);
+  cols_body<InT, LT, kArg>(J, static_cast<int64_t>(b % nbx) * blockDim.x + threadIdx.x, b / nbx, sD, sStage);
 }
 
 template <typename InT, int LT>
@@ -511,39 +537,50 @@ __global__ void __launch_bounds__(256, LT == 8 ? 3 : 2) project_cols_jobs_kernel
                                                                 const int* __restrict__ job_of) {
   __shared__ __align__(16) float sD[LT ? LT * LT : 64 * 64];
   __shared__ __align__(16) uint8_t sStage[LT == 8 ? 8 * 4096 : 16];
+  pdl_begin();
   const ColsJob& J = jobs[job_of[blockIdx.x]];
-  const int64_t b = static_cast<int64_t>(blockIdx.x) - J.block0;
-  cols_body<InT, LT>(J, (b % J.nbx) * blockDim.x + threadIdx.x, b / J.nbx, sD, sStage);
+  const uint32_t b = blockIdx.x - static_cast<uint32_t>(J.block0), nbx = static_cast<uint32_t>(J.nbx);
+  cols_body<InT, LT, false>(J, static_cast<int64_t>(b % nbx) * blockDim.x + threadIdx.x, b / nbx, sD, sStage);
 }
 
 // ---- FP64 path ------------------------------------------------------------
-__global__ void project_rows_f64_kernel(const double* __restrict__ A, int64_t lda, int64_t M, int64_t K, int L,
-                                        int lp1, int64_t NG, int64_t Kp, const double* __restrict__ Cs,
-                                        double* __restrict__ Ac) {
-  const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= M * NG) return;
-  const int64_t i = e / NG, gg = e - i * NG;
-  const double* a = A + i * lda + gg * L;
-  const int n = static_cast<int>(K - gg * L < L ? K - gg * L : L);
-  for (int p = 0; p < lp1; ++p) {
-    double acc = 0.0;
-    for (int t = 0; t < n; ++t) acc = fma(a[t], Cs[t * lp1 + p], acc);
-    Ac[i * Kp + gg * lp1 + p] = acc;
-  }
-}
+// Blocks [0, row_blocks): one thread per (row, group) of A; the rest: one thread per
+// (column, group) of B.
+struct PairF64 {
+  const double* A;
+  const double* B;
+  double* Ac;
+  double* Bd;
+  const double* Cs;
+  const double* Ds;
+  int64_t lda, ldb, M, N, K, NG, Kp, row_blocks;
+  int L, lp1;
+};
 
-__global__ void project_cols_f64_kernel(const double* __restrict__ B, int64_t ldb, int64_t N, int64_t K, int L,
-                                        int lp1, int64_t NG, const double* __restrict__ Ds,
-                                        double* __restrict__ Bd) {
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (j >= N) return;
-  for (int64_t gg = blockIdx.y; gg < NG; gg += gridDim.y) {
-    const int n = static_cast<int>(K - gg * L < L ? K - gg * L : L);
-    for (int p = 0; p < lp1; ++p) {
+__global__ void __launch_bounds__(128) project_pair_f64_kernel(const __grid_constant__ PairF64 p) {
+  pdl_begin();
+  const int L = p.L, lp1 = p.lp1;
+  if (static_cast<int64_t>(blockIdx.x) < p.row_blocks) {
+    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= p.M * p.NG) return;
+    const int64_t i = e / p.NG, gg = e - i * p.NG;
+    const double* a = p.A + i * p.lda + gg * L;
+    const int n = static_cast<int>(p.K - gg * L < L ? p.K - gg * L : L);
+    for (int q = 0; q < lp1; ++q) {
       double acc = 0.0;
-      for (int t = 0; t < n; ++t) acc = fma(Ds[p * L + t], B[(gg * L + t) * ldb + j], acc);
-      Bd[(gg * lp1 + p) * N + j] = acc;
+      for (int t = 0; t < n; ++t) acc = fma(a[t], p.Cs[t * lp1 + q], acc);
+      p.Ac[i * p.Kp + gg * lp1 + q] = acc;
     }
+    return;
+  }
+  const int64_t e = (static_cast<int64_t>(blockIdx.x) - p.row_blocks) * blockDim.x + threadIdx.x;
+  if (e >= p.N * p.NG) return;
+  const int64_t gg = e / p.N, j = e - gg * p.N;
+  const int n = static_cast<int>(p.K - gg * L < L ? p.K - gg * L : L);
+  for (int q = 0; q < lp1; ++q) {
+    double acc = 0.0;
+    for (int t = 0; t < n; ++t) acc = fma(p.Ds[q * L + t], p.B[(gg * L + t) * p.ldb + j], acc);
+    p.Bd[(gg * lp1 + q) * p.N + j] = acc;
   }
 }
 
@@ -741,6 +778,7 @@ __device__ __forceinline__ void conv_template_part(const ConvProjParams& p, int6
 template <int LB>
 __global__ void __launch_bounds__(256) conv_project_kernel(const __grid_constant__ ConvProjParams p) {
   __shared__ __align__(16) float buf[2][kConvBuf];
+  pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) *p.err = 0;
   if (blockIdx.x < p.sig_blocks)
     conv_signal_block<LB>(p, blockIdx.x, buf);
@@ -766,15 +804,27 @@ struct ConvGenParams {
   uint16_t* TP;
   const float* Cs;    // L x lp1, Cs[i * lp1 + p] = c[i, p]
   const float* Ds;    // lp1 x L, Ds[p * L + i] = d[p, i]
+  int inl;            // the kept vectors are in c8 (L = 8), and block 0 clears *err
+  Coef8 c8;
+  int* err;
 };
 
 template <int LP1>
 __global__ void __launch_bounds__(256) conv_project_general_kernel(const __grid_constant__ ConvGenParams p) {
   __shared__ float sC[kMaxL * LP1];
   __shared__ float sD[LP1 * kMaxL];
-  for (int e = threadIdx.x; e < p.L * LP1; e += blockDim.x) {
-    sC[e] = p.Cs[e];
-    sD[e] = p.Ds[e];
+  pdl_begin();
+  if (p.inl) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.err = 0;
+    for (int e = threadIdx.x; e < 8 * LP1; e += blockDim.x) {
+      sC[e] = p.c8.c[(e % LP1) * 8 + e / LP1 & 63];
+      sD[e] = p.c8.c[e & 63];
+    }
+  } else {
+    for (int e = threadIdx.x; e < p.L * LP1; e += blockDim.x) {
+      sC[e] = p.Cs[e];
+      sD[e] = p.Ds[e];
+    }
   }
   __syncthreads();
   const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -828,7 +878,8 @@ __global__ void __launch_bounds__(256) conv_project_general_kernel(const __grid_
 }  // namespace
 
 static cudaError_t launch_conv_project_general(const float* s, const float* k, const ConvGeom& g, uint16_t* G,
-                                               uint16_t* TP, const float* Cs, const float* Ds, cudaStream_t st) {
+                                               uint16_t* TP, const float* Cs, const float* Ds, const Coef8* c8,
+                                               int* err, cudaStream_t st) {
   ConvGenParams p{};
   p.s = s;
   p.S = g.S;
@@ -845,22 +896,24 @@ static cudaError_t launch_conv_project_general(const float* s, const float* k, c
   p.TP = TP;
   p.Cs = Cs;
   p.Ds = Ds;
+  if (c8) {
+    p.inl = 1;
+    p.c8 = *c8;
+  }
+  p.err = err;
   const int64_t threads = p.sig_threads + (k ? static_cast<int64_t>(g.Kc + 1) * 128 * 64 : 0);
   const unsigned blocks = static_cast<unsigned>(ceil_div(threads, 256));
   switch (g.lp1) {   // a power of two in [1, 64]
-    case 1: conv_project_general_kernel<1><<<blocks, 256, 0, st>>>(p); break;
-    case 2: conv_project_general_kernel<2><<<blocks, 256, 0, st>>>(p); break;
-    case 4: conv_project_general_kernel<4><<<blocks, 256, 0, st>>>(p); break;
-    case 8: conv_project_general_kernel<8><<<blocks, 256, 0, st>>>(p); break;
-    case 16: conv_project_general_kernel<16><<<blocks, 256, 0, st>>>(p); break;
-    case 32: conv_project_general_kernel<32><<<blocks, 256, 0, st>>>(p); break;
-    case 64: conv_project_general_kernel<64><<<blocks, 256, 0, st>>>(p); break;
+    case 1: return launch_plain(conv_project_general_kernel<1>, dim3(blocks), 256, 0, st, p);
+    case 2: return launch_plain(conv_project_general_kernel<2>, dim3(blocks), 256, 0, st, p);
+    case 4: return launch_plain(conv_project_general_kernel<4>, dim3(blocks), 256, 0, st, p);
+    case 8: return launch_plain(conv_project_general_kernel<8>, dim3(blocks), 256, 0, st, p);
+    case 16: return launch_plain(conv_project_general_kernel<16>, dim3(blocks), 256, 0, st, p);
+    case 32: return launch_plain(conv_project_general_kernel<32>, dim3(blocks), 256, 0, st, p);
+    case 64: return launch_plain(conv_project_general_kernel<64>, dim3(blocks), 256, 0, st, p);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
-
-static unsigned grid_y(int64_t n) { return static_cast<unsigned>(n < 65535 ? (n > 0 ? n : 1) : 65535); }
 
 RowsJob make_rows_job(const void* A, int64_t lda, int in_dtype, const GemmGeom& g, const float* Cs, uint16_t* Ac) {
   RowsJob J{};
@@ -910,80 +963,77 @@ int64_t cols_job_blocks(const ColsJob& J) { return J.nbx * ceil_div(J.NG, kColGr
 
 int projection_class(int in_bf16, int L) { return (in_bf16 ? 2 : 0) + (L == 8 ? 1 : 0); }
 
-cudaError_t launch_project_rows_simt(const void* A, int64_t lda, int in_dtype, const GemmGeom& g, const float* Cs,
-                                     uint16_t* Ac, cudaStream_t st) {
-  if (g.M == 0 || g.K == 0) return cudaSuccess;
-  const RowsJob J = make_rows_job(A, lda, in_dtype, g, Cs, Ac);
-  const unsigned blocks = static_cast<unsigned>(rows_job_blocks(J));
-  switch (projection_class(J.in_bf16, J.L)) {
-    case 0: project_rows_kernel<float, 0><<<blocks, 256, 0, st>>>(J); break;
-    case 1: project_rows_kernel<float, 8><<<blocks, 256, 0, st>>>(J); break;
-    case 2: project_rows_kernel<__nv_bfloat16, 0><<<blocks, 256, 0, st>>>(J); break;
-    default: project_rows_kernel<__nv_bfloat16, 8><<<blocks, 256, 0, st>>>(J); break;
+cudaError_t launch_project_pair_simt(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
+                                     const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
+                                     uint16_t* Ac, uint16_t* Bd, int* clear_err, cudaStream_t st) {
+  if (g.K == 0) return cudaSuccess;
+  const bool rows = A && g.M > 0, cols = B && g.N > 0;
+  if (!rows && !cols) return cudaSuccess;
+  SideArgs a{};
+  if (c8) a.c8 = *c8;
+  a.clear = clear_err;
+  if (rows) {
+    const RowsJob J = make_rows_job(A, lda, in_dtype, g, Cs, Ac);
+    const dim3 grid(static_cast<unsigned>(rows_job_blocks(J)));
+    void (*kern)(RowsJob, SideArgs) = nullptr;
+    switch (projection_class(J.in_bf16, J.L)) {
+      case 0: kern = project_rows_kernel<float, 0, false>; break;
+      case 1: kern = c8 ? project_rows_kernel<float, 8, true> : project_rows_kernel<float, 8, false>; break;
+      case 2: kern = project_rows_kernel<__nv_bfloat16, 0, false>; break;
+      default: kern = c8 ? project_rows_kernel<__nv_bfloat16, 8, true> : project_rows_kernel<__nv_bfloat16, 8, false>;
+    }
+    const cudaError_t e = launch_plain(kern, grid, 256, 0, st, J, a);
+    if (e != cudaSuccess) return e;
+    a.clear = nullptr;
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_project_cols_simt(const void* B, int64_t ldb, int in_dtype, const GemmGeom& g, const float* Ds,
-                                     uint16_t* Bd, cudaStream_t st) {
-  if (g.N == 0 || g.K == 0) return cudaSuccess;
+  if (!cols) return cudaSuccess;
   const ColsJob J = make_cols_job(B, ldb, in_dtype, g, Ds, Bd);
-  const unsigned blocks = static_cast<unsigned>(cols_job_blocks(J));
+  const dim3 grid(static_cast<unsigned>(cols_job_blocks(J)));
+  void (*kern)(ColsJob, SideArgs) = nullptr;
   switch (projection_class(J.in_bf16, J.L)) {
-    case 0: project_cols_kernel<float, 0><<<blocks, 256, 0, st>>>(J); break;
-    case 1: project_cols_kernel<float, 8><<<blocks, 256, 0, st>>>(J); break;
-    case 2: project_cols_kernel<__nv_bfloat16, 0><<<blocks, 256, 0, st>>>(J); break;
-    default: project_cols_kernel<__nv_bfloat16, 8><<<blocks, 256, 0, st>>>(J); break;
+    case 0: kern = project_cols_kernel<float, 0, false>; break;
+    case 1: kern = c8 ? project_cols_kernel<float, 8, true> : project_cols_kernel<float, 8, false>; break;
+    case 2: kern = project_cols_kernel<__nv_bfloat16, 0, false>; break;
+    default: kern = c8 ? project_cols_kernel<__nv_bfloat16, 8, true> : project_cols_kernel<__nv_bfloat16, 8, false>;
   }
-  return cudaGetLastError();
+  return launch_plain(kern, grid, 256, 0, st, J, a);
 }
 
 cudaError_t launch_project_rows_jobs(int cls, const RowsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st) {
   if (blocks == 0) return cudaSuccess;
   const unsigned nb = static_cast<unsigned>(blocks);
   switch (cls) {
-    case 0: project_rows_jobs_kernel<float, 0><<<nb, 256, 0, st>>>(jobs, job_of); break;
-    case 1: project_rows_jobs_kernel<float, 8><<<nb, 256, 0, st>>>(jobs, job_of); break;
-    case 2: project_rows_jobs_kernel<__nv_bfloat16, 0><<<nb, 256, 0, st>>>(jobs, job_of); break;
-    default: project_rows_jobs_kernel<__nv_bfloat16, 8><<<nb, 256, 0, st>>>(jobs, job_of); break;
+    case 0: return launch_plain(project_rows_jobs_kernel<float, 0>, dim3(nb), 256, 0, st, jobs, job_of);
+    case 1: return launch_plain(project_rows_jobs_kernel<float, 8>, dim3(nb), 256, 0, st, jobs, job_of);
+    case 2: return launch_plain(project_rows_jobs_kernel<__nv_bfloat16, 0>, dim3(nb), 256, 0, st, jobs, job_of);
+    default: return launch_plain(project_rows_jobs_kernel<__nv_bfloat16, 8>, dim3(nb), 256, 0, st, jobs, job_of);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_project_cols_jobs(int cls, const ColsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st) {
   if (blocks == 0) return cudaSuccess;
   const unsigned nb = static_cast<unsigned>(blocks);
   switch (cls) {
-    case 0: project_cols_jobs_kernel<float, 0><<<nb, 256, 0, st>>>(jobs, job_of); break;
-    case 1: project_cols_jobs_kernel<float, 8><<<nb, 256, 0, st>>>(jobs, job_of); break;
-    case 2: project_cols_jobs_kernel<__nv_bfloat16, 0><<<nb, 256, 0, st>>>(jobs, job_of); break;
-    default: project_cols_jobs_kernel<__nv_bfloat16, 8><<<nb, 256, 0, st>>>(jobs, job_of); break;
+    case 0: return launch_plain(project_cols_jobs_kernel<float, 0>, dim3(nb), 256, 0, st, jobs, job_of);
+    case 1: return launch_plain(project_cols_jobs_kernel<float, 8>, dim3(nb), 256, 0, st, jobs, job_of);
+    case 2: return launch_plain(project_cols_jobs_kernel<__nv_bfloat16, 0>, dim3(nb), 256, 0, st, jobs, job_of);
+    default: return launch_plain(project_cols_jobs_kernel<__nv_bfloat16, 8>, dim3(nb), 256, 0, st, jobs, job_of);
   }
-  return cudaGetLastError();
 }
 
 
-cudaError_t launch_project_rows_f64(const double* A, int64_t lda, const GemmGeom& g, const double* Cs, double* Ac,
-                                    cudaStream_t st) {
+cudaError_t launch_project_pair_f64(const double* A, int64_t lda, const double* B, int64_t ldb, const GemmGeom& g,
+                                    const double* Cs, const double* Ds, double* Ac, double* Bd, cudaStream_t st) {
   const int64_t NG = ceil_div(g.K, g.L);
-  if (g.M == 0 || NG == 0) return cudaSuccess;
-  project_rows_f64_kernel<<<static_cast<unsigned>(ceil_div(g.M * NG, 128)), 128, 0, st>>>(A, lda, g.M, g.K, g.L,
-                                                                                          g.lp1, NG, g.Kp, Cs, Ac);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_project_cols_f64(const double* B, int64_t ldb, const GemmGeom& g, const double* Ds, double* Bd,
-                                    cudaStream_t st) {
-  const int64_t NG = ceil_div(g.K, g.L);
-  if (g.N == 0 || NG == 0) return cudaSuccess;
-  dim3 grid(static_cast<unsigned>(ceil_div(g.N, 128)), grid_y(NG));
-  project_cols_f64_kernel<<<grid, 128, 0, st>>>(B, ldb, g.N, g.K, g.L, g.lp1, NG, Ds, Bd);
-  return cudaGetLastError();
+  const int64_t rb = A ? ceil_div(g.M * NG, 128) : 0, cb = B ? ceil_div(g.N * NG, 128) : 0;
+  if (rb + cb == 0) return cudaSuccess;
+  const PairF64 p{A, B, Ac, Bd, Cs, Ds, lda, ldb, g.M, g.N, g.K, NG, g.Kp, rb, g.L, g.lp1};
+  return launch_plain(project_pair_f64_kernel, dim3(static_cast<unsigned>(rb + cb)), 128, 0, st, p);
 }
 
 cudaError_t launch_conv_project(const float* s, const float* k, const ConvGeom& g, uint16_t* G, uint16_t* TP,
-                                int* err, cudaStream_t st, const float* Cs, const float* Ds) {
-  if (!g.box) return launch_conv_project_general(s, k, g, G, TP, Cs, Ds, st);
+                                int* err, cudaStream_t st, const float* Cs, const float* Ds, const Coef8* c8) {
+  if (!g.box) return launch_conv_project_general(s, k, g, G, TP, Cs, Ds, c8, err, st);
   ConvProjParams p{};
   p.s = s;
   p.S = g.S;
@@ -1003,16 +1053,15 @@ cudaError_t launch_conv_project(const float* s, const float* k, const ConvGeom& 
   const int64_t tpl_blocks = k ? ceil_div(tpl_threads, 256) : 0;
   const unsigned blocks = static_cast<unsigned>(p.sig_blocks + tpl_blocks);
   switch (g.Lb) {  // Lb = T / R is a power of two in [1, 64]
-    case 1: conv_project_kernel<1><<<blocks, 256, 0, st>>>(p); break;
-    case 2: conv_project_kernel<2><<<blocks, 256, 0, st>>>(p); break;
-    case 4: conv_project_kernel<4><<<blocks, 256, 0, st>>>(p); break;
-    case 8: conv_project_kernel<8><<<blocks, 256, 0, st>>>(p); break;
-    case 16: conv_project_kernel<16><<<blocks, 256, 0, st>>>(p); break;
-    case 32: conv_project_kernel<32><<<blocks, 256, 0, st>>>(p); break;
-    case 64: conv_project_kernel<64><<<blocks, 256, 0, st>>>(p); break;
+    case 1: return launch_plain(conv_project_kernel<1>, dim3(blocks), 256, 0, st, p);
+    case 2: return launch_plain(conv_project_kernel<2>, dim3(blocks), 256, 0, st, p);
+    case 4: return launch_plain(conv_project_kernel<4>, dim3(blocks), 256, 0, st, p);
+    case 8: return launch_plain(conv_project_kernel<8>, dim3(blocks), 256, 0, st, p);
+    case 16: return launch_plain(conv_project_kernel<16>, dim3(blocks), 256, 0, st, p);
+    case 32: return launch_plain(conv_project_kernel<32>, dim3(blocks), 256, 0, st, p);
+    case 64: return launch_plain(conv_project_kernel<64>, dim3(blocks), 256, 0, st, p);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace pj

@@ -22,6 +22,7 @@
 
 #include "common.hpp"
 #include "mx.cuh"
+#include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
 
@@ -52,6 +53,8 @@ struct ProjTmaParams {
   int64_t pitch, Kp_pad, Kt_pad;
   int64_t NG;           // groups along K
   int nsplit, tl;
+  int inl, clear;       // the kept vectors are in c8 (else side[].coef); block 0 clears *err
+  Coef8 c8;
   int* err;
 };
 
@@ -771,7 +774,7 @@ template <int NST>
 __device__ __forceinline__ bool pt_stage_free(const PtRing& r, int64_t k, int* err) {
   if (k < 0) return true;
   const int s = static_cast<int>(k % NST);
-  return mbar_wait(&r.empty[s], static_cast<uint32_t>((k / NST) & 1), err, DEV_TIMEOUT_EMPTY);
+  return mbar_wait_first(&r.empty[s], static_cast<uint32_t>((k / NST) & 1), err, DEV_TIMEOUT_EMPTY);
 }
 
 // Thread 0, after the loop: every issued copy must land before the block exits
@@ -814,11 +817,14 @@ __global__ void __launch_bounds__(kPtThreads, 2) project_tma_kernel(const __grid
     }
     fence_mbar_init();
   }
+  pdl_begin();
+  if (p.clear && blockIdx.x == 0 && threadIdx.x == 0) *p.err = 0;
   if (threadIdx.x < 128) {
     // Stage the kept basis vectors of side sd as sCoef[sd * 64 + q * 8 + t].
     const int sd = threadIdx.x >> 6, k = threadIdx.x & 63, q = k >> 3, t = k & 7;
     if (q < LP1 && p.side[sd].num_units > 0)
-      sCoef[threadIdx.x] = sd == 0 ? p.side[0].coef[t * LP1 + q] : p.side[1].coef[q * 8 + t];
+      sCoef[threadIdx.x] = p.inl ? p.c8.c[k]
+                                 : (sd == 0 ? p.side[0].coef[t * LP1 + q] : p.side[1].coef[q * 8 + t]);
   }
   __syncthreads();
 
@@ -844,7 +850,7 @@ __global__ void __launch_bounds__(kPtThreads, 2) project_tma_kernel(const __grid
   int64_t k = 0;
   for (; k < mine; ++k) {
     const int s = static_cast<int>(k % NST);
-    if (!mbar_wait(&ring.full[s], static_cast<uint32_t>((k / NST) & 1), p.err, DEV_TIMEOUT_FULL)) break;
+    if (!mbar_wait_first(&ring.full[s], static_cast<uint32_t>((k / NST) & 1), p.err, DEV_TIMEOUT_FULL)) break;
     const TileIn<InT, false> tin{tiles + s * TB, 0, 0, kPtBoxY, kPtBoxX};
     const int4 un = stage_unit[s];
     const int sd = un.x, ux = un.y, uy = un.z;
@@ -918,6 +924,7 @@ __global__ void __launch_bounds__(kPtThreads, 2) project_tma_jobs_kernel(const T
     }
     fence_mbar_init();
   }
+  pdl_begin();
   __syncthreads();
 
   auto fetch = [&](int64_t k, int4& u0, int4& u1) {
@@ -960,7 +967,7 @@ __global__ void __launch_bounds__(kPtThreads, 2) project_tma_jobs_kernel(const T
   int64_t k = 0;
   for (; k < mine; ++k) {
     const int s = static_cast<int>(k % NST);
-    if (!mbar_wait(&ring.full[s], static_cast<uint32_t>((k / NST) & 1), err, DEV_TIMEOUT_FULL)) break;
+    if (!mbar_wait_first(&ring.full[s], static_cast<uint32_t>((k / NST) & 1), err, DEV_TIMEOUT_FULL)) break;
     const int4 un = stage_unit[s];
     const TmaJob& J = jobs[un.x];
     const TileCtx c{J.out, J.n_out, J.NG, J.pitch, J.Kp_pad, J.Kt_pad, J.units_x, J.units_y, J.nsplit, J.tl};
@@ -1072,8 +1079,7 @@ cudaError_t launch_tma(const ProjTmaParams& p, int in_dtype, int lp1, int sms, c
   const int64_t units = p.side[0].num_units + p.side[1].num_units;
   const int64_t slots = static_cast<int64_t>(nb) * sms;
   const int64_t grid = units < slots ? units : slots;
-  kern<<<static_cast<unsigned>(grid), kPtThreads, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), kPtThreads, smem, st, 1, p);
 }
 
 // Fills side sd of p when the operand suits TMA; returns whether it does.
@@ -1095,8 +1101,8 @@ bool tma_side(ProjTmaParams& p, int sd, const void* X, int64_t ld, int in_dtype,
 }  // namespace
 
 cudaError_t launch_project_pair_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
-                                     const GemmGeom& g, const float* Cs, const float* Ds, uint16_t* Ac,
-                                     uint16_t* Bd, int* err, int sms, cudaStream_t st) {
+                                     const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
+                                     uint16_t* Ac, uint16_t* Bd, int* err, bool clear, int sms, cudaStream_t st) {
   if (g.K == 0) return cudaSuccess;
   if (g.M == 0) A = nullptr;
   if (g.N == 0) B = nullptr;
@@ -1110,19 +1116,21 @@ cudaError_t launch_project_pair_bf16(const void* A, int64_t lda, const void* B, 
     p.nsplit = g.nsplit;
     p.tl = g.tl;
     p.err = err;
+    if (c8) {
+      p.inl = 1;
+      p.c8 = *c8;
+    }
+    p.clear = clear;
     rows_tma = tma_side(p, 0, A, lda, in_dtype, g.K, g.M, g.M, Cs, Ac);
     cols_tma = tma_side(p, 1, B, ldb, in_dtype, g.N, g.K, g.N, Ds, Bd);
     if (rows_tma || cols_tma) {
       const cudaError_t e = launch_tma(p, in_dtype, g.lp1, sms, st);
       if (e != cudaSuccess) return e;
+      clear = false;
     }
   }
-  if (A && !rows_tma) {
-    const cudaError_t e = launch_project_rows_simt(A, lda, in_dtype, g, Cs, Ac, st);
-    if (e != cudaSuccess) return e;
-  }
-  if (B && !cols_tma) return launch_project_cols_simt(B, ldb, in_dtype, g, Ds, Bd, st);
-  return cudaSuccess;
+  return launch_project_pair_simt(rows_tma ? nullptr : A, lda, cols_tma ? nullptr : B, ldb, in_dtype, g, Cs, Ds, c8, Ac,
+                                  Bd, clear ? err : nullptr, st);
 }
 
 bool project_mx_fusable(const GemmGeom& g, int side) {
@@ -1131,9 +1139,9 @@ bool project_mx_fusable(const GemmGeom& g, int side) {
 }
 
 cudaError_t launch_project_pair_mx(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
-                                   const GemmGeom& g, const float* Cs, const float* Ds, const MxQuantSide* qa,
-                                   const MxQuantSide* qb, int* err, int sms, cudaStream_t st, bool* a_done,
-                                   bool* b_done) {
+                                   const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
+                                   const MxQuantSide* qa, const MxQuantSide* qb, int* err, bool clear, int sms,
+                                   cudaStream_t st, bool* a_done, bool* b_done) {
   *a_done = *b_done = false;
   if (g.K == 0) return cudaSuccess;
   if (g.M == 0) A = nullptr;
@@ -1146,6 +1154,11 @@ cudaError_t launch_project_pair_mx(const void* A, int64_t lda, const void* B, in
   p.nsplit = g.nsplit;
   p.tl = g.tl;
   p.err = err;
+  if (c8) {
+    p.inl = 1;
+    p.c8 = *c8;
+  }
+  p.clear = clear;
   if (A && qa && project_mx_fusable(g, 0) && tma_side(p, 0, A, lda, in_dtype, g.K, g.M, g.M, Cs, nullptr)) {
     p.q[0] = *qa;
     *a_done = true;
@@ -1161,16 +1174,6 @@ cudaError_t launch_project_pair_mx(const void* A, int64_t lda, const void* B, in
   if (!*b_done) p.side[1].num_units = 0;
   if (!*a_done && !*b_done) return cudaSuccess;
   return launch_tma(p, in_dtype, g.lp1, sms, st, true);
-}
-
-cudaError_t launch_project_rows_bf16(const void* A, int64_t lda, int in_dtype, const GemmGeom& g, const float* Cs,
-                                     uint16_t* Ac, int* err, int sms, cudaStream_t st) {
-  return launch_project_pair_bf16(A, lda, nullptr, 0, in_dtype, g, Cs, nullptr, Ac, nullptr, err, sms, st);
-}
-
-cudaError_t launch_project_cols_bf16(const void* B, int64_t ldb, int in_dtype, const GemmGeom& g, const float* Ds,
-                                     uint16_t* Bd, int* err, int sms, cudaStream_t st) {
-  return launch_project_pair_bf16(nullptr, 0, B, ldb, in_dtype, g, nullptr, Ds, nullptr, Bd, err, sms, st);
 }
 
 bool tma_projection_ok(const void* X, int in_dtype, int64_t inner, int64_t rows, int64_t ld) {
@@ -1299,8 +1302,7 @@ cudaError_t launch_project_tma_jobs(int in_bf16, int lp1, const TmaJob* jobs, co
   }
   const int64_t slots = static_cast<int64_t>(nb) * sms;
   const int64_t grid = total < slots ? total : slots;
-  kern<<<static_cast<unsigned>(grid), kPtThreads, smem, st>>>(jobs, units, total, err);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), kPtThreads, smem, st, 1, jobs, units, total, err);
 }
 
 }  // namespace pj

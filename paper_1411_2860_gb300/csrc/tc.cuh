@@ -101,6 +101,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   }
 }
 
+// The same, without reading the error word: for the first kernel of a call, one of
+// whose blocks clears what an earlier call may have left there.
+__device__ __forceinline__ bool mbar_wait_first(uint64_t* bar, uint32_t parity, int* err, int code) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 127u) == 0 && globaltimer_ns() - t0 > PJ_WAIT_LIMIT_NS) {
+      atomicCAS(err, 0, code);
+      return false;
+    }
+  }
+}
+
 // Wait for a phase that copies already issued will complete, ignoring the
 // error word (used before exit, so no copy is still writing shared memory).
 // Gives up after PJ_WAIT_LIMIT_NS and returns false.
