@@ -250,6 +250,14 @@ pj_status proj_gemm_backward(const void* A, int64_t lda, const void* B, int64_t 
                              const pj_basis* basis, const pj_precision* prec, void* workspace, size_t ws_bytes,
                              void* stream);
 
+/* The same with dY in a dtype of its own (PJ_F32 or PJ_BF16 for BF16 compute: an FP32
+ * dY of BF16 operands is rounded to BF16 here; PJ_F64 for F64). */
+pj_status proj_gemm_backward_mixed(const void* A, int64_t lda, const void* B, int64_t ldb, const void* dY,
+                                   int64_t lddy, void* dA, int64_t ldda, void* dB, int64_t lddb, int64_t M, int64_t N,
+                                   int64_t K, int32_t in_dtype, int32_t dy_dtype, int32_t out_dtype, int64_t block_k,
+                                   int64_t R, const pj_basis* basis, const pj_precision* prec, void* workspace,
+                                   size_t ws_bytes, void* stream);
+
 /* The same gradients from the projections a forward pass already made: A_c and
  * B_d are read from `fwd_workspace`, the workspace of a proj_gemm call (or of
  * proj_gemm_project with both operands) with the same M, N, K, block_k, R, basis

@@ -646,14 +646,20 @@ static bool bwd_fused(const GemmGeom& g, int compute, int64_t ldda, int64_t lddb
          (ldda * oes) % 16 == 0 && (lddb * oes) % 16 == 0;
 }
 
+// A BF16 dY whose rows are 16-byte aligned feeds both products as it is.
+static bool bwd_dy_direct(const void* dY, int64_t lddy, int32_t dy_dtype) {
+  return dy_dtype == PJ_BF16 && aligned16(dY) && lddy % 8 == 0;
+}
+
 // The two gradient products and their expansion, from projected operands Ac
 // (M x pitch) and Bd (N x pitch) -- computed by the backward itself or saved by
 // the forward -- and dY (dy_dtype).  The basis is staged in `workspace`, or given as c8
-// (fused products only).
+// (fused products only).  clear: dY's conversion, the call's first kernel, clears the
+// error word.
 static pj_status backward_products(const void* Ac_v, const void* Bd_v, const void* dY, int64_t lddy, int32_t dy_dtype,
                                    void* dA, int64_t ldda, void* dB, int64_t lddb, int32_t out_dtype,
                                    const GemmGeom& g, int compute, const BwdWs& w, const Coef8* c8, void* workspace,
-                                   int sms, cudaStream_t st) {
+                                   bool clear, int sms, cudaStream_t st) {
   BasisDev b = basis_area(workspace);
   if (compute == PJ_F64) {
     const double* Ac = static_cast<const double*>(Ac_v);
@@ -676,9 +682,10 @@ static pj_status backward_products(const void* Ac_v, const void* Bd_v, const voi
   GemmGeom g1 = g;
   g1.nsplit = 1;
   const int64_t pitch = gemm_pitch(g1);
-  // A BF16 dY whose rows are 16-byte aligned feeds both products as it is.
-  const bool dy_direct = dy_dtype == PJ_BF16 && aligned16(dY) && lddy % 8 == 0;
-  if (!dy_direct) PJ_CUDA_TRY(launch_convert_bf16(dY, dy_dtype, lddy, g.M, g.N, dYb, w.ldn, st));
+  const bool dy_direct = bwd_dy_direct(dY, lddy, dy_dtype);
+  if (!dy_direct)
+    PJ_CUDA_TRY(launch_convert_bf16(dY, dy_dtype, lddy, g.M, g.N, dYb, w.ldn, clear ? error_word(workspace) : nullptr,
+                                    st));
   const uint16_t* dYq = dy_direct ? static_cast<const uint16_t*>(dY) : dYb;
   const int64_t lddq = dy_direct ? lddy : w.ldn;
   const bool fuse = bwd_fused(g, compute, ldda, lddb, out_dtype);
@@ -755,10 +762,20 @@ pj_status proj_gemm_backward(const void* A, int64_t lda, const void* B, int64_t 
                              int32_t in_dtype, int32_t out_dtype, int64_t block_k, int64_t R,
                              const pj_basis* basis, const pj_precision* prec, void* workspace, size_t ws_bytes,
                              void* stream) {
+  return proj_gemm_backward_mixed(A, lda, B, ldb, dY, lddy, dA, ldda, dB, lddb, M, N, K, in_dtype, in_dtype, out_dtype,
+                                  block_k, R, basis, prec, workspace, ws_bytes, stream);
+}
+
+pj_status proj_gemm_backward_mixed(const void* A, int64_t lda, const void* B, int64_t ldb, const void* dY,
+                                   int64_t lddy, void* dA, int64_t ldda, void* dB, int64_t lddb, int64_t M, int64_t N,
+                                   int64_t K, int32_t in_dtype, int32_t dy_dtype, int32_t out_dtype, int64_t block_k,
+                                   int64_t R, const pj_basis* basis, const pj_precision* prec, void* workspace,
+                                   size_t ws_bytes, void* stream) {
   GemmGeom g{};
   PJ_TRY(gemm_geom(M, N, K, block_k, R, basis, prec, &g));
   PJ_TRY(backward_checks(g, prec, dY, lddy, dA, ldda, dB, lddb));
   PJ_TRY(check_gemm_dtypes(in_dtype, out_dtype, prec));
+  PJ_TRY(check_gemm_dtypes(dy_dtype, out_dtype, prec));
   const bool need_a = M > 0 && K > 0, need_b = K > 0 && N > 0;
   if ((need_a && !A) || (need_b && !B)) return fail(PJ_EINVAL, "A, B, dY, dA and dB must be non-NULL for non-empty operands");
   if (need_a && lda < K) return fail(PJ_EINVAL, "lda and ldda must be >= K");
@@ -788,7 +805,7 @@ pj_status proj_gemm_backward(const void* A, int64_t lda, const void* B, int64_t 
     PJ_CUDA_TRY(launch_project_pair_f64(static_cast<const double*>(A), lda, static_cast<const double*>(B), ldb, g, b.Cs64,
                                         b.Ds64, Ac, Bd, st));
     return backward_products(Ac, Bd, dY, lddy, PJ_F64, dA, ldda, dB, lddb, out_dtype, g, PJ_F64, w, nullptr, workspace,
-                             sms, st);
+                             false, sms, st);
   }
   uint16_t* Ac = at<uint16_t>(workspace, w.ac);
   uint16_t* Bd = at<uint16_t>(workspace, w.bd);
@@ -797,8 +814,8 @@ pj_status proj_gemm_backward(const void* A, int64_t lda, const void* B, int64_t 
   // A_c (M x Kp_pad) and B_d (N x Kp_pad) exactly as the forward projects them, in one launch
   PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g1, b.Cs32, b.Ds32, c8, Ac, Bd, error_word(workspace),
                                        c8 != nullptr, sms, st));
-  return backward_products(Ac, Bd, dY, lddy, in_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace,
-                           sms, st);
+  return backward_products(Ac, Bd, dY, lddy, dy_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace,
+                           false, sms, st);
 }
 
 pj_status proj_gemm_backward_saved(const void* fwd_workspace, size_t fwd_ws_bytes, const void* dY, int64_t lddy,
@@ -829,15 +846,19 @@ pj_status proj_gemm_backward_saved(const void* fwd_workspace, size_t fwd_ws_byte
   Coef8 c8v;
   const Coef8* c8 =
       bwd_fused(g, prec->compute, ldda, lddb, out_dtype) && coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
-  if (c8) {   // no kernel runs before the products, whose waits read the error word
+  // The products' waits read the error word: it is cleared by the basis kernel or by
+  // dY's conversion, whichever runs before them, else on its own.
+  const bool convert = prec->compute != PJ_F64 && !bwd_dy_direct(dY, lddy, dy_dtype);
+  if (c8 && !convert) {
     PJ_TRY(begin_call(workspace, st, &sms));
   } else {
     PJ_TRY(device_sms(&sms));
-    PJ_TRY(stage_basis(basis, g.lp1, workspace, st, nullptr, 0, true));
+    if (!c8) PJ_TRY(stage_basis(basis, g.lp1, workspace, st, nullptr, 0, true));
   }
   const void* fws = fwd_workspace;
   return backward_products(static_cast<const char*>(fws) + fw.off_ac, static_cast<const char*>(fws) + fw.off_bd, dY,
-                           lddy, dy_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace, sms, st);
+                           lddy, dy_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace,
+                           c8 != nullptr, sms, st);
 }
 
 // ------------------------------------------------------------------ CONV --

@@ -35,7 +35,9 @@ struct Groups {
 // X (rows x cols, pitch ldx) -> BF16 copy (pitch ldo).
 template <typename InT>
 __global__ void __launch_bounds__(256) convert_bf16_kernel(const InT* __restrict__ X, int64_t ldx, int64_t rows,
-                                                           int64_t cols, uint16_t* __restrict__ out, int64_t ldo) {
+                                                           int64_t cols, uint16_t* __restrict__ out, int64_t ldo,
+                                                           int* clear) {
+  if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
   const int64_t c = static_cast<int64_t>(blockIdx.y) * blockDim.x + threadIdx.x;
   const int64_t r = blockIdx.x;
   if (c < cols && r < rows) out[r * ldo + c] = __bfloat16_as_ushort(__float2bfloat16_rn(to_float(X[r * ldx + c])));
@@ -100,26 +102,17 @@ __device__ __forceinline__ void load8_bf16(const __nv_bfloat16* p, uint16_t (&v)
     v[2 * k + 1] = static_cast<uint16_t>(w[k] >> 16);
   }
 }
-__device__ __forceinline__ void load8_float(const float* p, float (&x)[8]) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-}
-__device__ __forceinline__ void load8_float(const __nv_bfloat16* p, float (&x)[8]) {
-  uint16_t v[8];
-  load8_bf16(p, v);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) x[k] = __uint_as_float(uint32_t(v[k]) << 16);
-}
-
-
 // X (rows x cols, pitch ldx) -> BF16 copy (pitch ldo), eight values per thread.
 template <typename InT>
 __global__ void __launch_bounds__(256) convert8_kernel(const InT* __restrict__ X, int64_t ldx, int64_t rows,
-                                                       int64_t cols, uint16_t* __restrict__ out, int64_t ldo) {
+                                                       int64_t cols, uint16_t* __restrict__ out, int64_t ldo,
+                                                       int* clear) {
+  if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
   const int64_t c8 = (cols + 7) / 8;
   const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= rows * c8) return;
-  const int64_t r = e / c8, c = (e - r * c8) * 8;
+  const int64_t r = rows * c8 < (int64_t(1) << 32) ? static_cast<uint32_t>(e) / static_cast<uint32_t>(c8) : e / c8;
+  const int64_t c = (e - r * c8) * 8;
   uint16_t v[8];
   if (c + 8 <= cols) {
     load8_bf16(X + r * ldx + c, v);
@@ -282,24 +275,24 @@ static bool rows16(const void* p, int64_t ld, size_t es) {
 }
 
 cudaError_t launch_convert_bf16(const void* X, int in_dtype, int64_t ldx, int64_t rows, int64_t cols, uint16_t* out,
-                                int64_t ldo, cudaStream_t st) {
+                                int64_t ldo, int* clear, cudaStream_t st) {
   if (rows == 0 || cols == 0) return cudaSuccess;
   const size_t es = in_dtype == PJ_F32 ? 4 : 2;
   if (rows16(X, ldx, es) && rows16(out, ldo, 2)) {
     const unsigned blocks = static_cast<unsigned>(ceil_div(rows * ceil_div(cols, 8), 256));
     if (in_dtype == PJ_F32)
-      convert8_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(X), ldx, rows, cols, out, ldo);
+      convert8_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(X), ldx, rows, cols, out, ldo, clear);
     else
       convert8_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(X), ldx, rows, cols,
-                                                             out, ldo);
+                                                             out, ldo, clear);
     return cudaGetLastError();
   }
   dim3 grid(static_cast<unsigned>(rows), static_cast<unsigned>(ceil_div(cols, 256)));
   if (in_dtype == PJ_F32)
-    convert_bf16_kernel<float><<<grid, 256, 0, st>>>(static_cast<const float*>(X), ldx, rows, cols, out, ldo);
+    convert_bf16_kernel<float><<<grid, 256, 0, st>>>(static_cast<const float*>(X), ldx, rows, cols, out, ldo, clear);
   else
     convert_bf16_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(X), ldx, rows, cols,
-                                                             out, ldo);
+                                                             out, ldo, clear);
   return cudaGetLastError();
 }
 

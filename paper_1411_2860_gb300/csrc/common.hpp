@@ -525,8 +525,9 @@ cudaError_t launch_gemm_mx_grouped(const MxInst* insts, const GemmTile* tiles, c
                                    int* err, cudaStream_t st);
 
 // backward.cu -----------------------------------------------------------
+// clear: an error word the kernel clears (NULL: none).
 cudaError_t launch_convert_bf16(const void* X, int in_dtype, int64_t ldx, int64_t rows, int64_t cols, uint16_t* out,
-                                int64_t ldo, cudaStream_t st);
+                                int64_t ldo, int* clear, cudaStream_t st);
 cudaError_t launch_expand_rows(const void* X, int acc_dtype, int64_t ldx, const GemmGeom& g, const void* Cs,
                                void* dA, int out_dtype, int64_t ldda, cudaStream_t st);
 cudaError_t launch_expand_cols(const void* X, int acc_dtype, int64_t ldx, const GemmGeom& g, const void* Ds,
