@@ -291,9 +291,10 @@ RowsJob make_rows_job(const void* A, int64_t lda, int in_dtype, const GemmGeom& 
 ColsJob make_cols_job(const void* B, int64_t ldb, int in_dtype, const GemmGeom& g, const float* Ds, uint16_t* Bd);
 int64_t rows_job_blocks(const RowsJob& J);
 int64_t cols_job_blocks(const ColsJob& J);
-// Jobs of one class (input dtype x group size, see projection_class) per launch.
-int projection_class(int in_bf16, int L);
-constexpr int kProjectionClasses = 4;
+// Jobs of one class (input dtype x (l+1 with groups of 8, or any other group size)) per
+// launch: class = 9 bf16_input + (L == 8 ? l+1 : 0).
+int projection_class(int in_bf16, int L, int lp1);
+constexpr int kProjectionClasses = 18;
 // job_of[b] = the job of block b (blocks of job j are [block0_j, block0_{j+1})).
 cudaError_t launch_project_rows_jobs(int cls, const RowsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st);
 cudaError_t launch_project_cols_jobs(int cls, const ColsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st);

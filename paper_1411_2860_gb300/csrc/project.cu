@@ -5,6 +5,8 @@
 // These kernels stream HBM; the arithmetic is FP32 (FP64 for the double path).
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "common.hpp"
 #include "pdl.cuh"
 
@@ -124,6 +126,30 @@ __device__ __forceinline__ void group8_pairs(const float (&x)[8], const float* c
   }
 }
 
+// The same for two groups (the same chains, so the same bits): each read of the basis
+// values feeds both.
+template <int LP1>
+__device__ __forceinline__ void group8_pairs2(const float (&x)[8], const float (&y)[8], const float* c,
+                                              float2 (&ax)[(LP1 + 1) / 2], float2 (&ay)[(LP1 + 1) / 2]) {
+  constexpr int NP = (LP1 + 1) / 2;
+#pragma unroll
+  for (int k = 0; k < NP; ++k) ax[k] = ay[k] = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const float2 xx = make_float2(x[t], x[t]), yy = make_float2(y[t], y[t]);
+#pragma unroll
+    for (int h = 0; h < (NP + 1) / 2; ++h) {
+      const float4 v = *reinterpret_cast<const float4*>(c + t * 8 + 4 * h);
+      ax[2 * h] = __ffma2_rn(xx, make_float2(v.x, v.y), ax[2 * h]);
+      ay[2 * h] = __ffma2_rn(yy, make_float2(v.x, v.y), ay[2 * h]);
+      if (2 * h + 1 < NP) {
+        ax[(2 * h + 1) % NP] = __ffma2_rn(xx, make_float2(v.z, v.w), ax[(2 * h + 1) % NP]);
+        ay[(2 * h + 1) % NP] = __ffma2_rn(yy, make_float2(v.z, v.w), ay[(2 * h + 1) % NP]);
+      }
+    }
+  }
+}
+
 // hi = bf16(component) and lo = bf16(component - hi), two components per conversion.
 template <int LP1>
 __device__ __forceinline__ void split_bf16(const float2 (&acc)[(LP1 + 1) / 2], uint16_t (&hi)[8], uint16_t (&lo)[8]) {
@@ -204,15 +230,35 @@ __device__ __forceinline__ void rows_span_odd(const RowsJob& J, const float (&x)
   }
 }
 
+// One group's components at the row's group gg, plain or with every lo term.
+template <int LP1>
+__device__ __forceinline__ void rows_store(uint16_t* row, int64_t gg, const float2 (&acc)[(LP1 + 1) / 2], bool two,
+                                           int64_t Kp_pad) {
+  uint16_t hi[8], lo[8];
+  split_bf16<LP1>(acc, hi, lo);
+  store_upto8(row + gg * LP1, hi, LP1);
+  if (two) store_upto8(row + Kp_pad + gg * LP1, lo, LP1);
+}
+
+// Group gx of row rx and group gy of row ry (NULL: not stored), l+1 in {1, 2, 4, 8}.
+template <int LP1>
+__device__ __forceinline__ void rows_two(uint16_t* rx, int64_t gx, const float (&x)[8], uint16_t* ry, int64_t gy,
+                                         const float (&y)[8], const float* sC, bool two, int64_t Kp_pad) {
+  float2 ax[(LP1 + 1) / 2], ay[(LP1 + 1) / 2];
+  group8_pairs2<LP1>(x, y, sC, ax, ay);
+  if (rx) rows_store<LP1>(rx, gx, ax, two, Kp_pad);
+  if (ry) rows_store<LP1>(ry, gy, ay, two, Kp_pad);
+}
+
 // Warp units w0 .. w0 + kRowUnits - 1 (each a run of one row): all their loads are
 // issued before any arithmetic.
 // kArg: the caller has staged the kept vectors in sC.
-template <typename InT, bool kArg>
+template <typename InT, int LP1, bool kArg>
 __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* sC, float* sX) {
   const int lane = threadIdx.x & 31;
   const int64_t nrun = (J.NG + kRowRun - 1) / kRowRun;
   const int64_t units = J.M * nrun;
-  const int lp1 = J.lp1;
+  constexpr int lp1 = LP1;
   // The row of the first run; the next run is the next one of the row or the first of
   // the next row.  (A 64-bit division per run, twice, was more instructions than the
   // projection itself.)
@@ -224,19 +270,46 @@ __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* 
   for (int v = 0; v < kRowUnits; ++v) {
     const bool live = w0 + v < units;
     const int64_t i = live ? row_of(v) : 0, run = live ? w0 + v - i * nrun : 0;
-    const InT* a = static_cast<const InT*>(J.A) + i * J.lda + run * (8 * kRowRun);
+    const InT* __restrict__ a = static_cast<const InT*>(J.A) + i * J.lda + run * (8 * kRowRun);
     const int64_t left = J.K - run * (8 * kRowRun);
     const int nk = static_cast<int>(left < 8 * kRowRun ? left : 8 * kRowRun);
-    float* buf = bufs + v * kRowBuf;
+    float* buf = bufs + v * kRowBuf + lane;
+    a += lane;
+    if (live && nk == 8 * kRowRun) {   // a whole run: no test per load
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int e = s * 32 + lane;
-      buf[e + s] = live && e < nk ? load_as_float(a + e) : 0.0f;
+      for (int s = 0; s < 8; ++s) buf[s * 33] = load_as_float(a + s * 32);
+    } else {
+#pragma unroll
+      for (int s = 0; s < 8; ++s) buf[s * 33] = live && s * 32 + lane < nk ? load_as_float(a + s * 32) : 0.0f;
     }
   }
   if (!kArg) stage_coef8(sC, lp1, [&](int t, int q) { return J.Cs[t * lp1 + q]; });
   __syncthreads();
-  const bool odd_span = (lp1 == 3 || lp1 == 5 || lp1 == 6 || lp1 == 7) && !(J.nsplit > 1 && J.tl < lp1);
+  const bool tiered = J.nsplit > 1 && J.tl < lp1;
+  constexpr bool kOdd = LP1 == 3 || LP1 == 5 || LP1 == 6 || LP1 == 7;
+  if (!kOdd && !tiered) {
+    // both runs together
+    if (w0 >= units) return;
+    const bool live1 = w0 + 1 < units;
+    const int64_t i1 = row_of(1);
+    const int64_t g0 = r0 * kRowRun + lane, g1 = (w0 + 1 - i1 * nrun) * kRowRun + lane;
+    uint16_t* const row0 = J.Ac + i0 * J.pitch;
+    uint16_t* const row1 = J.Ac + i1 * J.pitch;
+    float x[8], y[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      x[t] = bufs[8 * lane + t + (lane >> 2)];
+      y[t] = bufs[kRowBuf + 8 * lane + t + (lane >> 2)];
+    }
+    uint16_t* const o0 = g0 < J.NG ? row0 : nullptr;
+    uint16_t* const o1 = live1 && g1 < J.NG ? row1 : nullptr;
+    const bool two = J.nsplit > 1;
+    rows_two<LP1>(o0, g0, x, o1, g1, y, sC, two, J.Kp_pad);
+    if (g0 == 0) zero_split_rows(row0, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+    if (live1 && g1 == 0) zero_split_rows(row1, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+    return;
+  }
+  const bool odd_span = kOdd && !tiered;
 #pragma unroll 1
   for (int v = 0; v < kRowUnits; ++v) {
     if (w0 + v >= units) break;
@@ -251,12 +324,7 @@ __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* 
       uint16_t* o0 = row + run * (kRowRun * lp1);
       const int64_t room = 2 * (J.Kp_pad - run * (kRowRun * lp1));
       uint16_t* st = reinterpret_cast<uint16_t*>(fbuf);
-      switch (lp1) {
-        case 3: rows_span_odd<3>(J, x, sC, st, o0, room, lane); break;
-        case 5: rows_span_odd<5>(J, x, sC, st, o0, room, lane); break;
-        case 6: rows_span_odd<6>(J, x, sC, st, o0, room, lane); break;
-        default: rows_span_odd<7>(J, x, sC, st, o0, room, lane); break;
-      }
+      if constexpr (kOdd) rows_span_odd<LP1>(J, x, sC, st, o0, room, lane);
       if (gg == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
       continue;
     }
@@ -266,16 +334,7 @@ __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* 
 #pragma unroll
     for (int t = 0; t < 8; ++t) x[t] = buf[8 * lane + t + (lane >> 2)];
     uint16_t* row = J.Ac + i * J.pitch;
-    switch (lp1) {   // the same for the whole block
-      case 1: rows_group8<1>(J, row, gg, x, sC); break;
-      case 2: rows_group8<2>(J, row, gg, x, sC); break;
-      case 3: rows_group8<3>(J, row, gg, x, sC); break;
-      case 4: rows_group8<4>(J, row, gg, x, sC); break;
-      case 5: rows_group8<5>(J, row, gg, x, sC); break;
-      case 6: rows_group8<6>(J, row, gg, x, sC); break;
-      case 7: rows_group8<7>(J, row, gg, x, sC); break;
-      default: rows_group8<8>(J, row, gg, x, sC); break;
-    }
+    rows_group8<LP1>(J, row, gg, x, sC);   // (a tiered split)
     if (gg == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
   }
 }
@@ -305,12 +364,14 @@ __device__ __forceinline__ void rows_body_any(const RowsJob& J, int64_t e, float
   if (gg == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
 }
 
-// Thread t of block b handles unit b * 256 + t (LT = 0), or warp units
-// (b * 8 + t / 32) * kRowUnits onwards (LT = 8).
-template <typename InT, int LT, bool kArg>
+// LP = 0: any group size, thread t of block b handles unit b * 256 + t; LP > 0: groups
+// of 8 with l+1 = LP, warp units (b * 8 + t / 32) * kRowUnits onwards.  One
+// instantiation per l+1: with a switch over all of them in one kernel the column paths
+// shared one register allocation and spilled.
+template <typename InT, int LP, bool kArg>
 __device__ __forceinline__ void rows_body(const RowsJob& J, int64_t b, float* sC, float* sX) {
-  if (LT == 8)
-    rows_body8<InT, kArg>(J, (b * 8 + (threadIdx.x >> 5)) * kRowUnits, sC, sX);
+  if constexpr (LP > 0)
+    rows_body8<InT, LP, kArg>(J, (b * 8 + (threadIdx.x >> 5)) * kRowUnits, sC, sX);
   else
     rows_body_any<InT>(J, b * blockDim.x + threadIdx.x, sC);
 }
@@ -329,23 +390,23 @@ __device__ __forceinline__ void side_begin(const SideArgs& a, float* sC) {
   if (a.clear && blockIdx.x == 0 && threadIdx.x == 0) *a.clear = 0;
 }
 
-template <typename InT, int LT, bool kArg>
-__global__ void __launch_bounds__(256) project_rows_kernel(const __grid_constant__ RowsJob J,
+template <typename InT, int LP, bool kArg>
+__global__ void __launch_bounds__(256, LP ? 4 : 1) project_rows_kernel(const __grid_constant__ RowsJob J,
                                                            const __grid_constant__ SideArgs a) {
-  __shared__ __align__(16) float sC[LT ? LT * LT : 64 * 64];
-  __shared__ float sX[LT == 8 ? 8 * kRowUnits * kRowBuf : 1];
+  __shared__ __align__(16) float sC[LP ? 64 : 64 * 64];
+  __shared__ float sX[LP ? 8 * kRowUnits * kRowBuf : 1];
   side_begin<kArg>(a, sC);
-  rows_body<InT, LT, kArg>(J, blockIdx.x, sC, sX);
+  rows_body<InT, LP, kArg>(J, blockIdx.x, sC, sX);
 }
 
-template <typename InT, int LT>
-__global__ void __launch_bounds__(256) project_rows_jobs_kernel(const RowsJob* __restrict__ jobs,
+template <typename InT, int LP>
+__global__ void __launch_bounds__(256, LP ? 4 : 1) project_rows_jobs_kernel(const RowsJob* __restrict__ jobs,
                                                                 const int* __restrict__ job_of) {
-  __shared__ __align__(16) float sC[LT ? LT * LT : 64 * 64];
-  __shared__ float sX[LT == 8 ? 8 * kRowUnits * kRowBuf : 1];
+  __shared__ __align__(16) float sC[LP ? 64 : 64 * 64];
+  __shared__ float sX[LP ? 8 * kRowUnits * kRowBuf : 1];
   pdl_begin();
-  const RowsJob& J = jobs[job_of[blockIdx.x]];
-  rows_body<InT, LT, false>(J, static_cast<int64_t>(blockIdx.x) - J.block0, sC, sX);
+  const RowsJob J = jobs[job_of[blockIdx.x]];   // a copy: read once, not again after every store
+  rows_body<InT, LP, false>(J, static_cast<int64_t>(blockIdx.x) - J.block0, sC, sX);
 }
 
 // ---- columns of B -> B_d stored transposed (N x pitch, K-major) -----------
@@ -368,17 +429,23 @@ __device__ __forceinline__ void cols_staged(const ColsJob& J, int64_t j, int64_t
   uint16_t* row = J.Bd + (live ? j : 0) * J.pitch;
   uint8_t* base = stage + (threadIdx.x >> 5) * 4096;
 #pragma unroll
-  for (int q = 0; q < kColGroups; ++q) {
-    float x8[8];
+  for (int q = 0; q < kColGroups; q += 2) {   // two groups per read of the basis values
+    float x8[8], y8[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) x8[t] = xa[q * 8 + t];
-    float2 acc[(LP1 + 1) / 2];
-    group8_pairs<LP1>(x8, sD, acc);
-    uint16_t hi[8], lo[8];
-    split_bf16<LP1>(acc, hi, lo);
-    run_put_group<LP1>(base, 128, 0, lane, q, hi);
-    if (two) run_put_group<LP1>(base, 128, 1, lane, q, lo);
-    if (tiered && live) store_split_part(row, g0 + q, hi, lo, LP1, J.tl, J.Kp_pad, J.Kt_pad, StoreUpto8{});
+    for (int t = 0; t < 8; ++t) {
+      x8[t] = xa[q * 8 + t];
+      y8[t] = xa[q * 8 + 8 + t];
+    }
+    float2 ax[(LP1 + 1) / 2], ay[(LP1 + 1) / 2];
+    group8_pairs2<LP1>(x8, y8, sD, ax, ay);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint16_t hi[8], lo[8];
+      split_bf16<LP1>(h ? ay : ax, hi, lo);
+      run_put_group<LP1>(base, 128, 0, lane, q + h, hi);
+      if (two) run_put_group<LP1>(base, 128, 1, lane, q + h, lo);
+      if (tiered && live) store_split_part(row, g0 + q + h, hi, lo, LP1, J.tl, J.Kp_pad, J.Kt_pad, StoreUpto8{});
+    }
   }
   __syncwarp();
   const int64_t jw = j - lane;
@@ -389,37 +456,58 @@ __device__ __forceinline__ void cols_staged(const ColsJob& J, int64_t j, int64_t
   if (g0 == 0 && live) zero_split_rows(row, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
 }
 
-// L = 8, l+1 in {3, 5, 6, 7}, four whole groups, no tiered split: the 4 (l+1)
-// components of the column's groups packed into words and stored as (l+1) 8-byte
-// chunks (the run starts 8 (l+1) qd bytes into the row).
+// L = 8, l+1 in {3, 5, 6, 7}, four whole groups, no tiered split: a column's run of
+// 4 (l+1) components (8 (l+1) bytes of its row) packed into words, staged in the warp's
+// area (2 KB per part; runs an odd number of 8 bytes apart, so the lanes' words fall in
+// different banks but for pairs) and written by the warp run after run, in 8-byte
+// chunks.  Stored by the lanes themselves, every chunk went to 32 rows at once and the
+// words of all four groups were held in registers and spilled.  Every lane of the warp
+// takes part; columns past N are not written back.
 template <int LP1>
-__device__ __forceinline__ void cols_quad_odd(const ColsJob& J, uint16_t* row, int64_t g0,
-                                              const float (&xa)[kColGroups * 8], const float* sD) {
-  uint32_t wh[2 * LP1], wl[2 * LP1];
+__device__ __forceinline__ void cols_quad_odd(const ColsJob& J, int64_t j, int64_t g0,
+                                              const float (&xa)[kColGroups * 8], const float* sD, uint8_t* stage) {
+  constexpr int kPitch = 8 * (LP1 | 1);
+  static_assert(32 * kPitch <= 2048, "the runs of a warp fit their area");
+  const int lane = threadIdx.x & 31;
+  const bool two = J.nsplit > 1;
+  uint8_t* base = stage + (threadIdx.x >> 5) * 4096;
 #pragma unroll
-  for (int k = 0; k < 2 * LP1; ++k) wh[k] = wl[k] = 0u;
+  for (int q = 0; q < kColGroups; q += 2) {
+    float x8[8], y8[8];
 #pragma unroll
-  for (int q = 0; q < kColGroups; ++q) {
-    float x8[8];
+    for (int t = 0; t < 8; ++t) {
+      x8[t] = xa[q * 8 + t];
+      y8[t] = xa[q * 8 + 8 + t];
+    }
+    float2 ax[(LP1 + 1) / 2], ay[(LP1 + 1) / 2];
+    group8_pairs2<LP1>(x8, y8, sD, ax, ay);
+    uint16_t hx[8], lx[8], hy[8], ly[8];
+    split_bf16<LP1>(ax, hx, lx);
+    split_bf16<LP1>(ay, hy, ly);
+    uint32_t* wh = reinterpret_cast<uint32_t*>(base + lane * kPitch + q * 2 * LP1);
+    uint32_t* wl = wh + 2048 / 4;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) x8[t] = xa[q * 8 + t];
-    float2 acc[(LP1 + 1) / 2];
-    group8_pairs<LP1>(x8, sD, acc);
-    uint16_t hi[8], lo[8];
-    split_bf16<LP1>(acc, hi, lo);
-#pragma unroll
-    for (int p = 0; p < LP1; ++p) {
-      const int e = q * LP1 + p;
-      wh[e >> 1] |= uint32_t(hi[p]) << (16 * (e & 1));
-      wl[e >> 1] |= uint32_t(lo[p]) << (16 * (e & 1));
+    for (int k = 0; k < LP1; ++k) {   // word k: components 2k and 2k + 1 of the two groups' 2 (l+1)
+      const int a = 2 * k, b = 2 * k + 1;
+      wh[k] = (a < LP1 ? hx[a % 8] : hy[(a + 8 - LP1) % 8]) | (uint32_t(b < LP1 ? hx[b % 8] : hy[(b + 8 - LP1) % 8]) << 16);
+      if (two)
+        wl[k] = (a < LP1 ? lx[a % 8] : ly[(a + 8 - LP1) % 8]) |
+                (uint32_t(b < LP1 ? lx[b % 8] : ly[(b + 8 - LP1) % 8]) << 16);
     }
   }
-  uint16_t* o = row + g0 * LP1;
+  __syncwarp();
+  const int64_t jw = j - lane;
+  const int ncols = J.N - jw < 32 ? static_cast<int>(J.N - jw) : 32;
+  uint16_t* o0 = J.Bd + jw * J.pitch + g0 * LP1;
+  for (int part = 0; part < (two ? 2 : 1); ++part)
 #pragma unroll
-  for (int k = 0; k < LP1; ++k) reinterpret_cast<uint2*>(o)[k] = make_uint2(wh[2 * k], wh[2 * k + 1]);
-  if (J.nsplit > 1)
-#pragma unroll
-    for (int k = 0; k < LP1; ++k) reinterpret_cast<uint2*>(o + J.Kp_pad)[k] = make_uint2(wl[2 * k], wl[2 * k + 1]);
+    for (int s = 0; s < LP1; ++s) {
+      const int gi = s * 32 + lane, c = gi / LP1, k = gi - c * LP1;
+      if (c < ncols)
+        *reinterpret_cast<uint2*>(o0 + part * J.Kp_pad + c * J.pitch + k * 4) =
+            *reinterpret_cast<const uint2*>(base + part * 2048 + c * kPitch + k * 8);
+    }
+  if (g0 == 0 && j < J.N) zero_split_rows(J.Bd + j * J.pitch, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
 }
 
 // L = 8, unstaged: group gg of one column, l+1 components.
@@ -434,18 +522,24 @@ __device__ __forceinline__ void col_group8(const ColsJob& J, uint16_t* row, int6
   if (J.nsplit > 1) store_split_part(row, gg, hi, lo, LP1, J.tl, J.Kp_pad, J.Kt_pad, StoreUpto8{});
 }
 
-template <typename InT, int LT, bool kArg>
+template <typename InT, int LP, bool kArg>
 __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t qd, float* sD, uint8_t* stage) {
-  constexpr int LMAX = LT ? LT : 64;
-  const int L = LT ? LT : J.L;
-  const int lp1 = J.lp1;
+  constexpr int LMAX = LP ? 8 : 64;
+  const int L = LP ? 8 : J.L;
+  const int lp1 = LP ? LP : J.lp1;
   const bool live = j < J.N;
   const InT* B = static_cast<const InT*>(J.B);
   const int64_t g0 = qd * kColGroups;
   const int ng = static_cast<int>(J.NG - g0 < kColGroups ? J.NG - g0 : kColGroups);
   // L = 8: all kColGroups * 8 inputs are loaded before the staging barrier.
-  float xa[LT == 8 ? kColGroups * 8 : 1];
-  if (LT == 8) {
+  float xa[LP ? kColGroups * 8 : 1];
+  if (LP && (g0 + kColGroups) * 8 <= J.K) {
+    // whole groups: no test per load (a column past N reads the last one, and is not written)
+    const InT* __restrict__ b = B + g0 * 8 * J.ldb + (live ? j : J.N - 1);
+    const int64_t ldb = J.ldb;
+#pragma unroll
+    for (int e = 0; e < (LP ? kColGroups * 8 : 1); ++e, b += ldb) xa[e] = load_as_float(b);
+  } else if (LP) {
 #pragma unroll
     for (int q = 0; q < kColGroups; ++q) {
       const int64_t k0 = (g0 + q) * 8;
@@ -455,49 +549,33 @@ __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t q
     }
   }
   if (kArg) {
-  } else if (LT == 8)
+  } else if (LP)
     stage_coef8(sD, lp1, [&](int t, int q) { return J.Ds[q * 8 + t]; });
   else
     for (int k = threadIdx.x; k < L * lp1; k += blockDim.x) sD[k] = J.Ds[k];
   __syncthreads();
-  if constexpr (LT == 8) {
-    if (ng == kColGroups && (lp1 == 8 || lp1 == 4)) {  // the same for the whole block
-      if (lp1 == 8)
-        cols_staged<8>(J, j, g0, xa, sD, stage);
-      else
-        cols_staged<4>(J, j, g0, xa, sD, stage);
+  if constexpr (LP == 4 || LP == 8) {
+    if (ng == kColGroups) {  // the same for the whole block
+      cols_staged<LP>(J, j, g0, xa, sD, stage);
+      return;
+    }
+  }
+  if constexpr (LP == 3 || LP == 5 || LP == 6 || LP == 7) {
+    if (ng == kColGroups && !(J.nsplit > 1 && J.tl < LP)) {
+      cols_quad_odd<LP>(J, j, g0, xa, sD, stage);
       return;
     }
   }
   if (!live) return;
   uint16_t* row = J.Bd + j * J.pitch;
-  if constexpr (LT == 8) {
-    if (ng == kColGroups && (lp1 == 3 || lp1 == 5 || lp1 == 6 || lp1 == 7) && !(J.nsplit > 1 && J.tl < lp1)) {
-      switch (lp1) {
-        case 3: cols_quad_odd<3>(J, row, g0, xa, sD); break;
-        case 5: cols_quad_odd<5>(J, row, g0, xa, sD); break;
-        case 6: cols_quad_odd<6>(J, row, g0, xa, sD); break;
-        default: cols_quad_odd<7>(J, row, g0, xa, sD); break;
-      }
-      if (qd == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
-      return;
-    }
+  if constexpr (LP > 0) {
 #pragma unroll
     for (int q = 0; q < kColGroups; ++q) {
       if (q >= ng) break;
       float x8[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) x8[t] = xa[(q * 8 + t) % (LT == 8 ? kColGroups * 8 : 1)];
-      switch (lp1) {   // the same for the whole block
-        case 1: col_group8<1>(J, row, g0 + q, x8, sD); break;
-        case 2: col_group8<2>(J, row, g0 + q, x8, sD); break;
-        case 3: col_group8<3>(J, row, g0 + q, x8, sD); break;
-        case 4: col_group8<4>(J, row, g0 + q, x8, sD); break;
-        case 5: col_group8<5>(J, row, g0 + q, x8, sD); break;
-        case 6: col_group8<6>(J, row, g0 + q, x8, sD); break;
-        case 7: col_group8<7>(J, row, g0 + q, x8, sD); break;
-        default: col_group8<8>(J, row, g0 + q, x8, sD); break;
-      }
+      for (int t = 0; t < 8; ++t) x8[t] = xa[(q * 8 + t) % (LP ? kColGroups * 8 : 1)];
+      col_group8<LP>(J, row, g0 + q, x8, sD);
     }
   } else {
     for (int q = 0; q < ng; ++q) {
@@ -522,25 +600,25 @@ __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t q
   if (qd == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
 }
 
-template <typename InT, int LT, bool kArg>
-__global__ void __launch_bounds__(256, LT == 8 ? 3 : 2) project_cols_kernel(const __grid_constant__ ColsJob J,
+template <typename InT, int LP, bool kArg>
+__global__ void __launch_bounds__(256, LP == 7 ? 2 : LP ? 3 : 2) project_cols_kernel(const __grid_constant__ ColsJob J,
                                                                             const __grid_constant__ SideArgs a) {
-  __shared__ __align__(16) float sD[LT ? LT * LT : 64 * 64];
-  __shared__ __align__(16) uint8_t sStage[LT == 8 ? 8 * 4096 : 16];
+  __shared__ __align__(16) float sD[LP ? 64 : 64 * 64];
+  __shared__ __align__(16) uint8_t sStage[LP ? 8 * 4096 : 16];
   side_begin<kArg>(a, sD);
   const uint32_t b = blockIdx.x, nbx = static_cast<uint32_t>(J.nbx);
-  cols_body<InT, LT, kArg>(J, static_cast<int64_t>(b % nbx) * blockDim.x + threadIdx.x, b / nbx, sD, sStage);
+  cols_body<InT, LP, kArg>(J, static_cast<int64_t>(b % nbx) * blockDim.x + threadIdx.x, b / nbx, sD, sStage);
 }
 
-template <typename InT, int LT>
-__global__ void __launch_bounds__(256, LT == 8 ? 3 : 2) project_cols_jobs_kernel(const ColsJob* __restrict__ jobs,
+template <typename InT, int LP>
+__global__ void __launch_bounds__(256, LP == 7 ? 2 : LP ? 3 : 2) project_cols_jobs_kernel(const ColsJob* __restrict__ jobs,
                                                                 const int* __restrict__ job_of) {
-  __shared__ __align__(16) float sD[LT ? LT * LT : 64 * 64];
-  __shared__ __align__(16) uint8_t sStage[LT == 8 ? 8 * 4096 : 16];
+  __shared__ __align__(16) float sD[LP ? 64 : 64 * 64];
+  __shared__ __align__(16) uint8_t sStage[LP ? 8 * 4096 : 16];
   pdl_begin();
-  const ColsJob& J = jobs[job_of[blockIdx.x]];
+  const ColsJob J = jobs[job_of[blockIdx.x]];   // (as for rows)
   const uint32_t b = blockIdx.x - static_cast<uint32_t>(J.block0), nbx = static_cast<uint32_t>(J.nbx);
-  cols_body<InT, LT, false>(J, static_cast<int64_t>(b % nbx) * blockDim.x + threadIdx.x, b / nbx, sD, sStage);
+  cols_body<InT, LP, false>(J, static_cast<int64_t>(b % nbx) * blockDim.x + threadIdx.x, b / nbx, sD, sStage);
 }
 
 // ---- FP64 path ------------------------------------------------------------
@@ -961,7 +1039,27 @@ int64_t rows_job_blocks(const RowsJob& J) {
 }
 int64_t cols_job_blocks(const ColsJob& J) { return J.nbx * ceil_div(J.NG, kColGroups); }
 
-int projection_class(int in_bf16, int L) { return (in_bf16 ? 2 : 0) + (L == 8 ? 1 : 0); }
+int projection_class(int in_bf16, int L, int lp1) { return (in_bf16 ? 9 : 0) + (L == 8 ? lp1 : 0); }
+
+// f(InT value, std::integral_constant<int, LP>) for the kernels of one class.
+template <typename InT, typename F>
+static cudaError_t with_lp(int lp, F f) {
+  switch (lp) {
+    case 0: return f(InT(), std::integral_constant<int, 0>());
+    case 1: return f(InT(), std::integral_constant<int, 1>());
+    case 2: return f(InT(), std::integral_constant<int, 2>());
+    case 3: return f(InT(), std::integral_constant<int, 3>());
+    case 4: return f(InT(), std::integral_constant<int, 4>());
+    case 5: return f(InT(), std::integral_constant<int, 5>());
+    case 6: return f(InT(), std::integral_constant<int, 6>());
+    case 7: return f(InT(), std::integral_constant<int, 7>());
+    default: return f(InT(), std::integral_constant<int, 8>());
+  }
+}
+template <typename F>
+static cudaError_t with_class(int cls, F f) {
+  return cls >= 9 ? with_lp<__nv_bfloat16>(cls - 9, f) : with_lp<float>(cls, f);
+}
 
 cudaError_t launch_project_pair_simt(const void* A, int64_t lda, const void* B, int64_t ldb, int in_dtype,
                                      const GemmGeom& g, const float* Cs, const float* Ds, const Coef8* c8,
@@ -975,50 +1073,40 @@ cudaError_t launch_project_pair_simt(const void* A, int64_t lda, const void* B, 
   if (rows) {
     const RowsJob J = make_rows_job(A, lda, in_dtype, g, Cs, Ac);
     const dim3 grid(static_cast<unsigned>(rows_job_blocks(J)));
-    void (*kern)(RowsJob, SideArgs) = nullptr;
-    switch (projection_class(J.in_bf16, J.L)) {
-      case 0: kern = project_rows_kernel<float, 0, false>; break;
-      case 1: kern = c8 ? project_rows_kernel<float, 8, true> : project_rows_kernel<float, 8, false>; break;
-      case 2: kern = project_rows_kernel<__nv_bfloat16, 0, false>; break;
-      default: kern = c8 ? project_rows_kernel<__nv_bfloat16, 8, true> : project_rows_kernel<__nv_bfloat16, 8, false>;
-    }
-    const cudaError_t e = launch_plain(kern, grid, 256, 0, st, J, a);
+    const cudaError_t e = with_class(projection_class(J.in_bf16, J.L, J.lp1), [&](auto in, auto lp) {
+      using InT = decltype(in);
+      constexpr int LP = decltype(lp)::value;
+      return launch_plain(c8 ? project_rows_kernel<InT, LP, (LP > 0)> : project_rows_kernel<InT, LP, false>, grid, 256, 0,
+                          st, J, a);
+    });
     if (e != cudaSuccess) return e;
     a.clear = nullptr;
   }
   if (!cols) return cudaSuccess;
   const ColsJob J = make_cols_job(B, ldb, in_dtype, g, Ds, Bd);
   const dim3 grid(static_cast<unsigned>(cols_job_blocks(J)));
-  void (*kern)(ColsJob, SideArgs) = nullptr;
-  switch (projection_class(J.in_bf16, J.L)) {
-    case 0: kern = project_cols_kernel<float, 0, false>; break;
-    case 1: kern = c8 ? project_cols_kernel<float, 8, true> : project_cols_kernel<float, 8, false>; break;
-    case 2: kern = project_cols_kernel<__nv_bfloat16, 0, false>; break;
-    default: kern = c8 ? project_cols_kernel<__nv_bfloat16, 8, true> : project_cols_kernel<__nv_bfloat16, 8, false>;
-  }
-  return launch_plain(kern, grid, 256, 0, st, J, a);
+  return with_class(projection_class(J.in_bf16, J.L, J.lp1), [&](auto in, auto lp) {
+    using InT = decltype(in);
+    constexpr int LP = decltype(lp)::value;
+    return launch_plain(c8 ? project_cols_kernel<InT, LP, (LP > 0)> : project_cols_kernel<InT, LP, false>, grid, 256, 0,
+                        st, J, a);
+  });
 }
 
 cudaError_t launch_project_rows_jobs(int cls, const RowsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st) {
   if (blocks == 0) return cudaSuccess;
   const unsigned nb = static_cast<unsigned>(blocks);
-  switch (cls) {
-    case 0: return launch_plain(project_rows_jobs_kernel<float, 0>, dim3(nb), 256, 0, st, jobs, job_of);
-    case 1: return launch_plain(project_rows_jobs_kernel<float, 8>, dim3(nb), 256, 0, st, jobs, job_of);
-    case 2: return launch_plain(project_rows_jobs_kernel<__nv_bfloat16, 0>, dim3(nb), 256, 0, st, jobs, job_of);
-    default: return launch_plain(project_rows_jobs_kernel<__nv_bfloat16, 8>, dim3(nb), 256, 0, st, jobs, job_of);
-  }
+  return with_class(cls, [&](auto in, auto lp) {
+    return launch_plain(project_rows_jobs_kernel<decltype(in), decltype(lp)::value>, dim3(nb), 256, 0, st, jobs, job_of);
+  });
 }
 
 cudaError_t launch_project_cols_jobs(int cls, const ColsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st) {
   if (blocks == 0) return cudaSuccess;
   const unsigned nb = static_cast<unsigned>(blocks);
-  switch (cls) {
-    case 0: return launch_plain(project_cols_jobs_kernel<float, 0>, dim3(nb), 256, 0, st, jobs, job_of);
-    case 1: return launch_plain(project_cols_jobs_kernel<float, 8>, dim3(nb), 256, 0, st, jobs, job_of);
-    case 2: return launch_plain(project_cols_jobs_kernel<__nv_bfloat16, 0>, dim3(nb), 256, 0, st, jobs, job_of);
-    default: return launch_plain(project_cols_jobs_kernel<__nv_bfloat16, 8>, dim3(nb), 256, 0, st, jobs, job_of);
-  }
+  return with_class(cls, [&](auto in, auto lp) {
+    return launch_plain(project_cols_jobs_kernel<decltype(in), decltype(lp)::value>, dim3(nb), 256, 0, st, jobs, job_of);
+  });
 }
 
 
