@@ -210,6 +210,7 @@ struct RowsJob {
   const float* Cs;
   int64_t lda, M, K, NG, pitch, Kp_pad, block0, Kt_pad;
   int L, lp1, nsplit, in_bf16, tl;
+  int upw;   // L = 8: runs (32 groups of a row) per warp, even
 };
 struct ColsJob {
   const void* B;

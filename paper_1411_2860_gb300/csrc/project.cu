@@ -5,6 +5,7 @@
 // These kernels stream HBM; the arithmetic is FP32 (FP64 for the double path).
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "common.hpp"
@@ -100,6 +101,20 @@ __device__ __forceinline__ void zero_split_rows(uint16_t* row, int64_t NG, int l
   } else {
     for (int sg = 0; sg < nsplit; ++sg) zero_run(row + sg * Kp_pad, NG * lp1, Kp_pad);
   }
+}
+
+// 4-byte asynchronous copy global -> shared (bytes = 4, or 0 to write zeros).
+__device__ __forceinline__ void cp_async4(float* dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Waits until at most N of this thread's groups are pending.
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // ---- L = 8: components in pairs ------------------------------------------
@@ -250,92 +265,114 @@ __device__ __forceinline__ void rows_two(uint16_t* rx, int64_t gx, const float (
   if (ry) rows_store<LP1>(ry, gy, ay, two, Kp_pad);
 }
 
-// Warp units w0 .. w0 + kRowUnits - 1 (each a run of one row): all their loads are
-// issued before any arithmetic.
-// kArg: the caller has staged the kept vectors in sC.
+// Projects and stores run `run` of row i from buffer `buf` and, when live1, run `run1` of
+// row i1 from buf1 (which may be overwritten).  Every lane of the warp takes part.
+template <int LP1>
+__device__ __forceinline__ void rows_two_runs(const RowsJob& J, int64_t i, int64_t run, float* buf, bool live1,
+                                              int64_t i1, int64_t run1, float* buf1, const float* sC) {
+  const int lane = threadIdx.x & 31;
+  const int64_t g0 = run * kRowRun + lane, g1 = run1 * kRowRun + lane;
+  uint16_t* const row0 = J.Ac + i * J.pitch;
+  uint16_t* const row1 = J.Ac + i1 * J.pitch;
+  const bool tiered = J.nsplit > 1 && J.tl < LP1;
+  constexpr bool kOdd = LP1 == 3 || LP1 == 5 || LP1 == 6 || LP1 == 7;
+  float x[8], y[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    x[t] = buf[8 * lane + t + (lane >> 2)];
+    y[t] = buf1[8 * lane + t + (lane >> 2)];
+  }
+  if (tiered) {
+    if (g0 < J.NG) rows_group8<LP1>(J, row0, g0, x, sC);
+    if (live1 && g1 < J.NG) rows_group8<LP1>(J, row1, g1, y, sC);
+  } else if constexpr (kOdd) {
+    rows_span_odd<LP1>(J, x, sC, reinterpret_cast<uint16_t*>(buf), row0 + run * (kRowRun * LP1),
+                       2 * (J.Kp_pad - run * (kRowRun * LP1)), lane);
+    if (live1)   // the same for the whole warp
+      rows_span_odd<LP1>(J, y, sC, reinterpret_cast<uint16_t*>(buf1), row1 + run1 * (kRowRun * LP1),
+                         2 * (J.Kp_pad - run1 * (kRowRun * LP1)), lane);
+  } else {
+    rows_two<LP1>(g0 < J.NG ? row0 : nullptr, g0, x, live1 && g1 < J.NG ? row1 : nullptr, g1, y, sC, J.nsplit > 1,
+                  J.Kp_pad);
+  }
+  if (g0 == 0) zero_split_rows(row0, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+  if (live1 && g1 == 0) zero_split_rows(row1, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+}
+
+// The runs of one warp, w0 .. w0 + n - 1 (consecutive runs of a row, then of the next),
+// two at a time.  FP32: a ring of kRowRing pairs filled by 4-byte asynchronous copies
+// (rows start anywhere, and the copies need no registers), so a warp keeps two pairs in
+// flight while it projects a third.  With one pair per warp, loaded, projected and
+// stored before the block left, the kernel moved 0.56 of the copy rate however few
+// instructions it took.  BF16 (rows may start at odd 2-byte offsets): plain loads, one
+// pair at a time.
+constexpr int kRowRing = 3;
+constexpr int kRowsSmem = 8 * kRowRing * kRowUnits * kRowBuf * 4;   // bytes a block of either kind reserves (L = 8)
+
 template <typename InT, int LP1, bool kArg>
 __device__ __forceinline__ void rows_body8(const RowsJob& J, int64_t w0, float* sC, float* sX) {
+  static_assert(kRowUnits == 2, "runs go in pairs");
+  constexpr bool kAsync = sizeof(InT) == 4;
   const int lane = threadIdx.x & 31;
   const int64_t nrun = (J.NG + kRowRun - 1) / kRowRun;
   const int64_t units = J.M * nrun;
-  constexpr int lp1 = LP1;
-  // The row of the first run; the next run is the next one of the row or the first of
-  // the next row.  (A 64-bit division per run, twice, was more instructions than the
-  // projection itself.)
-  const int64_t i0 = units < (int64_t(1) << 32) ? static_cast<uint32_t>(w0) / static_cast<uint32_t>(nrun) : w0 / nrun;
-  const int64_t r0 = w0 - i0 * nrun;
-  auto row_of = [&](int v) { return i0 + (r0 + v >= nrun ? 1 : 0); };
-  float* bufs = sX + (threadIdx.x >> 5) * (kRowUnits * kRowBuf);
-#pragma unroll
-  for (int v = 0; v < kRowUnits; ++v) {
-    const bool live = w0 + v < units;
-    const int64_t i = live ? row_of(v) : 0, run = live ? w0 + v - i * nrun : 0;
-    const InT* __restrict__ a = static_cast<const InT*>(J.A) + i * J.lda + run * (8 * kRowRun);
-    const int64_t left = J.K - run * (8 * kRowRun);
+  const int n = static_cast<int>(units - w0 < J.upw ? (units > w0 ? units - w0 : 0) : J.upw);
+  // (one 32-bit division per warp: 64-bit ones per run were more instructions than the
+  // projection itself)
+  int64_t li = units < (int64_t(1) << 32) ? static_cast<uint32_t>(w0) / static_cast<uint32_t>(nrun) : w0 / nrun;
+  int64_t lr = w0 - li * nrun;      // the next run to load ...
+  int64_t pi = li, pr = lr;         // ... and to project
+  float* const bufs = sX + (threadIdx.x >> 5) * (kRowRing * kRowUnits * kRowBuf);
+  auto load_run = [&](float* buf, bool live) {
+    const InT* a = static_cast<const InT*>(J.A) + (live ? li * J.lda + lr * (8 * kRowRun) : 0);
+    const int64_t left = live ? J.K - lr * (8 * kRowRun) : 0;
     const int nk = static_cast<int>(left < 8 * kRowRun ? left : 8 * kRowRun);
-    float* buf = bufs + v * kRowBuf + lane;
-    a += lane;
-    if (live && nk == 8 * kRowRun) {   // a whole run: no test per load
 #pragma unroll
-      for (int s = 0; s < 8; ++s) buf[s * 33] = load_as_float(a + s * 32);
-    } else {
-#pragma unroll
-      for (int s = 0; s < 8; ++s) buf[s * 33] = live && s * 32 + lane < nk ? load_as_float(a + s * 32) : 0.0f;
+    for (int s = 0; s < 8; ++s) {
+      const bool in = s * 32 + lane < nk;
+      if constexpr (kAsync)
+        cp_async4(buf + s * 33 + lane, in ? a + s * 32 + lane : a, in ? 4 : 0);
+      else
+        buf[s * 33 + lane] = in ? load_as_float(a + s * 32 + lane) : 0.0f;
     }
-  }
-  if (!kArg) stage_coef8(sC, lp1, [&](int t, int q) { return J.Cs[t * lp1 + q]; });
+    if (++lr == nrun) {
+      lr = 0;
+      ++li;
+    }
+  };
+  auto load_pair = [&](int k) {   // runs 2k and 2k + 1 into ring slot k % kRowRing
+    if (2 * k < n) {
+      float* b = bufs + (k % kRowRing) * (kRowUnits * kRowBuf);
+      load_run(b, true);
+      load_run(b + kRowBuf, 2 * k + 1 < n);
+    }
+    if constexpr (kAsync) cp_async_commit();
+  };
+  if constexpr (kAsync)
+    for (int k = 0; k < kRowRing - 1; ++k) load_pair(k);
+  if (!kArg) stage_coef8(sC, LP1, [&](int t, int q) { return J.Cs[t * LP1 + q]; });
   __syncthreads();
-  const bool tiered = J.nsplit > 1 && J.tl < lp1;
-  constexpr bool kOdd = LP1 == 3 || LP1 == 5 || LP1 == 6 || LP1 == 7;
-  if (!kOdd && !tiered) {
-    // both runs together
-    if (w0 >= units) return;
-    const bool live1 = w0 + 1 < units;
-    const int64_t i1 = row_of(1);
-    const int64_t g0 = r0 * kRowRun + lane, g1 = (w0 + 1 - i1 * nrun) * kRowRun + lane;
-    uint16_t* const row0 = J.Ac + i0 * J.pitch;
-    uint16_t* const row1 = J.Ac + i1 * J.pitch;
-    float x[8], y[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      x[t] = bufs[8 * lane + t + (lane >> 2)];
-      y[t] = bufs[kRowBuf + 8 * lane + t + (lane >> 2)];
-    }
-    uint16_t* const o0 = g0 < J.NG ? row0 : nullptr;
-    uint16_t* const o1 = live1 && g1 < J.NG ? row1 : nullptr;
-    const bool two = J.nsplit > 1;
-    rows_two<LP1>(o0, g0, x, o1, g1, y, sC, two, J.Kp_pad);
-    if (g0 == 0) zero_split_rows(row0, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
-    if (live1 && g1 == 0) zero_split_rows(row1, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
-    return;
-  }
-  const bool odd_span = kOdd && !tiered;
 #pragma unroll 1
-  for (int v = 0; v < kRowUnits; ++v) {
-    if (w0 + v >= units) break;
-    const int64_t i = row_of(v), run = w0 + v - i * nrun;
-    const int64_t gg = run * kRowRun + lane;
-    if (odd_span) {   // the same for the whole warp
-      float* fbuf = bufs + v * kRowBuf;
-      float x[8];
-#pragma unroll
-      for (int t = 0; t < 8; ++t) x[t] = fbuf[8 * lane + t + (lane >> 2)];
-      uint16_t* row = J.Ac + i * J.pitch;
-      uint16_t* o0 = row + run * (kRowRun * lp1);
-      const int64_t room = 2 * (J.Kp_pad - run * (kRowRun * lp1));
-      uint16_t* st = reinterpret_cast<uint16_t*>(fbuf);
-      if constexpr (kOdd) rows_span_odd<LP1>(J, x, sC, st, o0, room, lane);
-      if (gg == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
-      continue;
+  for (int k = 0; 2 * k < n; ++k) {
+    if constexpr (kAsync) {
+      load_pair(k + kRowRing - 1);   // into the slot projected last
+      cp_async_wait<kRowRing - 1>();
+    } else {
+      load_pair(k);
     }
-    if (gg >= J.NG) continue;
-    const float* buf = bufs + v * kRowBuf;
-    float x[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) x[t] = buf[8 * lane + t + (lane >> 2)];
-    uint16_t* row = J.Ac + i * J.pitch;
-    rows_group8<LP1>(J, row, gg, x, sC);   // (a tiered split)
-    if (gg == 0) zero_split_rows(row, J.NG, lp1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+    __syncwarp();
+    const int64_t i0 = pi, r0 = pr;
+    if (++pr == nrun) {
+      pr = 0;
+      ++pi;
+    }
+    float* b = bufs + (k % kRowRing) * (kRowUnits * kRowBuf);
+    rows_two_runs<LP1>(J, i0, r0, b, 2 * k + 1 < n, pi, pr, b + kRowBuf, sC);
+    if (++pr == nrun) {
+      pr = 0;
+      ++pi;
+    }
+    __syncwarp();   // the pair's buffers are read
   }
 }
 
@@ -365,13 +402,13 @@ __device__ __forceinline__ void rows_body_any(const RowsJob& J, int64_t e, float
 }
 
 // LP = 0: any group size, thread t of block b handles unit b * 256 + t; LP > 0: groups
-// of 8 with l+1 = LP, warp units (b * 8 + t / 32) * kRowUnits onwards.  One
+// of 8 with l+1 = LP, warp units (b * 8 + t / 32) * upw onwards.  One
 // instantiation per l+1: with a switch over all of them in one kernel the column paths
 // shared one register allocation and spilled.
 template <typename InT, int LP, bool kArg>
 __device__ __forceinline__ void rows_body(const RowsJob& J, int64_t b, float* sC, float* sX) {
   if constexpr (LP > 0)
-    rows_body8<InT, LP, kArg>(J, (b * 8 + (threadIdx.x >> 5)) * kRowUnits, sC, sX);
+    rows_body8<InT, LP, kArg>(J, (b * 8 + (threadIdx.x >> 5)) * J.upw, sC, sX);
   else
     rows_body_any<InT>(J, b * blockDim.x + threadIdx.x, sC);
 }
@@ -394,7 +431,7 @@ template <typename InT, int LP, bool kArg>
 __global__ void __launch_bounds__(256, LP ? 4 : 1) project_rows_kernel(const __grid_constant__ RowsJob J,
                                                            const __grid_constant__ SideArgs a) {
   __shared__ __align__(16) float sC[LP ? 64 : 64 * 64];
-  __shared__ float sX[LP ? 8 * kRowUnits * kRowBuf : 1];
+  extern __shared__ __align__(16) float sX[];   // kRowsSmem bytes for groups of 8
   side_begin<kArg>(a, sC);
   rows_body<InT, LP, kArg>(J, blockIdx.x, sC, sX);
 }
@@ -403,7 +440,7 @@ template <typename InT, int LP>
 __global__ void __launch_bounds__(256, LP ? 4 : 1) project_rows_jobs_kernel(const RowsJob* __restrict__ jobs,
                                                                 const int* __restrict__ job_of) {
   __shared__ __align__(16) float sC[LP ? 64 : 64 * 64];
-  __shared__ float sX[LP ? 8 * kRowUnits * kRowBuf : 1];
+  extern __shared__ __align__(16) float sX[];   // kRowsSmem bytes for groups of 8
   pdl_begin();
   const RowsJob J = jobs[job_of[blockIdx.x]];   // a copy: read once, not again after every store
   rows_body<InT, LP, false>(J, static_cast<int64_t>(blockIdx.x) - J.block0, sC, sX);
@@ -1010,6 +1047,10 @@ RowsJob make_rows_job(const void* A, int64_t lda, int in_dtype, const GemmGeom& 
   J.lp1 = g.lp1;
   J.nsplit = g.nsplit;
   J.in_bf16 = in_dtype == PJ_BF16;
+  // Runs per warp: eight where that leaves the chip full (152 SMs x 4 blocks x 8 warps),
+  // fewer for small operands; BF16 input loads one pair at a time, so its warps take one.
+  const int64_t units = J.M * ceil_div(J.NG, kRowRun), warps = 152 * 32;
+  J.upw = J.in_bf16 || units <= 2 * warps ? 2 : (units >= 8 * warps ? 8 : static_cast<int>(units / warps / 2 * 2));
   return J;
 }
 
@@ -1035,7 +1076,7 @@ ColsJob make_cols_job(const void* B, int64_t ldb, int in_dtype, const GemmGeom& 
 }
 
 int64_t rows_job_blocks(const RowsJob& J) {
-  return J.L == 8 ? ceil_div(J.M * ceil_div(J.NG, kRowRun), 8 * kRowUnits) : ceil_div(J.M * J.NG, 256);
+  return J.L == 8 ? ceil_div(J.M * ceil_div(J.NG, kRowRun), 8 * J.upw) : ceil_div(J.M * J.NG, 256);
 }
 int64_t cols_job_blocks(const ColsJob& J) { return J.nbx * ceil_div(J.NG, kColGroups); }
 
@@ -1055,6 +1096,30 @@ static cudaError_t with_lp(int lp, F f) {
     case 7: return f(InT(), std::integral_constant<int, 7>());
     default: return f(InT(), std::integral_constant<int, 8>());
   }
+}
+// The shared-memory opt-in of a row kernel (a block's static share is added to the ring:
+// above 48 KB), recorded per kernel and device; a racing repeat is harmless.
+template <typename K>
+static cudaError_t rows_smem(K* kern, int smem) {
+  static std::atomic<const void*> done[64][80] = {};
+  if (smem == 0) return cudaSuccess;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const void* key = reinterpret_cast<const void*>(kern);
+  if (dev >= 0 && dev < 64)
+    for (auto& d : done[dev]) {
+      const void* k = d.load(std::memory_order_acquire);
+      if (k == key) return cudaSuccess;
+      if (!k) break;
+    }
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess && dev >= 0 && dev < 64)
+    for (auto& d : done[dev]) {
+      const void* none = nullptr;
+      if (d.compare_exchange_strong(none, key) || none == key) break;
+    }
+  return e;
 }
 template <typename F>
 static cudaError_t with_class(int cls, F f) {
@@ -1076,8 +1141,10 @@ cudaError_t launch_project_pair_simt(const void* A, int64_t lda, const void* B, 
     const cudaError_t e = with_class(projection_class(J.in_bf16, J.L, J.lp1), [&](auto in, auto lp) {
       using InT = decltype(in);
       constexpr int LP = decltype(lp)::value;
-      return launch_plain(c8 ? project_rows_kernel<InT, LP, (LP > 0)> : project_rows_kernel<InT, LP, false>, grid, 256, 0,
-                          st, J, a);
+      auto kern = c8 ? project_rows_kernel<InT, LP, (LP > 0)> : project_rows_kernel<InT, LP, false>;
+      const int smem = LP ? kRowsSmem : 0;
+      const cudaError_t e = rows_smem(kern, smem);
+      return e != cudaSuccess ? e : launch_plain(kern, grid, 256, smem, st, J, a);
     });
     if (e != cudaSuccess) return e;
     a.clear = nullptr;
@@ -1097,7 +1164,10 @@ cudaError_t launch_project_rows_jobs(int cls, const RowsJob* jobs, const int* jo
   if (blocks == 0) return cudaSuccess;
   const unsigned nb = static_cast<unsigned>(blocks);
   return with_class(cls, [&](auto in, auto lp) {
-    return launch_plain(project_rows_jobs_kernel<decltype(in), decltype(lp)::value>, dim3(nb), 256, 0, st, jobs, job_of);
+    auto kern = project_rows_jobs_kernel<decltype(in), decltype(lp)::value>;
+    const int smem = decltype(lp)::value ? kRowsSmem : 0;
+    const cudaError_t e = rows_smem(kern, smem);
+    return e != cudaSuccess ? e : launch_plain(kern, dim3(nb), 256, smem, st, jobs, job_of);
   });
 }
 
