@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256) batch_sigquant_kernel(const SigQJob* __re
 #pragma unroll
   for (int k = 0; k < 32; ++k) am = fmaxf(am, fabsf(x[k]));
   const int e = mx_exponent(am);
-  const float inv = ldexpf(1.0f, -e);
+  const float inv = mx_pow2(-e);
   uint32_t q[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k)

@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
 // Quantises x[0..31] with scale 2^e into 32 E4M3 bytes (q) and returns the
 // dequantised values in x (x becomes the residual x - deq when `residual`).
 __device__ __forceinline__ void quant32(float (&x)[32], int e, uint32_t (&q)[8], bool residual) {
-  const float inv = ldexpf(1.0f, -e), s = ldexpf(1.0f, e);
+  const float inv = mx_pow2(-e), s = mx_pow2(e);
 #pragma unroll
   for (int w = 0; w < 8; ++w) {
     const uint32_t a = e4m3x2(x[4 * w], x[4 * w + 1], inv);

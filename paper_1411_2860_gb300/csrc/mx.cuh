@@ -33,13 +33,25 @@ __device__ __forceinline__ float2 e4m3x2_value(uint32_t q) {
       __half2(__nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(q & 0xFFFFu), __NV_E4M3)));
 }
 
+// 2^e for e in [-127, 127], from its bits (2^-127 is subnormal).
+__device__ __forceinline__ float mx_pow2(int e) {
+  return __uint_as_float(e > -127 ? static_cast<uint32_t>(e + 127) << 23 : 0x00400000u);
+}
+
 // Byte of the scale of run cg (32 components) of row r: per tile of rows and
 // 128-component stage, row r of a 128-row group and K block b at byte
-// (r % 32) * 16 + (r / 32) * 4 + b.
+// (r % 32) * 16 + (r / 32) * 4 + b.  The row's part and the run's part are separate,
+// so that a thread divides once for all its runs (rows number below 2^31).
+__device__ __forceinline__ int64_t mx_sf_row(const MxQuantSide& a, int64_t r) {
+  const uint32_t tr = static_cast<uint32_t>(a.tile_rows), tile = static_cast<uint32_t>(r) / tr;
+  const uint32_t rr = static_cast<uint32_t>(r) - tile * tr, atom = rr >> 7, ar = rr & 127;
+  return (static_cast<int64_t>(tile) * a.sf_stages * a.atoms + atom) * 512 + (ar & 31) * 16 + (ar >> 5) * 4;
+}
+__device__ __forceinline__ int64_t mx_sf_run(const MxQuantSide& a, int64_t cg) {
+  return (cg >> 2) * a.atoms * 512 + (cg & 3);
+}
 __device__ __forceinline__ int64_t mx_sf_offset(const MxQuantSide& a, int64_t r, int64_t cg) {
-  const int64_t tile = r / a.tile_rows, rr = r - tile * a.tile_rows;
-  const int64_t atom = rr >> 7, ar = rr & 127;
-  return ((tile * a.sf_stages + (cg >> 2)) * a.atoms + atom) * 512 + (ar & 31) * 16 + (ar >> 5) * 4 + (cg & 3);
+  return mx_sf_row(a, r) + mx_sf_run(a, cg);
 }
 
 }  // namespace pj

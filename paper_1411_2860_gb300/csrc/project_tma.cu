@@ -404,9 +404,10 @@ __device__ __forceinline__ void mx_zero_tail(const MxQuantSide& q, int64_t r, in
     *reinterpret_cast<uint4*>(row + c) = make_uint4(0u, 0u, 0u, 0u);
     if (q.qsplit > 1) *reinterpret_cast<uint4*>(row + q.Kq_pad + c) = make_uint4(0u, 0u, 0u, 0u);
   }
+  uint8_t* const sf = q.sf + mx_sf_row(q, r);
   for (int64_t cg = c0 / 32; cg < q.Kq_pad / 32; ++cg) {
-    q.sf[mx_sf_offset(q, r, cg)] = 127;
-    if (q.qsplit > 1) q.sf[mx_sf_offset(q, r, q.Kq_pad / 32 + cg)] = 127;
+    sf[mx_sf_run(q, cg)] = 127;
+    if (q.qsplit > 1) sf[mx_sf_run(q, q.Kq_pad / 32 + cg)] = 127;
   }
 }
 
@@ -488,25 +489,26 @@ __device__ __forceinline__ void rows_tile_q(const TileCtx& c, const TileIn<InT, 
     for (int o = RL / 2; o >= 1; o >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
     const int e = mx_exponent(am);
     uint32_t qw[LP1 > 1 ? LP1 / 2 : 1];
-    mx_quant<LP1>(v, ldexpf(1.0f, -e), qw);
+    mx_quant<LP1>(v, mx_pow2(-e), qw);
     const bool live = i < c.n_out && in_k;
     uint8_t* row = q.dst + (i < c.n_out ? i : 0) * q.dst_pitch;
+    uint8_t* sf = q.sf + mx_sf_row(q, i < c.n_out ? i : 0);
     if (live) {
       mx_put<LP1>(row + comp0, qw);
-      if (lane % RL == 0) q.sf[mx_sf_offset(q, i, comp0 / 32)] = static_cast<uint8_t>(e + 127);
+      if (lane % RL == 0) sf[mx_sf_run(q, comp0 / 32)] = static_cast<uint8_t>(e + 127);
     }
     if (q.qsplit > 1) {
-      mx_residual<LP1>(v, qw, ldexpf(1.0f, e));
+      mx_residual<LP1>(v, qw, mx_pow2(e));
       float am2 = 0.0f;
 #pragma unroll
       for (int p = 0; p < LP1; ++p) am2 = fmaxf(am2, fabsf(v[p]));
 #pragma unroll
       for (int o = RL / 2; o >= 1; o >>= 1) am2 = fmaxf(am2, __shfl_xor_sync(0xffffffffu, am2, o));
       const int e2 = mx_exponent(am2);
-      mx_quant<LP1>(v, ldexpf(1.0f, -e2), qw);
+      mx_quant<LP1>(v, mx_pow2(-e2), qw);
       if (live) {
         mx_put<LP1>(row + q.Kq_pad + comp0, qw);
-        if (lane % RL == 0) q.sf[mx_sf_offset(q, i, q.Kq_pad / 32 + comp0 / 32)] = static_cast<uint8_t>(e2 + 127);
+        if (lane % RL == 0) sf[mx_sf_run(q, q.Kq_pad / 32 + comp0 / 32)] = static_cast<uint8_t>(e2 + 127);
       }
     }
   }
@@ -533,34 +535,68 @@ __device__ __forceinline__ void cols_tile_q(const TileCtx& c, const TileIn<InT, 
   if (ux == c.units_x - 1)   // padding rows: this tile's run, and the last tile also the runs past the tiles
     mx_pad_rows(q, c.n_out, uy, uy == c.units_y - 1 ? q.Kq_pad / 32 : uy + 1);
   if (j >= c.n_out) return;
-  const PtCoef<8, kG, false> cf(sCoef);
   float v[32];
   float am = 0.0f;
+  if constexpr (kG) {
+    const PtCoef<8, kG, false> cf(sCoef);
 #pragma unroll
-  for (int g4 = 0; g4 < 4; ++g4) {
-    float2 x[4];
+    for (int g4 = 0; g4 < 4; ++g4) {
+      float2 x[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      x[e] = make_float2(tin.elem(g4 * 8 + 2 * e, t), tin.elem(g4 * 8 + 2 * e + 1, t));
+      for (int e = 0; e < 4; ++e)
+        x[e] = make_float2(tin.elem(g4 * 8 + 2 * e, t), tin.elem(g4 * 8 + 2 * e + 1, t));
 #pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      v[g4 * 8 + p] = hi_lo_value(project_one(x, cf, p));
-      am = fmaxf(am, fabsf(v[g4 * 8 + p]));
+      for (int p = 0; p < 8; ++p) v[g4 * 8 + p] = project_one(x, cf, p);
     }
+  } else {
+    // sCoef as [t * 8 + p]: components in pairs, each one chain over the elements in order
+    // (the chain of project_one), every read of the values feeding two groups
+#pragma unroll
+    for (int g4 = 0; g4 < 4; g4 += 2) {
+      float2 a[4], b[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) a[p] = b[p] = make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float x = tin.elem(g4 * 8 + e, t), y = tin.elem(g4 * 8 + 8 + e, t);
+        const float4 c0 = reinterpret_cast<const float4*>(sCoef + e * 8)[0];
+        const float4 c1 = reinterpret_cast<const float4*>(sCoef + e * 8)[1];
+        const float2 cc[4] = {make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), make_float2(c1.x, c1.y),
+                              make_float2(c1.z, c1.w)};
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          a[p] = __ffma2_rn(make_float2(x, x), cc[p], a[p]);
+          b[p] = __ffma2_rn(make_float2(y, y), cc[p], b[p]);
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        v[g4 * 8 + 2 * p] = a[p].x;
+        v[g4 * 8 + 2 * p + 1] = a[p].y;
+        v[g4 * 8 + 8 + 2 * p] = b[p].x;
+        v[g4 * 8 + 8 + 2 * p + 1] = b[p].y;
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    v[k] = hi_lo_value(v[k]);
+    am = fmaxf(am, fabsf(v[k]));
   }
   uint8_t* row = q.dst + j * q.dst_pitch;
   const int64_t comp0 = static_cast<int64_t>(uy) * 32;
   if (comp0 < q.Kq_pad) {
     const int e = mx_exponent(am);
-    const float inv = ldexpf(1.0f, -e);
+    const float inv = mx_pow2(-e);
     uint32_t w[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) w[k] = e4m3x2(v[4 * k], v[4 * k + 1], inv) | (e4m3x2(v[4 * k + 2], v[4 * k + 3], inv) << 16);
     reinterpret_cast<uint4*>(row + comp0)[0] = make_uint4(w[0], w[1], w[2], w[3]);
     reinterpret_cast<uint4*>(row + comp0)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    q.sf[mx_sf_offset(q, j, uy)] = static_cast<uint8_t>(e + 127);
+    uint8_t* const sf = q.sf + mx_sf_row(q, j);
+    sf[mx_sf_run(q, uy)] = static_cast<uint8_t>(e + 127);
     if (q.qsplit > 1) {
-      const float sc = ldexpf(1.0f, e);
+      const float sc = mx_pow2(e);
       float am2 = 0.0f;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -572,13 +608,13 @@ __device__ __forceinline__ void cols_tile_q(const TileCtx& c, const TileIn<InT, 
         am2 = fmaxf(am2, fmaxf(fmaxf(fabsf(v[4 * k]), fabsf(v[4 * k + 1])), fmaxf(fabsf(v[4 * k + 2]), fabsf(v[4 * k + 3]))));
       }
       const int e2 = mx_exponent(am2);
-      const float inv2 = ldexpf(1.0f, -e2);
+      const float inv2 = mx_pow2(-e2);
 #pragma unroll
       for (int k = 0; k < 8; ++k)
         w[k] = e4m3x2(v[4 * k], v[4 * k + 1], inv2) | (e4m3x2(v[4 * k + 2], v[4 * k + 3], inv2) << 16);
       reinterpret_cast<uint4*>(row + q.Kq_pad + comp0)[0] = make_uint4(w[0], w[1], w[2], w[3]);
       reinterpret_cast<uint4*>(row + q.Kq_pad + comp0)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-      q.sf[mx_sf_offset(q, j, q.Kq_pad / 32 + uy)] = static_cast<uint8_t>(e2 + 127);
+      sf[mx_sf_run(q, q.Kq_pad / 32 + uy)] = static_cast<uint8_t>(e2 + 127);
     }
   }
   if (uy == c.units_y - 1) mx_zero_tail(q, j, static_cast<int64_t>(c.units_y) * 32);
@@ -822,8 +858,10 @@ __global__ void __launch_bounds__(kPtThreads, 2) project_tma_kernel(const __grid
   if (threadIdx.x < 128) {
     // Stage the kept basis vectors of side sd as sCoef[sd * 64 + q * 8 + t].
     const int sd = threadIdx.x >> 6, k = threadIdx.x & 63, q = k >> 3, t = k & 7;
+    // (the E4M3 columns of side 1 read them as [t * 8 + q])
+    const int at = kQ && sd == 1 ? 64 + t * 8 + q : static_cast<int>(threadIdx.x);
     if (q < LP1 && p.side[sd].num_units > 0)
-      sCoef[threadIdx.x] = p.inl ? p.c8.c[k]
+      sCoef[at] = p.inl ? p.c8.c[k]
                                  : (sd == 0 ? p.side[0].coef[t * LP1 + q] : p.side[1].coef[q * 8 + t]);
   }
   __syncthreads();
