@@ -397,8 +397,10 @@ static pj_status gemm_project_impl(const void* A, int64_t lda, const void* B, in
   // basis of groups of 8 (whose vectors are kernel arguments) the projection itself.
   Coef8 c8v;
   const Coef8* c8 = prec->compute != PJ_F64 && coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
+  Coef8d c8dv;
+  const Coef8d* c8d = prec->compute == PJ_F64 && coef8(basis, g.lp1, 0, &c8dv) ? &c8dv : nullptr;
   bool clear = false;
-  if (c8) {
+  if (c8 || c8d) {
     clear = A || B;
     if (!clear) PJ_CUDA_TRY(cudaMemsetAsync(ws, 0, sizeof(int), st));
   } else {
@@ -407,7 +409,8 @@ static pj_status gemm_project_impl(const void* A, int64_t lda, const void* B, in
   BasisDev b = basis_area(ws);
   if (prec->compute == PJ_F64) {
     PJ_CUDA_TRY(launch_project_pair_f64(static_cast<const double*>(A), lda, static_cast<const double*>(B), ldb, g, b.Cs64,
-                                        b.Ds64, at<double>(ws, w.off_ac), at<double>(ws, w.off_bd), st));
+                                        b.Ds64, c8d, at<double>(ws, w.off_ac), at<double>(ws, w.off_bd),
+                                        clear ? error_word(ws) : nullptr, st));
   } else {
     if (prec->compute == PJ_E4M3) {
       const MxQuantSide qa = make_mx_side(at<uint16_t>(ws, w.off_ac), g.Kp_pad, g.M, at<uint8_t>(ws, w.off_aq),
@@ -792,18 +795,20 @@ pj_status proj_gemm_backward_mixed(const void* A, int64_t lda, const void* B, in
     return backward_zero(dA, ldda, dB, lddb, g, out_dtype, st);
   }
   PJ_TRY(device_sms(&sms));
-  // the first kernel clears the error word (as in gemm_project_impl); the expansion
-  // kernels read the staged tables
+  // The first kernel clears the error word (as in gemm_project_impl).  The projections
+  // take their vectors as the forward does, so that they are the forward's bit for bit;
+  // the expansion kernels read the staged tables.
   Coef8 c8v;
-  const Coef8* c8 =
-      bwd_fused(g, prec->compute, ldda, lddb, out_dtype) && coef8(basis, g.lp1, 0, &c8v) ? &c8v : nullptr;
+  const bool arg8 = prec->compute != PJ_F64 && coef8(basis, g.lp1, 0, &c8v);
+  const Coef8* c8 = arg8 && bwd_fused(g, prec->compute, ldda, lddb, out_dtype) ? &c8v : nullptr;
   if (!c8) PJ_TRY(stage_basis(basis, g.lp1, workspace, st, nullptr, 0, true));
   BasisDev b = basis_area(workspace);
   if (prec->compute == PJ_F64) {
     double* Ac = at<double>(workspace, w.ac);
     double* Bd = at<double>(workspace, w.bd);
+    Coef8d c8d;
     PJ_CUDA_TRY(launch_project_pair_f64(static_cast<const double*>(A), lda, static_cast<const double*>(B), ldb, g, b.Cs64,
-                                        b.Ds64, Ac, Bd, st));
+                                        b.Ds64, coef8(basis, g.lp1, 0, &c8d) ? &c8d : nullptr, Ac, Bd, nullptr, st));
     return backward_products(Ac, Bd, dY, lddy, PJ_F64, dA, ldda, dB, lddb, out_dtype, g, PJ_F64, w, nullptr, workspace,
                              false, sms, st);
   }
@@ -812,8 +817,8 @@ pj_status proj_gemm_backward_mixed(const void* A, int64_t lda, const void* B, in
   GemmGeom g1 = g;
   g1.nsplit = 1;
   // A_c (M x Kp_pad) and B_d (N x Kp_pad) exactly as the forward projects them, in one launch
-  PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g1, b.Cs32, b.Ds32, c8, Ac, Bd, error_word(workspace),
-                                       c8 != nullptr, sms, st));
+  PJ_CUDA_TRY(launch_project_pair_bf16(A, lda, B, ldb, in_dtype, g1, b.Cs32, b.Ds32, arg8 ? &c8v : nullptr, Ac, Bd,
+                                       error_word(workspace), c8 != nullptr, sms, st));
   return backward_products(Ac, Bd, dY, lddy, dy_dtype, dA, ldda, dB, lddb, out_dtype, g, prec->compute, w, c8, workspace,
                            false, sms, st);
 }

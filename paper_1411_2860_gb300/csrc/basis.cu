@@ -143,7 +143,8 @@ cudaError_t launch_basis_build(int kind, int L, int lp1, BasisDev b, int* err, c
   return launch_plain(basis_kernel, dim3(1), kBasisThreads, 0, st, kind, L, lp1, p0, b, err, clear ? 1 : 0);
 }
 
-bool coef8(const pj_basis* basis, int lp1, int p0, Coef8* out) {
+template <typename T, typename Out>
+static bool fill_coef8(const pj_basis* basis, int lp1, int p0, Out* out) {
   if (basis->L != 8 || basis->kind == PJ_BASIS_USER) return false;
   // cos(k pi / 16), k = 0 .. 8; cos(m pi / 16) follows from the cosine's symmetries.
   static const double kCos[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
@@ -166,9 +167,12 @@ bool coef8(const pj_basis* basis, int lp1, int p0, Coef8* out) {
           if (i >= start && i < start + width) v = (j == 0 || i < start + width / 2) ? h : -h;
         }
       }
-      out->c[q * 8 + i] = static_cast<float>(v);
+      out->c[q * 8 + i] = static_cast<T>(v);
     }
   return true;
 }
+
+bool coef8(const pj_basis* basis, int lp1, int p0, Coef8* out) { return fill_coef8<float>(basis, lp1, p0, out); }
+bool coef8(const pj_basis* basis, int lp1, int p0, Coef8d* out) { return fill_coef8<double>(basis, lp1, p0, out); }
 
 }  // namespace pj

@@ -58,6 +58,10 @@ struct Coef8 {
   float c[64];
 };
 bool coef8(const pj_basis* basis, int lp1, int p0, Coef8* out);
+struct Coef8d {   // the same in FP64
+  double c[64];
+};
+bool coef8(const pj_basis* basis, int lp1, int p0, Coef8d* out);
 pj_status gemm_geom(int64_t M, int64_t N, int64_t K, int64_t block_k, int64_t R, const pj_basis* basis,
                     const pj_precision* prec, GemmGeom* g);
 pj_status conv_geom(int64_t S, int64_t T, int64_t nt, int64_t block, int64_t R, const pj_basis* basis,
@@ -300,9 +304,11 @@ constexpr int kProjectionClasses = 18;
 cudaError_t launch_project_rows_jobs(int cls, const RowsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st);
 cudaError_t launch_project_cols_jobs(int cls, const ColsJob* jobs, const int* job_of, int64_t blocks, cudaStream_t st);
 // FP64 path: A_c (M x Kp, pitch Kp) and B_d (Kp x N, pitch N), both double, in one
-// launch (A or B may be NULL).
+// launch (A or B may be NULL).  c8 (NULL: the tables Cs and Ds): the kept vectors as
+// arguments; clear_err: an error word the kernel clears (NULL: none).
 cudaError_t launch_project_pair_f64(const double* A, int64_t lda, const double* B, int64_t ldb, const GemmGeom& g,
-                                    const double* Cs, const double* Ds, double* Ac, double* Bd, cudaStream_t st);
+                                    const double* Cs, const double* Ds, const Coef8d* c8, double* Ac, double* Bd,
+                                    int* clear_err, cudaStream_t st);
 
 // gemm_f64.cu: Y = Ac (M x Kp) * Bd (Kp x N) in double.
 cudaError_t launch_gemm_f64(const double* Ac, const double* Bd, double* Y, int64_t ldy, int64_t M, int64_t N,

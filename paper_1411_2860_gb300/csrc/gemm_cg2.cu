@@ -339,17 +339,8 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             pending = true;
           }
           if (++sbuf == nbuf) sbuf = 0;
-        } else if (out_bf16) {
-          __nv_bfloat16* Y = static_cast<__nv_bfloat16*>(Yout);
-#pragma unroll
-          for (int u = 0; u < 32; ++u)
-            if (jok && i0 + u < M)
-              Y[static_cast<int64_t>(i0 + u) * ldy + j] = __float2bfloat16_rn(__uint_as_float(r[u]));
-        } else {
-          float* Y = static_cast<float*>(Yout);
-#pragma unroll
-          for (int u = 0; u < 32; ++u)
-            if (jok && i0 + u < M) __stcs(Y + static_cast<int64_t>(i0 + u) * ldy + j, __uint_as_float(r[u]));
+        } else if (jok) {
+          store_rows<32>(r, Yout, ldy, out_bf16, false, i0, M, j);
         }
       }
       tc_fence_before();

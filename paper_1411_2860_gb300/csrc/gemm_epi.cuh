@@ -19,6 +19,37 @@ __device__ __forceinline__ int expand_c8_index(const ExpandArgs& ex, int e) {
   return ex.mode == 1 ? (e % ex.lp1) * 8 + e / ex.lp1 : e;
 }
 
+// Element stores of a chunk: NR accumulator values of output column j (one per row from
+// i0 on), for outputs whose rows TMA cannot address.  A chunk whose rows all exist is
+// walked by pointer; tested and addressed one by one, the stores took the epilogue
+// warps (one per scheduler) three times the instructions.  add: atomic additions.
+template <int NR, typename Op>
+__device__ __forceinline__ void walk_rows(const uint32_t (&r)[NR], int64_t ldy, int i0, int M, Op op) {
+  if (i0 + NR <= M) {
+    int64_t off = 0;
+#pragma unroll
+    for (int u = 0; u < NR; ++u, off += ldy) op(off, __uint_as_float(r[u]));
+  } else {
+#pragma unroll
+    for (int u = 0; u < NR; ++u)
+      if (i0 + u < M) op(u * ldy, __uint_as_float(r[u]));
+  }
+}
+template <int NR>
+__device__ __forceinline__ void store_rows(const uint32_t (&r)[NR], void* Yv, int64_t ldy, bool out_bf16, bool add, int i0,
+                                           int M, int j) {
+  if (out_bf16) {
+    __nv_bfloat16* Y = static_cast<__nv_bfloat16*>(Yv) + i0 * ldy + j;
+    walk_rows(r, ldy, i0, M, [&](int64_t off, float v) { Y[off] = __float2bfloat16_rn(v); });
+  } else if (add) {
+    float* Y = static_cast<float*>(Yv) + i0 * ldy + j;
+    walk_rows(r, ldy, i0, M, [&](int64_t off, float v) { atomicAdd(Y + off, v); });
+  } else {
+    float* Y = static_cast<float*>(Yv) + i0 * ldy + j;
+    walk_rows(r, ldy, i0, M, [&](int64_t off, float v) { __stcs(Y + off, v); });
+  }
+}
+
 template <bool kBF16>
 __device__ __forceinline__ void store_run(void* out, int64_t off, const float (&y)[8], int n, int per) {
   if (kBF16) {

@@ -43,6 +43,7 @@
 #include <string.h>
 
 #include "common.hpp"
+#include "gemm_epi.cuh"
 #include "mx.cuh"
 #include "pdl.cuh"
 #include "tc.cuh"
@@ -362,17 +363,21 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
       const int* v = vote + (it & 1) * 4;
       if (!(v[0] && v[1] && v[2] && v[3])) break;
       tc_fence_after();
-      const int M = I->M, N = I->N;
+      const int M = I->M, N = I->N, bn = I->bn;   // read once (as in gemm_tc.cu)
+      const bool out_bf16 = I->out_bf16 != 0, conv = I->conv_mode != 0;
+      const int64_t ldy = I->ldy;
+      void* const Yout = I->Y;
+      const bool tma = I->tma_out && (tj + 1) * XBM <= I->tma_cols;
       const int jl = q * 32 + lane;
       const int j = tj * XBM + jl;
       const bool jok = j < N;
-      for (int c0 = 0; c0 < I->bn; c0 += kXEpiRows) {
+      for (int c0 = 0; c0 < bn; c0 += kXEpiRows) {
         uint32_t r[kXEpiRows];
         tmem_ld_x16(tmem + acc * 256 + c0 + (static_cast<uint32_t>(q * 32) << 16), r);
         tmem_wait_ld();
-        const int i0 = ti * I->bn + c0;
+        const int i0 = ti * bn + c0;
         if (i0 >= M) continue;
-        if (I->conv_mode) {
+        if (conv) {
           // lowered correlation: element (i, j) is output sample i * 128 + j of this phase
           float* Y = static_cast<float*>(I->Y);
 #pragma unroll
@@ -380,10 +385,10 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
             const int64_t flat = static_cast<int64_t>(i0 + u) * XBM + j;
             if (jok && flat < I->conv_limit) __stcs(Y + flat * I->conv_stride, __uint_as_float(r[u]));
           }
-        } else if (I->tma_out && (tj + 1) * XBM <= I->tma_cols) {
+        } else if (tma) {
           if (leader && pending) bulk_wait_read_all();
           named_barrier(1, 128);
-          if (I->out_bf16) {
+          if (out_bf16) {
             __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(stage_out);
 #pragma unroll
             for (int u = 0; u < kXEpiRows; ++u) st[u * XBM + jl] = __float2bfloat16_rn(__uint_as_float(r[u]));
@@ -402,22 +407,8 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
             bulk_commit_group();
             pending = true;
           }
-        } else if (I->out_bf16) {
-          __nv_bfloat16* Y = static_cast<__nv_bfloat16*>(I->Y);
-#pragma unroll
-          for (int u = 0; u < kXEpiRows; ++u)
-            if (jok && i0 + u < M)
-              Y[static_cast<int64_t>(i0 + u) * I->ldy + j] = __float2bfloat16_rn(__uint_as_float(r[u]));
-        } else if (red) {
-          float* Y = static_cast<float*>(I->Y);
-#pragma unroll
-          for (int u = 0; u < kXEpiRows; ++u)
-            if (jok && i0 + u < M) atomicAdd(Y + static_cast<int64_t>(i0 + u) * I->ldy + j, __uint_as_float(r[u]));
-        } else {
-          float* Y = static_cast<float*>(I->Y);
-#pragma unroll
-          for (int u = 0; u < kXEpiRows; ++u)
-            if (jok && i0 + u < M) __stcs(Y + static_cast<int64_t>(i0 + u) * I->ldy + j, __uint_as_float(r[u]));
+        } else if (jok) {
+          store_rows<kXEpiRows>(r, Yout, ldy, out_bf16, red, i0, M, j);
         }
       }
       tc_fence_before();

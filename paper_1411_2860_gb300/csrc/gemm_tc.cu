@@ -377,7 +377,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       const int* v = vote + (it & 1) * 4;
       if (!(v[0] && v[1] && v[2] && v[3])) break;
       tc_fence_after();
-      const int M = I->M, N = I->N;
+      // read once: the stores go through generic pointers, after which a field read
+      // through I would be read again
+      const int M = I->M, N = I->N, bn = I->bn;
+      const bool out_bf16 = I->out_bf16 != 0;
+      const int64_t ldy = I->ldy;
+      void* const Yout = I->Y;
+      const int tma_rows = I->tma_out && (tj + 1) * BM <= I->tma_cols ? I->tma_rows : 0;
       const int jl = q * 32 + lane;
       const int j = tj * BM + jl;
       const bool jok = j < N;
@@ -393,16 +399,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         continue;
       }
       // a stand-in tile of a pair (grouped launch) writes nothing
-      for (int c0 = 0; c0 < ((T.pad0 & 2) ? 0 : I->bn); c0 += 32) {
+      for (int c0 = 0; c0 < ((T.pad0 & 2) ? 0 : bn); c0 += 32) {
         uint32_t r[32];
         tmem_ld_x32(tmem + acc * BN + c0 + (static_cast<uint32_t>(q * 32) << 16), r);
         tmem_wait_ld();
-        const int i0 = ti * I->bn + c0;
+        const int i0 = ti * bn + c0;
         if (i0 >= M) continue;  // uniform: no rows of this chunk exist
-        if (I->tma_out && i0 + 32 <= I->tma_rows && (tj + 1) * BM <= I->tma_cols) {
+        if (i0 + 32 <= tma_rows) {
           if (leader && pending) bulk_wait_read_all();
           named_barrier(1, 128);  // staging free
-          if (I->out_bf16) {
+          if (out_bf16) {
             __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(stage);
 #pragma unroll
             for (int u = 0; u < 32; ++u) st[u * BM + jl] = __float2bfloat16_rn(__uint_as_float(r[u]));
@@ -429,24 +435,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             const int64_t flat = static_cast<int64_t>(i0 + u) * BM + j;
             if (jok && flat < I->conv_limit) __stcs(Y + flat * I->conv_stride, __uint_as_float(r[u]));
           }
-        } else if (I->out_bf16) {
-          __nv_bfloat16* Y = static_cast<__nv_bfloat16*>(I->Y);
-          const int64_t ldy = I->ldy;
-#pragma unroll
-          for (int u = 0; u < 32; ++u)
-            if (jok && i0 + u < M) Y[static_cast<int64_t>(i0 + u) * ldy + j] = __float2bfloat16_rn(__uint_as_float(r[u]));
-        } else if (red) {
-          float* Y = static_cast<float*>(I->Y);
-          const int64_t ldy = I->ldy;
-#pragma unroll
-          for (int u = 0; u < 32; ++u)
-            if (jok && i0 + u < M) atomicAdd(Y + static_cast<int64_t>(i0 + u) * ldy + j, __uint_as_float(r[u]));
-        } else {
-          float* Y = static_cast<float*>(I->Y);
-          const int64_t ldy = I->ldy;
-#pragma unroll
-          for (int u = 0; u < 32; ++u)
-            if (jok && i0 + u < M) __stcs(Y + static_cast<int64_t>(i0 + u) * ldy + j, __uint_as_float(r[u]));
+        } else if (jok) {
+          store_rows<32>(r, Yout, ldy, out_bf16, red, i0, M, j);
         }
       }
       tc_fence_before();

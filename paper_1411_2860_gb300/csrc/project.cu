@@ -670,32 +670,41 @@ struct PairF64 {
   const double* Ds;
   int64_t lda, ldb, M, N, K, NG, Kp, row_blocks;
   int L, lp1;
+  int* clear;   // the call's error word (NULL: not cleared here)
+  Coef8d c8;    // the kept vectors (kArg: groups of 8)
 };
 
+template <bool kArg>
 __global__ void __launch_bounds__(128) project_pair_f64_kernel(const __grid_constant__ PairF64 p) {
   pdl_begin();
-  const int L = p.L, lp1 = p.lp1;
-  if (static_cast<int64_t>(blockIdx.x) < p.row_blocks) {
-    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (e >= p.M * p.NG) return;
-    const int64_t i = e / p.NG, gg = e - i * p.NG;
-    const double* a = p.A + i * p.lda + gg * L;
-    const int n = static_cast<int>(p.K - gg * L < L ? p.K - gg * L : L);
+  if (p.clear && blockIdx.x == 0 && threadIdx.x == 0) *p.clear = 0;
+  const int L = kArg ? 8 : p.L, lp1 = p.lp1;
+  const bool rows = static_cast<int64_t>(blockIdx.x) < p.row_blocks;
+  const int64_t e = (static_cast<int64_t>(blockIdx.x) - (rows ? 0 : p.row_blocks)) * blockDim.x + threadIdx.x;
+  if (e >= (rows ? p.M : p.N) * p.NG) return;
+  const int64_t i = rows ? e / p.NG : 0, j = rows ? 0 : e % p.N;
+  const int64_t gg = rows ? e - i * p.NG : e / p.N;
+  const double* x = rows ? p.A + i * p.lda + gg * L : p.B + gg * L * p.ldb + j;
+  const int64_t xs = rows ? 1 : p.ldb;
+  double* o = rows ? p.Ac + i * p.Kp + gg * lp1 : p.Bd + gg * lp1 * p.N + j;
+  const int64_t os = rows ? 1 : p.N;
+  const int n = static_cast<int>(p.K - gg * L < L ? p.K - gg * L : L);
+  if constexpr (kArg) {
+    double v[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = t < n ? x[t * xs] : 0.0;
     for (int q = 0; q < lp1; ++q) {
       double acc = 0.0;
-      for (int t = 0; t < n; ++t) acc = fma(a[t], p.Cs[t * lp1 + q], acc);
-      p.Ac[i * p.Kp + gg * lp1 + q] = acc;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) acc = fma(v[t], p.c8.c[q * 8 + t], acc);
+      o[q * os] = acc;
     }
-    return;
-  }
-  const int64_t e = (static_cast<int64_t>(blockIdx.x) - p.row_blocks) * blockDim.x + threadIdx.x;
-  if (e >= p.N * p.NG) return;
-  const int64_t gg = e / p.N, j = e - gg * p.N;
-  const int n = static_cast<int>(p.K - gg * L < L ? p.K - gg * L : L);
-  for (int q = 0; q < lp1; ++q) {
-    double acc = 0.0;
-    for (int t = 0; t < n; ++t) acc = fma(p.Ds[q * L + t], p.B[(gg * L + t) * p.ldb + j], acc);
-    p.Bd[(gg * lp1 + q) * p.N + j] = acc;
+  } else {
+    for (int q = 0; q < lp1; ++q) {
+      double acc = 0.0;
+      for (int t = 0; t < n; ++t) acc = fma(x[t * xs], rows ? p.Cs[t * lp1 + q] : p.Ds[q * L + t], acc);
+      o[q * os] = acc;
+    }
   }
 }
 
@@ -1181,12 +1190,15 @@ cudaError_t launch_project_cols_jobs(int cls, const ColsJob* jobs, const int* jo
 
 
 cudaError_t launch_project_pair_f64(const double* A, int64_t lda, const double* B, int64_t ldb, const GemmGeom& g,
-                                    const double* Cs, const double* Ds, double* Ac, double* Bd, cudaStream_t st) {
+                                    const double* Cs, const double* Ds, const Coef8d* c8, double* Ac, double* Bd,
+                                    int* clear_err, cudaStream_t st) {
   const int64_t NG = ceil_div(g.K, g.L);
   const int64_t rb = A ? ceil_div(g.M * NG, 128) : 0, cb = B ? ceil_div(g.N * NG, 128) : 0;
   if (rb + cb == 0) return cudaSuccess;
-  const PairF64 p{A, B, Ac, Bd, Cs, Ds, lda, ldb, g.M, g.N, g.K, NG, g.Kp, rb, g.L, g.lp1};
-  return launch_plain(project_pair_f64_kernel, dim3(static_cast<unsigned>(rb + cb)), 128, 0, st, p);
+  PairF64 p{A, B, Ac, Bd, Cs, Ds, lda, ldb, g.M, g.N, g.K, NG, g.Kp, rb, g.L, g.lp1, clear_err, {}};
+  if (c8) p.c8 = *c8;
+  return launch_plain(c8 ? project_pair_f64_kernel<true> : project_pair_f64_kernel<false>,
+                      dim3(static_cast<unsigned>(rb + cb)), 128, 0, st, p);
 }
 
 cudaError_t launch_conv_project(const float* s, const float* k, const ConvGeom& g, uint16_t* G, uint16_t* TP,
