@@ -43,18 +43,25 @@ namespace {
 constexpr int CM = 128;   // P rows per CTA (the pair's MMA M is 256)
 constexpr int CN = 256;   // most Q rows per pair tile (MMA N); each CTA holds half
 constexpr int CK = 64;
-constexpr int CSTAGES = 6;
+// The ring holds as many slots as its memory takes: six at 256 Q rows, eight at 128.
+constexpr int kCMaxStages = 8;
 // warp 0: TMA producer; warp 1: MMA issuer (leader CTA); warps 2-9: epilogue.
 // Eight epilogue warps (two per TMEM lane quadrant) split an expansion tile's
 // columns in halves; the plain epilogue runs on warps 2-5.
 constexpr int kCThreads = 320;
 constexpr uint32_t kCStageP = CM * CK * 2;
-constexpr uint32_t kCStageQ = (CN / 2) * CK * 2;
 // Output staging of the TMA-store epilogue: 32 KB, four 32-column chunks of BF16
 // or two of FP32 in flight, so a chunk is staged while earlier ones are stored.
 constexpr uint32_t kCStageOut = 2 * 32 * CM * 4;
-constexpr size_t kCSmemBytes = 1024 + CSTAGES * (kCStageP + kCStageQ) + kCStageOut + 256;
+constexpr uint32_t kCCtl = 320;
+constexpr uint32_t kCRing = 6 * (kCStageP + (CN / 2) * CK * 2);
+constexpr size_t kCSmemBytes = 1024 + kCRing + kCStageOut + kCCtl;
 static_assert(kCSmemBytes + 64 * sizeof(float) <= 232448, "shared memory per block (dynamic + static)");
+
+__host__ __device__ constexpr int cg2_slots(int bn) {
+  const int n = static_cast<int>(kCRing / (kCStageP + static_cast<uint32_t>(bn / 2) * CK * 2));
+  return n < kCMaxStages ? n : kCMaxStages;
+}
 
 struct Cg2Params {
   GemmInst I;       // P map box {CK, CM} (MN-major: {64, CK}); Q map box {CK, bn/2} (MN-major: {64, CK})
@@ -71,18 +78,18 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  uint8_t* sP = sm;
-  uint8_t* sQ = sP + CSTAGES * kCStageP;
-  uint8_t* stage_out = sQ + CSTAGES * kCStageQ;
+  const int nst = cg2_slots(p.I.bn);
+  const uint32_t slot_bytes = kCStageP + static_cast<uint32_t>(p.I.bn / 2) * CK * 2;   // P rows, then Q rows
+  uint8_t* stage_out = sm + kCRing;
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + kCStageOut);
   uint64_t* full = bars;
-  uint64_t* empty = bars + CSTAGES;
-  uint64_t* acc_full = bars + 2 * CSTAGES;
+  uint64_t* empty = bars + kCMaxStages;
+  uint64_t* acc_full = bars + 2 * kCMaxStages;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
   int* vote = reinterpret_cast<int*>(tslot + 4);   // 2 x 8 flags
-  static_assert(17 * 8 + 16 + 16 * 4 <= 256, "barriers, TMEM slot and votes fit their 256 bytes");
+  static_assert((2 * kCMaxStages + 5) * 8 + 16 + 16 * 4 <= kCCtl, "barriers, TMEM slot and votes");
   __shared__ float s_coef[64];
   const GemmInst* I = &p.I;
 
@@ -90,7 +97,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < CSTAGES; ++s) {
+    for (int s = 0; s < nst; ++s) {
       mbar_init(&full[s], 1);    // the leader's expect_tx; both CTAs' copies count their bytes on it
       mbar_init(&empty[s], 1);   // the leader's MMA commit, delivered to both CTAs
     }
@@ -163,8 +170,8 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
           const int px = oP + kin * CK, qx = oQ + kin * CK;
           if (leader) mbar_arrive_expect_tx(&full[stage], pair_bytes);
           const uint32_t bar = full_leader + stage * 8;
-          uint8_t* const dP = sP + stage * kCStageP;
-          uint8_t* const dQ = sQ + stage * kCStageQ;
+          uint8_t* const dP = sm + stage * slot_bytes;
+          uint8_t* const dQ = dP + kCStageP;
           if (mnP) {
             tma_load_2d_cg2(dP, mapP, bar, prow, px);
             tma_load_2d_cg2(dP + 8192, mapP, bar, prow + 64, px);
@@ -178,7 +185,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
           }
           used |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
-          if (++stage == CSTAGES) {
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
@@ -188,7 +195,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
       // issued phase complete, no copy of either CTA is still writing shared memory
       // (the peer leaves only after the cluster barrier below).
       if (leader)
-        for (int s = 0; s < CSTAGES; ++s)
+        for (int s = 0; s < nst; ++s)
           if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
             atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
@@ -199,8 +206,9 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
       const uint32_t idesc = idesc_bf16_f32(2 * CM, I->bn) | (static_cast<uint32_t>(mnP) << 15) |
                              (static_cast<uint32_t>(mnQ) << 16);
       // (A K step of 16 moves a K-major start by 32 bytes, an MN-major one by 2048.)
-      const uint64_t bP = mnP ? sdesc_sw128_mn(smem_u32(sP), 8192) : sdesc_sw128(smem_u32(sP), 0);
-      const uint64_t bQ = mnQ ? sdesc_sw128_mn(smem_u32(sQ), 8192) : sdesc_sw128(smem_u32(sQ), 0);
+      const uint32_t a0 = smem_u32(sm), slot_units = slot_bytes / 16;
+      const uint64_t bP = mnP ? sdesc_sw128_mn(a0, 8192) : sdesc_sw128(a0, 0);
+      const uint64_t bQ = mnQ ? sdesc_sw128_mn(a0 + kCStageP, 8192) : sdesc_sw128(a0 + kCStageP, 0);
       const uint32_t kP = mnP ? 128 : 2, kQ = mnQ ? 128 : 2;
       const bool share = I->share != 0;
       const int chunks = share ? I->kc / 3 : I->kc;
@@ -219,7 +227,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
         const uint32_t d = tmem + acc * CN;
         // One 64-component product of the P tiles in slot sp and the Q tiles in slot sq.
         auto products = [&](int sp, int sq, bool first) {
-          const uint64_t dp = sdesc_advance(bP, sp * (kCStageP / 16)), dq = sdesc_advance(bQ, sq * (kCStageQ / 16));
+          const uint64_t dp = sdesc_advance(bP, sp * slot_units), dq = sdesc_advance(bQ, sq * slot_units);
 #pragma unroll
           for (int k = 0; k < CK / 16; ++k)
             umma_f16_cg2(d, sdesc_advance(dp, k * kP), sdesc_advance(dq, k * kQ), idesc, !first || (k != 0));
@@ -234,7 +242,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
           issued_any = true;
           if (share) {
             const int hi = stage;
-            if (++stage == CSTAGES) {
+            if (++stage == nst) {
               stage = 0;
               phase ^= 1u;
             }
@@ -248,7 +256,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             umma_commit_cg2_mc(&empty[hi], 0x3);
           }
           umma_commit_cg2_mc(&empty[stage], 0x3);
-          if (++stage == CSTAGES) {
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }

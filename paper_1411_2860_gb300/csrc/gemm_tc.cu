@@ -44,12 +44,24 @@ namespace {
 constexpr int BM = 128;  // output columns per tile (MMA M)
 constexpr int BN = 256;  // output rows per tile (MMA N)
 constexpr int BK = 64;
-constexpr int STAGES = 4;
+// The ring holds as many slots of (128 + tile height) operand rows as its memory takes:
+// four at 256 rows, eight at 64.  (With four slots at every height, the 64-row tiles of a
+// 1000 x 777 product over 2256 split components waited on their loads: 28.6 us.)
+constexpr int kMaxStages = 8;
 constexpr int kThreads = 192;
 constexpr uint32_t kStageP = BM * BK * 2;
-constexpr uint32_t kStageQ = BN * BK * 2;
 constexpr uint32_t kStageOut = 32 * BM * 4;          // output staging: 32 rows x 128 columns (FP32 max)
-constexpr size_t kSmemBytes = 1024 + STAGES * (kStageP + kStageQ) + kStageOut + 256;
+constexpr uint32_t kCtl = 256;                       // barriers, TMEM slot and votes
+constexpr size_t kSmemBytes = 232448 - 512;          // a block's shared memory less the static coefficients
+constexpr uint32_t kRing = 232448 - 512 - 1024 - kStageOut - kCtl;
+static_assert((2 * kMaxStages + 5) * 8 + 16 + 8 * 4 <= kCtl, "control area");
+
+// Ring slots at a tile height of bn rows (a multiple of 32).
+__host__ __device__ constexpr int ring_slots(int bn) {
+  const int n = static_cast<int>(kRing / (kStageP + static_cast<uint32_t>(bn) * BK * 2));
+  return n < kMaxStages ? n : kMaxStages;
+}
+static_assert(ring_slots(BN) >= 4, "at least two K chunks of a split product");
 
 struct GemmParams {
   GemmInst single;           // the instance when `tiles` is null
@@ -58,6 +70,7 @@ struct GemmParams {
   const int* cta_off;        // grouped launch: tiles of CTA c are [cta_off[c], cta_off[c+1])
   int num_tiles;             // single instance: tiles, walked with a grid stride
   int streamk;               // single instance: CTAs share the K stages of all tiles evenly
+  int slot_rows;             // tile height the ring slots are sized for (the instance's, or 256 when grouped)
   int stall;                 // failure-detection self-test: the producer stops after this many stages (-1: never)
   int* err;
   ExpandArgs ex;             // single instance: expansion to samples in the epilogue (mode 0: none)
@@ -130,13 +143,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  uint8_t* sP = sm;
-  uint8_t* sQ = sm + STAGES * kStageP;
-  uint8_t* stage = sQ + STAGES * kStageQ;              // output staging
+  const int nst = ring_slots(p.slot_rows);
+  const uint32_t slot_bytes = kStageP + static_cast<uint32_t>(p.slot_rows) * BK * 2;   // P rows, then Q rows
+  uint8_t* stage = sm + kRing;                         // output staging
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage + kStageOut);
   uint64_t* full = bars;
-  uint64_t* empty = bars + STAGES;
-  uint64_t* acc_full = bars + 2 * STAGES;
+  uint64_t* empty = bars + kMaxStages;
+  uint64_t* acc_full = bars + 2 * kMaxStages;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
@@ -145,7 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int rank = kPair ? static_cast<int>(cluster_ctarank()) : 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < nst; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kPair ? 2 : 1);
     }
@@ -223,8 +236,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           const int qx = conv ? (kin & 1) * BK : oQ + kin * BK;
           const int qy = conv ? y0 + (kin >> 1) + oQ : y0;
           uint64_t* const bar = &full[stage];
-          uint8_t* const dP = sP + stage * kStageP;
-          uint8_t* const dQ = sQ + stage * kStageQ;
+          uint8_t* const dP = sm + stage * slot_bytes;
+          uint8_t* const dQ = dP + kStageP;
           mbar_arrive_expect_tx(bar, stage_bytes);
           if (mnP) {  // 64-wide MN chunks of 64 K rows (8 KB each)
             tma_load_2d(dP, mapP, bar, tj * BM, px);
@@ -255,20 +268,21 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           }
           used |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
-          if (++stage == STAGES) {
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
       }
       // Every issued copy must land before the CTA may exit.
-      for (int s = 0; s < STAGES; ++s)
+      for (int s = 0; s < nst; ++s)
         if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
           atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // ---------------- UMMA issuer
+      const uint32_t slot_units = slot_bytes / 16;
       int stage = 0;
       uint32_t phase = 0;
       int it = 0;
@@ -288,11 +302,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         const uint32_t d = tmem + acc * BN;
         // One 64-component product of the P tile in slot sp and the Q tile in slot sq.
         // (A K step of 16 moves a K-major start by 32 bytes, an MN-major one by 2048.)
-        const uint64_t bP = mnP ? sdesc_sw128_mn(smem_u32(sP), 8192) : sdesc_sw128(smem_u32(sP), 0);
-        const uint64_t bQ = mnQ ? sdesc_sw128_mn(smem_u32(sQ), 8192) : sdesc_sw128(smem_u32(sQ), 0);
+        const uint32_t a0 = smem_u32(sm);
+        const uint64_t bP = mnP ? sdesc_sw128_mn(a0, 8192) : sdesc_sw128(a0, 0);
+        const uint64_t bQ = mnQ ? sdesc_sw128_mn(a0 + kStageP, 8192) : sdesc_sw128(a0 + kStageP, 0);
         const uint32_t kP = mnP ? 128 : 2, kQ = mnQ ? 128 : 2;
         auto products = [&](int sp, int sq, bool first) {
-          const uint64_t dp = sdesc_advance(bP, sp * (kStageP / 16)), dq = sdesc_advance(bQ, sq * (kStageQ / 16));
+          const uint64_t dp = sdesc_advance(bP, sp * slot_units), dq = sdesc_advance(bQ, sq * slot_units);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
             umma_f16(d, sdesc_advance(dp, k * kP), sdesc_advance(dq, k * kQ), idesc, !first || (k != 0));
@@ -317,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           issued_any = true;
           if (share) {  // hi*hi issued; then lo(P)*hi(Q) and hi(P)*lo(Q) from the same four tiles
             const int hi = stage;
-            if (++stage == STAGES) {
+            if (++stage == nst) {
               stage = 0;
               phase ^= 1u;
             }
@@ -331,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             release(hi);
           }
           release(stage);
-          if (++stage == STAGES) {
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
@@ -588,6 +603,7 @@ cudaError_t launch_gemm_tc_generic(const GemmTcArgs& a_in, int* err, int num_sms
   p.tiles = nullptr;
   p.cta_off = nullptr;
   p.num_tiles = gemm_tiles_of(p.single);
+  p.slot_rows = a.bn;
   p.err = err;
   p.stall = a.stall_stage;
   p.ex = a.ex;
@@ -623,6 +639,7 @@ cudaError_t launch_gemm_tc_grouped(const GemmInst* insts, const GemmTile* tiles,
   p.cta_off = cta_off;
   p.num_tiles = 0;
   p.streamk = 0;
+  p.slot_rows = BN;   // instances of any height share the ring
   p.stall = -1;
   p.err = err;
   p.ex = ExpandArgs{};

@@ -83,17 +83,33 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Bounded waits.  Reading %globaltimer takes about 680 clocks on this GPU, so a wait
+// polls first and reads the time only every kPolls failed polls: when every wait that was
+// not ready at once began with a read, each step of a ring took those 680 clocks whatever
+// it loaded (a probe streaming boxes of 64, 128 or 256 rows of 128 bytes on 1 or 152 SMs:
+// 12, 24 and 48 bytes a clock), and so did every K stage of the products.
+constexpr uint32_t kPolls = 128;
+
+// The time of the first call, and whether PJ_WAIT_LIMIT_NS have passed since then.
+struct WaitClock {
+  uint64_t t0 = 0;
+  __device__ __forceinline__ bool expired() {
+    const uint64_t t = globaltimer_ns();
+    if (t0 == 0) t0 = t;
+    return t - t0 > PJ_WAIT_LIMIT_NS;
+  }
+};
+
 // Wait for the phase with the given parity to complete.  Gives up after
 // PJ_WAIT_LIMIT_NS (recording `code` in *err) or as soon as another thread
 // has recorded an error; returns false in both cases.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int code) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
+  WaitClock clk;
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 127u) == 0) {
+    if (it % kPolls == 0) {
       if (*reinterpret_cast<volatile int*>(err) != 0) return false;
-      if (globaltimer_ns() - t0 > PJ_WAIT_LIMIT_NS) {
+      if (clk.expired()) {
         atomicCAS(err, 0, code);
         return false;
       }
@@ -104,11 +120,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
 // The same, without reading the error word: for the first kernel of a call, one of
 // whose blocks clears what an earlier call may have left there.
 __device__ __forceinline__ bool mbar_wait_first(uint64_t* bar, uint32_t parity, int* err, int code) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
+  WaitClock clk;
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 127u) == 0 && globaltimer_ns() - t0 > PJ_WAIT_LIMIT_NS) {
+    if (it % kPolls == 0 && clk.expired()) {
       atomicCAS(err, 0, code);
       return false;
     }
@@ -119,10 +134,11 @@ __device__ __forceinline__ bool mbar_wait_first(uint64_t* bar, uint32_t parity, 
 // error word (used before exit, so no copy is still writing shared memory).
 // Gives up after PJ_WAIT_LIMIT_NS and returns false.
 __device__ __forceinline__ bool mbar_wait_drain(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = globaltimer_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (globaltimer_ns() - t0 > PJ_WAIT_LIMIT_NS) return false;
-  return true;
+  WaitClock clk;
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (it % kPolls == 0 && clk.expired()) return false;
+  }
 }
 
 __device__ __forceinline__ bool dev_failed(const int* err) {
