@@ -137,33 +137,38 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
   const int nchunks = p.Kc + 1;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer: template chunks, one per K step
+    {
+      // ---------------- TMA producer (the whole warp; one lane issues): template chunks,
+      // one per K step
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t last_phase[STAGES];
-      bool used[STAGES];
-      for (int s = 0; s < STAGES; ++s) used[s] = false;
+      uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
       bool ok = true;
-      tma_prefetch(&p.mapTP);
-      for (int tile = blockIdx.x; tile < p.num_tiles && ok; tile += gridDim.x) {
+      const int nst = p.nst, num_tiles = p.num_tiles;
+      if (lane == 0) tma_prefetch(&p.mapTP);
+      __syncwarp();
+      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         for (int c = 0; c < nchunks; ++c) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
+          if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&full[stage], kStageA);
-          tma_load_2d(sA + stage * kStageA, &p.mapTP, &full[stage], 0, c * 128);
-          used[stage] = true;
-          last_phase[stage] = phase;
-          if (++stage == p.nst) {
+          if (elect_one()) {
+            mbar_arrive_expect_tx(&full[stage], kStageA);
+            tma_load_2d(sA + stage * kStageA, &p.mapTP, &full[stage], 0, c * 128);
+          }
+          __syncwarp();
+          used |= 1u << stage;
+          last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
       }
       for (int s = 0; s < STAGES; ++s)
-        if (used[s] && !mbar_wait_drain(&full[s], last_phase[s])) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+        if (lane == 0 && (used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
+          atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 6) {
     if (lane == 0) {
@@ -190,49 +195,55 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
         if (ring_used[r] && !mbar_wait_drain(&ring_full[r], ring_last[r])) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- UMMA issuer
+    {
+      // ---------------- UMMA issuer (the whole warp; one lane issues)
+      const int nst = p.nst, num_tiles = p.num_tiles;
+      const uint64_t bA = sdesc_sw128(smem_u32(sA), 0), bR = sdesc_sw128(smem_u32(ring), 0);
       int stage = 0;
       uint32_t phase = 0;
       int it = 0;
       bool ok = true;
       bool issued_any = false;
-      for (int tile = blockIdx.x; tile < p.num_tiles && ok; tile += gridDim.x, ++it) {
+      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++it) {
         const int buf = it & 1;
         const uint32_t bphase = (it >> 1) & 1;
-        if (!mbar_wait(&acc_empty[buf], bphase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
-        if (!mbar_wait(&ring_full[buf], bphase, p.err, DEV_TIMEOUT_RING)) break;
+        if (!mbar_wait_warp(&acc_empty[buf], bphase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
+        if (!mbar_wait_warp(&ring_full[buf], bphase, p.err, DEV_TIMEOUT_RING)) break;
         tc_fence_after();
         const uint32_t d = tmem + buf * 256;
-        const uint32_t ring0 = smem_u32(ring + buf * kRingBuf);
         for (int c = 0; c < nchunks; ++c) {
-          if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+          if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t aA = smem_u32(sA + stage * kStageA);
+          const uint64_t dA = sdesc_advance(bA, stage * (kStageA / 16));
           // rows a0 + 2i + c for i < 256: parity (c & 1), ring row (c >> 1) + i
-          const uint32_t aB = ring0 + (c & 1) * kRingParity + (c >> 1) * 128;
+          const uint64_t dB = sdesc_advance(bR, (buf * kRingBuf + (c & 1) * kRingParity + (c >> 1) * 128) / 16);
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma_f16(d, sdesc_sw128(aA + k * 32, 0), sdesc_sw128(aB + k * 32, 0), kIdesc, (c | k) != 0);
+            for (int k = 0; k < 4; ++k)
+              umma_f16(d, sdesc_advance(dA, 2 * k), sdesc_advance(dB, 2 * k), kIdesc, (c | k) != 0);
+            umma_commit(&empty[stage]);
+          }
+          __syncwarp();
           issued_any = true;
-          umma_commit(&empty[stage]);
-          if (++stage == p.nst) {
+          if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) {
+        if (ok && elect_one()) {
           umma_commit(&ring_empty[buf]);
           umma_commit(&acc_full[buf]);
         }
+        __syncwarp();
       }
       // Commit only behind issued MMAs: a commit with nothing to track is never issued.
       if (issued_any) {
-        umma_commit(drain);
-        if (!mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+        if (elect_one()) umma_commit(drain);
+        __syncwarp();
+        if (lane == 0 && !mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
       }
     }
   } else if ((warp >= 2 && warp <= 5) || (NEPI == 2 && warp >= 7)) {

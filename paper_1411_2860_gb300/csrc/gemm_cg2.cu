@@ -122,10 +122,14 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
   pdl_begin();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer (both CTAs): this CTA's P rows and half of the Q rows
-      tma_prefetch(&I->mapP);
-      tma_prefetch(&I->mapQ);
+    {
+      // ---------------- TMA producer (both CTAs; the whole warp, one lane issues): this
+      // CTA's P rows and half of the Q rows
+      if (lane == 0) {
+        tma_prefetch(&I->mapP);
+        tma_prefetch(&I->mapQ);
+      }
+      __syncwarp();
       int stage = 0;
       uint32_t phase = 0;
       uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
@@ -153,7 +157,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             ok = false;
             break;
           }
-          if (!mbar_wait(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
+          if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
@@ -168,21 +172,24 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             oQ = kk < e0 ? sQ0 : (kk < e1 ? sQ1 : sQ2);
           }
           const int px = oP + kin * CK, qx = oQ + kin * CK;
-          if (leader) mbar_arrive_expect_tx(&full[stage], pair_bytes);
           const uint32_t bar = full_leader + stage * 8;
           uint8_t* const dP = sm + stage * slot_bytes;
           uint8_t* const dQ = dP + kCStageP;
-          if (mnP) {
-            tma_load_2d_cg2(dP, mapP, bar, prow, px);
-            tma_load_2d_cg2(dP + 8192, mapP, bar, prow + 64, px);
-          } else {
-            tma_load_2d_cg2(dP, mapP, bar, px, prow);
+          if (elect_one()) {
+            if (leader) mbar_arrive_expect_tx(&full[stage], pair_bytes);
+            if (mnP) {
+              tma_load_2d_cg2(dP, mapP, bar, prow, px);
+              tma_load_2d_cg2(dP + 8192, mapP, bar, prow + 64, px);
+            } else {
+              tma_load_2d_cg2(dP, mapP, bar, px, prow);
+            }
+            if (mnQ) {
+              for (int c = 0; c < half / 64; ++c) tma_load_2d_cg2(dQ + c * 8192, mapQ, bar, qrow + 64 * c, qx);
+            } else {
+              tma_load_2d_cg2(dQ, mapQ, bar, qx, qrow);
+            }
           }
-          if (mnQ) {
-            for (int c = 0; c < half / 64; ++c) tma_load_2d_cg2(dQ + c * 8192, mapQ, bar, qrow + 64 * c, qx);
-          } else {
-            tma_load_2d_cg2(dQ, mapQ, bar, qx, qrow);
-          }
+          __syncwarp();
           used |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == nst) {
@@ -194,14 +201,14 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
       // The leader's barriers count both CTAs' copies: once the leader has seen every
       // issued phase complete, no copy of either CTA is still writing shared memory
       // (the peer leaves only after the cluster barrier below).
-      if (leader)
+      if (leader && lane == 0)
         for (int s = 0; s < nst; ++s)
           if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
             atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
-      // ---------------- MMA issuer (the leader only)
+    if (leader) {
+      // ---------------- MMA issuer (the leader's whole warp; one lane issues)
       const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
       const uint32_t idesc = idesc_bf16_f32(2 * CM, I->bn) | (static_cast<uint32_t>(mnP) << 15) |
                              (static_cast<uint32_t>(mnQ) << 16);
@@ -222,7 +229,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
         if (pi >= num_pairs) break;
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
+        if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * CN;
         // One 64-component product of the P tiles in slot sp and the Q tiles in slot sq.
@@ -233,12 +240,16 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             umma_f16_cg2(d, sdesc_advance(dp, k * kP), sdesc_advance(dq, k * kQ), idesc, !first || (k != 0));
         };
         for (int kk = 0; kk < chunks; ++kk) {
-          if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+          if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          products(stage, stage, kk == 0);
+          if (elect_one()) {
+            products(stage, stage, kk == 0);
+            if (!share) umma_commit_cg2_mc(&empty[stage], 0x3);
+          }
+          __syncwarp();
           issued_any = true;
           if (share) {
             const int hi = stage;
@@ -246,26 +257,31 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
               stage = 0;
               phase ^= 1u;
             }
-            if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+            if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            products(stage, hi, false);
-            products(hi, stage, false);
-            umma_commit_cg2_mc(&empty[hi], 0x3);
+            if (elect_one()) {
+              products(stage, hi, false);
+              products(hi, stage, false);
+              umma_commit_cg2_mc(&empty[hi], 0x3);
+              umma_commit_cg2_mc(&empty[stage], 0x3);
+            }
+            __syncwarp();
           }
-          umma_commit_cg2_mc(&empty[stage], 0x3);
           if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) umma_commit_cg2_mc(&acc_full[acc], 0x3);
+        if (ok && elect_one()) umma_commit_cg2_mc(&acc_full[acc], 0x3);
+        __syncwarp();
       }
       if (issued_any) {
-        umma_commit_cg2_mc(drain, 0x1);
-        if (!mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+        if (elect_one()) umma_commit_cg2_mc(drain, 0x1);
+        __syncwarp();
+        if (lane == 0 && !mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
       }
     }
   } else {

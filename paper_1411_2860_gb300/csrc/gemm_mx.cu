@@ -193,8 +193,9 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
   pdl_begin();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- producer: operand tiles by TMA, scale blocks by bulk copy
+    {
+      // ---------------- producer (the whole warp; one lane issues): operand tiles by TMA,
+      // scale blocks by bulk copy
       int stage = 0;
       uint32_t phase = 0;
       uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
@@ -206,8 +207,11 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         // read once (see gemm_tc.cu: a value read through I would be read again after every copy)
         const CUtensorMap* const mapP = &I->mapP;
         const CUtensorMap* const mapQ = &I->mapQ;
-        tma_prefetch(mapP);
-        tma_prefetch(mapQ);
+        if (lane == 0) {
+          tma_prefetch(mapP);
+          tma_prefetch(mapQ);
+        }
+        __syncwarp();
         const int bn = I->bn, half = bn / 2, y0 = T.ti * bn, p0 = T.tj * XBM;
         const bool conv = I->conv_mode != 0;
         const uint32_t stage_bytes = kXStageP + static_cast<uint32_t>(bn) * XBK + kXStageSF;
@@ -218,7 +222,7 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         const uint8_t* const sfP = I->sfP + static_cast<int64_t>(T.tj) * I->sf_stages * 512;
         const uint8_t* const sfQ = I->sfQ + static_cast<int64_t>(T.ti) * I->sf_stages * 1024;
         for (int kk = f0; kk < f1; ++kk) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
+          if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
@@ -228,22 +232,25 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
           uint8_t* const sQ = sP + kXStageP;
           uint8_t* const sf = sSF + stage * kXStageSF;
           uint64_t* const bar = &full[stage];
-          mbar_arrive_expect_tx(bar, stage_bytes);
-          tma_load_2d(sP, mapP, bar, xp, p0);
+          if (elect_one()) {
+            mbar_arrive_expect_tx(bar, stage_bytes);
+            tma_load_2d(sP, mapP, bar, xp, p0);
 #if PJ_CTA_PAIRS
-          if (kPair) {  // this CTA's half of the Q tile, for both CTAs of the pair
-            tma_load_2d_mc(sQ + rank * half * XBK, mapQ, bar, xq, y0 + rank * half, 0x3);
-          } else
+            if (kPair) {  // this CTA's half of the Q tile, for both CTAs of the pair
+              tma_load_2d_mc(sQ + rank * half * XBK, mapQ, bar, xq, y0 + rank * half, 0x3);
+            } else
 #endif
-          {
-            // (lowered correlation: stage kk of output rows r reads Q rows r + kk)
-            if (conv)
-              tma_load_2d(sQ, mapQ, bar, 0, y0 + kk);
-            else
-              tma_load_2d(sQ, mapQ, bar, xq, y0);
+            {
+              // (lowered correlation: stage kk of output rows r reads Q rows r + kk)
+              if (conv)
+                tma_load_2d(sQ, mapQ, bar, 0, y0 + kk);
+              else
+                tma_load_2d(sQ, mapQ, bar, xq, y0);
+            }
+            bulk_load(sf, sfP + static_cast<int64_t>(xp / XBK) * 512, 512, bar);
+            bulk_load(sf + 512, sfQ + static_cast<int64_t>(xq / XBK) * 1024, 1024, bar);
           }
-          bulk_load(sf, sfP + static_cast<int64_t>(xp / XBK) * 512, 512, bar);
-          bulk_load(sf + 512, sfQ + static_cast<int64_t>(xq / XBK) * 1024, 1024, bar);
+          __syncwarp();
           used |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == nst) {
@@ -253,12 +260,12 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         }
       }
       for (int s = 0; s < nst; ++s)
-        if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
+        if (lane == 0 && (used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
           atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
+    {
+      // ---------------- MMA issuer (the whole warp; one lane issues)
       const uint64_t b0 = sdesc_sw128(smem_u32(sm), 0), bS = sdesc_rows16(smem_u32(sSF));
       const uint32_t slot_units = slot_bytes / 16;
       int stage = 0;
@@ -273,18 +280,17 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         if (!I) break;
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
+        if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * 256;
         const uint32_t idesc = idesc_mx_e4m3(XBM, I->bn, 0, 0);
         // The scales of ring slot sl into TMEM (two sets of columns, used in turn).
-        auto scales = [&](int sl) {
-          const uint32_t cols = tmem + ((nslot++ & 1u) ? kSlot1 : kSlot0);
+        auto next_cols = [&]() { return tmem + ((nslot++ & 1u) ? kSlot1 : kSlot0); };
+        auto scales = [&](int sl, uint32_t cols) {
           const uint64_t ds = sdesc_advance(bS, sl * (kXStageSF / 16));
           tmem_cp_32x128b_warpx4(cols, ds);
           tmem_cp_32x128b_warpx4(cols + 4, sdesc_advance(ds, 512 / 16));
           tmem_cp_32x128b_warpx4(cols + 8, sdesc_advance(ds, 1024 / 16));
-          return cols;
         };
         // One 128-component product of the P tile in slot sp (scales at columns cp) and
         // the Q tile in slot sq (scales at cq).
@@ -306,13 +312,18 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         const bool share = I->share != 0;
         const int c0 = share ? share_chunk(T.k0) : T.k0, c1 = share ? share_chunk(T.k1) : T.k1;
         for (int kk = c0; kk < c1; ++kk) {
-          if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+          if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t ch = scales(stage);
-          products(stage, ch, stage, ch, kk == c0);
+          const uint32_t ch = next_cols();
+          if (elect_one()) {
+            scales(stage, ch);
+            products(stage, ch, stage, ch, kk == c0);
+            if (!share) release(stage);
+          }
+          __syncwarp();
           issued_any = true;
           if (share) {  // hi*hi issued; then hi(P)*lo(Q) and lo(P)*hi(Q) from the same four tiles
             const int hi = stage;
@@ -320,27 +331,33 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
               stage = 0;
               phase ^= 1u;
             }
-            if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+            if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t cl = scales(stage);
-            products(hi, ch, stage, cl, false);
-            products(stage, cl, hi, ch, false);
-            release(hi);
+            const uint32_t cl = next_cols();
+            if (elect_one()) {
+              scales(stage, cl);
+              products(hi, ch, stage, cl, false);
+              products(stage, cl, hi, ch, false);
+              release(hi);
+              release(stage);
+            }
+            __syncwarp();
           }
-          release(stage);
           if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) umma_commit(&acc_full[acc]);
+        if (ok && elect_one()) umma_commit(&acc_full[acc]);
+        __syncwarp();
       }
       if (issued_any) {
-        umma_commit(drain);
-        if (!mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+        if (elect_one()) umma_commit(drain);
+        __syncwarp();
+        if (lane == 0 && !mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
       }
     }
   } else {

@@ -181,8 +181,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   pdl_begin();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer
+    {
+      // ---------------- TMA producer (the whole warp; one lane issues)
       int stage = 0;
       uint32_t phase = 0;
       uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
@@ -197,8 +197,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         // and this thread's chain of loads would set the pace of the whole CTA.
         const CUtensorMap* const mapP = &I->mapP;
         const CUtensorMap* const mapQ = &I->mapQ;
-        tma_prefetch(mapP);
-        tma_prefetch(mapQ);
+        if (lane == 0) {
+          tma_prefetch(mapP);
+          tma_prefetch(mapQ);
+        }
+        __syncwarp();
         const int tj = T.tj, bn = I->bn, half = bn / 2;
         const int y0 = T.ti * bn;
         const bool conv = I->conv_mode != 0, mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
@@ -215,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             ok = false;
             break;
           }
-          if (!mbar_wait(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
+          if (!mbar_wait_warp(&empty[stage], phase ^ 1u, p.err, DEV_TIMEOUT_EMPTY)) {
             ok = false;
             break;
           }
@@ -238,34 +241,37 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           uint64_t* const bar = &full[stage];
           uint8_t* const dP = sm + stage * slot_bytes;
           uint8_t* const dQ = dP + kStageP;
-          mbar_arrive_expect_tx(bar, stage_bytes);
-          if (mnP) {  // 64-wide MN chunks of 64 K rows (8 KB each)
-            tma_load_2d(dP, mapP, bar, tj * BM, px);
-            tma_load_2d(dP + 8192, mapP, bar, tj * BM + 64, px);
-          } else {
-            tma_load_2d(dP, mapP, bar, px, tj * BM);
-          }
-          if (mnQ) {
+          if (elect_one()) {
+            mbar_arrive_expect_tx(bar, stage_bytes);
+            if (mnP) {  // 64-wide MN chunks of 64 K rows (8 KB each)
+              tma_load_2d(dP, mapP, bar, tj * BM, px);
+              tma_load_2d(dP + 8192, mapP, bar, tj * BM + 64, px);
+            } else {
+              tma_load_2d(dP, mapP, bar, px, tj * BM);
+            }
+            if (mnQ) {
 #if PJ_CTA_PAIRS
-            if (kPair) {  // this CTA's half of the Q chunks, for both CTAs of the pair
-              const int hc = qchunks / 2;
-              for (int c = rank * hc; c < (rank + 1) * hc; ++c)
-                tma_load_2d_mc(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx, 0x3);
-            } else
+              if (kPair) {  // this CTA's half of the Q chunks, for both CTAs of the pair
+                const int hc = qchunks / 2;
+                for (int c = rank * hc; c < (rank + 1) * hc; ++c)
+                  tma_load_2d_mc(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx, 0x3);
+              } else
 #endif
-            for (int c = 0; c < qchunks; ++c) tma_load_2d(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx);
+              for (int c = 0; c < qchunks; ++c) tma_load_2d(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx);
 #if PJ_CTA_PAIRS
-          } else if (kPair && !(T.pad0 & 1)) {
-            // this CTA's half of the Q tile, for both CTAs of the pair
-            tma_load_2d_mc(dQ + rank * half * (BK * 2), mapQ, bar, qx, qy + rank * half, 0x3);
+            } else if (kPair && !(T.pad0 & 1)) {
+              // this CTA's half of the Q tile, for both CTAs of the pair
+              tma_load_2d_mc(dQ + rank * half * (BK * 2), mapQ, bar, qx, qy + rank * half, 0x3);
 #endif
-          } else if (kPair) {
-            // a tile of its own (grouped launch): both halves for this CTA only
-            tma_load_2d(dQ, mapQ, bar, qx, qy);
-            tma_load_2d(dQ + half * (BK * 2), mapQ, bar, qx, qy + half);
-          } else {
-            tma_load_2d(dQ, mapQ, bar, qx, qy);
+            } else if (kPair) {
+              // a tile of its own (grouped launch): both halves for this CTA only
+              tma_load_2d(dQ, mapQ, bar, qx, qy);
+              tma_load_2d(dQ + half * (BK * 2), mapQ, bar, qx, qy + half);
+            } else {
+              tma_load_2d(dQ, mapQ, bar, qx, qy);
+            }
           }
+          __syncwarp();
           used |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == nst) {
@@ -276,12 +282,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       }
       // Every issued copy must land before the CTA may exit.
       for (int s = 0; s < nst; ++s)
-        if ((used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
+        if (lane == 0 && (used >> s & 1u) && !mbar_wait_drain(&full[s], last_phase >> s & 1u))
           atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- UMMA issuer
+    {
+      // ---------------- UMMA issuer (the whole warp; one lane issues)
       const uint32_t slot_units = slot_bytes / 16;
       int stage = 0;
       uint32_t phase = 0;
@@ -297,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                                (static_cast<uint32_t>(mnQ) << 16);
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
+        if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
         tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         // One 64-component product of the P tile in slot sp and the Q tile in slot sq.
@@ -323,12 +329,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         const bool share = I->share != 0;
         const int c0 = share ? share_chunk(T.k0) : T.k0, c1 = share ? share_chunk(T.k1) : T.k1;
         for (int kk = c0; kk < c1; ++kk) {
-          if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+          if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          products(stage, stage, kk == c0);
+          if (elect_one()) {
+            products(stage, stage, kk == c0);
+            if (!share) release(stage);
+          }
+          __syncwarp();
           issued_any = true;
           if (share) {  // hi*hi issued; then lo(P)*hi(Q) and hi(P)*lo(Q) from the same four tiles
             const int hi = stage;
@@ -336,27 +346,32 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
               stage = 0;
               phase ^= 1u;
             }
-            if (!mbar_wait(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
+            if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            products(stage, hi, false);
-            products(hi, stage, false);
-            release(hi);
+            if (elect_one()) {
+              products(stage, hi, false);
+              products(hi, stage, false);
+              release(hi);
+              release(stage);
+            }
+            __syncwarp();
           }
-          release(stage);
           if (++stage == nst) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) umma_commit(&acc_full[acc]);
+        if (ok && elect_one()) umma_commit(&acc_full[acc]);
+        __syncwarp();
       }
       // Commit only behind issued MMAs: a commit with nothing to track is never issued.
       if (issued_any) {
-        umma_commit(drain);
-        if (!mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
+        if (elect_one()) umma_commit(drain);
+        __syncwarp();
+        if (lane == 0 && !mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
       }
     }
   } else {

@@ -46,7 +46,16 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
-__device__ __forceinline__ bool elect_lane0() { return (threadIdx.x & 31) == 0; }
+// True in one lane of the (whole, converged) warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(is));
+  return is != 0;
+}
 
 // ------------------------------------------------------------- mbarrier ---
 
@@ -83,11 +92,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded waits.  Reading %globaltimer takes about 680 clocks on this GPU, so a wait
-// polls first and reads the time only every kPolls failed polls: when every wait that was
-// not ready at once began with a read, each step of a ring took those 680 clocks whatever
-// it loaded (a probe streaming boxes of 64, 128 or 256 rows of 128 bytes on 1 or 152 SMs:
-// 12, 24 and 48 bytes a clock), and so did every K stage of the products.
+// Bounded waits poll, and read %globaltimer only every kPolls failed polls.
 constexpr uint32_t kPolls = 128;
 
 // The time of the first call, and whether PJ_WAIT_LIMIT_NS have passed since then.
@@ -126,6 +131,32 @@ __device__ __forceinline__ bool mbar_wait_first(uint64_t* bar, uint32_t parity, 
     if (it % kPolls == 0 && clk.expired()) {
       atomicCAS(err, 0, code);
       return false;
+    }
+  }
+}
+
+// The same for a whole warp (every lane calls it, and all get one answer).
+//
+// The copy producers and MMA issuers are warps that run their loop together and elect a
+// lane for each copy or MMA.  A loop that one lane runs inside a branch keeps its operands
+// in vector registers, and each copy or MMA first moves them to uniform ones: a ring step
+// with one TMA load took 343 clocks that way and 248 this way, whatever it loaded (a probe
+// streaming boxes of 64 to 256 rows of 128 bytes on 1 and on 152 SMs; +70 clocks for a
+// second load), against 448 to 512 clocks of MMAs per 64-deep K stage.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, int code) {
+  WaitClock clk;
+  for (uint32_t it = 1;; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (it % kPolls == 0) {
+      bool stop = false;
+      if ((threadIdx.x & 31) == 0) {
+        stop = *reinterpret_cast<volatile int*>(err) != 0;
+        if (!stop && clk.expired()) {
+          atomicCAS(err, 0, code);
+          stop = true;
+        }
+      }
+      if (__any_sync(0xffffffffu, stop)) return false;
     }
   }
 }
