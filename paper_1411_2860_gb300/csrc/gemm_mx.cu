@@ -688,7 +688,7 @@ cudaError_t launch_gemm_mx(const MxGemmArgs& a_in, int* err, int num_sms, cudaSt
   MxGemmArgs a = a_in;
   const int64_t tiles_n = ceil_div(a.rowsP, XBM), tiles = tiles_n * ceil_div(a.rowsQ, a.bn);
   const int stages = static_cast<int>(a.Kq_pad / XBK) * (a.qsplit == 1 ? 1 : 3);
-  const bool streamk = a.out_dtype != PJ_BF16 && use_stream_k(static_cast<int>(tiles), stages, num_sms);
+  const bool streamk = a.out_dtype != PJ_BF16 && use_stream_k(tiles, stages, num_sms, false);
   // CTA pairs share the Q tiles when the tile columns pair up (half-tiles of whole 8-row atoms).
   a.pair = PJ_CTA_PAIRS && !streamk && tiles_n % 2 == 0 && a.bn % 16 == 0 && num_sms >= 2;
   MxParams p;

@@ -604,7 +604,7 @@ cudaError_t launch_gemm_tc_generic(const GemmTcArgs& a_in, int* err, int num_sms
   const int64_t tiles = tiles_n * ceil_div(a.rowsQ, a.bn);
   // (the expansion writes samples, which partial products could not be added into)
   const bool streamk = !a.conv_mode && !a.ex.mode && a.out_dtype != PJ_BF16 &&
-                       use_stream_k(static_cast<int>(tiles), args_stages(a), num_sms);
+                       use_stream_k(tiles, args_stages(a), num_sms, a.nseg > 1);
   // CTA pairs share the Q tiles of a K-major product with an even number of tile
   // columns (half-tiles of whole 8-row swizzle atoms).
   // 256-row tiles on 2-SM MMAs wherever the tile columns pair up (gemm_cg2.cu).
