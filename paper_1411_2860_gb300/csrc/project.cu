@@ -92,14 +92,16 @@ __device__ __forceinline__ void split_part_one(uint16_t* row, int64_t gg, int p,
 }
 
 // Zero padding of every segment of one output row.
+// from: the first component no other thread writes (at least NG (l+1); plain split only).
 __device__ __forceinline__ void zero_split_rows(uint16_t* row, int64_t NG, int lp1, int nsplit, int tl,
-                                                int64_t Kp_pad, int64_t Kt_pad) {
+                                                int64_t Kp_pad, int64_t Kt_pad, int64_t from = 0) {
   if (nsplit > 1 && tl < lp1) {
     zero_run(row, NG * lp1, Kp_pad);
     zero_run(row + Kp_pad, NG * tl, Kt_pad);
     zero_run(row + Kp_pad + Kt_pad, NG * tl, Kt_pad);
   } else {
-    for (int sg = 0; sg < nsplit; ++sg) zero_run(row + sg * Kp_pad, NG * lp1, Kp_pad);
+    const int64_t c0 = from > NG * lp1 ? from : NG * lp1;
+    for (int sg = 0; sg < nsplit; ++sg) zero_run(row + sg * Kp_pad, c0, Kp_pad);
   }
 }
 
@@ -453,6 +455,13 @@ __global__ void __launch_bounds__(256, LP ? 4 : 1) project_rows_jobs_kernel(cons
 // group quad also zero their column's padding.
 constexpr int kColGroups = 4;
 
+// The components the quads of a column write: whole quads when they fit the row.
+template <int LP1>
+__device__ __forceinline__ int64_t staged_end(const ColsJob& J) {
+  const int64_t end = (J.NG + kColGroups - 1) / kColGroups * kColGroups * LP1;
+  return end <= J.Kp_pad ? end : J.NG * LP1;
+}
+
 // L = 8, l+1 = 4 or 8, four whole groups: the warp's 32 columns stage their
 // runs in `stage` (4 KB per warp) and write them row by row (run_put_group /
 // runs_write).  Every lane of the warp takes part; columns past N are not
@@ -490,7 +499,8 @@ __device__ __forceinline__ void cols_staged(const ColsJob& J, int64_t j, int64_t
   uint16_t* o0 = J.Bd + jw * J.pitch + g0 * LP1;
   runs_write<LP1>(base, 128, 0, lane, o0, J.pitch, ncols);
   if (two) runs_write<LP1>(base, 128, 1, lane, o0 + J.Kp_pad, J.pitch, ncols);
-  if (g0 == 0 && live) zero_split_rows(row, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+  if (g0 == 0 && live)
+    zero_split_rows(row, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad, tiered ? 0 : staged_end<LP1>(J));
 }
 
 // L = 8, l+1 in {3, 5, 6, 7}, four whole groups, no tiered split: a column's run of
@@ -544,7 +554,8 @@ __device__ __forceinline__ void cols_quad_odd(const ColsJob& J, int64_t j, int64
         *reinterpret_cast<uint2*>(o0 + part * J.Kp_pad + c * J.pitch + k * 4) =
             *reinterpret_cast<const uint2*>(base + part * 2048 + c * kPitch + k * 8);
     }
-  if (g0 == 0 && j < J.N) zero_split_rows(J.Bd + j * J.pitch, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad);
+  if (g0 == 0 && j < J.N)
+    zero_split_rows(J.Bd + j * J.pitch, J.NG, LP1, J.nsplit, J.tl, J.Kp_pad, J.Kt_pad, staged_end<LP1>(J));
 }
 
 // L = 8, unstaged: group gg of one column, l+1 components.
@@ -591,14 +602,17 @@ __device__ __forceinline__ void cols_body(const ColsJob& J, int64_t j, int64_t q
   else
     for (int k = threadIdx.x; k < L * lp1; k += blockDim.x) sD[k] = J.Ds[k];
   __syncthreads();
+  // Four whole groups, or fewer whose missing components (zeros) still lie in the row's
+  // padding (as in project_tma.cu); the same for the whole block.
+  const bool tiered = J.nsplit > 1 && J.tl < lp1;
   if constexpr (LP == 4 || LP == 8) {
-    if (ng == kColGroups) {  // the same for the whole block
+    if (ng == kColGroups || (!tiered && (g0 + kColGroups) * LP <= J.Kp_pad)) {
       cols_staged<LP>(J, j, g0, xa, sD, stage);
       return;
     }
   }
   if constexpr (LP == 3 || LP == 5 || LP == 6 || LP == 7) {
-    if (ng == kColGroups && !(J.nsplit > 1 && J.tl < LP)) {
+    if (!tiered && (g0 + kColGroups) * LP <= J.Kp_pad) {
       cols_quad_odd<LP>(J, j, g0, xa, sD, stage);
       return;
     }

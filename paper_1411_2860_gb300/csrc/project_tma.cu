@@ -93,13 +93,15 @@ __device__ __forceinline__ void zero_tail(uint16_t* row, int64_t c0, int64_t c1)
 }
 
 // Padding of every segment of one output row (see gemm_tiered for the layout).
-__device__ __forceinline__ void zero_row_tails(const TileCtx& c, uint16_t* row, int lp1) {
+// from: the first component not written yet (at least NG (l+1); plain split only).
+__device__ __forceinline__ void zero_row_tails(const TileCtx& c, uint16_t* row, int lp1, int64_t from = 0) {
   if (c.nsplit > 1 && c.tl < lp1) {
     zero_tail(row, c.NG * lp1, c.Kp_pad);
     zero_tail(row + c.Kp_pad, c.NG * c.tl, c.Kt_pad);
     zero_tail(row + c.Kp_pad + c.Kt_pad, c.NG * c.tl, c.Kt_pad);
   } else {
-    for (int sg = 0; sg < c.nsplit; ++sg) zero_tail(row + sg * c.Kp_pad, c.NG * lp1, c.Kp_pad);
+    const int64_t c0 = from > c.NG * lp1 ? from : c.NG * lp1;
+    for (int sg = 0; sg < c.nsplit; ++sg) zero_tail(row + sg * c.Kp_pad, c0, c.Kp_pad);
   }
 }
 
@@ -648,8 +650,12 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
   const int t = threadIdx.x;
   const int64_t j = static_cast<int64_t>(ux) * kPtBoxX + t;
   const int64_t g0 = static_cast<int64_t>(uy) * 4;
-  const bool full = g0 + 4 <= c.NG;
   constexpr bool tiered = kTiered;
+  // Four whole groups, or fewer whose missing components (zeros: the copies fill past K
+  // with zeros) still lie in the row's padding: the last quad then takes the same stores.
+  // Group by group, a last quad of three cost the columns of a 3000 x 776 operand 16 us
+  // at l+1 = 6: its 2-byte stores each go to 32 rows.
+  const bool full = g0 + 4 <= c.NG || (!tiered && (g0 + 4) * LP1 <= c.Kp_pad);
   constexpr bool kStaged = sizeof(InT) == 4 && (LP1 == 4 || LP1 == 8);
   const PtCoef<LP1, kG, (LP1 <= 4)> cf(sCoef);
   const bool need_lo = c.nsplit > 1;   // (the tiered lead terms are split as well)
@@ -697,7 +703,57 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
       if (two) runs_write<LP1>(base, row_bytes, 1, lane, o0 + c.Kp_pad, c.pitch, ncols);
       // the staging writes must be ordered before the next TMA fill of this stage
       fence_proxy_async_smem();
-      if (uy == c.units_y - 1 && j < c.n_out) zero_row_tails(c, c.out + j * c.pitch, LP1);
+      if (uy == c.units_y - 1 && j < c.n_out) zero_row_tails(c, c.out + j * c.pitch, LP1, (g0 + 4) * LP1);
+      return;
+    }
+  }
+  if constexpr (kOddRun<LP1> && !tiered) {
+    if (full) {
+      // l+1 in {3, 5, 6, 7}, four whole groups: the column's 4 (l+1) components packed into
+      // words, one part (hi, then lo) at a time staged in the warp's own columns of the
+      // tile (read by now; runs an odd number of 8 bytes apart) and written run after run
+      // in 8-byte chunks.  Stored by the lanes themselves, every chunk went to 32 rows.
+      constexpr int kSeg = 32 * static_cast<int>(sizeof(InT)), kPitch = 8 * (LP1 | 1);
+      static_assert(32 * kPitch <= 32 * kSeg, "the runs of a warp fit its columns");
+      const int lane = t & 31, w = t >> 5;
+      uint8_t* const base = tin.base + w * kSeg;
+      auto at = [&](int b) { return base + (b / kSeg) * row_bytes + b % kSeg; };
+      uint32_t wh[2 * LP1], wl[2 * LP1];
+#pragma unroll
+      for (int k = 0; k < 2 * LP1; ++k) wh[k] = wl[k] = 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float2 x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = make_float2(tin.elem(q * 8 + 2 * e, t), tin.elem(q * 8 + 2 * e + 1, t));
+        uint16_t hi[8], lo[8];
+        project8(x, cf, need_lo, hi, lo);
+#pragma unroll
+        for (int p = 0; p < LP1; ++p) {
+          const int e = q * LP1 + p;
+          wh[e >> 1] |= uint32_t(hi[p]) << (16 * (e & 1));
+          wl[e >> 1] |= uint32_t(lo[p]) << (16 * (e & 1));
+        }
+      }
+      const int64_t jw = static_cast<int64_t>(ux) * kPtBoxX + w * 32;
+      const int ncols = c.n_out - jw < 32 ? static_cast<int>(c.n_out - jw) : 32;
+      uint16_t* o0 = c.out + jw * c.pitch + g0 * LP1;
+#pragma unroll 1
+      for (int part = 0; part < (need_lo ? 2 : 1); ++part) {
+        __syncwarp();   // the columns (or the previous part's runs) are read
+#pragma unroll
+        for (int k = 0; k < 2 * LP1; ++k) *reinterpret_cast<uint32_t*>(at(lane * kPitch + 4 * k)) = part ? wl[k] : wh[k];
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < LP1; ++s) {
+          const int gi = s * 32 + lane, cc = gi / LP1, k = gi - cc * LP1;
+          if (cc < ncols)
+            *reinterpret_cast<uint2*>(o0 + part * c.Kp_pad + cc * c.pitch + k * 4) =
+                *reinterpret_cast<const uint2*>(at(cc * kPitch + 8 * k));
+        }
+      }
+      fence_proxy_async_smem();   // before the stage's next TMA fill
+      if (uy == c.units_y - 1 && j < c.n_out) zero_row_tails(c, c.out + j * c.pitch, LP1, (g0 + 4) * LP1);
       return;
     }
   }
@@ -706,12 +762,6 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
   uint16_t* o = orow + g0 * LP1;
   uint32_t ph[4] = {0u, 0u, 0u, 0u}, pl[4] = {0u, 0u, 0u, 0u};  // packed runs for l+1 <= 2
   uint32_t lh[4] = {0u, 0u, 0u, 0u}, ll[4] = {0u, 0u, 0u, 0u};  // packed lead runs for tl <= 2
-  // l+1 in {3, 5, 6, 7}, four whole groups: the 4 (l+1) components packed into words,
-  // stored as (l+1) 8-byte chunks (the run starts 8 (l+1) uy bytes into the row)
-  constexpr int kW = kOddRun<LP1> ? 2 * LP1 : 1;
-  uint32_t wh[kW], wl[kW];
-#pragma unroll
-  for (int k = 0; k < kW; ++k) wh[k] = wl[k] = 0u;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     float2 x[4];
@@ -727,15 +777,7 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
       ph[q] = pack2(hi[0], hi[1]);
       pl[q] = pack2(lo[0], lo[1]);
     }
-    if (kOddRun<LP1> && full) {
-#pragma unroll
-      for (int p = 0; p < 8; ++p) {
-        if (p >= LP1) break;
-        const int e = (q * LP1 + p) % (2 * kW);   // (the modulus only keeps non-odd l+1 in range)
-        wh[(e >> 1) % kW] |= uint32_t(hi[p]) << (16 * (e & 1));
-        wl[(e >> 1) % kW] |= uint32_t(lo[p]) << (16 * (e & 1));
-      }
-    } else if ((LP1 > 2 || !full) && g0 + q < c.NG) {
+    if ((LP1 > 2 || !full) && g0 + q < c.NG) {
       store_upto8(o + q * LP1, hi, LP1);
       if (!tiered && c.nsplit > 1) store_upto8(o + c.Kp_pad + q * LP1, lo, LP1);
     }
@@ -755,14 +797,6 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
       }
     }
   }
-  if (kOddRun<LP1> && full) {
-#pragma unroll
-    for (int k = 0; k < kW / 2; ++k) reinterpret_cast<uint2*>(o)[k] = make_uint2(wh[2 * k], wh[2 * k + 1]);
-    if (!tiered && c.nsplit > 1)
-#pragma unroll
-      for (int k = 0; k < kW / 2; ++k)
-        reinterpret_cast<uint2*>(o + c.Kp_pad)[k] = make_uint2(wl[2 * k], wl[2 * k + 1]);
-  }
   if (full && LP1 == 1) {
     *reinterpret_cast<uint2*>(o) = make_uint2(ph[0], ph[1]);
     if (c.nsplit > 1 && !tiered) *reinterpret_cast<uint2*>(o + c.Kp_pad) = make_uint2(pl[0], pl[1]);
@@ -771,7 +805,7 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
     if (c.nsplit > 1 && !tiered) *reinterpret_cast<uint4*>(o + c.Kp_pad) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
   }
   if (tiered && full && c.tl <= 2) store_lead_runs(c, orow, g0, lh, ll);
-  if (uy == c.units_y - 1) zero_row_tails(c, orow, LP1);
+  if (uy == c.units_y - 1) zero_row_tails(c, orow, LP1, full && LP1 <= 2 ? (g0 + 4) * LP1 : 0);
 }
 
 // The ring of one block: NST tile buffers with a full and an empty barrier
