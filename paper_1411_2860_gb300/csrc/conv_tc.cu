@@ -39,21 +39,25 @@ namespace pj {
 namespace {
 
 constexpr int STAGES = 4;       // template-chunk stages at most (p.nst at run time)
-// Warps: 0 chunk TMA, 1 UMMA, 2-5 epilogue, 6 ring TMA, and with NEPI = 2 a
-// second epilogue set 7-10.
+// Warps: 0 chunk TMA, 1 UMMA, 2-5 epilogue, 6 ring TMA, and with NEPI = 4 three more
+// epilogue sets 7-18.
 template <int NEPI>
-constexpr int conv_threads() { return NEPI == 2 ? 352 : 224; }
+constexpr int conv_threads() { return 224 + (NEPI - 1) * 128; }
 constexpr int kRowsPerTile = 512;
 constexpr uint32_t kStageA = 128 * 64 * 2;         // one template-pair chunk
 constexpr int kMaxRingRows = 288;                   // per parity, Kc <= 64
 constexpr uint32_t kRingParity = kMaxRingRows * 128;
 constexpr uint32_t kRingBuf = 2 * kRingParity;
 constexpr uint32_t kIdesc = idesc_bf16_f32(128, 256);
-constexpr uint32_t kStageWarp = 2 * 16 * 32 * 4;   // one epilogue warp's staging: [2 buffers][16 rows][32 templates] FP32
+// One epilogue warp's staging: [buffers][16 rows][32 templates] FP32, two buffers with one
+// set of warps, one with four.
+template <int NEPI>
+constexpr int kStageBufs = NEPI == 1 ? 2 : 1;
+constexpr uint32_t kStageBuf = 16 * 32 * 4;
 // After the rings: nst template stages, then nepi x 4 warps' staging; both
-// splits (4 stages + 4 warps, 3 stages + 8 warps) fill the same 80 KB.
-constexpr uint32_t kChunkArea = STAGES * kStageA + 4 * kStageWarp;
-static_assert(3 * kStageA + 8 * kStageWarp == kChunkArea, "the two shared-memory splits must coincide");
+// splits (4 stages + 4 warps x 2 buffers, 3 stages + 16 warps x 1) fill the same 80 KB.
+constexpr uint32_t kChunkArea = STAGES * kStageA + 4 * 2 * kStageBuf;
+static_assert(3 * kStageA + 16 * kStageBuf == kChunkArea, "the two shared-memory splits must coincide");
 constexpr size_t kSmemBytes = 1024 + 2 * kRingBuf + kChunkArea + 256;
 
 struct ConvParams {
@@ -246,11 +250,10 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
         if (lane == 0 && !mbar_wait_drain(drain, 0)) atomicCAS(p.err, 0, DEV_TIMEOUT_DRAIN);
       }
     }
-  } else if ((warp >= 2 && warp <= 5) || (NEPI == 2 && warp >= 7)) {
+  } else if ((warp >= 2 && warp <= 5) || warp >= 7) {
     // ---------------- epilogue: warp q drains TMEM lanes 32q .. 32q+31, i.e. the
     // output rows of parity e = q / 2 for templates t0 .. t0+31, column = row pair;
-    // with two sets, set 0 (warps 2-5) takes the even 32-column chunks and set 1
-    // (warps 7-10) the odd ones.
+    // with four sets, set s takes the 32-column chunks s and s + 4.
     // Full row pairs leave through the warp's own TMA bulk stores of 16 rows x
     // 32 templates from two alternating 2 KB staging buffers, so a buffer is
     // only waited for when the store issued two before it still reads it, and
@@ -263,13 +266,14 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
     // about 35 us.  (With 64 templates direct stores are slower than the TMA path:
     // 78 against 72 us for the call at R = 256.)
     const int q = warp & 3;
-    const int set = warp >= 7 ? 1 : 0;
+    const int set = warp >= 7 ? (warp - 3) >> 2 : 0;
     const int e = q >> 1;
     const int t0 = (q & 1) * 32;
     const int t = t0 + lane;
     const bool tok = t < p.nt;
     const bool wlive = t0 < p.nt;
-    float* stg = stage + (set * 4 + q) * 2 * 16 * 32;   // [2 buffers][16 rows][32 templates]
+    constexpr int kBufs = kStageBufs<NEPI>;
+    float* stg = stage + (set * 4 + q) * kBufs * 16 * 32;   // [buffers][16 rows][32 templates]
     bool issued = false;
     int it = 0;
     // read once: the stores go through a generic pointer, after which a parameter
@@ -300,8 +304,11 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
           if (wlive) {
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-              float* sb = stg + hh * 16 * 32;
-              if (lane == 0) bulk_wait_read_1();  // the store that last read buffer hh is done
+              float* sb = stg + (hh % kBufs) * 16 * 32;
+              if (lane == 0) {   // the store that last read this buffer is done
+                if (kBufs == 2) bulk_wait_read_1();
+                else bulk_wait_read_all();
+              }
               __syncwarp();
 #pragma unroll
               for (int u = 0; u < 16; ++u) sb[u * 32 + lane] = __uint_as_float(r[hh * 16 + u]);
@@ -347,8 +354,11 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
 
 // Reductions of 16 chunks or more (R >= 1024) keep the MMA busy: four template
 // stages and one epilogue set.  Shorter ones are bound by the output write and
-// drain the accumulators with two epilogue sets (three template stages).
-int conv_epilogue_sets(int Kc) { return Kc >= 16 ? 1 : 2; }
+// drain the accumulators with four epilogue sets (three template stages): with two
+// sets of two buffers each, R = 256 on 2^20 samples and 64 templates took 70.0 us a
+// call, with four of one buffer (the same memory) 68.0.  (Rows TMA cannot address
+// gain nothing from more sets: 37 templates at R = 1024 47.1 us with one, 49.0 with four.)
+int conv_epilogue_sets(int Kc) { return Kc >= 16 ? 1 : 4; }
 
 }  // namespace
 
@@ -432,19 +442,19 @@ cudaError_t launch_conv_tc(const uint16_t* G, const uint16_t* TP, float* out, co
     p.tma_out = make_tmap_f32(&p.mapOut, out, 4, dims, strides, box) ? 1 : 0;
   }
   const int nepi = conv_epilogue_sets(g.Kc);
-  static bool attr_set[2][64] = {};
+  static bool attr_set[4][64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !attr_set[nepi - 1][dev]) {
-    e = cudaFuncSetAttribute(nepi == 2 ? conv_tc_kernel<2> : conv_tc_kernel<1>,
+    e = cudaFuncSetAttribute(nepi == 4 ? conv_tc_kernel<4> : conv_tc_kernel<1>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) attr_set[nepi - 1][dev] = true;
   }
   const int grid = p.num_tiles < num_sms ? p.num_tiles : num_sms;
-  if (nepi == 2)
-    return launch_pdl(conv_tc_kernel<2>, dim3(static_cast<unsigned>(grid)), conv_threads<2>(), kSmemBytes, st, 1, p);
+  if (nepi == 4)
+    return launch_pdl(conv_tc_kernel<4>, dim3(static_cast<unsigned>(grid)), conv_threads<4>(), kSmemBytes, st, 1, p);
   return launch_pdl(conv_tc_kernel<1>, dim3(static_cast<unsigned>(grid)), conv_threads<1>(), kSmemBytes, st, 1, p);
 }
 
