@@ -419,13 +419,13 @@ pj_status proj_batch_plan_create(const pj_batch_desc* descs, int32_t n, void* wo
  * chosen by test runs on the target core; here tile heights, K splits and the
  * tile order are chosen per instance by a cost model or by measurement.
  *   schedule:  0 = the cost model splits the reduced dimensions that would set the
- *                  makespan (below); tiles sorted by reduced K, longest first, and
- *                  dealt to the persistent CTAs round-robin, so the tiles of one
- *                  instance run side by side and share their operands in L2;
+ *                  makespan (below); tiles sorted by reduced K, longest first, each to
+ *                  the CTA the model sees least loaded, so the tiles of one instance
+ *                  run side by side and share their operands in L2;
  *              1 = no cost model: tiles sorted by reduced K and dealt round-robin,
  *                  no splits (with tile_rows = 256, the plain longest-K-first order);
- *              2 = as 0, but each tile goes to the CTA the model sees least loaded
- *                  (longest processing time first).
+ *              2 = as 0, but the tiles sorted by their modelled time (longest
+ *                  processing time first).
  *   tile_rows: rows of A_c per GEMM tile (the MMA N): 0 = per instance, the
  *              fewest tiles of at most 256 (E4M3: 240) rows with the least padding;
  *              otherwise a fixed height, a multiple of 32 in [32, 256].

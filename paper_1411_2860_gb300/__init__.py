@@ -844,7 +844,7 @@ class BatchPlan:
 # --------------------------------------------------------------- autotuner --
 
 DEFAULT_CANDIDATES = (
-    None,                                            # cost-model splits, fitted heights, round-robin by K
+    None,                                            # cost-model splits, fitted heights, longest K first
     {"tile_rows": 256},                              # the same with full-height tiles
     {"schedule": 2},                                 # cost-model splits, least-loaded CTA first (LPT)
     {"schedule": 1},                                 # no model: round-robin by reduced K, fitted heights

@@ -5,13 +5,14 @@
 // GEMM instances are the projected products of Sec. III-B.  A correlation
 // instance (valid cross-correlation with the box/Haar projection, Sec. III-A,
 // Eq. 11-13) is lowered to GEMMs, one per (phase, template): with the
-// projected signal b^phi viewed as rows of 128 samples and the projected
-// template kb in a 128 x (R + 127) Toeplitz matrix Kt[p][j] = kb[j - p],
-//   r[phi + Lb (128 i + p)] = sum_j b^phi[128 i + j] Kt[p][j],
-// i.e. output row i of the GEMM holds 128 consecutive lags of that phase.
-// The signal operand is read in the row-split mode of the grouped GEMM (chunk
-// k of row i = view row i + k/2, half k mod 2), so nothing is materialised
-// per lag; the Toeplitz matrix of each template is built once per run.
+// projected signal b^phi viewed as rows of W samples and the projected
+// template kb in a W x (R + W - 1) Toeplitz matrix Kt[p][j] = kb[j - p],
+//   r[phi + Lb (W i + p)] = sum_j b^phi[W i + j] Kt[p][j],
+// i.e. output row i of the GEMM holds W consecutive lags of that phase: W = 256,
+// the width of a CTA pair's tile, or 128 on solo CTAs and for E4M3.
+// The signal operand is read in the row-split mode of the grouped GEMM (with
+// c = W / 64, chunk k of row i = view row i + k / c, column 64 (k mod c)), so nothing
+// is materialised per lag; the Toeplitz matrix of each template is built once per run.
 // GEMM instances with E4M3 compute are quantised after the projections and
 // multiplied by a second persistent grouped launch of the block-scaled kernel.
 //
@@ -19,9 +20,9 @@
 // covers its rows with the least padding, long reduced dimensions may be cut
 // into pieces (by a cost model) whose partial products are added into the
 // (zeroed) FP32 output, and the tiles are dealt to the persistent CTAs sorted
-// by reduced length, round-robin (or, as an option, longest first onto the
-// least-loaded CTA).  By default the BF16 tiles go to clusters of two CTAs in
-// pairs that share their A_c tiles (see schedule_kind).  The cost model's
+// by reduced length (or, as an option, by cost), each onto the least-loaded
+// one.  By default the BF16 products run on 2-SM MMAs (gemm_cg2.cu): clusters
+// of two CTAs take two tile columns at once (see schedule_kind).  The cost model's
 // constants, the height policy, the largest split, the order and the pairing
 // are knobs (pj_batch_tuning) that a measuring autotuner can search.
 #include <cuda_bf16.h>
@@ -55,7 +56,7 @@ struct TplJob {
   const float* k;
   uint16_t* Kt;
   int64_t R, Kpad, ldk, block0;  // row p: hi at [0, Kpad), split residual at [Kpad, 2 Kpad)
-  int Lb, nsplit;
+  int Lb, nsplit, rows;          // rows: samples per output row of the lowering (128 or 256)
   float scale;
 };
 
@@ -119,11 +120,13 @@ __global__ void __launch_bounds__(256) batch_toeplitz_kernel(const TplJob* __res
                                                              const int* __restrict__ job_of) {
   pdl_begin();
   const TplJob J = jobs[job_of[blockIdx.x]];
-  const uint32_t per = static_cast<uint32_t>(J.Kpad / 8);   // Kpad < 2^31, so 128 per fits
-  const uint32_t e = (blockIdx.x - static_cast<uint32_t>(J.block0)) * 256u + threadIdx.x;
-  if (e >= 128u * per) return;
-  const int p = static_cast<int>(e / per);
-  const int64_t jj = static_cast<int64_t>(e - p * per) * 8;
+  const int64_t per = J.Kpad / 8;
+  const int64_t e = (static_cast<int64_t>(blockIdx.x) - J.block0) * 256 + threadIdx.x;
+  if (e >= J.rows * per) return;
+  // (a 32-bit division wherever the entries can be counted in 32 bits)
+  const int p = static_cast<int>(J.rows * per <= 0xffffffffll
+                                     ? static_cast<uint32_t>(e) / static_cast<uint32_t>(per) : e / per);
+  const int64_t jj = (e - p * per) * 8;
   uint16_t h[8], l[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -342,6 +345,9 @@ int pick_bn(int64_t M, int gran, int bnmax, const Tuning& t) {
   const int64_t b = round_up(ceil_div(M > 0 ? M : 1, tiles), gran);
   return static_cast<int>(b < bnmax ? b : bnmax);
 }
+
+// Whether the BF16 instances run on CTA pairs (2-SM MMAs, 256 output columns per tile).
+bool batch_pairs(const Tuning& t) { return PJ_CTA_PAIRS && !t.solo; }
 
 // The largest split the tuner may give an instance: FP32 output, >= 8 K stages a piece.
 int split_cap(int64_t stages, bool fp32_out, const Tuning& t) {
@@ -578,16 +584,20 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
       // E4M3: the BF16 hi + lo of the projected signal and templates feed the quantisers
       const bool e4 = x.prec.compute == PJ_E4M3;
       const int nsplit = e4 ? 2 : x.prec.split_terms;
-      const int64_t Kpad = round_up(g.R + 127, 64);
+      // Samples per output row of the lowering: 256 on CTA pairs, whose tiles are 256 wide
+      // (128 would leave half of every tile empty), else 128.
+      const int W = !e4 && batch_pairs(b.tune) ? 256 : 128;
+      const int64_t Kpad = round_up(g.R + W - 1, 64);
       const int64_t Kq = round_up(Kpad, 128);
       const float scale = 1.0f / sqrtf(static_cast<float>(g.Lb));
       std::vector<uint16_t*> kts(g.nt);
       for (int64_t t = 0; t < g.nt; ++t) {
-        const size_t kt = L.take(2 * 128 * Kpad * nsplit);
+        const size_t kt = L.take(2 * W * Kpad * nsplit);
         TplJob tj{};
         tj.k = static_cast<const float*>(x.B) + t * g.T;
         tj.Kt = ptr<uint16_t>(ws, kt);
-        tj.R = g.R; tj.Kpad = Kpad; tj.ldk = Kpad * nsplit; tj.Lb = g.Lb; tj.nsplit = nsplit; tj.scale = scale;
+        tj.R = g.R; tj.Kpad = Kpad; tj.ldk = Kpad * nsplit; tj.Lb = g.Lb; tj.nsplit = nsplit; tj.rows = W;
+        tj.scale = scale;
         b.tpl.push_back(tj);
         kts[t] = tj.Kt;
       }
@@ -603,12 +613,12 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
       for (int phi = 0; phi < g.Lb; ++phi) {
         const int64_t lags_phi = g.lags > phi ? ceil_div(g.lags - phi, g.Lb) : 0;
         if (lags_phi == 0) continue;
-        const int64_t rows_alloc = ceil_div(lags_phi + g.R - 1, 128) + 1;
-        const size_t q = L.take(2 * 128 * rows_alloc * nsplit);
+        const int64_t rows_alloc = ceil_div(lags_phi + g.R - 1, W) + 1;
+        const size_t q = L.take(2 * W * rows_alloc * nsplit);
         SigJob sj{};
         sj.s = static_cast<const float*>(x.A); sj.Q = ptr<uint16_t>(ws, q);
-        sj.Qlo = nsplit > 1 ? ptr<uint16_t>(ws, q + 2 * 128 * rows_alloc) : nullptr;
-        sj.S = g.S; sj.n = rows_alloc * 128; sj.Lb = g.Lb; sj.phi = phi; sj.scale = scale;
+        sj.Qlo = nsplit > 1 ? ptr<uint16_t>(ws, q + 2 * W * rows_alloc) : nullptr;
+        sj.S = g.S; sj.n = rows_alloc * W; sj.Lb = g.Lb; sj.phi = phi; sj.scale = scale;
         b.sig.push_back(sj);
         if (e4) {
           const int64_t rowsQ = ceil_div(lags_phi, 128);
@@ -639,8 +649,8 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
         }
         for (int64_t t = 0; t < g.nt; ++t) {
           GemmTcArgs a;
-          a.Q = sj.Q; a.ldq = 128; a.rowsQ = ceil_div(lags_phi, 128);
-          a.P = kts[t]; a.ldp = Kpad * nsplit; a.rowsP = 128;
+          a.Q = sj.Q; a.ldq = W; a.rowsQ = ceil_div(lags_phi, W);
+          a.P = kts[t]; a.ldp = Kpad * nsplit; a.rowsP = W;
           a.xdim = Kpad * nsplit; a.kdim = Kpad;
           if (nsplit == 1) {
             a.nseg = 1;
@@ -653,14 +663,14 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
             a.segQ[2] = rows_alloc; a.segP[2] = 0;
           }
           a.Y = static_cast<float*>(x.Y) + phi * g.nt + t;
-          a.ldy = 128; a.out_dtype = PJ_F32;
-          a.conv_mode = 1; a.q_rows_alloc = rows_alloc * nsplit;
+          a.ldy = W; a.out_dtype = PJ_F32;
+          a.conv_mode = 1; a.conv_w = W; a.q_rows_alloc = rows_alloc * nsplit;
           a.conv_stride = static_cast<int64_t>(g.Lb) * g.nt;
           a.conv_limit = lags_phi;
           a.bn = 256;
           const int stages = static_cast<int>(ceil_div(Kpad, 64)) * a.nseg;
           b.planned.push_back(GemmPlanned{0, static_cast<int>(b.gemms.size()),
-                                          static_cast<int>(ceil_div(a.rowsQ, 256)), 1, stages, 256, 1, false});
+                                          static_cast<int>(ceil_div(a.rowsQ, 256)), W / 128, stages, 256, 1, false});
           b.gemms.push_back(a);
         }
       }
@@ -680,7 +690,7 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
   for (auto& s : b.sig) { s.block0 = blk; blk += ceil_div(s.n, kSigPerBlock); }
   b.sig_total = blk;
   blk = 0;
-  for (auto& t : b.tpl) { t.block0 = blk; blk += ceil_div(128 * t.Kpad, kTplPerBlock); }
+  for (auto& t : b.tpl) { t.block0 = blk; blk += ceil_div(t.rows * t.Kpad, kTplPerBlock); }
   b.tpl_total = blk;
   blk = 0;
   for (auto& q : b.sigq) { q.block0 = blk; blk += ceil_div(q.nblk, 256); }
@@ -731,8 +741,7 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
   b.mx_off = L.take(sizeof(MxInst) * (b.mx.size() + 1));
   // tile lists sized for the largest split the tuner may choose
   int tiles = 0, mx_tiles = 0;
-  // (plus, for paired BF16 tiles, at most one stand-in tile per piece of an instance)
-  for (const auto& pl : b.planned) (pl.kind ? mx_tiles : tiles) += pl.tiles_m * pl.tiles_n * pl.cap + (pl.kind ? 0 : pl.cap);
+  for (const auto& pl : b.planned) (pl.kind ? mx_tiles : tiles) += pl.tiles_m * pl.tiles_n * pl.cap;
   b.tiles_cap = tiles;
   b.mx_tiles_cap = mx_tiles;
   b.tiles_off = L.take(sizeof(GemmTile) * (tiles + 1));
@@ -752,10 +761,11 @@ double tile_cost(const Tuning& t, int stages, int bn, bool out_bf16, bool red) {
 
 struct Schedule {
   std::vector<GemmTile> tiles;  // CTA by CTA
-  std::vector<int> cta_off;     // ctas + 1 entries
+  std::vector<int> cta_off;     // ctas (paired: clusters of two) + 1 entries
   double makespan = 0, total = 0;
   int splits = 0;
-  bool paired = false;          // CTAs 2c and 2c + 1 form a cluster (see schedule_kind)
+  int64_t count = 0;            // tiles of 128 output columns, split pieces counted
+  bool paired = false;          // the lists are those of clusters of two CTAs
 };
 
 // Tiles of the instances of one kernel (kind), with the splits chosen, dealt to
@@ -800,15 +810,10 @@ Schedule schedule_kind(const Built& b, int kind, int sms, bool paired) {
       if (!changed) break;
     }
   }
-  // An item is the work of one CTA or, paired, of the two CTAs of a cluster:
-  // t[0] for the CTA of rank 0, t[1] for rank 1.  Paired tiles are neighbouring
-  // tile columns of one tile row (they share that row's A_c tiles); the last
-  // column of an odd number of columns pairs with the same column of the next
-  // tile row, each CTA loading its own A_c tile (flag 1), and a last one left
-  // over pairs with a stand-in copy of itself whose output is not written
-  // (flags 1 | 2).  Both tiles of an item have the same K stages.
+  // An item is the work of one CTA or, paired, of the two CTAs of a cluster on the two
+  // tile columns of one pair column (a last single column leaves its second CTA idle).
   struct Item {
-    GemmTile t[2];
+    GemmTile t;
     double cost;
   };
   std::vector<Item> items;
@@ -817,25 +822,15 @@ Schedule schedule_kind(const Built& b, int kind, int sms, bool paired) {
     const GemmPlanned& pl = *ins[i];
     const int sp = split[i];
     if (sp > 1) ++S.splits;
+    S.count += static_cast<int64_t>(pl.tiles_m) * pl.tiles_n * sp;
+    const int cols = paired ? (pl.tiles_n + 1) / 2 : pl.tiles_n;
     for (int k = 0; k < sp; ++k) {
       const int k0 = static_cast<int>(static_cast<int64_t>(pl.stages) * k / sp);
       const int k1 = static_cast<int>(static_cast<int64_t>(pl.stages) * (k + 1) / sp);
       const double cost = tile_cost(t, k1 - k0, pl.bn, pl.out_bf16, sp > 1);
-      auto tile = [&](int ti, int tj, int flags) {
-        return GemmTile{pl.index, ti, tj, k0, k1, sp > 1 ? 1 : 0, flags, 0};
-      };
-      if (!paired) {
-        for (int ti = 0; ti < pl.tiles_m; ++ti)
-          for (int tj = 0; tj < pl.tiles_n; ++tj) items.push_back(Item{{tile(ti, tj, 0), tile(ti, tj, 0)}, cost});
-        continue;
-      }
       for (int ti = 0; ti < pl.tiles_m; ++ti)
-        for (int tj = 0; tj + 1 < pl.tiles_n; tj += 2) items.push_back(Item{{tile(ti, tj, 0), tile(ti, tj + 1, 0)}, cost});
-      if (pl.tiles_n % 2) {
-        const int tj = pl.tiles_n - 1;
-        for (int ti = 0; ti + 1 < pl.tiles_m; ti += 2) items.push_back(Item{{tile(ti, tj, 1), tile(ti + 1, tj, 1)}, cost});
-        if (pl.tiles_m % 2) items.push_back(Item{{tile(pl.tiles_m - 1, tj, 1), tile(pl.tiles_m - 1, tj, 3)}, cost});
-      }
+        for (int tj = 0; tj < cols; ++tj)
+          items.push_back(Item{GemmTile{pl.index, ti, tj, k0, k1, sp > 1 ? 1 : 0, 0, 0}, cost});
     }
   }
   // units that take items: CTAs, or clusters of two when paired
@@ -843,46 +838,41 @@ Schedule schedule_kind(const Built& b, int kind, int sms, bool paired) {
   const int units = static_cast<int>(items.size() < static_cast<size_t>(slots) ? items.size() : slots);
   std::vector<std::vector<int>> per(units);
   std::vector<double> load(units, 0.0);
-  if (t.schedule != 2) {
-    // longest reduced K first (measured faster than costliest first), dealt
-    // round-robin, so the tiles of one instance run side by side and share
-    // their operand panels in L2
-    std::vector<int> order(items.size());
-    for (size_t k = 0; k < order.size(); ++k) order[k] = static_cast<int>(k);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
-      return items[a].t[0].k1 - items[a].t[0].k0 > items[c].t[0].k1 - items[c].t[0].k0;
-    });
-    for (size_t k = 0; k < order.size(); ++k) {
-      per[k % units].push_back(order[k]);
-      load[k % units] += items[order[k]].cost;
+  // Longest reduced K first, each item onto the least-loaded unit: the tiles of one
+  // instance run side by side and share their operand panels in L2, and the loads even
+  // out (dealt round-robin, the busiest pair of a 60-product batch worked 8 % longer than
+  // the mean: 1424 us for the call against 1384).  schedule 2 takes the costliest item first (LPT),
+  // schedule 1 has no costs and deals round-robin.
+  std::vector<int> order(items.size());
+  for (size_t k = 0; k < order.size(); ++k) order[k] = static_cast<int>(k);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
+    return t.schedule == 2 ? items[a].cost > items[c].cost : items[a].t.k1 - items[a].t.k0 > items[c].t.k1 - items[c].t.k0;
+  });
+  std::vector<std::pair<double, int>> heap;
+  for (int c = 0; c < units; ++c) heap.push_back({0.0, c});
+  auto cmp = [](const std::pair<double, int>& a, const std::pair<double, int>& c) {
+    return a.first > c.first || (a.first == c.first && a.second > c.second);
+  };
+  std::make_heap(heap.begin(), heap.end(), cmp);
+  for (size_t n = 0; n < order.size(); ++n) {
+    const int k = order[n];
+    if (t.schedule == 1) {   // the plan without a cost model
+      per[n % units].push_back(k);
+      load[n % units] += items[k].cost;
+      continue;
     }
-  } else {
-    // LPT: costliest item first onto the least-loaded unit
-    std::vector<int> order(items.size());
-    for (size_t k = 0; k < order.size(); ++k) order[k] = static_cast<int>(k);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return items[a].cost > items[c].cost; });
-    std::vector<std::pair<double, int>> heap;
-    for (int c = 0; c < units; ++c) heap.push_back({0.0, c});
-    auto cmp = [](const std::pair<double, int>& a, const std::pair<double, int>& c) {
-      return a.first > c.first || (a.first == c.first && a.second > c.second);
-    };
-    std::make_heap(heap.begin(), heap.end(), cmp);
-    for (int k : order) {
-      std::pop_heap(heap.begin(), heap.end(), cmp);
-      auto& top = heap.back();
-      per[top.second].push_back(k);
-      top.first += items[k].cost;
-      load[top.second] = top.first;
-      std::push_heap(heap.begin(), heap.end(), cmp);
-    }
+    std::pop_heap(heap.begin(), heap.end(), cmp);
+    auto& top = heap.back();
+    per[top.second].push_back(k);
+    top.first += items[k].cost;
+    load[top.second] = top.first;
+    std::push_heap(heap.begin(), heap.end(), cmp);
   }
   S.cta_off.push_back(0);
   for (int c = 0; c < units; ++c) {
-    for (int r = 0; r < (paired ? 2 : 1); ++r) {
-      for (int k : per[c]) S.tiles.push_back(items[k].t[r]);
-      S.cta_off.push_back(static_cast<int>(S.tiles.size()));
-      S.total += load[c];
-    }
+    for (int k : per[c]) S.tiles.push_back(items[k].t);
+    S.cta_off.push_back(static_cast<int>(S.tiles.size()));
+    S.total += load[c] * (paired ? 2 : 1);
     S.makespan = load[c] > S.makespan ? load[c] : S.makespan;
   }
   S.paired = paired;
@@ -954,7 +944,7 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   }
   // instance tables and the tuned schedules of the two grouped launches
   // BF16 products on CTA pairs unless the tuning asks for solo CTAs
-  const bool paired = PJ_CTA_PAIRS && !w.tune.solo && sms >= 2;
+  const bool paired = batch_pairs(w.tune);
   std::vector<GemmInst> insts(w.gemms.size());
   for (size_t i = 0; i < w.gemms.size(); ++i) {
     w.gemms[i].pair = paired ? 1 : 0;
@@ -1079,7 +1069,7 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   p->sig_of = ptr<int>(workspace, w.sig_map_off);
   p->tpl_of = ptr<int>(workspace, w.tpl_map_off);
   for (const auto& s : w.sig) p->sig_blocks = s.block0 + ceil_div(s.n, kSigPerBlock);
-  for (const auto& t : w.tpl) p->tpl_blocks = t.block0 + ceil_div(128 * t.Kpad, kTplPerBlock);
+  for (const auto& t : w.tpl) p->tpl_blocks = t.block0 + ceil_div(t.rows * t.Kpad, kTplPerBlock);
   p->d_sigq = ptr<SigQJob>(workspace, w.sigq_off);
   p->d_sfx = ptr<SfExpJob>(workspace, w.sfx_off);
   p->sigq_of = ptr<int>(workspace, w.sigq_map_off);
@@ -1089,7 +1079,7 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   p->d_insts = ptr<GemmInst>(workspace, w.insts_off);
   p->d_tiles = ptr<GemmTile>(workspace, w.tiles_off);
   p->d_cta_off = ptr<int>(workspace, w.cta_off_off);
-  p->ctas = static_cast<int>(S0.cta_off.size()) - 1;
+  p->ctas = static_cast<int>(S0.cta_off.size()) - 1;   // clusters of two when paired
   p->paired = S0.paired ? 1 : 0;
   p->d_mx = ptr<MxInst>(workspace, w.mx_off);
   p->d_mx_tiles = ptr<GemmTile>(workspace, w.mx_tiles_off);
@@ -1102,9 +1092,10 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   p->zero_of = ptr<int>(workspace, w.zero_map_off);
   p->zero_blocks = zero_blocks;
   p->sms = sms;
-  p->info.gemm_tiles = static_cast<int32_t>(S0.tiles.size());
-  p->info.mx_tiles = static_cast<int32_t>(S1.tiles.size());
-  p->info.ctas = p->ctas > p->mx_ctas ? p->ctas : p->mx_ctas;
+  p->info.gemm_tiles = static_cast<int32_t>(S0.count);
+  p->info.mx_tiles = static_cast<int32_t>(S1.count);
+  const int main_ctas = p->ctas * (p->paired ? 2 : 1);
+  p->info.ctas = main_ctas > p->mx_ctas ? main_ctas : p->mx_ctas;
   p->info.split_instances = S0.splits + S1.splits;
   p->info.model_makespan_us = S0.makespan + S1.makespan;
   p->info.model_total_us = S0.total + S1.total;
@@ -1147,8 +1138,10 @@ pj_status proj_batch_run(const pj_batch_plan* plan, void* stream) {
   if (plan->zero_blocks > 0) {
     PJ_CUDA_TRY(launch_plain(batch_zero_kernel, dim3(static_cast<unsigned>(plan->zero_blocks)), 256, 0, st, plan->d_zero, plan->zero_of));
   }
-  PJ_CUDA_TRY(launch_gemm_tc_grouped(plan->d_insts, plan->d_tiles, plan->d_cta_off, plan->ctas, plan->paired,
-                                     error_word(plan->ws), st));
+  PJ_CUDA_TRY(plan->paired ? launch_gemm_cg2_grouped(plan->d_insts, plan->d_tiles, plan->d_cta_off, plan->ctas,
+                                                     error_word(plan->ws), st)
+                           : launch_gemm_tc_grouped(plan->d_insts, plan->d_tiles, plan->d_cta_off, plan->ctas,
+                                                    error_word(plan->ws), st));
   PJ_CUDA_TRY(launch_gemm_mx_grouped(plan->d_mx, plan->d_mx_tiles, plan->d_mx_cta_off, plan->mx_ctas,
                                      error_word(plan->ws), st));
   return PJ_OK;

@@ -350,18 +350,19 @@ struct GemmTcArgs {
   void* Y;
   int64_t ldy;
   int out_dtype;
-  // Row-split mode (a lowered correlation): Q is a 128-wide view with q_rows_alloc
-  // rows; K chunk k of output row r reads view row r + k/2 at column 64 (k mod 2).
-  // Output element (i, j) is sample i*128 + j < conv_limit, at Y[(i*128 + j) * conv_stride].
+  // Row-split mode (a lowered correlation): Q is a conv_w-wide view with q_rows_alloc
+  // rows; with c = conv_w / 64, K chunk k of output row r reads view row r + k / c at
+  // column 64 (k mod c).  Output element (i, j) is sample i * conv_w + j < conv_limit, at
+  // Y[(i * conv_w + j) * conv_stride].
   int conv_mode = 0;
   int64_t q_rows_alloc = 0, conv_stride = 1, conv_limit = 0;
+  int conv_w = 128;   // width of that view and samples per output row: 128, or 256 for CTA pairs
   int bn = 256;   // rows of Q per tile: a multiple of 32 (64 for an MN-major Q), at most 256
   // MN-major operands: Q (P) is stored transposed, as xdim rows of the reduced
   // dimension by rowsQ (rowsP) contiguous values with pitch ldq (ldp); the tensor
   // cores read it as it is, so no transposed copy is made.
   int mnQ = 0, mnP = 0;
-  // Set by launch_gemm_tc_generic: CTA pairs (clusters of two) share each Q tile,
-  // each loading half of it for both; the Q tensor map then has half-height boxes.
+  // 2-SM MMAs: each CTA of a pair loads half of the Q tile (half-height boxes).
   int pair = 0;
   // Failure-detection self-test only (pj_selftest_timeout): the copy producer stops
   // after this many K stages, so the waits of the MMA and epilogue warps run out.
@@ -428,7 +429,7 @@ struct GemmInst {  // 128-byte aligned through its tensor maps
   int M, N, kc, nseg;     // kc: K stages of all segments together
   int segP[3], segQ[3];
   int segKc[3];           // K stages of each segment
-  int tiles_n, out_bf16, tma_out, tma_rows, conv_mode;
+  int tiles_n, out_bf16, tma_out, tma_rows, conv_mode, conv_w;
   // TMA boxes may store (or add into) tile columns that end at or before this
   // column.  A TMA store writes the whole 16-byte chunk that holds a row's last
   // element, so when a row of Y does not end on a 16-byte boundary the ragged
@@ -453,16 +454,18 @@ int share_chunk(int k) { return (k + 2) / 3; }
 // instance's reduced dimension is split), and red = 1 when its partial product
 // is added to the output (the output is zeroed first) instead of stored.
 struct GemmTile {
-  int inst, ti, tj, k0, k1, red, pad0, pad1;   // pad0: pair flags (see launch_gemm_tc_grouped)
+  int inst, ti, tj, k0, k1, red, pad0, pad1;   // tj: tile column, or pair column on CTA pairs
 };
 bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I);
 int gemm_tiles_of(const GemmInst& I);
 // Tiles of CTA c are tiles[cta_off[c] .. cta_off[c+1]); `ctas` blocks.
-// pair: the lists were planned for clusters of two CTAs (2c, 2c + 1), whose tile
-// i share their rows of A_c unless flagged (pad0 bit 0: loads its own A_c tile;
-// bit 1: a stand-in that writes nothing); every instance then has pair = 1.
 cudaError_t launch_gemm_tc_grouped(const GemmInst* insts, const GemmTile* tiles, const int* cta_off, int ctas,
-                                   int pair, int* err, cudaStream_t st);
+                                   int* err, cudaStream_t st);
+// The same on 2-SM MMAs (gemm_cg2.cu): `pairs` clusters of two CTAs, tj counting pairs of
+// tile columns (the second column of the last pair may not exist); every instance was
+// built with pair = 1.
+cudaError_t launch_gemm_cg2_grouped(const GemmInst* insts, const GemmTile* tiles, const int* pair_off, int pairs,
+                                    int* err, cudaStream_t st);
 
 // Forward reduced product: Y (M x N) = A_c * B_d^T with split segments.
 cudaError_t launch_gemm_tc(const uint16_t* Ac, const uint16_t* Bd, void* Y, int64_t ldy, int out_dtype,

@@ -18,11 +18,17 @@
 // commit frees the stage in both CTAs.  Both CTAs' epilogue warps arrive on the
 // leader's accumulator barriers.
 //
-// The producer and the issuer are one thread each, and their instruction chains
-// set the pace: with the instance's fields read in the loop (again after every
-// copy) and descriptors built per MMA, a slot of the 4096 x 2048 product over
-// 12,880 components took 0.34 us whatever was prefetched; with everything held
-// in registers it takes 0.30 us (137 -> 122 us, 1.77 PFLOP/s).
+// The producer's and the issuer's instruction chains set the pace: with the instance's
+// fields read in the loop (again after every copy) and descriptors built per MMA, a slot
+// of the 4096 x 2048 product over 12,880 components took 0.34 us whatever was
+// prefetched; with everything held in registers it takes 0.30 us (137 -> 122 us, 1.77
+// PFLOP/s).
+//
+// A batch's products run here too (kGrouped): on CTAs of their own (gemm_tc.cu) they
+// drew 96 KB of operands per 64-component chunk through an SM that can take in about 74
+// bytes a clock, and the grouped launch of 40 products and 20 correlations took 818 us;
+// here it takes 64 KB and 733 us at 98 % of the tensor pipe's cycles, under the power
+// cap (1.74 GHz).
 #include <cuda_bf16.h>
 #include <string.h>
 
@@ -65,6 +71,10 @@ __host__ __device__ constexpr int cg2_slots(int bn) {
 
 struct Cg2Params {
   GemmInst I;       // P map box {CK, CM} (MN-major: {64, CK}); Q map box {CK, bn/2} (MN-major: {64, CK})
+  const GemmInst* insts;   // grouped launch: the instances, the tiles pair by pair (tj counts pair
+  const GemmTile* tiles;   // columns), and where each pair's tiles start
+  const int* pair_off;
+  int slot_rows;    // tile height the ring slots are sized for (the instance's, or 256 when grouped)
   ExpandArgs ex;
   Coef8 ex_c8;      // the expansion's vectors when ex.coef is null
   int npp;          // pair columns: P tile columns of 256
@@ -73,13 +83,35 @@ struct Cg2Params {
   int* err;
 };
 
-template <bool kMN>
+// The n-th tile of this pair: instance, pair column tj, tile row ti and K-stage range;
+// null past the last.
+template <bool kGrouped>
+__device__ __forceinline__ const GemmInst* cg2_tile(const Cg2Params& p, int n, GemmTile& t) {
+  if (kGrouped) {
+    const int k = p.pair_off[blockIdx.x / 2] + n;
+    if (k >= p.pair_off[blockIdx.x / 2 + 1]) return nullptr;
+    t = p.tiles[k];
+    return p.insts + t.inst;
+  }
+  const int pi = static_cast<int>(blockIdx.x / 2) + n * static_cast<int>(gridDim.x / 2);
+  if (pi >= p.num_pairs) return nullptr;
+  t.tj = pi % p.npp;
+  t.ti = pi / p.npp;
+  t.k0 = 0;
+  t.k1 = p.I.kc;
+  t.red = 0;
+  return &p.I;
+}
+
+// kGrouped: the batch's launch, many instances (K-major, no expansion) over planned tile
+// lists; see launch_gemm_cg2_grouped.
+template <bool kMN, bool kGrouped>
 __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_constant__ Cg2Params p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  const int nst = cg2_slots(p.I.bn);
-  const uint32_t slot_bytes = kCStageP + static_cast<uint32_t>(p.I.bn / 2) * CK * 2;   // P rows, then Q rows
+  const int nst = cg2_slots(p.slot_rows);
+  const uint32_t slot_bytes = kCStageP + static_cast<uint32_t>(p.slot_rows / 2) * CK * 2;   // P rows, then Q rows
   uint8_t* stage_out = sm + kCRing;
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage_out + kCStageOut);
   uint64_t* full = bars;
@@ -91,7 +123,6 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
   int* vote = reinterpret_cast<int*>(tslot + 4);   // 2 x 8 flags
   static_assert((2 * kCMaxStages + 5) * 8 + 16 + 16 * 4 <= kCCtl, "barriers, TMEM slot and votes");
   __shared__ float s_coef[64];
-  const GemmInst* I = &p.I;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const uint32_t rank = cluster_ctarank();
@@ -125,34 +156,37 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
     {
       // ---------------- TMA producer (both CTAs; the whole warp, one lane issues): this
       // CTA's P rows and half of the Q rows
-      if (lane == 0) {
-        tma_prefetch(&I->mapP);
-        tma_prefetch(&I->mapQ);
-      }
-      __syncwarp();
       int stage = 0;
       uint32_t phase = 0;
       uint32_t used = 0, last_phase = 0;   // bit s: slot s was filled; the phase of its last fill
       bool ok = true;
       int issued = 0;
-      // read once (see gemm_tc.cu: a value read through I would be read again after every copy)
-      const CUtensorMap* const mapP = &I->mapP;
-      const CUtensorMap* const mapQ = &I->mapQ;
-      const int bn = I->bn, half = bn / 2, npp = p.npp, num_pairs = p.num_pairs, stall = p.stall;
-      const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
-      const bool share = I->share != 0;   // hi and lo tiles in alternate slots (GemmInst::share)
-      const int fills = share ? I->kc / 3 * 2 : I->kc;
-      const int sP0 = I->segP[0], sP1 = I->segP[1], sP2 = I->segP[2];
-      const int sQ0 = I->segQ[0], sQ1 = I->segQ[1], sQ2 = I->segQ[2];
-      const int e0 = I->nseg > 1 ? I->segKc[0] : 0x7fffffff, e1 = I->nseg > 2 ? e0 + I->segKc[1] : 0x7fffffff;
-      const uint32_t pair_bytes = 2 * (kCStageP + static_cast<uint32_t>(half) * CK * 2);
+      const int stall = p.stall;
+      GemmTile T{};
       for (int n = 0; ok; ++n) {
-        const int pi = static_cast<int>(blockIdx.x / 2) + n * static_cast<int>(gridDim.x / 2);
-        if (pi >= num_pairs) break;
-        const int pc = pi % npp, ti = pi / npp;
-        const int prow = pc * 2 * CM + static_cast<int>(rank) * CM;
-        const int qrow = ti * bn + static_cast<int>(rank) * half;
-        for (int kk = 0; kk < fills; ++kk, ++issued) {
+        const GemmInst* I = cg2_tile<kGrouped>(p, n, T);
+        if (!I) break;
+        // read once (see gemm_tc.cu: a value read through I would be read again after every copy)
+        const CUtensorMap* const mapP = &I->mapP;
+        const CUtensorMap* const mapQ = &I->mapQ;
+        if (lane == 0 && (kGrouped || n == 0)) {
+          tma_prefetch(mapP);
+          tma_prefetch(mapQ);
+        }
+        __syncwarp();
+        const int bn = I->bn, half = bn / 2;
+        const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
+        const bool share = I->share != 0;   // hi and lo tiles in alternate slots (GemmInst::share)
+        const bool conv = kGrouped && I->conv_mode != 0;
+        const int cmask = conv ? I->conv_w / CK - 1 : 0, cshift = conv ? 31 - __clz(I->conv_w / CK) : 0;
+        const int f0 = share ? 2 * share_chunk(T.k0) : T.k0, f1 = share ? 2 * share_chunk(T.k1) : T.k1;
+        const int sP0 = I->segP[0], sP1 = I->segP[1], sP2 = I->segP[2];
+        const int sQ0 = I->segQ[0], sQ1 = I->segQ[1], sQ2 = I->segQ[2];
+        const int e0 = I->nseg > 1 ? I->segKc[0] : 0x7fffffff, e1 = I->nseg > 2 ? e0 + I->segKc[1] : 0x7fffffff;
+        const uint32_t pair_bytes = 2 * (kCStageP + static_cast<uint32_t>(half) * CK * 2);
+        const int prow = T.tj * 2 * CM + static_cast<int>(rank) * CM;
+        const int qrow0 = T.ti * bn + static_cast<int>(rank) * half;
+        for (int kk = f0; kk < f1; ++kk, ++issued) {
           if (issued == stall) {
             ok = false;
             break;
@@ -171,7 +205,10 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             oP = kk < e0 ? sP0 : (kk < e1 ? sP1 : sP2);
             oQ = kk < e0 ? sQ0 : (kk < e1 ? sQ1 : sQ2);
           }
-          const int px = oP + kin * CK, qx = oQ + kin * CK;
+          const int px = oP + kin * CK;
+          // (a lowered correlation's Q: see gemm_tc.cu)
+          const int qx = conv ? (kin & cmask) * CK : oQ + kin * CK;
+          const int qrow = conv ? qrow0 + (kin >> cshift) + oQ : qrow0;
           const uint32_t bar = full_leader + stage * 8;
           uint8_t* const dP = sm + stage * slot_bytes;
           uint8_t* const dQ = dP + kCStageP;
@@ -209,24 +246,24 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
   } else if (warp == 1) {
     if (leader) {
       // ---------------- MMA issuer (the leader's whole warp; one lane issues)
-      const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
-      const uint32_t idesc = idesc_bf16_f32(2 * CM, I->bn) | (static_cast<uint32_t>(mnP) << 15) |
-                             (static_cast<uint32_t>(mnQ) << 16);
-      // (A K step of 16 moves a K-major start by 32 bytes, an MN-major one by 2048.)
       const uint32_t a0 = smem_u32(sm), slot_units = slot_bytes / 16;
-      const uint64_t bP = mnP ? sdesc_sw128_mn(a0, 8192) : sdesc_sw128(a0, 0);
-      const uint64_t bQ = mnQ ? sdesc_sw128_mn(a0 + kCStageP, 8192) : sdesc_sw128(a0 + kCStageP, 0);
-      const uint32_t kP = mnP ? 128 : 2, kQ = mnQ ? 128 : 2;
-      const bool share = I->share != 0;
-      const int chunks = share ? I->kc / 3 : I->kc;
-      const int num_pairs = p.num_pairs;
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
       bool issued_any = false;
+      GemmTile T{};
       for (int n = 0, it = 0; ok; ++n, ++it) {
-        const int pi = static_cast<int>(blockIdx.x / 2) + n * static_cast<int>(gridDim.x / 2);
-        if (pi >= num_pairs) break;
+        const GemmInst* I = cg2_tile<kGrouped>(p, n, T);
+        if (!I) break;
+        const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
+        const uint32_t idesc = idesc_bf16_f32(2 * CM, I->bn) | (static_cast<uint32_t>(mnP) << 15) |
+                               (static_cast<uint32_t>(mnQ) << 16);
+        // (A K step of 16 moves a K-major start by 32 bytes, an MN-major one by 2048.)
+        const uint64_t bP = mnP ? sdesc_sw128_mn(a0, 8192) : sdesc_sw128(a0, 0);
+        const uint64_t bQ = mnQ ? sdesc_sw128_mn(a0 + kCStageP, 8192) : sdesc_sw128(a0 + kCStageP, 0);
+        const uint32_t kP = mnP ? 128 : 2, kQ = mnQ ? 128 : 2;
+        const bool share = I->share != 0;
+        const int c0 = share ? share_chunk(T.k0) : T.k0, c1 = share ? share_chunk(T.k1) : T.k1;
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
         if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, p.err, DEV_TIMEOUT_ACC_FREE)) break;
@@ -239,14 +276,14 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
           for (int k = 0; k < CK / 16; ++k)
             umma_f16_cg2(d, sdesc_advance(dp, k * kP), sdesc_advance(dq, k * kQ), idesc, !first || (k != 0));
         };
-        for (int kk = 0; kk < chunks; ++kk) {
+        for (int kk = c0; kk < c1; ++kk) {
           if (!mbar_wait_warp(&full[stage], phase, p.err, DEV_TIMEOUT_FULL)) {
             ok = false;
             break;
           }
           tc_fence_after();
           if (elect_one()) {
-            products(stage, stage, kk == 0);
+            products(stage, stage, kk == c0);
             if (!share) umma_commit_cg2_mc(&empty[stage], 0x3);
           }
           __syncwarp();
@@ -294,24 +331,32 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
     // Everything the stores need, read from the parameters once: the stores go
     // through generic pointers, so values read through a pointer to the
     // parameters would be read again after every store.
-    const ExpandArgs ex = p.ex;
-    const int M = I->M, N = I->N, bn = I->bn;
-    const bool out_bf16 = I->out_bf16 != 0;
-    const bool tma_out = I->tma_out != 0;
-    const int tma_cols = I->tma_cols;
-    const int64_t ldy = I->ldy;
-    void* const Yout = I->Y;
-    const uint32_t chunk_bytes = 32u * CM * (out_bf16 ? 2u : 4u);
-    const int nbuf = static_cast<int>(kCStageOut / chunk_bytes);
-    int sbuf = 0;
+    const ExpandArgs ex = kGrouped ? ExpandArgs{} : p.ex;
+    int sbuf = 0, last_nbuf = 0;
+    bool relaid = false;
     if (ex.mode)
       for (int e = threadIdx.x - 64; e < 8 * ex.lp1; e += 256)
         s_coef[e] = ex.coef ? ex.coef[e] : p.ex_c8.c[expand_c8_index(ex, e)];
     named_barrier(1, 256);
+    GemmTile T{};
     for (int n = 0, it = 0;; ++n, ++it) {
-      const int pi = static_cast<int>(blockIdx.x / 2) + n * static_cast<int>(gridDim.x / 2);
-      if (pi >= p.num_pairs) break;
-      const int ti = pi / p.npp, tj = (pi % p.npp) * 2 + static_cast<int>(rank);
+      const GemmInst* I = cg2_tile<kGrouped>(p, n, T);
+      if (!I) break;
+      const int ti = T.ti, tj = T.tj * 2 + static_cast<int>(rank);
+      const bool red = T.red != 0;
+      const int M = I->M, N = I->N, bn = I->bn;
+      const bool out_bf16 = I->out_bf16 != 0;
+      const int tma_rows = I->tma_out && (tj + 1) * CM <= I->tma_cols ? I->tma_rows : 0;
+      const int64_t ldy = I->ldy;
+      void* const Yout = I->Y;
+      const uint32_t chunk_bytes = 32u * CM * (out_bf16 ? 2u : 4u);
+      const int nbuf = static_cast<int>(kCStageOut / chunk_bytes);
+      // another element size lays the staging out anew: the next store waits for all under way
+      if (kGrouped && last_nbuf != 0 && nbuf != last_nbuf) {
+        relaid = true;
+        sbuf = 0;
+      }
+      last_nbuf = nbuf;
       const int acc = it & 1;
       const uint32_t acc_phase = (it >> 1) & 1;
       const bool okw = __all_sync(0xffffffffu, mbar_wait(&acc_full[acc], acc_phase, p.err, DEV_TIMEOUT_ACC));
@@ -332,18 +377,21 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
         expand_tile(tmem + acc * CN + h * hb + (static_cast<uint32_t>(q * 32) << 16), hb, ex, s_coef, lane,
                     j, ncomp, ti * bn + h * hb, M, j, jok);
       }
-      for (int c0 = 0; c0 < (ex.mode || h ? 0 : bn); c0 += 32) {
+      // (a pair's second column past an odd number of columns writes nothing)
+      for (int c0 = 0; c0 < (ex.mode || h || tj * CM >= N ? 0 : bn); c0 += 32) {
         uint32_t r[32];
         tmem_ld_x32(tmem + acc * CN + c0 + (static_cast<uint32_t>(q * 32) << 16), r);
         tmem_wait_ld();
         const int i0 = ti * bn + c0;
         if (i0 >= M) continue;  // uniform: no rows of this chunk exist
-        if (tma_out && (tj + 1) * CM <= tma_cols) {
+        if (i0 + 32 <= tma_rows) {
           // buffer sbuf was last read by the store nbuf chunks ago
           if (store_leader && pending) {
-            if (nbuf == 4) bulk_wait_read_3();
+            if (relaid) bulk_wait_read_all();
+            else if (nbuf == 4) bulk_wait_read_3();
             else bulk_wait_read_1();
           }
+          relaid = false;
           named_barrier(2, 128);  // staging buffer free
           uint8_t* buf = stage_out + sbuf * chunk_bytes;
           if (out_bf16) {
@@ -358,13 +406,19 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
           fence_proxy_async_smem();
           named_barrier(2, 128);  // staging written
           if (store_leader) {
-            tma_store_2d(&I->mapY, buf, tj * CM, i0);
+            if (kGrouped && red)
+              tma_reduce_add_2d(&I->mapY, buf, tj * CM, i0);
+            else
+              tma_store_2d(&I->mapY, buf, tj * CM, i0);
             bulk_commit_group();
             pending = true;
           }
           if (++sbuf == nbuf) sbuf = 0;
+        } else if (kGrouped && I->conv_mode) {
+          // lowered correlation: element (i, j) is output sample i * conv_w + j of this phase
+          store_samples<32>(r, static_cast<float*>(Yout), I->conv_w, I->conv_stride, I->conv_limit, i0, j, jok);
         } else if (jok) {
-          store_rows<32>(r, Yout, ldy, out_bf16, false, i0, M, j);
+          store_rows<32>(r, Yout, ldy, out_bf16, kGrouped && red, i0, M, j);
         }
       }
       tc_fence_before();
@@ -393,9 +447,11 @@ cudaError_t set_cg2_smem_attr() {
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
   const int bytes = static_cast<int>(kCSmemBytes);
-  e = cudaFuncSetAttribute(gemm_cg2_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  e = cudaFuncSetAttribute(gemm_cg2_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gemm_cg2_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    e = cudaFuncSetAttribute(gemm_cg2_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_cg2_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
   return e;
 }
@@ -436,7 +492,7 @@ static cudaError_t launch_cg2(Cg2Params& p, bool mn, int num_sms, cudaStream_t s
   cudaError_t e = set_cg2_smem_attr();
   if (e != cudaSuccess) return e;
   const int slots = num_sms / 2;
-  return launch_pdl(mn ? gemm_cg2_kernel<true> : gemm_cg2_kernel<false>,
+  return launch_pdl(mn ? gemm_cg2_kernel<true, false> : gemm_cg2_kernel<false, false>,
                     dim3(static_cast<unsigned>(2 * (p.num_pairs < slots ? p.num_pairs : slots))), kCThreads, kCSmemBytes,
                     st, 2, p);
 }
@@ -450,6 +506,7 @@ cudaError_t launch_gemm_cg2(const GemmTcArgs& a_in, int* err, int num_sms, cudaS
   if (!build_gemm_inst(a, &p.I)) return cudaErrorInvalidValue;
   p.npp = static_cast<int>(pair_cols);
   p.num_pairs = static_cast<int>(pair_cols * ceil_div(a.rowsQ, a.bn));
+  p.slot_rows = a.bn;
   p.stall = a.stall_stage;
   p.err = err;
   p.ex = a.ex;
@@ -457,7 +514,26 @@ cudaError_t launch_gemm_cg2(const GemmTcArgs& a_in, int* err, int num_sms, cudaS
   return launch_cg2(p, a.mnP || a.mnQ, num_sms, st);
 }
 
+cudaError_t launch_gemm_cg2_grouped(const GemmInst* insts, const GemmTile* tiles, const int* pair_off, int pairs,
+                                    int* err, cudaStream_t st) {
+  if (pairs == 0) return cudaSuccess;
+  cudaError_t e = set_cg2_smem_attr();
+  if (e != cudaSuccess) return e;
+  Cg2Params p{};
+  p.insts = insts;
+  p.tiles = tiles;
+  p.pair_off = pair_off;
+  p.slot_rows = CN;   // instances of any height share the ring
+  p.stall = -1;
+  p.err = err;
+  return launch_pdl(gemm_cg2_kernel<false, true>, dim3(static_cast<unsigned>(2 * pairs)), kCThreads, kCSmemBytes, st, 2, p);
+}
+
 #else   // the solo build has no CTA pairs
+
+cudaError_t launch_gemm_cg2_grouped(const GemmInst*, const GemmTile*, const int*, int, int*, cudaStream_t) {
+  return cudaErrorNotSupported;   // a build without CTA pairs plans none
+}
 
 bool gemm_cg2_eligible(const GemmTcArgs&, int) { return false; }
 cudaError_t launch_gemm_cg2(const GemmTcArgs&, int*, int, cudaStream_t) { return cudaErrorNotSupported; }

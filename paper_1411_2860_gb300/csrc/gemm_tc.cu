@@ -15,9 +15,9 @@
 // so each warp's stores of one output row are 128 contiguous bytes.
 //
 // A tile moves (128 + rows) x 128 bytes from L2 per K stage; at the tensor
-// rate that is more than the SMs can draw from L2, so K-major products run in
-// clusters of two CTAs on neighbouring tile columns of one tile row: each CTA
-// loads half of the shared A_c rows and multicasts them to both (kPair).
+// rate that is more than the SMs can draw from L2, so products whose tile columns
+// pair up, and batches, run on 2-SM MMAs instead (gemm_cg2.cu); this kernel serves
+// the odd ones, stream-K and solo CTAs.
 // With the hi/lo split, the hi and lo tiles of a K chunk take two ring slots and
 // serve all three products (hi*hi, lo*hi, hi*lo) from there: four tile loads per
 // chunk instead of six, and the same shared memory covers 1.5x the MMA time.
@@ -34,9 +34,6 @@
 #include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
-#if PJ_CTA_PAIRS
-#include "tc_pair.cuh"
-#endif
 
 namespace pj {
 namespace {
@@ -78,23 +75,7 @@ struct GemmParams {
 };
 
 // The n-th tile of this CTA: instance, coordinates and K-stage range; false past the last.
-// kPair (a single instance with an even number of tile columns, clusters of two CTAs):
-// the CTAs of cluster c take the tile columns 2 c' and 2 c' + 1 (by cluster rank) of the
-// same tile row, so both read the same rows of A_c.
-template <bool kPair>
-__device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, GemmTile& t, int rank) {
-  if (kPair && !p.tiles) {
-    const int npp = p.single.tiles_n / 2;
-    const int pi = static_cast<int>(blockIdx.x / 2) + n * static_cast<int>(gridDim.x / 2);
-    if (pi >= p.num_tiles / 2) return nullptr;
-    t.tj = (pi % npp) * 2 + rank;
-    t.ti = pi / npp;
-    t.k0 = 0;
-    t.k1 = p.single.kc;
-    t.red = 0;
-    t.pad0 = 0;
-    return &p.single;
-  }
+__device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, GemmTile& t) {
   if (p.tiles) {
     const int k = p.cta_off[blockIdx.x] + n;
     if (k >= p.cta_off[blockIdx.x + 1]) return nullptr;
@@ -132,13 +113,9 @@ __device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, G
   return &p.single;
 }
 
-// kMN: the launch may hold MN-major operands (the K-major instantiation carries
-// none of their branches).  kPair: launched in clusters of two CTAs that share
-// every Q tile (see tile_of): each CTA loads half of the tile's rows and the
-// copy is multicast to both, so the pair reads the rows of A_c once.  A stage
-// is then free only when both CTAs' MMAs have read it: every MMA commit
-// arrives on the stage's empty barrier in both CTAs (initial count 2).
-template <bool kMN, bool kPair>
+// kMN: the launch may hold MN-major operands (the K-major instantiation carries none of
+// their branches).
+template <bool kMN>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -156,11 +133,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   int* vote = reinterpret_cast<int*>(tslot + 4);       // [2][4] epilogue warps' wait outcomes
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int rank = kPair ? static_cast<int>(cluster_ctarank()) : 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], kPair ? 2 : 1);
+      mbar_init(&empty[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
@@ -175,7 +151,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   }
   tc_fence_before();
   __syncthreads();
-  if (kPair) cluster_sync_all();  // the peer's barriers exist before any copy or commit reaches them
   tc_fence_after();
   const uint32_t tmem = *tslot;
   pdl_begin();
@@ -190,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       int issued = 0;
       GemmTile T{};
       for (int n = 0; ok; ++n) {
-        const GemmInst* I = tile_of<kPair>(p, n, T, rank);
+        const GemmInst* I = tile_of(p, n, T);
         if (!I) break;
         // Everything the loop needs, read once: the copies are asm volatile with a memory
         // clobber, so a value read through I would be read again for every one of them,
@@ -202,9 +177,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           tma_prefetch(mapQ);
         }
         __syncwarp();
-        const int tj = T.tj, bn = I->bn, half = bn / 2;
+        const int tj = T.tj, bn = I->bn;
         const int y0 = T.ti * bn;
-        const bool conv = I->conv_mode != 0, mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
+        const bool conv = I->conv_mode != 0;
+        const int cmask = conv ? I->conv_w / BK - 1 : 0, cshift = conv ? 31 - __clz(I->conv_w / BK) : 0;
+        const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
         const uint32_t stage_bytes = kStageP + static_cast<uint32_t>(bn) * BK * 2;
         const int qchunks = bn / 64;
         // Shared tiles: K chunk c is ring slots 2c (hi P, hi Q) and 2c + 1 (lo P, lo Q).
@@ -233,11 +210,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             oQ = kk < e0 ? sQ0 : (kk < e1 ? sQ1 : sQ2);
           }
           const int px = oP + kin * BK;
-          // Row-split mode: Q row r, K chunk k lives at row r + k/2, column 64 (k mod 2) of
-          // a 128-wide view (the signal segments of a lowered correlation); there a
-          // segment's Q offset counts rows (the split residual rows follow the hi rows).
-          const int qx = conv ? (kin & 1) * BK : oQ + kin * BK;
-          const int qy = conv ? y0 + (kin >> 1) + oQ : y0;
+          // Row-split mode: Q row r, K chunk k lives at row r + k / c, column 64 (k mod c) of
+          // a view c = conv_w / 64 chunks wide (the signal segments of a lowered correlation);
+          // there a segment's Q offset counts rows (the split residual rows follow the hi rows).
+          const int qx = conv ? (kin & cmask) * BK : oQ + kin * BK;
+          const int qy = conv ? y0 + (kin >> cshift) + oQ : y0;
           uint64_t* const bar = &full[stage];
           uint8_t* const dP = sm + stage * slot_bytes;
           uint8_t* const dQ = dP + kStageP;
@@ -250,23 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
               tma_load_2d(dP, mapP, bar, px, tj * BM);
             }
             if (mnQ) {
-#if PJ_CTA_PAIRS
-              if (kPair) {  // this CTA's half of the Q chunks, for both CTAs of the pair
-                const int hc = qchunks / 2;
-                for (int c = rank * hc; c < (rank + 1) * hc; ++c)
-                  tma_load_2d_mc(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx, 0x3);
-              } else
-#endif
               for (int c = 0; c < qchunks; ++c) tma_load_2d(dQ + c * 8192, mapQ, bar, y0 + 64 * c, qx);
-#if PJ_CTA_PAIRS
-            } else if (kPair && !(T.pad0 & 1)) {
-              // this CTA's half of the Q tile, for both CTAs of the pair
-              tma_load_2d_mc(dQ + rank * half * (BK * 2), mapQ, bar, qx, qy + rank * half, 0x3);
-#endif
-            } else if (kPair) {
-              // a tile of its own (grouped launch): both halves for this CTA only
-              tma_load_2d(dQ, mapQ, bar, qx, qy);
-              tma_load_2d(dQ + half * (BK * 2), mapQ, bar, qx, qy + half);
             } else {
               tma_load_2d(dQ, mapQ, bar, qx, qy);
             }
@@ -296,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       bool issued_any = false;
       GemmTile T{};
       for (int n = 0; ok; ++n, ++it) {
-        const GemmInst* I = tile_of<kPair>(p, n, T, rank);
+        const GemmInst* I = tile_of(p, n, T);
         if (!I) break;
         const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
         const uint32_t idesc = idesc_bf16_f32(BM, I->bn) | (static_cast<uint32_t>(mnP) << 15) |
@@ -318,14 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           for (int k = 0; k < BK / 16; ++k)
             umma_f16(d, sdesc_advance(dp, k * kP), sdesc_advance(dq, k * kQ), idesc, !first || (k != 0));
         };
-        auto release = [&](int sl) {
-#if PJ_CTA_PAIRS
-          if (kPair)
-            umma_commit_mc(&empty[sl], 0x3);
-          else
-#endif
-            umma_commit(&empty[sl]);
-        };
+        auto release = [&](int sl) { umma_commit(&empty[sl]); };
         const bool share = I->share != 0;
         const int c0 = share ? share_chunk(T.k0) : T.k0, c1 = share ? share_chunk(T.k1) : T.k1;
         for (int kk = c0; kk < c1; ++kk) {
@@ -394,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     int it = 0;
     GemmTile T{};
     for (int n = 0;; ++n, ++it) {
-      const GemmInst* I = tile_of<kPair>(p, n, T, rank);
+      const GemmInst* I = tile_of(p, n, T);
       if (!I) break;
       const int ti = T.ti, tj = T.tj;
       const bool red = T.red != 0;
@@ -428,8 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         if (lane == 0) mbar_arrive(&acc_empty[acc]);
         continue;
       }
-      // a stand-in tile of a pair (grouped launch) writes nothing
-      for (int c0 = 0; c0 < ((T.pad0 & 2) ? 0 : bn); c0 += 32) {
+      for (int c0 = 0; c0 < bn; c0 += 32) {
         uint32_t r[32];
         tmem_ld_x32(tmem + acc * BN + c0 + (static_cast<uint32_t>(q * 32) << 16), r);
         tmem_wait_ld();
@@ -458,13 +411,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             pending = true;
           }
         } else if (I->conv_mode) {
-          // lowered correlation: element (i, j) is output sample i * 128 + j of this phase
-          float* Y = static_cast<float*>(I->Y);
-#pragma unroll
-          for (int u = 0; u < 32; ++u) {
-            const int64_t flat = static_cast<int64_t>(i0 + u) * BM + j;
-            if (jok && flat < I->conv_limit) __stcs(Y + flat * I->conv_stride, __uint_as_float(r[u]));
-          }
+          // lowered correlation: element (i, j) is output sample i * conv_w + j of this phase
+          store_samples<32>(r, static_cast<float*>(Yout), I->conv_w, I->conv_stride, I->conv_limit, i0, j, jok);
         } else if (jok) {
           store_rows<32>(r, Yout, ldy, out_bf16, red, i0, M, j);
         }
@@ -478,8 +426,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 
   tc_fence_before();
   __syncthreads();
-  // Neither CTA of a pair leaves while the other's MMAs may still arrive on its barriers.
-  if (kPair) cluster_sync_all();
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
@@ -509,7 +455,7 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
     const uint32_t box[2] = {64, BK};
     if (!make_tmap_bf16(&I->mapQ, a.Q, 2, dims, strides, box)) return false;
   } else {
-    const uint64_t dims[2] = {static_cast<uint64_t>(a.conv_mode ? 128 : a.xdim),
+    const uint64_t dims[2] = {static_cast<uint64_t>(a.conv_mode ? a.conv_w : a.xdim),
                               static_cast<uint64_t>(a.conv_mode ? a.q_rows_alloc : a.rowsQ)};
     const uint64_t strides[1] = {static_cast<uint64_t>(a.ldq) * 2};
     const uint32_t box[2] = {BK, static_cast<uint32_t>(a.pair ? a.bn / 2 : a.bn)};
@@ -537,6 +483,7 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
              I->segQ[0] == I->segQ[1];
   I->tiles_n = static_cast<int>(ceil_div(a.rowsP, BM));
   I->conv_mode = a.conv_mode;
+  I->conv_w = a.conv_w;
   I->conv_stride = a.conv_stride;
   I->conv_limit = a.conv_limit;
   I->tma_out = 0;
@@ -544,11 +491,11 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
   I->tma_cols = 1 << 30;
   const size_t es = I->out_bf16 ? 2 : 4;
   if (a.conv_mode) {
-    // contiguous output rows of 128 samples only when samples are adjacent in memory
-    const int64_t full_rows = a.conv_limit / BM;
+    // contiguous output rows of conv_w samples only when samples are adjacent in memory
+    const int64_t full_rows = a.conv_limit / a.conv_w;
     if (a.conv_stride == 1 && !I->out_bf16 && full_rows > 0 && reinterpret_cast<uintptr_t>(a.Y) % 16 == 0) {
-      const uint64_t dims[2] = {static_cast<uint64_t>(BM), static_cast<uint64_t>(full_rows)};
-      const uint64_t strides[1] = {static_cast<uint64_t>(BM) * 4};
+      const uint64_t dims[2] = {static_cast<uint64_t>(a.conv_w), static_cast<uint64_t>(full_rows)};
+      const uint64_t strides[1] = {static_cast<uint64_t>(a.conv_w) * 4};
       const uint32_t box[2] = {BM, 32};
       I->tma_out = make_tmap_f32(&I->mapY, a.Y, 2, dims, strides, box) ? 1 : 0;
       I->tma_rows = static_cast<int>(full_rows);
@@ -581,15 +528,9 @@ static cudaError_t set_smem_attr() {
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
   const int bytes = static_cast<int>(kSmemBytes);
-  e = cudaFuncSetAttribute(gemm_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  e = cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gemm_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-#if PJ_CTA_PAIRS
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gemm_tc_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-#endif
+    e = cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
   return e;
 }
@@ -605,14 +546,8 @@ cudaError_t launch_gemm_tc_generic(const GemmTcArgs& a_in, int* err, int num_sms
   // (the expansion writes samples, which partial products could not be added into)
   const bool streamk = !a.conv_mode && !a.ex.mode && a.out_dtype != PJ_BF16 &&
                        use_stream_k(tiles, args_stages(a), num_sms, a.nseg > 1);
-  // CTA pairs share the Q tiles of a K-major product with an even number of tile
-  // columns (half-tiles of whole 8-row swizzle atoms).
   // 256-row tiles on 2-SM MMAs wherever the tile columns pair up (gemm_cg2.cu).
   if (!streamk && gemm_cg2_eligible(a, num_sms)) return launch_gemm_cg2(a, err, num_sms, st);
-  // An MN-major Q tile is bn / 64 chunks of 64 values: the pair splits the chunks.
-  const bool q_pair_ok = !a.mnQ || (a.bn / 64) % 2 == 0;
-  a.pair = PJ_CTA_PAIRS && !a.conv_mode && q_pair_ok && !streamk && tiles_n % 2 == 0 && a.bn % 16 == 0 &&
-           num_sms >= 2;
   if (!build_gemm_inst(a, &p.single)) return cudaErrorInvalidValue;
   p.insts = nullptr;
   p.tiles = nullptr;
@@ -633,19 +568,12 @@ cudaError_t launch_gemm_tc_generic(const GemmTcArgs& a_in, int* err, int num_sms
     p.streamk = 1;
     grid = num_sms;
   }
-#if PJ_CTA_PAIRS
-  if (a.pair) {
-    const int pairs = p.num_tiles / 2, slots = num_sms / 2;
-    return launch_pdl(a.mnQ || a.mnP ? gemm_tc_kernel<true, true> : gemm_tc_kernel<false, true>,
-                      dim3(static_cast<unsigned>(2 * (pairs < slots ? pairs : slots))), kThreads, kSmemBytes, st, 2, p);
-  }
-#endif
-  return launch_pdl(a.mnP || a.mnQ ? gemm_tc_kernel<true, false> : gemm_tc_kernel<false, false>,
+  return launch_pdl(a.mnP || a.mnQ ? gemm_tc_kernel<true> : gemm_tc_kernel<false>,
                     dim3(static_cast<unsigned>(grid)), kThreads, kSmemBytes, st, 1, p);
 }
 
 cudaError_t launch_gemm_tc_grouped(const GemmInst* insts, const GemmTile* tiles, const int* cta_off, int ctas,
-                                   int pair, int* err, cudaStream_t st) {
+                                   int* err, cudaStream_t st) {
   if (ctas == 0) return cudaSuccess;
   GemmParams p;
   memset(&p.single, 0, sizeof(GemmInst));
@@ -661,15 +589,8 @@ cudaError_t launch_gemm_tc_grouped(const GemmInst* insts, const GemmTile* tiles,
   p.ex_c8 = Coef8{};
   cudaError_t e = set_smem_attr();
   if (e != cudaSuccess) return e;
-  if (pair) {  // CTAs 2c and 2c + 1 form a cluster; their tile lists are paired
-#if !PJ_CTA_PAIRS
-    return cudaErrorNotSupported;   // a build without CTA pairs plans none
-#else
-    return launch_pdl(gemm_tc_kernel<false, true>, dim3(static_cast<unsigned>(ctas)), kThreads, kSmemBytes, st, 2, p);
-#endif
-  }
   // grouped instances are K-major
-  return launch_pdl(gemm_tc_kernel<false, false>, dim3(static_cast<unsigned>(ctas)), kThreads, kSmemBytes, st, 1, p);
+  return launch_pdl(gemm_tc_kernel<false>, dim3(static_cast<unsigned>(ctas)), kThreads, kSmemBytes, st, 1, p);
 }
 
 cudaError_t launch_gemm_tc(const uint16_t* Ac, const uint16_t* Bd, void* Y, int64_t ldy, int out_dtype,
