@@ -34,6 +34,9 @@
 #include "pdl.cuh"
 #include "tc.cuh"
 #include "tmap.hpp"
+#if PJ_CTA_PAIRS
+#include "tc_pair.cuh"   // as in every GEMM of the build with CTA pairs
+#endif
 
 namespace pj {
 namespace {
