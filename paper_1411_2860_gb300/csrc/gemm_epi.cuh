@@ -176,15 +176,68 @@ __device__ __forceinline__ void expand_cols_x8(const uint32_t (&r)[8], int k0, i
   }
 }
 
+// Mode 1 on a chunk of 8 rows and a warp of groups that all exist, walked by pointer with
+// the coefficients held by the caller's loop.  With an address, two bounds and the
+// coefficients' shared loads per row, the instructions of the eight epilogue warps bound
+// the expansion: the backward of an 8192 x 4096 x 4096 BF16 layer (l+1 = 2) takes 147 us
+// so, 152 before, and a 2048 x 2048 x 4096 FP32 one (l+1 = 8) 105 us, 113 before.  Not for
+// l+1 = 1, whose rows exchange nothing (190 against 184 us), not for BF16 at l+1 = 8, whose
+// lanes store two bytes each (526 against 520 us), nor for mode 2, whose stores in bursts
+// slowed the products they overlap (l+1 = 4: 282 against 278 us).
+template <int LP1, bool kBF16>
+__device__ __forceinline__ void expand_rows_full(const uint32_t (&r)[8], int lbase, const float (&cf)[8 / LP1][LP1],
+                                                 void* out, int64_t off, int64_t ld) {
+  constexpr int per = 8 / LP1;
+#pragma unroll
+  for (int u = 0; u < 8; ++u, off += ld) {
+    float v[LP1], y[8];
+#pragma unroll
+    for (int pp = 0; pp < LP1; ++pp) v[pp] = __shfl_sync(0xffffffffu, __uint_as_float(r[u]), lbase + pp);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      y[t] = 0.0f;
+      if (t < per) {
+#pragma unroll
+        for (int pp = 0; pp < LP1; ++pp) y[t] = fmaf(v[pp], cf[t < per ? t : 0][pp], y[t]);
+      }
+    }
+    store_run<kBF16>(out, off, y, per, per);
+  }
+}
+
 template <int LP1, bool kBF16>
 __device__ __noinline__ void expand_tile_cols(uint32_t taddr, int ncols, const ExpandArgs ex, const float* sc,
                                               int lane, int kk_lane, int Kp, int i0, int M, int j, bool jok) {
+  uint32_t r[8];
+  constexpr bool kWhole = LP1 > 1 && !(LP1 == 8 && kBF16);
+  if constexpr (kWhole) {
+    if (ex.mode == 1) {
+      constexpr int per = 8 / LP1;
+      const int g = kk_lane / LP1, t0 = (kk_lane - g * LP1) * per;
+      const int64_t col0 = static_cast<int64_t>(g) * 8 + t0;
+      const bool whole = __all_sync(0xffffffffu, kk_lane < Kp && col0 + per <= ex.K);
+      float cf[per][LP1];
+#pragma unroll
+      for (int t = 0; t < per; ++t)
+#pragma unroll
+        for (int pp = 0; pp < LP1; ++pp) cf[t][pp] = sc[(t0 + t) * LP1 + pp];
+#pragma unroll 1
+      for (int c = 0; c < ncols && i0 + c < M; c += 8) {
+        tmem_ld_x8(taddr + c, r);
+        tmem_wait_ld();
+        if (whole && i0 + c + 8 <= M)
+          expand_rows_full<LP1, kBF16>(r, lane & ~(LP1 - 1), cf, ex.out, (i0 + c) * ex.ld + col0, ex.ld);
+        else
+          expand_rows_x8<LP1, kBF16>(r, lane, kk_lane, Kp, i0 + c, M, ex, sc);
+      }
+      return;
+    }
+  }
 #pragma unroll 1
   for (int c = 0; c < ncols; c += 8) {
-    uint32_t r[8];
     tmem_ld_x8(taddr + c, r);
     tmem_wait_ld();
-    if (ex.mode == 1) {
+    if (!kWhole && ex.mode == 1) {
       if (i0 + c < M) expand_rows_x8<LP1, kBF16>(r, lane, kk_lane, Kp, i0 + c, M, ex, sc);
     } else if (jok && i0 + c < Kp) {
       expand_cols_x8<LP1, kBF16>(r, i0 + c, Kp, j, ex, sc);
