@@ -29,6 +29,14 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// A launch that the runtime refuses also leaves its error behind for whoever asks for the
+// last one next (the caller's framework after a launch of its own): it is taken back here,
+// and returned.
+inline cudaError_t launched(cudaError_t e) {
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
+}
+
 template <typename... P, typename... A>
 inline cudaError_t launch_plain(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
                                 const A&... args) {
@@ -37,7 +45,7 @@ inline cudaError_t launch_plain(void (*kernel)(P...), dim3 grid, int threads, si
   cfg.blockDim = dim3(static_cast<unsigned>(threads));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  return launched(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
 template <typename... P, typename... A>
@@ -57,7 +65,7 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  return launched(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
 }  // namespace pj
