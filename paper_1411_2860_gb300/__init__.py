@@ -252,9 +252,10 @@ def _prec(compute: str, split: int, split_lead: int = 0, fp8_tier: int = 0):
 # which the GPU worked 55; what follows keeps the per-call Python short: descriptors
 # of built-in bases and precisions made once per value (the library only reads them),
 # workspace sizes remembered by their arguments, plain integers for pointers and
-# streams, and no device switch when the device is current.  The step now takes
-# 235 us, of which some 150 are autograd's hand-over to its device thread and back;
-# a product of 64 x 512 x 96 went from 30 to 23.5 us.
+# streams, and no device switch when the device is current.  The step then took
+# 235 us, and a product of 64 x 512 x 96 went from 30 to 23.5 us.  What is remembered is
+# remembered for plain integers alone: another object that stands for one (a NumPy or
+# torch scalar) may be unhashable, or hash by identity and change its value.
 
 @functools.lru_cache(maxsize=256)
 def _basis_ref(kind: str, L: int):
@@ -263,24 +264,34 @@ def _basis_ref(kind: str, L: int):
 
 
 @functools.lru_cache(maxsize=256)
-def _prec_ref(compute: str, split: int, split_lead: int = 0, fp8_tier: int = 0):
+def _prec_of(compute: str, split: int, split_lead: int, fp8_tier: int):
     return ctypes.byref(_prec(compute, split, split_lead, fp8_tier))
+
+
+def _prec_ref(compute: str, split: int, split_lead: int = 0, fp8_tier: int = 0):
+    return _prec_of(compute, int(split), int(split_lead), int(fp8_tier))
 
 
 def _basis_arg(kind, L, user_C=None, holder=None):
     """(reference for a call, object to keep alive meanwhile) of a basis."""
     if kind != "user":
-        return _basis_ref(kind, L), None
+        return _basis_ref(kind, int(L)), None
     b, keep = _basis(kind, L, user_C, holder)
     return ctypes.byref(b), (b, keep)
 
 
 @functools.lru_cache(maxsize=1024)
-def _gemm_size(fn: str, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier) -> int:
-    n = getattr(_load(), fn)(M, N, K, block_k, R, _basis_ref(basis, L), _prec_ref(compute, split, split_lead, fp8_tier))
+def _gemm_size_of(fn: str, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier) -> int:
+    n = getattr(_load(), fn)(M, N, K, block_k, R, _basis_ref(basis, L), _prec_of(compute, split, split_lead, fp8_tier))
     if n == 0:
         raise ProjError(PJ_EINVAL, fn[:-len("_workspace_size")], last_error())   # (an exception is not remembered)
     return int(n)
+
+
+def _gemm_size(fn: str, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier) -> int:
+    plain = type(M) is int and type(N) is int and type(K) is int and type(block_k) is int and type(R) is int
+    size = _gemm_size_of if plain else _gemm_size_of.__wrapped__
+    return size(fn, M, N, K, block_k, R, basis, int(L), compute, int(split), int(split_lead), int(fp8_tier))
 
 
 def _stream(stream, device):
