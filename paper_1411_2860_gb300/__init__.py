@@ -316,9 +316,10 @@ def _on(device, fn, *args):
 
 def _dy_arg(dY, dtype):
     """dY as the library takes it: contiguous, in the operands' dtype, or FP32 as it is
-    for BF16 operands (the library rounds it as dY.to(bfloat16) would)."""
+    for BF16 operands (the library rounds it as dY.to(bfloat16) would).  A view that negates
+    its memory when it is read goes through that copy, which applies the sign."""
     if dY.dtype != dtype and not (dY.dtype == torch.float32 and dtype == torch.bfloat16 and dY.is_cuda
-                                  and dY.is_contiguous() and dY.data_ptr() % 16 == 0):
+                                  and dY.is_contiguous() and not dY.is_neg() and dY.data_ptr() % 16 == 0):
         dY = dY.to(dtype)
     return dY.contiguous()
 

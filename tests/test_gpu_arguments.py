@@ -1,4 +1,5 @@
-"""Arguments that stand for others: scalars of NumPy and torch in place of integers."""
+"""Arguments that stand for others: scalars of NumPy and torch in place of integers, and a
+gradient that is a negating view."""
 import numpy as np
 import pytest
 import torch
@@ -34,3 +35,20 @@ def test_sizes_that_change_in_place():
     R.fill_(16)     # more components: a larger workspace
     L.fill_(4)
     assert torch.equal(pj.proj_gemm(A, B, block, R, "dct2", L), pj.proj_gemm(A, B, 16, 16, "dct2", 4))
+
+
+def test_negated_gradient():
+    """A contiguous FP32 view that negates its memory when it is read."""
+    X, W = _operands(torch.bfloat16)
+    dY = torch.randn(60, 72, device="cuda")
+    neg = torch._neg_view(dY)
+    assert neg.is_neg() and neg.is_contiguous()
+    for g, w in zip(pj.proj_gemm_backward(X, W, neg, 16, 8), pj.proj_gemm_backward(X, W, -dY, 16, 8)):
+        assert torch.equal(g, w)
+    X.requires_grad_()
+    W.requires_grad_()
+    for save in (False, True):
+        Y = pj.proj_matmul(X, W, 16, 8, save_projections=save)
+        for g, w in zip(torch.autograd.grad(Y, (X, W), neg, retain_graph=not save),
+                        pj.proj_gemm_backward(X.detach(), W.detach(), -dY, 16, 8)):
+            assert torch.equal(g, w)
