@@ -622,19 +622,39 @@ __device__ __forceinline__ void cols_tile_q(const TileCtx& c, const TileIn<InT, 
   if (uy == c.units_y - 1) mx_zero_tail(q, j, static_cast<int64_t>(c.units_y) * 32);
 }
 
-// The packed lead hi and lo terms of four whole groups (tiered split, tl <= 2).
-__device__ __forceinline__ void store_lead_runs(const TileCtx& c, uint16_t* orow, int64_t g0, const uint32_t (&lh)[4],
-                                                const uint32_t (&ll)[4]) {
-  uint16_t* lhp = orow + c.Kp_pad + g0 * c.tl;
-  uint16_t* llp = orow + c.Kp_pad + c.Kt_pad + g0 * c.tl;
-  if (c.tl == 1) {
-    *reinterpret_cast<uint2*>(lhp) = make_uint2(lh[0], lh[1]);
-    *reinterpret_cast<uint2*>(llp) = make_uint2(ll[0], ll[1]);
-  } else {
-    *reinterpret_cast<uint4*>(lhp) = make_uint4(lh[0], lh[1], lh[2], lh[3]);
-    *reinterpret_cast<uint4*>(llp) = make_uint4(ll[0], ll[1], ll[2], ll[3]);
+// The lead hi and lo terms of a column's quad of groups (tiered split).  Those of four
+// whole groups are contiguous in their segments: packed (h, l) and stored at the end when
+// tl <= 2, one run per group otherwise.
+struct LeadTerms {
+  uint32_t h[4] = {0u, 0u, 0u, 0u}, l[4] = {0u, 0u, 0u, 0u};
+
+  __device__ __forceinline__ void put(const TileCtx& c, uint16_t* orow, int64_t g0, int q, bool full,
+                                      const uint16_t (&hi)[8], const uint16_t (&lo)[8]) {
+    if (c.tl == 1) {
+      h[q >> 1] |= uint32_t(hi[0]) << (16 * (q & 1));
+      l[q >> 1] |= uint32_t(lo[0]) << (16 * (q & 1));
+    } else if (c.tl == 2) {
+      h[q] = pack2(hi[0], hi[1]);
+      l[q] = pack2(lo[0], lo[1]);
+    }
+    if ((c.tl > 2 || !full) && g0 + q < c.NG) {
+      store_upto8(orow + c.Kp_pad + (g0 + q) * c.tl, hi, c.tl);
+      store_upto8(orow + c.Kp_pad + c.Kt_pad + (g0 + q) * c.tl, lo, c.tl);
+    }
   }
-}
+  __device__ __forceinline__ void finish(const TileCtx& c, uint16_t* orow, int64_t g0, bool full) const {
+    if (!full || c.tl > 2) return;
+    uint16_t* hp = orow + c.Kp_pad + g0 * c.tl;
+    uint16_t* lp = orow + c.Kp_pad + c.Kt_pad + g0 * c.tl;
+    if (c.tl == 1) {
+      *reinterpret_cast<uint2*>(hp) = make_uint2(h[0], h[1]);
+      *reinterpret_cast<uint2*>(lp) = make_uint2(l[0], l[1]);
+    } else {
+      *reinterpret_cast<uint4*>(hp) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(lp) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+  }
+};
 
 // Cols: tile = 32 rows of B (4 groups) x 256 columns.  Thread t owns column
 // t of the tile and writes its 4 (l+1) components contiguously into row j of
@@ -666,7 +686,8 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
       const int lane = t & 31, w = t >> 5;
       uint8_t* base = tin.base + w * 128;
       const bool two = !tiered && c.nsplit > 1;
-      uint32_t lh[4] = {0u, 0u, 0u, 0u}, ll[4] = {0u, 0u, 0u, 0u};  // packed lead runs for tl <= 2
+      uint16_t* const orow = c.out + j * c.pitch;   // (of a column that exists)
+      LeadTerms lead;
       float x[32];
   #pragma unroll
       for (int e = 0; e < 32; ++e) x[e] = tin.elem(e, t);
@@ -680,21 +701,9 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
         project8(xq, cf, need_lo, hi, lo);
         run_put_group<LP1>(base, row_bytes, 0, lane, q, hi);
         if (two) run_put_group<LP1>(base, row_bytes, 1, lane, q, lo);
-        if (tiered) {
-          if (c.tl == 1) {
-            lh[q >> 1] |= uint32_t(hi[0]) << (16 * (q & 1));
-            ll[q >> 1] |= uint32_t(lo[0]) << (16 * (q & 1));
-          } else if (c.tl == 2) {
-            lh[q] = pack2(hi[0], hi[1]);
-            ll[q] = pack2(lo[0], lo[1]);
-          } else if (j < c.n_out) {
-            uint16_t* orow = c.out + j * c.pitch;
-            store_upto8(orow + c.Kp_pad + (g0 + q) * c.tl, hi, c.tl);
-            store_upto8(orow + c.Kp_pad + c.Kt_pad + (g0 + q) * c.tl, lo, c.tl);
-          }
-        }
+        if (tiered && j < c.n_out) lead.put(c, orow, g0, q, true, hi, lo);
       }
-      if (tiered && c.tl <= 2 && j < c.n_out) store_lead_runs(c, c.out + j * c.pitch, g0, lh, ll);
+      if (tiered && j < c.n_out) lead.finish(c, orow, g0, true);
       __syncwarp();
       const int64_t jw = static_cast<int64_t>(ux) * kPtBoxX + w * 32;
       const int ncols = c.n_out - jw < 32 ? static_cast<int>(c.n_out - jw) : 32;
@@ -707,17 +716,22 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
       return;
     }
   }
-  if constexpr (kOddRun<LP1> && !tiered) {
+  if constexpr (kOddRun<LP1>) {
     if (full) {
       // l+1 in {3, 5, 6, 7}, four whole groups: the column's 4 (l+1) components packed into
       // words, one part (hi, then lo) at a time staged in the warp's own columns of the
       // tile (read by now; runs an odd number of 8 bytes apart) and written run after run
       // in 8-byte chunks.  Stored by the lanes themselves, every chunk went to 32 rows.
+      // (A tiered split stages its hi part; the lead terms are few and stored as below.
+      // With the hi part stored element by element too, a product of 4096 x 2048 over
+      // 10,304 with l+1 = 6 and one lead term took 292 us, so 180.)
       constexpr int kSeg = 32 * static_cast<int>(sizeof(InT)), kPitch = 8 * (LP1 | 1);
       static_assert(32 * kPitch <= 32 * kSeg, "the runs of a warp fit its columns");
       const int lane = t & 31, w = t >> 5;
       uint8_t* const base = tin.base + w * kSeg;
       auto at = [&](int b) { return base + (b / kSeg) * row_bytes + b % kSeg; };
+      uint16_t* const orow = c.out + j * c.pitch;   // (of a column that exists)
+      LeadTerms lead;
       uint32_t wh[2 * LP1], wl[2 * LP1];
 #pragma unroll
       for (int k = 0; k < 2 * LP1; ++k) wh[k] = wl[k] = 0u;
@@ -734,12 +748,14 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
           wh[e >> 1] |= uint32_t(hi[p]) << (16 * (e & 1));
           wl[e >> 1] |= uint32_t(lo[p]) << (16 * (e & 1));
         }
+        if (tiered && j < c.n_out) lead.put(c, orow, g0, q, true, hi, lo);
       }
+      if (tiered && j < c.n_out) lead.finish(c, orow, g0, true);
       const int64_t jw = static_cast<int64_t>(ux) * kPtBoxX + w * 32;
       const int ncols = c.n_out - jw < 32 ? static_cast<int>(c.n_out - jw) : 32;
       uint16_t* o0 = c.out + jw * c.pitch + g0 * LP1;
 #pragma unroll 1
-      for (int part = 0; part < (need_lo ? 2 : 1); ++part) {
+      for (int part = 0; part < (need_lo && !tiered ? 2 : 1); ++part) {
         __syncwarp();   // the columns (or the previous part's runs) are read
 #pragma unroll
         for (int k = 0; k < 2 * LP1; ++k) *reinterpret_cast<uint32_t*>(at(lane * kPitch + 4 * k)) = part ? wl[k] : wh[k];
@@ -761,7 +777,7 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
   uint16_t* orow = c.out + j * c.pitch;
   uint16_t* o = orow + g0 * LP1;
   uint32_t ph[4] = {0u, 0u, 0u, 0u}, pl[4] = {0u, 0u, 0u, 0u};  // packed runs for l+1 <= 2
-  uint32_t lh[4] = {0u, 0u, 0u, 0u}, ll[4] = {0u, 0u, 0u, 0u};  // packed lead runs for tl <= 2
+  LeadTerms lead;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     float2 x[4];
@@ -781,21 +797,7 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
       store_upto8(o + q * LP1, hi, LP1);
       if (!tiered && c.nsplit > 1) store_upto8(o + c.Kp_pad + q * LP1, lo, LP1);
     }
-    if (tiered) {
-      // the lead terms of the four groups are contiguous in their segments:
-      // packed like the l+1 <= 2 runs when tl <= 2, one run per group otherwise
-      if (c.tl == 1) {
-        lh[q >> 1] |= uint32_t(hi[0]) << (16 * (q & 1));
-        ll[q >> 1] |= uint32_t(lo[0]) << (16 * (q & 1));
-      } else if (c.tl == 2) {
-        lh[q] = pack2(hi[0], hi[1]);
-        ll[q] = pack2(lo[0], lo[1]);
-      }
-      if ((c.tl > 2 || !full) && g0 + q < c.NG) {
-        store_upto8(orow + c.Kp_pad + (g0 + q) * c.tl, hi, c.tl);
-        store_upto8(orow + c.Kp_pad + c.Kt_pad + (g0 + q) * c.tl, lo, c.tl);
-      }
-    }
+    if (tiered) lead.put(c, orow, g0, q, full, hi, lo);
   }
   if (full && LP1 == 1) {
     *reinterpret_cast<uint2*>(o) = make_uint2(ph[0], ph[1]);
@@ -804,7 +806,7 @@ __device__ __forceinline__ void cols_tile(const TileCtx& c, const TileIn<InT, fa
     *reinterpret_cast<uint4*>(o) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
     if (c.nsplit > 1 && !tiered) *reinterpret_cast<uint4*>(o + c.Kp_pad) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
   }
-  if (tiered && full && c.tl <= 2) store_lead_runs(c, orow, g0, lh, ll);
+  if (tiered) lead.finish(c, orow, g0, full);
   if (uy == c.units_y - 1) zero_row_tails(c, orow, LP1, full && LP1 <= 2 ? (g0 + 4) * LP1 : 0);
 }
 
