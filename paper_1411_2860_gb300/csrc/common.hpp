@@ -382,18 +382,6 @@ cudaError_t launch_gemm_fused(const void* A, int64_t lda, int in_dtype, const ui
                               const float* Cs, void* Y, int64_t ldy, int out_dtype, int* err, int num_sms,
                               cudaStream_t st);
 
-// Whether a single-instance launch of `tiles` tiles of `stages` K stages each
-// should share the stages evenly over all SMs (stream-K; FP32 output zeroed
-// first): when the tiles fill less than half of one wave, and every SM still
-// gets at least 16 stages.  From half a wave on, the zeroing, the additions of
-// partial tiles and (2-SM MMAs cannot share) the solo kernel cost more than the
-// idle SMs: 2048 x 2048 x 2048 (128 tiles) 25.7 us shared, 15.1 on pairs; 2000 x
-// 1000 x 4000 23.2 against 18.9; below half, 300 x 300 x 8000 (15 tiles) 14.3
-// against 78.9.  With a wave or more, CTAs that start in the middle of tiles also
-// lose the L2 sharing of operand slices.
-// Products with BF16 hi/lo terms (split) share up to 0.9 of a wave: their error is
-// that of the accumulation, which sums cut in pieces keep smaller (1000 x 777 over
-// 2256 components, 112 tiles: 6.2e-6 relative shared, 9.0e-6 whole, for 4 us less).
 // Tile height (rows of A_c per tile, a multiple of gran, at most bnmax) for a
 // single-instance launch: the height whose whole waves of tiles over the SMs
 // finish first, counting each tile as its K stages scaled by its height plus a
@@ -414,9 +402,23 @@ inline int single_launch_bn(int64_t rows, int64_t tiles_n, int64_t stages, int s
   return best;
 }
 
+// Whether a single-instance launch of `tiles` tiles of `stages` K stages each
+// should share the stages evenly over all SMs (stream-K; FP32 output zeroed
+// first): when every SM still gets at least 16 stages and the tiles fill less than half
+// of one wave, or less than 0.9 of one and sharing takes at least 32 stages off every SM.
+// The zeroing, the additions of partial tiles and (2-SM MMAs cannot share) the solo
+// kernel cost what some 25 stages do.  Calls, shared and whole: BF16, 80 tiles of 161
+// stages 102 and 109 us (on pairs 58 and 69), 100 of 128 55 and 59, 110 of 64 67 and 65,
+// 112 of 36 46 and 38; E4M3 (stages of 128 components), 80 of 243 176 and 187, 100 of 192
+// 68 and 74, 110 of 96 112 and 109, 128 of 32 40 and 34.  With a wave or more, CTAs that start in the middle of tiles also lose the L2 sharing of
+// operand slices.
+// Products with BF16 hi/lo terms (split) share up to 0.9 of a wave: their error is
+// that of the accumulation, which sums cut in pieces keep smaller (1000 x 777 over
+// 2256 components, 112 tiles: 6.2e-6 relative shared, 9.0e-6 whole, for 4 us less).
 inline bool use_stream_k(int64_t tiles, int64_t stages, int sms, bool split) {
   if (tiles < 1 || stages < 16 || tiles * stages < 16 * static_cast<int64_t>(sms)) return false;
-  return split ? 10 * tiles < 9 * sms : 2 * tiles < sms;
+  if (2 * tiles < sms) return true;
+  return 10 * tiles < 9 * sms && (split || stages * (sms - tiles) >= 32 * static_cast<int64_t>(sms));
 }
 
 // One instance of the grouped GEMM: tensor maps and output description, laid out
