@@ -70,34 +70,96 @@ __device__ __forceinline__ float from_bf16(uint16_t b) { return __uint_as_float(
 // Eight consecutive positions per thread (n is a multiple of 128), stored in 16 bytes:
 // with one position and a 2-byte store a thread, 20 signals of 530,000 samples took
 // 64 us at 13 % of the memory rate.
+//
+// Lb > 2: the eight windows of a thread are 8 Lb samples of their own, so lanes that read
+// them for themselves sit 32 Lb bytes apart (20 signals of 500,000 samples, R = 128 of
+// T = 1024: 376 us for the call so, 163 with the code below, 194 with one position a
+// thread).  A warp instead fetches 32 windows at a time, at most eight samples of each per
+// turn (whole 32-byte sectors), transposes them through shared memory while the next
+// turn's loads are under way, and each lane sums one window in order.
 constexpr int kSigPerBlock = 8 * 256;
+constexpr int kSigTurn = 8;               // samples of a window fetched per turn
+constexpr int kSigFetch = 32 * (kSigTurn + 1);
 
 __device__ __forceinline__ uint4 pack8(const uint16_t (&v)[8]) {
   return make_uint4(v[0] | (uint32_t(v[1]) << 16), v[2] | (uint32_t(v[3]) << 16), v[4] | (uint32_t(v[5]) << 16),
                     v[6] | (uint32_t(v[7]) << 16));
 }
 
-__global__ void __launch_bounds__(256) batch_signal_kernel(const SigJob* __restrict__ jobs,
+// The box sums of a warp's positions w0 .. w0 + 255 (Lb > 2, a power of two), eight
+// consecutive ones per lane; 0 where the window passes the end of the signal.  fetch and
+// sums: the warp's buffers.
+__device__ __forceinline__ void box_sums_warp(const SigJob& J, int64_t w0, float* fetch, float* sums, float (&v)[8]) {
+  const int lane = threadIdx.x & 31, Lb = J.Lb;
+  const int lc = Lb < kSigTurn ? 31 - __clz(Lb) : 3, C = 1 << lc;   // samples per window and turn
+  const int64_t x0 = J.phi + w0 * Lb, rest = J.S - x0;
+  const int left = rest < 256 * Lb ? static_cast<int>(rest) : 256 * Lb;   // samples from x0 on (may be <= 0)
+  const float* __restrict__ s = J.s + x0;
+  const int at = (lane >> lc) * Lb + (lane & (C - 1)), step = (32 >> lc) * Lb;   // this lane's first, and to its next
+  const int to = (lane >> lc) * (C + 1) + (lane & (C - 1)), to_step = (32 >> lc) * (C + 1);
+  float r[kSigTurn];
+  auto load = [&](int base) {   // the samples of one turn: 32 windows from `base` on, C of each
+#pragma unroll
+    for (int j = 0; j < kSigTurn; ++j) {
+      const int o = base + at + j * step;
+      r[j] = j < C && o < left ? __ldg(s + o) : 0.0f;
+    }
+  };
+  load(0);
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k) {
+    float sum = 0.0f;
+#pragma unroll 1
+    for (int t = 0; t < Lb; t += C) {
+#pragma unroll
+      for (int j = 0; j < kSigTurn; ++j)
+        if (j < C) fetch[to + j * to_step] = r[j];
+      __syncwarp();
+      if (t + C < Lb) load(32 * k * Lb + t + C);
+      else if (k < 7) load(32 * (k + 1) * Lb);
+#pragma unroll
+      for (int e = 0; e < kSigTurn; ++e)
+        if (e < C) sum += fetch[lane * (C + 1) + e];
+      __syncwarp();
+    }
+    sums[32 * k + lane] = (32 * k + lane + 1) * Lb <= left ? sum * J.scale : 0.0f;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = sums[8 * lane + k];
+}
+
+__global__ void __launch_bounds__(256, 6) batch_signal_kernel(const SigJob* __restrict__ jobs,
                                                            const int* __restrict__ job_of) {
+  __shared__ float s_fetch[8][kSigFetch];
+  __shared__ float s_sums[8][256];
   pdl_begin();
   const SigJob J = jobs[job_of[blockIdx.x]];
   const int64_t u0 = (static_cast<int64_t>(blockIdx.x) - J.block0) * kSigPerBlock + 8 * threadIdx.x;
-  if (u0 >= J.n) return;
-  const int64_t x0 = J.phi + static_cast<int64_t>(J.Lb) * u0;
-  const float* __restrict__ s = J.s + x0;
+  const int warp = threadIdx.x / 32;
+  const int64_t w0 = u0 - 8 * (threadIdx.x & 31);
+  if (w0 >= J.n) return;   // the same for the whole warp
   float v[8];
-  if (J.Lb == 1 && x0 + 8 <= J.S && reinterpret_cast<uintptr_t>(s) % 16 == 0) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(s)), b = __ldg(reinterpret_cast<const float4*>(s) + 1);
-    const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = (0.0f + w[k]) * J.scale;
+  if (J.Lb > 2) {
+    box_sums_warp(J, w0, s_fetch[warp], s_sums[warp], v);
+    if (u0 >= J.n) return;
   } else {
+    if (u0 >= J.n) return;
+    const int64_t x0 = J.phi + J.Lb * u0;
+    const float* __restrict__ s = J.s + x0;
+    if (J.Lb == 1 && x0 + 8 <= J.S && reinterpret_cast<uintptr_t>(s) % 16 == 0) {
+      const float4 a = __ldg(reinterpret_cast<const float4*>(s)), b = __ldg(reinterpret_cast<const float4*>(s) + 1);
+      const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      v[k] = 0.0f;
-      if (x0 + static_cast<int64_t>(J.Lb) * (k + 1) <= J.S) {
-        for (int w = 0; w < J.Lb; ++w) v[k] += __ldg(s + k * J.Lb + w);
-        v[k] *= J.scale;
+      for (int k = 0; k < 8; ++k) v[k] = (0.0f + w[k]) * J.scale;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = 0.0f;
+        if (x0 + J.Lb * (k + 1) <= J.S) {
+          for (int w = 0; w < J.Lb; ++w) v[k] += __ldg(s + k * J.Lb + w);
+          v[k] *= J.scale;
+        }
       }
     }
   }
