@@ -436,12 +436,13 @@ pj_status proj_batch_plan_create(const pj_batch_desc* descs, int32_t n, void* wo
  *   us_per_tile, us_per_stage, us_per_out_kb: the cost model of one tile, in
  *              microseconds: fixed, per K stage of a 128 x 256 tile (scaled by the
  *              tile's height) and per KB of output; 0 = built-in values.
- *   solo:      0 = the BF16 products run on pairs of CTAs (clusters of two) that
- *                  take neighbouring tiles of one tile row and share its rows of
- *                  A_c, each loading half and multicasting it to both (the
- *                  "solo" build of the library has no pairs and ignores this);
- *              1 = every CTA loads its own tiles.
- *   Correlation instances always use 256-row tiles and no split.
+ *   solo:      0 = the BF16 products run on pairs of CTAs (2-SM MMAs over two
+ *                  neighbouring tile columns) and the correlations beside them in a
+ *                  launch on single CTAs, unless the cost model finds one launch on
+ *                  single CTAs for both shorter (the "solo" build of the library has
+ *                  no pairs and ignores this);
+ *              1 = every product and correlation on single CTAs, in one launch.
+ *   Correlation instances always use 256-row tiles of 128 lags and no split.
  * The schedule, splits and tiles are decided when the plan is created. */
 typedef struct {
   int32_t schedule;
@@ -455,7 +456,7 @@ typedef struct {
 
 /* What a plan's tuner decided: tiles of the BF16 and E4M3 grouped launches, the
  * persistent CTAs of the larger launch, instances whose reduced dimension was
- * split, and the cost model's makespan (the most loaded CTA, summed over the two
+ * split, and the cost model's makespan (the most loaded CTA, summed over the
  * launches) and total (all CTAs), in microseconds. */
 typedef struct {
   int32_t gemm_tiles;

@@ -5,14 +5,22 @@
 // GEMM instances are the projected products of Sec. III-B.  A correlation
 // instance (valid cross-correlation with the box/Haar projection, Sec. III-A,
 // Eq. 11-13) is lowered to GEMMs, one per (phase, template): with the
-// projected signal b^phi viewed as rows of W samples and the projected
-// template kb in a W x (R + W - 1) Toeplitz matrix Kt[p][j] = kb[j - p],
-//   r[phi + Lb (W i + p)] = sum_j b^phi[W i + j] Kt[p][j],
-// i.e. output row i of the GEMM holds W consecutive lags of that phase: W = 256,
-// the width of a CTA pair's tile, or 128 on solo CTAs and for E4M3.
-// The signal operand is read in the row-split mode of the grouped GEMM (with
-// c = W / 64, chunk k of row i = view row i + k / c, column 64 (k mod c)), so nothing
-// is materialised per lag; the Toeplitz matrix of each template is built once per run.
+// projected signal b^phi viewed as rows of 128 samples and the projected
+// template kb in a 128 x (R + 127) Toeplitz matrix Kt[p][j] = kb[j - p],
+//   r[phi + Lb (128 i + p)] = sum_j b^phi[128 i + j] Kt[p][j],
+// i.e. output row i of the GEMM holds 128 consecutive lags of that phase.
+// The signal operand is read in the row-split mode of the grouped GEMM (chunk
+// k of row i = view row i + k/2, half k mod 2), so nothing is materialised
+// per lag; the Toeplitz matrix of each template is built once per run.
+//
+// Those rows are one tile column wide, so beside products on CTA pairs the correlations
+// take a grouped launch of their own, on single CTAs.  Rows of 256 lags, the pairs' tile
+// width, put them in the products' launch, but the reduced dimension grows to R + 255,
+// and a sample that is not finite spoils 255 lags before its windows and past them
+// instead of 127 (every lag of a row whose Toeplitz zeros meet it).  20 signals of
+// 500,000 samples, T = 1024, split, at R = 1024, 512 and 64: 97, 110 and 211 us with rows
+// of 256 lags, 90, 102 and 196 so.
+//
 // GEMM instances with E4M3 compute are quantised after the projections and
 // multiplied by a second persistent grouped launch of the block-scaled kernel.
 //
@@ -22,7 +30,7 @@
 // (zeroed) FP32 output, and the tiles are dealt to the persistent CTAs sorted
 // by reduced length (or, as an option, by cost), each onto the least-loaded
 // one.  By default the BF16 products run on 2-SM MMAs (gemm_cg2.cu): clusters
-// of two CTAs take two tile columns at once (see schedule_kind).  The cost model's
+// of two CTAs take two tile columns at once (see Schedule).  The cost model's
 // constants, the height policy, the largest split, the order and the pairing
 // are knobs (pj_batch_tuning) that a measuring autotuner can search.
 #include <cuda_bf16.h>
@@ -56,7 +64,7 @@ struct TplJob {
   const float* k;
   uint16_t* Kt;
   int64_t R, Kpad, ldk, block0;  // row p: hi at [0, Kpad), split residual at [Kpad, 2 Kpad)
-  int Lb, nsplit, rows;          // rows: samples per output row of the lowering (128 or 256)
+  int Lb, nsplit;
   float scale;
 };
 
@@ -73,7 +81,7 @@ __device__ __forceinline__ float from_bf16(uint16_t b) { return __uint_as_float(
 //
 // Lb > 2: the eight windows of a thread are 8 Lb samples of their own, so lanes that read
 // them for themselves sit 32 Lb bytes apart (20 signals of 500,000 samples, R = 128 of
-// T = 1024: 376 us for the call so, 163 with the code below, 194 with one position a
+// T = 1024: 376 us for the call so, 153 with the code below, 194 with one position a
 // thread).  A warp instead fetches 32 windows at a time, at most eight samples of each per
 // turn (whole 32-byte sectors), transposes them through shared memory while the next
 // turn's loads are under way, and each lane sums one window in order.
@@ -184,9 +192,9 @@ __global__ void __launch_bounds__(256) batch_toeplitz_kernel(const TplJob* __res
   const TplJob J = jobs[job_of[blockIdx.x]];
   const int64_t per = J.Kpad / 8;
   const int64_t e = (static_cast<int64_t>(blockIdx.x) - J.block0) * 256 + threadIdx.x;
-  if (e >= J.rows * per) return;
+  if (e >= 128 * per) return;
   // (a 32-bit division wherever the entries can be counted in 32 bits)
-  const int p = static_cast<int>(J.rows * per <= 0xffffffffll
+  const int p = static_cast<int>(128 * per <= 0xffffffffll
                                      ? static_cast<uint32_t>(e) / static_cast<uint32_t>(per) : e / per);
   const int64_t jj = (e - p * per) * 8;
   uint16_t h[8], l[8];
@@ -324,7 +332,10 @@ struct pj_batch_plan {
   GemmTile* d_tiles = nullptr;
   int* d_cta_off = nullptr;
   int ctas = 0;
-  int paired = 0;        // BF16 launch in clusters of two CTAs
+  int paired = 0;        // BF16 products in clusters of two CTAs (the correlations in a launch of their own)
+  GemmTile* d_conv_tiles = nullptr;
+  int* d_conv_cta_off = nullptr;
+  int conv_ctas = 0;
   MxInst* d_mx = nullptr;
   GemmTile* d_mx_tiles = nullptr;
   int* d_mx_cta_off = nullptr;
@@ -419,9 +430,13 @@ int split_cap(int64_t stages, bool fp32_out, const Tuning& t) {
   return s;
 }
 
+// Kinds of GEMMs: the BF16 products, everything on the block-scaled MMA, and the lowered
+// BF16 correlations.
+constexpr int kProduct = 0, kE4m3 = 1, kConv = 2;
+
 // One GEMM of the grouped launches, before tiling.
 struct GemmPlanned {
-  int kind;             // 0 = BF16 kernel, 1 = E4M3 kernel
+  int kind;             // kProduct, kE4m3 or kConv
   int index;            // into Built::gemms or Built::mx
   int tiles_m, tiles_n; // tile rows (of bn A_c rows) and columns (of 128 B_d rows)
   int stages;           // K stages of a whole tile
@@ -435,7 +450,7 @@ struct Built {
   std::vector<MxQuantSide> qsides;
   std::vector<ZeroJob> zeros;
   std::vector<GemmPlanned> planned;
-  size_t mx_off = 0, mx_tiles_off = 0, mx_cta_off = 0, cta_off_off = 0, qsides_off = 0, qsides_map_off = 0,
+  size_t mx_off = 0, mx_tiles_off = 0, mx_cta_off = 0, conv_cta_off = 0, cta_off_off = 0, qsides_off = 0, qsides_map_off = 0,
          zero_off = 0, zero_map_off = 0;
   int64_t qsides_total = 0, zero_total = 0;
   int tiles_cap = 0, mx_tiles_cap = 0;
@@ -615,7 +630,7 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
         m.rowsQ = g.M; m.rowsP = g.N; m.pitch = qpitch; m.Kq_pad = g.Kq_pad; m.qsplit = g.qsplit;
         m.Y = x.Y; m.ldy = x.ldy; m.out_dtype = x.out_dtype; m.bn = bn;
         const int stages = static_cast<int>(g.Kq_pad / 128) * (g.qsplit == 1 ? 1 : 3);
-        b.planned.push_back(GemmPlanned{1, static_cast<int>(b.mx.size()), static_cast<int>(ceil_div(g.M, bn)),
+        b.planned.push_back(GemmPlanned{kE4m3, static_cast<int>(b.mx.size()), static_cast<int>(ceil_div(g.M, bn)),
                                         static_cast<int>(ceil_div(g.N, 128)), stages, bn,
                                         split_cap(stages, x.out_dtype == PJ_F32, b.tune), x.out_dtype == PJ_BF16});
         b.mx.push_back(m);
@@ -636,7 +651,7 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
         }
         a.bn = pick_bn(g.M, 32, 256, b.tune);
         const int stages = static_cast<int>(ceil_div(g.Kp_pad, 64)) * a.nseg;
-        b.planned.push_back(GemmPlanned{0, static_cast<int>(b.gemms.size()), static_cast<int>(ceil_div(g.M, a.bn)),
+        b.planned.push_back(GemmPlanned{kProduct, static_cast<int>(b.gemms.size()), static_cast<int>(ceil_div(g.M, a.bn)),
                                         static_cast<int>(ceil_div(g.N, 128)), stages, a.bn,
                                         split_cap(stages, x.out_dtype == PJ_F32, b.tune), x.out_dtype == PJ_BF16});
         b.gemms.push_back(a);
@@ -646,20 +661,16 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
       // E4M3: the BF16 hi + lo of the projected signal and templates feed the quantisers
       const bool e4 = x.prec.compute == PJ_E4M3;
       const int nsplit = e4 ? 2 : x.prec.split_terms;
-      // Samples per output row of the lowering: 256 on CTA pairs, whose tiles are 256 wide
-      // (128 would leave half of every tile empty), else 128.
-      const int W = !e4 && batch_pairs(b.tune) ? 256 : 128;
-      const int64_t Kpad = round_up(g.R + W - 1, 64);
+      const int64_t Kpad = round_up(g.R + 127, 64);
       const int64_t Kq = round_up(Kpad, 128);
       const float scale = 1.0f / sqrtf(static_cast<float>(g.Lb));
       std::vector<uint16_t*> kts(g.nt);
       for (int64_t t = 0; t < g.nt; ++t) {
-        const size_t kt = L.take(2 * W * Kpad * nsplit);
+        const size_t kt = L.take(2 * 128 * Kpad * nsplit);
         TplJob tj{};
         tj.k = static_cast<const float*>(x.B) + t * g.T;
         tj.Kt = ptr<uint16_t>(ws, kt);
-        tj.R = g.R; tj.Kpad = Kpad; tj.ldk = Kpad * nsplit; tj.Lb = g.Lb; tj.nsplit = nsplit; tj.rows = W;
-        tj.scale = scale;
+        tj.R = g.R; tj.Kpad = Kpad; tj.ldk = Kpad * nsplit; tj.Lb = g.Lb; tj.nsplit = nsplit; tj.scale = scale;
         b.tpl.push_back(tj);
         kts[t] = tj.Kt;
       }
@@ -675,12 +686,12 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
       for (int phi = 0; phi < g.Lb; ++phi) {
         const int64_t lags_phi = g.lags > phi ? ceil_div(g.lags - phi, g.Lb) : 0;
         if (lags_phi == 0) continue;
-        const int64_t rows_alloc = ceil_div(lags_phi + g.R - 1, W) + 1;
-        const size_t q = L.take(2 * W * rows_alloc * nsplit);
+        const int64_t rows_alloc = ceil_div(lags_phi + g.R - 1, 128) + 1;
+        const size_t q = L.take(2 * 128 * rows_alloc * nsplit);
         SigJob sj{};
         sj.s = static_cast<const float*>(x.A); sj.Q = ptr<uint16_t>(ws, q);
-        sj.Qlo = nsplit > 1 ? ptr<uint16_t>(ws, q + 2 * W * rows_alloc) : nullptr;
-        sj.S = g.S; sj.n = rows_alloc * W; sj.Lb = g.Lb; sj.phi = phi; sj.scale = scale;
+        sj.Qlo = nsplit > 1 ? ptr<uint16_t>(ws, q + 2 * 128 * rows_alloc) : nullptr;
+        sj.S = g.S; sj.n = rows_alloc * 128; sj.Lb = g.Lb; sj.phi = phi; sj.scale = scale;
         b.sig.push_back(sj);
         if (e4) {
           const int64_t rowsQ = ceil_div(lags_phi, 128);
@@ -703,7 +714,7 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
             m.conv_mode = 1;
             m.conv_stride = static_cast<int64_t>(g.Lb) * g.nt;
             m.conv_limit = lags_phi;
-            b.planned.push_back(GemmPlanned{1, static_cast<int>(b.mx.size()), static_cast<int>(tiles_m), 1, kc, bn,
+            b.planned.push_back(GemmPlanned{kE4m3, static_cast<int>(b.mx.size()), static_cast<int>(tiles_m), 1, kc, bn,
                                             1, false});
             b.mx.push_back(m);
           }
@@ -711,8 +722,8 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
         }
         for (int64_t t = 0; t < g.nt; ++t) {
           GemmTcArgs a;
-          a.Q = sj.Q; a.ldq = W; a.rowsQ = ceil_div(lags_phi, W);
-          a.P = kts[t]; a.ldp = Kpad * nsplit; a.rowsP = W;
+          a.Q = sj.Q; a.ldq = 128; a.rowsQ = ceil_div(lags_phi, 128);
+          a.P = kts[t]; a.ldp = Kpad * nsplit; a.rowsP = 128;
           a.xdim = Kpad * nsplit; a.kdim = Kpad;
           if (nsplit == 1) {
             a.nseg = 1;
@@ -725,14 +736,14 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
             a.segQ[2] = rows_alloc; a.segP[2] = 0;
           }
           a.Y = static_cast<float*>(x.Y) + phi * g.nt + t;
-          a.ldy = W; a.out_dtype = PJ_F32;
-          a.conv_mode = 1; a.conv_w = W; a.q_rows_alloc = rows_alloc * nsplit;
+          a.ldy = 128; a.out_dtype = PJ_F32;
+          a.conv_mode = 1; a.q_rows_alloc = rows_alloc * nsplit;
           a.conv_stride = static_cast<int64_t>(g.Lb) * g.nt;
           a.conv_limit = lags_phi;
           a.bn = 256;
           const int stages = static_cast<int>(ceil_div(Kpad, 64)) * a.nseg;
-          b.planned.push_back(GemmPlanned{0, static_cast<int>(b.gemms.size()),
-                                          static_cast<int>(ceil_div(a.rowsQ, 256)), W / 128, stages, 256, 1, false});
+          b.planned.push_back(GemmPlanned{kConv, static_cast<int>(b.gemms.size()),
+                                          static_cast<int>(ceil_div(a.rowsQ, 256)), 1, stages, 256, 1, false});
           b.gemms.push_back(a);
         }
       }
@@ -752,7 +763,7 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
   for (auto& s : b.sig) { s.block0 = blk; blk += ceil_div(s.n, kSigPerBlock); }
   b.sig_total = blk;
   blk = 0;
-  for (auto& t : b.tpl) { t.block0 = blk; blk += ceil_div(t.rows * t.Kpad, kTplPerBlock); }
+  for (auto& t : b.tpl) { t.block0 = blk; blk += ceil_div(128 * t.Kpad, kTplPerBlock); }
   b.tpl_total = blk;
   blk = 0;
   for (auto& q : b.sigq) { q.block0 = blk; blk += ceil_div(q.nblk, 256); }
@@ -786,10 +797,10 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
   b.qsides_total = blk;
   for (const auto& pl : b.planned)
     if (pl.cap > 1) {
-      const int64_t M = pl.kind ? b.mx[pl.index].rowsQ : b.gemms[pl.index].rowsQ;
-      const int64_t N = pl.kind ? b.mx[pl.index].rowsP : b.gemms[pl.index].rowsP;
-      const int64_t ld = pl.kind ? b.mx[pl.index].ldy : b.gemms[pl.index].ldy;
-      void* Y = pl.kind ? b.mx[pl.index].Y : b.gemms[pl.index].Y;
+      const int64_t M = pl.kind == kE4m3 ? b.mx[pl.index].rowsQ : b.gemms[pl.index].rowsQ;
+      const int64_t N = pl.kind == kE4m3 ? b.mx[pl.index].rowsP : b.gemms[pl.index].rowsP;
+      const int64_t ld = pl.kind == kE4m3 ? b.mx[pl.index].ldy : b.gemms[pl.index].ldy;
+      void* Y = pl.kind == kE4m3 ? b.mx[pl.index].Y : b.gemms[pl.index].Y;
       b.zeros.push_back(ZeroJob{static_cast<float*>(Y), M, N, ld, 0});
     }
   blk = 0;
@@ -803,13 +814,14 @@ pj_status layout(const pj_batch_desc* d, int n, const pj_batch_tuning* tuning, v
   b.mx_off = L.take(sizeof(MxInst) * (b.mx.size() + 1));
   // tile lists sized for the largest split the tuner may choose
   int tiles = 0, mx_tiles = 0;
-  for (const auto& pl : b.planned) (pl.kind ? mx_tiles : tiles) += pl.tiles_m * pl.tiles_n * pl.cap;
+  for (const auto& pl : b.planned) (pl.kind == kE4m3 ? mx_tiles : tiles) += pl.tiles_m * pl.tiles_n * pl.cap;
   b.tiles_cap = tiles;
   b.mx_tiles_cap = mx_tiles;
   b.tiles_off = L.take(sizeof(GemmTile) * (tiles + 1));
   b.mx_tiles_off = L.take(sizeof(GemmTile) * (mx_tiles + 1));
   b.cta_off_off = L.take(sizeof(int) * (kMaxCtas + 1));
   b.mx_cta_off = L.take(sizeof(int) * (kMaxCtas + 1));
+  b.conv_cta_off = L.take(sizeof(int) * (kMaxCtas + 1));
   b.total = L.off;
   return PJ_OK;
 }
@@ -830,13 +842,13 @@ struct Schedule {
   bool paired = false;          // the lists are those of clusters of two CTAs
 };
 
-// Tiles of the instances of one kernel (kind), with the splits chosen, dealt to
+// Tiles of the instances of one launch (of kind a or c), with the splits chosen, dealt to
 // the CTAs (paired: to clusters of two CTAs, see Item).
-Schedule schedule_kind(const Built& b, int kind, int sms, bool paired) {
+Schedule schedule_kinds(const Built& b, int a, int c, int sms, bool paired) {
   const Tuning& t = b.tune;
   std::vector<const GemmPlanned*> ins;
   for (const auto& pl : b.planned)
-    if (pl.kind == kind) ins.push_back(&pl);
+    if (pl.kind == a || pl.kind == c) ins.push_back(&pl);
   std::vector<int> split(ins.size(), 1);
   int64_t ntiles = 0;
   double total = 0;
@@ -1004,20 +1016,39 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
       PJ_CUDA_TRY(cudaMemcpyAsync(area.U64, std::get<3>(key), sizeof(double) * L * L, cudaMemcpyHostToDevice, st));
     PJ_CUDA_TRY(launch_basis_build(kind, L, lp1, area, error_word(workspace), st));
   }
-  // instance tables and the tuned schedules of the two grouped launches
-  // BF16 products on CTA pairs unless the tuning asks for solo CTAs
-  const bool paired = batch_pairs(w.tune);
+  // The tuned schedules of the grouped launches.  BF16 products go to CTA pairs unless the
+  // tuning asks for solo CTAs, and the correlations, whose tiles are one column wide, to a
+  // launch of their own.  Of a batch with both, one launch on solo CTAs takes all where
+  // the pairs' gain on the products (the grouped product of 40 products and 20
+  // correlations 818 us on solo CTAs, 733 on pairs) is less than what two unfilled
+  // launches lose by the model.  Calls, two launches and one: 4 products with 20
+  // correlations 136 us and 110, 8 with 20 224 and 201, 10 with 11 259 and 250; 30 with
+  // 15 614 and 626, 40 with 20 1367 and 1425.
+  Schedule S0, S2;
+  bool paired = batch_pairs(w.tune);
+  if (paired) {
+    S0 = schedule_kinds(w, kProduct, kProduct, sms, true);
+    S2 = schedule_kinds(w, kConv, kConv, sms, false);
+  }
+  if (!paired || (w.tune.schedule != 1 && S0.count > 0 && S2.count > 0)) {
+    Schedule one = schedule_kinds(w, kProduct, kConv, sms, false);
+    if (!paired || one.makespan * 818 < (S0.makespan + S2.makespan) * 733) {
+      paired = false;
+      S0 = std::move(one);
+      S2 = Schedule{};
+      S2.cta_off.assign(1, 0);
+    }
+  }
+  const Schedule S1 = schedule_kinds(w, kE4m3, kE4m3, sms, false);
   std::vector<GemmInst> insts(w.gemms.size());
   for (size_t i = 0; i < w.gemms.size(); ++i) {
-    w.gemms[i].pair = paired ? 1 : 0;
+    w.gemms[i].pair = paired && !w.gemms[i].conv_mode ? 1 : 0;
     if (!build_gemm_inst(w.gemms[i], &insts[i])) return fail(PJ_EINVAL, "could not encode tensor maps for batch entry");
   }
   std::vector<MxInst> mxi(w.mx.size());
   for (size_t i = 0; i < w.mx.size(); ++i)
     if (!build_mx_inst(w.mx[i], &mxi[i])) return fail(PJ_EINVAL, "could not encode tensor maps for batch entry");
-  const Schedule S0 = schedule_kind(w, 0, sms, paired);
-  const Schedule S1 = schedule_kind(w, 1, sms, false);
-  if (S0.tiles.size() > static_cast<size_t>(w.tiles_cap) || S1.tiles.size() > static_cast<size_t>(w.mx_tiles_cap))
+  if (S0.tiles.size() + S2.tiles.size() > static_cast<size_t>(w.tiles_cap) || S1.tiles.size() > static_cast<size_t>(w.mx_tiles_cap))
     return fail(PJ_EINVAL, "internal: schedule exceeds its reserved tile list");
   // zero jobs are needed only for the instances the schedules actually split
   std::vector<ZeroJob> zeros;
@@ -1027,9 +1058,9 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
     for (const auto& t : S1.tiles) if (t.red) split1[t.inst] = 1;
     int64_t blk = 0;
     for (const auto& pl : w.planned) {
-      if (!(pl.kind ? split1[pl.index] : split0[pl.index])) continue;
+      if (!(pl.kind == kE4m3 ? split1[pl.index] : split0[pl.index])) continue;
       ZeroJob z{};
-      if (pl.kind) {
+      if (pl.kind == kE4m3) {
         z.Y = static_cast<float*>(w.mx[pl.index].Y); z.rows = w.mx[pl.index].rowsQ;
         z.cols = w.mx[pl.index].rowsP; z.ld = w.mx[pl.index].ldy;
       } else {
@@ -1098,10 +1129,13 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   PJ_TRY(upload(zeros, workspace, w.zero_off, st));
   PJ_TRY(upload(insts, workspace, w.insts_off, st));
   PJ_TRY(upload(mxi, workspace, w.mx_off, st));
-  PJ_TRY(upload(S0.tiles, workspace, w.tiles_off, st));
+  std::vector<GemmTile> tiles = S0.tiles;   // the correlations' after the products'
+  tiles.insert(tiles.end(), S2.tiles.begin(), S2.tiles.end());
+  PJ_TRY(upload(tiles, workspace, w.tiles_off, st));
   PJ_TRY(upload(S1.tiles, workspace, w.mx_tiles_off, st));
   PJ_TRY(upload(S0.cta_off, workspace, w.cta_off_off, st));
   PJ_TRY(upload(S1.cta_off, workspace, w.mx_cta_off, st));
+  PJ_TRY(upload(S2.cta_off, workspace, w.conv_cta_off, st));
   PJ_CUDA_TRY(cudaStreamSynchronize(st));
   int code = 0;
   PJ_CUDA_TRY(cudaMemcpy(&code, workspace, sizeof(int), cudaMemcpyDeviceToHost));
@@ -1131,7 +1165,7 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   p->sig_of = ptr<int>(workspace, w.sig_map_off);
   p->tpl_of = ptr<int>(workspace, w.tpl_map_off);
   for (const auto& s : w.sig) p->sig_blocks = s.block0 + ceil_div(s.n, kSigPerBlock);
-  for (const auto& t : w.tpl) p->tpl_blocks = t.block0 + ceil_div(t.rows * t.Kpad, kTplPerBlock);
+  for (const auto& t : w.tpl) p->tpl_blocks = t.block0 + ceil_div(128 * t.Kpad, kTplPerBlock);
   p->d_sigq = ptr<SigQJob>(workspace, w.sigq_off);
   p->d_sfx = ptr<SfExpJob>(workspace, w.sfx_off);
   p->sigq_of = ptr<int>(workspace, w.sigq_map_off);
@@ -1143,6 +1177,9 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   p->d_cta_off = ptr<int>(workspace, w.cta_off_off);
   p->ctas = static_cast<int>(S0.cta_off.size()) - 1;   // clusters of two when paired
   p->paired = S0.paired ? 1 : 0;
+  p->d_conv_tiles = p->d_tiles + S0.tiles.size();
+  p->d_conv_cta_off = ptr<int>(workspace, w.conv_cta_off);
+  p->conv_ctas = static_cast<int>(S2.cta_off.size()) - 1;
   p->d_mx = ptr<MxInst>(workspace, w.mx_off);
   p->d_mx_tiles = ptr<GemmTile>(workspace, w.mx_tiles_off);
   p->d_mx_cta_off = ptr<int>(workspace, w.mx_cta_off);
@@ -1154,13 +1191,12 @@ pj_status proj_batch_plan_create_tuned(const pj_batch_desc* descs, int32_t n, co
   p->zero_of = ptr<int>(workspace, w.zero_map_off);
   p->zero_blocks = zero_blocks;
   p->sms = sms;
-  p->info.gemm_tiles = static_cast<int32_t>(S0.count);
+  p->info.gemm_tiles = static_cast<int32_t>(S0.count + S2.count);
   p->info.mx_tiles = static_cast<int32_t>(S1.count);
-  const int main_ctas = p->ctas * (p->paired ? 2 : 1);
-  p->info.ctas = main_ctas > p->mx_ctas ? main_ctas : p->mx_ctas;
+  p->info.ctas = std::max({p->ctas * (p->paired ? 2 : 1), p->mx_ctas, p->conv_ctas});
   p->info.split_instances = S0.splits + S1.splits;
-  p->info.model_makespan_us = S0.makespan + S1.makespan;
-  p->info.model_total_us = S0.total + S1.total;
+  p->info.model_makespan_us = S0.makespan + S1.makespan + S2.makespan;
+  p->info.model_total_us = S0.total + S1.total + S2.total;
   *plan = p;
   return PJ_OK;
 }
@@ -1204,6 +1240,8 @@ pj_status proj_batch_run(const pj_batch_plan* plan, void* stream) {
                                                      error_word(plan->ws), st)
                            : launch_gemm_tc_grouped(plan->d_insts, plan->d_tiles, plan->d_cta_off, plan->ctas,
                                                     error_word(plan->ws), st));
+  PJ_CUDA_TRY(launch_gemm_tc_grouped(plan->d_insts, plan->d_conv_tiles, plan->d_conv_cta_off, plan->conv_ctas,
+                                     error_word(plan->ws), st));
   PJ_CUDA_TRY(launch_gemm_mx_grouped(plan->d_mx, plan->d_mx_tiles, plan->d_mx_cta_off, plan->mx_ctas,
                                      error_word(plan->ws), st));
   return PJ_OK;

@@ -350,13 +350,11 @@ struct GemmTcArgs {
   void* Y;
   int64_t ldy;
   int out_dtype;
-  // Row-split mode (a lowered correlation): Q is a conv_w-wide view with q_rows_alloc
-  // rows; with c = conv_w / 64, K chunk k of output row r reads view row r + k / c at
-  // column 64 (k mod c).  Output element (i, j) is sample i * conv_w + j < conv_limit, at
-  // Y[(i * conv_w + j) * conv_stride].
+  // Row-split mode (a lowered correlation): Q is a 128-wide view with q_rows_alloc
+  // rows; K chunk k of output row r reads view row r + k/2 at column 64 (k mod 2).
+  // Output element (i, j) is sample i*128 + j < conv_limit, at Y[(i*128 + j) * conv_stride].
   int conv_mode = 0;
   int64_t q_rows_alloc = 0, conv_stride = 1, conv_limit = 0;
-  int conv_w = 128;   // width of that view and samples per output row: 128, or 256 for CTA pairs
   int bn = 256;   // rows of Q per tile: a multiple of 32 (64 for an MN-major Q), at most 256
   // MN-major operands: Q (P) is stored transposed, as xdim rows of the reduced
   // dimension by rowsQ (rowsP) contiguous values with pitch ldq (ldp); the tensor
@@ -431,7 +429,7 @@ struct GemmInst {  // 128-byte aligned through its tensor maps
   int M, N, kc, nseg;     // kc: K stages of all segments together
   int segP[3], segQ[3];
   int segKc[3];           // K stages of each segment
-  int tiles_n, out_bf16, tma_out, tma_rows, conv_mode, conv_w;
+  int tiles_n, out_bf16, tma_out, tma_rows, conv_mode;
   // TMA boxes may store (or add into) tile columns that end at or before this
   // column.  A TMA store writes the whole 16-byte chunk that holds a row's last
   // element, so when a row of Y does not end on a 16-byte boundary the ragged

@@ -177,15 +177,13 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
         const int bn = I->bn, half = bn / 2;
         const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
         const bool share = I->share != 0;   // hi and lo tiles in alternate slots (GemmInst::share)
-        const bool conv = kGrouped && I->conv_mode != 0;
-        const int cmask = conv ? I->conv_w / CK - 1 : 0, cshift = conv ? 31 - __clz(I->conv_w / CK) : 0;
         const int f0 = share ? 2 * share_chunk(T.k0) : T.k0, f1 = share ? 2 * share_chunk(T.k1) : T.k1;
         const int sP0 = I->segP[0], sP1 = I->segP[1], sP2 = I->segP[2];
         const int sQ0 = I->segQ[0], sQ1 = I->segQ[1], sQ2 = I->segQ[2];
         const int e0 = I->nseg > 1 ? I->segKc[0] : 0x7fffffff, e1 = I->nseg > 2 ? e0 + I->segKc[1] : 0x7fffffff;
         const uint32_t pair_bytes = 2 * (kCStageP + static_cast<uint32_t>(half) * CK * 2);
         const int prow = T.tj * 2 * CM + static_cast<int>(rank) * CM;
-        const int qrow0 = T.ti * bn + static_cast<int>(rank) * half;
+        const int qrow = T.ti * bn + static_cast<int>(rank) * half;
         for (int kk = f0; kk < f1; ++kk, ++issued) {
           if (issued == stall) {
             ok = false;
@@ -206,9 +204,7 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             oQ = kk < e0 ? sQ0 : (kk < e1 ? sQ1 : sQ2);
           }
           const int px = oP + kin * CK;
-          // (a lowered correlation's Q: see gemm_tc.cu)
-          const int qx = conv ? (kin & cmask) * CK : oQ + kin * CK;
-          const int qrow = conv ? qrow0 + (kin >> cshift) + oQ : qrow0;
+          const int qx = oQ + kin * CK;
           const uint32_t bar = full_leader + stage * 8;
           uint8_t* const dP = sm + stage * slot_bytes;
           uint8_t* const dQ = dP + kCStageP;
@@ -414,9 +410,6 @@ __global__ void __launch_bounds__(kCThreads, 1) gemm_cg2_kernel(const __grid_con
             pending = true;
           }
           if (++sbuf == nbuf) sbuf = 0;
-        } else if (kGrouped && I->conv_mode) {
-          // lowered correlation: element (i, j) is output sample i * conv_w + j of this phase
-          store_samples<32>(r, static_cast<float*>(Yout), I->conv_w, I->conv_stride, I->conv_limit, i0, j, jok);
         } else if (jok) {
           store_rows<32>(r, Yout, ldy, out_bf16, kGrouped && red, i0, M, j);
         }

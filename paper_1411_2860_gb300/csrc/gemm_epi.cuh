@@ -50,14 +50,14 @@ __device__ __forceinline__ void store_rows(const uint32_t (&r)[NR], void* Yv, in
   }
 }
 
-// The same for a lowered correlation: element (i, j) is output sample i * w + j of a
+// The same for a lowered correlation: element (i, j) is output sample i * 128 + j of a
 // phase, `stride` floats apart, below `limit`.
 template <int NR>
-__device__ __forceinline__ void store_samples(const uint32_t (&r)[NR], float* Y, int w, int64_t stride, int64_t limit,
+__device__ __forceinline__ void store_samples(const uint32_t (&r)[NR], float* Y, int64_t stride, int64_t limit,
                                               int i0, int j, bool jok) {
 #pragma unroll
   for (int u = 0; u < NR; ++u) {
-    const int64_t flat = static_cast<int64_t>(i0 + u) * w + j;
+    const int64_t flat = static_cast<int64_t>(i0 + u) * 128 + j;
     if (jok && flat < limit) __stcs(Y + flat * stride, __uint_as_float(r[u]));
   }
 }

@@ -183,7 +183,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         const int tj = T.tj, bn = I->bn;
         const int y0 = T.ti * bn;
         const bool conv = I->conv_mode != 0;
-        const int cmask = conv ? I->conv_w / BK - 1 : 0, cshift = conv ? 31 - __clz(I->conv_w / BK) : 0;
         const bool mnP = kMN && I->mnP != 0, mnQ = kMN && I->mnQ != 0;
         const uint32_t stage_bytes = kStageP + static_cast<uint32_t>(bn) * BK * 2;
         const int qchunks = bn / 64;
@@ -213,11 +212,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             oQ = kk < e0 ? sQ0 : (kk < e1 ? sQ1 : sQ2);
           }
           const int px = oP + kin * BK;
-          // Row-split mode: Q row r, K chunk k lives at row r + k / c, column 64 (k mod c) of
-          // a view c = conv_w / 64 chunks wide (the signal segments of a lowered correlation);
-          // there a segment's Q offset counts rows (the split residual rows follow the hi rows).
-          const int qx = conv ? (kin & cmask) * BK : oQ + kin * BK;
-          const int qy = conv ? y0 + (kin >> cshift) + oQ : y0;
+          // Row-split mode: Q row r, K chunk k lives at row r + k / 2, half k mod 2 of a
+          // 128-wide view (the signal segments of a lowered correlation); there a segment's
+          // Q offset counts rows (the split residual rows follow the hi rows).
+          const int qx = conv ? (kin & 1) * BK : oQ + kin * BK;
+          const int qy = conv ? y0 + (kin >> 1) + oQ : y0;
           uint64_t* const bar = &full[stage];
           uint8_t* const dP = sm + stage * slot_bytes;
           uint8_t* const dQ = dP + kStageP;
@@ -414,8 +413,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             pending = true;
           }
         } else if (I->conv_mode) {
-          // lowered correlation: element (i, j) is output sample i * conv_w + j of this phase
-          store_samples<32>(r, static_cast<float*>(Yout), I->conv_w, I->conv_stride, I->conv_limit, i0, j, jok);
+          // lowered correlation: element (i, j) is output sample i * 128 + j of this phase
+          store_samples<32>(r, static_cast<float*>(Yout), I->conv_stride, I->conv_limit, i0, j, jok);
         } else if (jok) {
           store_rows<32>(r, Yout, ldy, out_bf16, red, i0, M, j);
         }
@@ -458,7 +457,7 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
     const uint32_t box[2] = {64, BK};
     if (!make_tmap_bf16(&I->mapQ, a.Q, 2, dims, strides, box)) return false;
   } else {
-    const uint64_t dims[2] = {static_cast<uint64_t>(a.conv_mode ? a.conv_w : a.xdim),
+    const uint64_t dims[2] = {static_cast<uint64_t>(a.conv_mode ? BM : a.xdim),
                               static_cast<uint64_t>(a.conv_mode ? a.q_rows_alloc : a.rowsQ)};
     const uint64_t strides[1] = {static_cast<uint64_t>(a.ldq) * 2};
     const uint32_t box[2] = {BK, static_cast<uint32_t>(a.pair ? a.bn / 2 : a.bn)};
@@ -486,7 +485,6 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
              I->segQ[0] == I->segQ[1];
   I->tiles_n = static_cast<int>(ceil_div(a.rowsP, BM));
   I->conv_mode = a.conv_mode;
-  I->conv_w = a.conv_w;
   I->conv_stride = a.conv_stride;
   I->conv_limit = a.conv_limit;
   I->tma_out = 0;
@@ -494,11 +492,11 @@ bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I) {
   I->tma_cols = 1 << 30;
   const size_t es = I->out_bf16 ? 2 : 4;
   if (a.conv_mode) {
-    // contiguous output rows of conv_w samples only when samples are adjacent in memory
-    const int64_t full_rows = a.conv_limit / a.conv_w;
+    // contiguous output rows of 128 samples only when samples are adjacent in memory
+    const int64_t full_rows = a.conv_limit / BM;
     if (a.conv_stride == 1 && !I->out_bf16 && full_rows > 0 && reinterpret_cast<uintptr_t>(a.Y) % 16 == 0) {
-      const uint64_t dims[2] = {static_cast<uint64_t>(a.conv_w), static_cast<uint64_t>(full_rows)};
-      const uint64_t strides[1] = {static_cast<uint64_t>(a.conv_w) * 4};
+      const uint64_t dims[2] = {static_cast<uint64_t>(BM), static_cast<uint64_t>(full_rows)};
+      const uint64_t strides[1] = {static_cast<uint64_t>(BM) * 4};
       const uint32_t box[2] = {BM, 32};
       I->tma_out = make_tmap_f32(&I->mapY, a.Y, 2, dims, strides, box) ? 1 : 0;
       I->tma_rows = static_cast<int>(full_rows);
