@@ -281,17 +281,29 @@ def _basis_arg(kind, L, user_C=None, holder=None):
 
 
 @functools.lru_cache(maxsize=1024)
-def _gemm_size_of(fn: str, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier) -> int:
-    n = getattr(_load(), fn)(M, N, K, block_k, R, _basis_ref(basis, L), _prec_of(compute, split, split_lead, fp8_tier))
+def _gemm_call_of(where: str, size_fn: str, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier):
+    b, p = _basis_ref(basis, L), _prec_of(compute, split, split_lead, fp8_tier)
+    n = getattr(_load(), size_fn)(M, N, K, block_k, R, b, p)
     if n == 0:
-        raise ProjError(PJ_EINVAL, fn[:-len("_workspace_size")], last_error())   # (an exception is not remembered)
-    return int(n)
+        raise ProjError(PJ_EINVAL, where, last_error())   # (an exception is not remembered)
+    return b, p, int(n), None
 
 
-def _gemm_size(fn: str, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier) -> int:
-    plain = type(M) is int and type(N) is int and type(K) is int and type(block_k) is int and type(R) is int
-    size = _gemm_size_of if plain else _gemm_size_of.__wrapped__
-    return size(fn, M, N, K, block_k, R, basis, int(L), compute, int(split), int(split_lead), int(fp8_tier))
+def _gemm_call(where: str, size_fn: str, M, N, K, block_k, R, basis, L, user_C, holder, compute, split=1, split_lead=0,
+               fp8_tier=0):
+    """What a product's call passes: (basis, precision, workspace bytes, object to keep alive meanwhile)."""
+    if basis != "user":
+        if (type(block_k) is int and type(R) is int and type(K) is int and type(L) is int and type(split) is int
+                and type(split_lead) is int and type(fp8_tier) is int):
+            return _gemm_call_of(where, size_fn, M, N, K, block_k, R, basis, L, compute, split, split_lead, fp8_tier)
+        return _gemm_call_of.__wrapped__(where, size_fn, M, N, K, block_k, R, basis, int(L), compute, int(split),
+                                         int(split_lead), int(fp8_tier))
+    b, keep = _basis_arg(basis, L, user_C, holder)
+    p = _prec_ref(compute, split, split_lead, fp8_tier)
+    n = getattr(_load(), size_fn)(M, N, K, block_k, R, b, p)
+    if n == 0:
+        raise ProjError(PJ_EINVAL, where, last_error())
+    return b, p, n, keep
 
 
 def _stream(stream, device):
@@ -392,16 +404,9 @@ def proj_gemm(A, B, block_k: int, R: int, basis: str = "dct2", L: int = 8, compu
     if out is None:
         out = torch.empty((M, N), dtype=out_dtype, device=A.device)
     ldy = _rows(out)
-    b, _keep = _basis_arg(basis, L, user_C, workspace)
-    p = _prec_ref(compute, split, split_lead, fp8_tier)
     lib = _load()
-    if _keep is None:
-        nbytes = _gemm_size("proj_gemm_workspace_size", M, N, K, block_k, R, basis, L, compute, split, split_lead,
-                            fp8_tier)
-    else:
-        nbytes = lib.proj_gemm_workspace_size(M, N, K, block_k, R, b, p)
-        if nbytes == 0:
-            raise ProjError(PJ_EINVAL, "proj_gemm", last_error())
+    b, p, nbytes, _keep = _gemm_call("proj_gemm", "proj_gemm_workspace_size", M, N, K, block_k, R, basis, L, user_C,
+                                     workspace, compute, split, split_lead, fp8_tier)
     device = A.device
     ws = _workspace(nbytes, device, workspace)
     st = _on(device, lib.proj_gemm, A.data_ptr(), lda, B.data_ptr(), ldb, out.data_ptr(), ldy, M, N, K, _DT[A.dtype],
@@ -458,18 +463,6 @@ def proj_gemm_fused(A, out, block_k: int, R: int, workspace, basis="dct2", L=8, 
     return out
 
 
-def _backward_bytes(where, M, N, K, block_k, R, basis, L, compute, b, p, keep) -> int:
-    if keep is None:
-        try:
-            return _gemm_size("proj_gemm_backward_workspace_size", M, N, K, block_k, R, basis, L, compute, 1, 0, 0)
-        except ProjError as e:
-            raise ProjError(PJ_EINVAL, where, last_error()) from e
-    n = _load().proj_gemm_backward_workspace_size(M, N, K, block_k, R, b, p)
-    if n == 0:
-        raise ProjError(PJ_EINVAL, where, last_error())
-    return n
-
-
 def proj_gemm_backward(A, B, dY, block_k: int, R: int, basis: str = "dct2", L: int = 8,
                        compute: str | None = None, out_dtype=None, user_C=None, workspace=None, stream=None,
                        dA=None, dB=None):
@@ -489,10 +482,9 @@ def proj_gemm_backward(A, B, dY, block_k: int, R: int, basis: str = "dct2", L: i
         dA = torch.empty((M, K), dtype=out_dtype, device=A.device)
     if dB is None:
         dB = torch.empty((K, N), dtype=out_dtype, device=A.device)
-    b, _keep = _basis_arg(basis, L, user_C)
-    p = _prec_ref(compute, 1)
     lib = _load()
-    nbytes = _backward_bytes("proj_gemm_backward", M, N, K, block_k, R, basis, L, compute, b, p, _keep)
+    b, p, nbytes, _keep = _gemm_call("proj_gemm_backward", "proj_gemm_backward_workspace_size", M, N, K, block_k, R,
+                                     basis, L, user_C, None, compute)
     device = A.device
     ws = _workspace(nbytes, device, workspace)
     st = _on(device, lib.proj_gemm_backward_mixed, A.data_ptr(), _rows(A), B.data_ptr(), _rows(B), dY.data_ptr(),
@@ -516,10 +508,9 @@ def proj_gemm_backward_saved(fwd_workspace, dY, K: int, block_k: int, R: int, ba
         dA = torch.empty((M, K), dtype=out_dtype, device=dY.device)
     if dB is None:
         dB = torch.empty((K, N), dtype=out_dtype, device=dY.device)
-    b, _keep = _basis_arg(basis, L, user_C)
-    p = _prec_ref(compute, 1)
     lib = _load()
-    nbytes = _backward_bytes("proj_gemm_backward_saved", M, N, K, block_k, R, basis, L, compute, b, p, _keep)
+    b, p, nbytes, _keep = _gemm_call("proj_gemm_backward_saved", "proj_gemm_backward_workspace_size", M, N, K, block_k,
+                                     R, basis, L, user_C, None, compute)
     device = dY.device
     ws = _workspace(nbytes, device, workspace)
     st = _on(device, lib.proj_gemm_backward_saved, fwd_workspace.data_ptr(), fwd_workspace.numel(), dY.data_ptr(),
@@ -547,9 +538,8 @@ class ProjGemmFn(torch.autograd.Function):
                 raise ValueError("save_projections needs split = 1")
             compute = "f64" if A.dtype == torch.float64 else "bf16"
             M, K = A.shape
-            nbytes = (_gemm_size("proj_gemm_workspace_size", M, B.shape[1], K, block_k, R, basis, L, compute, 1, 0, 0)
-                      if basis != "user" else
-                      gemm_workspace_size(M, B.shape[1], K, block_k, R, basis, L, compute, user_C=user_C))
+            nbytes = _gemm_call("proj_gemm", "proj_gemm_workspace_size", M, B.shape[1], K, block_k, R, basis, L, user_C,
+                                None, compute)[2]
             ws = torch.empty(nbytes, dtype=torch.uint8, device=A.device)
             ctx.fwd_ws = ws
             ctx.shape = (K, A.dtype, B.dtype)
