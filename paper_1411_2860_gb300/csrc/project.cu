@@ -1070,9 +1070,11 @@ RowsJob make_rows_job(const void* A, int64_t lda, int in_dtype, const GemmGeom& 
   J.lp1 = g.lp1;
   J.nsplit = g.nsplit;
   J.in_bf16 = in_dtype == PJ_BF16;
-  // Runs per warp: eight where that leaves the chip full (152 SMs x 4 blocks x 8 warps),
+  // Runs per warp: eight where that leaves the chip full (4 blocks of 8 warps an SM),
   // fewer for small operands; BF16 input loads one pair at a time, so its warps take one.
-  const int64_t units = J.M * ceil_div(J.NG, kRowRun), warps = 152 * 32;
+  int sms = 0;
+  if (device_sms(&sms) != PJ_OK) sms = 152;
+  const int64_t units = J.M * ceil_div(J.NG, kRowRun), warps = static_cast<int64_t>(sms) * 32;
   J.upw = J.in_bf16 || units <= 2 * warps ? 2 : (units >= 8 * warps ? 8 : static_cast<int>(units / warps / 2 * 2));
   return J;
 }
