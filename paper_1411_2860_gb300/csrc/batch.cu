@@ -904,7 +904,7 @@ Schedule schedule_kinds(const Built& b, int a, int c, int sms, bool paired) {
       const double cost = tile_cost(t, k1 - k0, pl.bn, pl.out_bf16, sp > 1);
       for (int ti = 0; ti < pl.tiles_m; ++ti)
         for (int tj = 0; tj < cols; ++tj)
-          items.push_back(Item{GemmTile{pl.index, ti, tj, k0, k1, sp > 1 ? 1 : 0, 0, 0}, cost});
+          items.push_back(Item{GemmTile{pl.index, ti, tj, k0, k1, sp > 1 ? 1 : 0}, cost});
     }
   }
   // units that take items: CTAs, or clusters of two when paired

@@ -454,7 +454,7 @@ int share_chunk(int k) { return (k + 2) / 3; }
 // instance's reduced dimension is split), and red = 1 when its partial product
 // is added to the output (the output is zeroed first) instead of stored.
 struct GemmTile {
-  int inst, ti, tj, k0, k1, red, pad0, pad1;   // tj: tile column, or pair column on CTA pairs
+  int inst, ti, tj, k0, k1, red;   // tj: tile column, or pair column on CTA pairs
 };
 bool build_gemm_inst(const GemmTcArgs& a, GemmInst* I);
 int gemm_tiles_of(const GemmInst& I);

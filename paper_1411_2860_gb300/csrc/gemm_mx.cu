@@ -105,7 +105,6 @@ __device__ __forceinline__ const MxInst* mx_tile_of(const MxParams& p, int n, Ge
     t.k0 = 0;
     t.k1 = p.single.kc * p.single.nseg;
     t.red = p.single.accum;
-    t.pad0 = 0;
     return &p.single;
   }
   if (p.tiles) {
@@ -131,7 +130,6 @@ __device__ __forceinline__ const MxInst* mx_tile_of(const MxParams& p, int n, Ge
     t.k0 = unit * static_cast<int>(start - static_cast<int64_t>(tile) * S);
     t.k1 = unit * static_cast<int>(end - static_cast<int64_t>(tile) * S);
     t.red = (t.k0 != 0 || t.k1 != unit * S || p.single.accum) ? 1 : 0;
-    t.pad0 = 0;
     return &p.single;
   }
   const int tile = blockIdx.x + n * gridDim.x;
@@ -141,7 +139,6 @@ __device__ __forceinline__ const MxInst* mx_tile_of(const MxParams& p, int n, Ge
   t.k0 = 0;
   t.k1 = unit * S;
   t.red = p.single.accum;
-  t.pad0 = 0;
   return &p.single;
 }
 
@@ -396,12 +393,7 @@ __global__ void __launch_bounds__(kXThreads, 1) gemm_mx_kernel(const __grid_cons
         if (i0 >= M) continue;
         if (conv) {
           // lowered correlation: element (i, j) is output sample i * 128 + j of this phase
-          float* Y = static_cast<float*>(I->Y);
-#pragma unroll
-          for (int u = 0; u < kXEpiRows; ++u) {
-            const int64_t flat = static_cast<int64_t>(i0 + u) * XBM + j;
-            if (jok && flat < I->conv_limit) __stcs(Y + flat * I->conv_stride, __uint_as_float(r[u]));
-          }
+          store_samples<kXEpiRows>(r, static_cast<float*>(Yout), I->conv_stride, I->conv_limit, i0, j, jok);
         } else if (tma) {
           if (leader && pending) bulk_wait_read_all();
           named_barrier(1, 128);
@@ -659,10 +651,11 @@ bool build_mx_inst(const MxGemmArgs& a, MxInst* I) {
 
 // Tile height of a single product of `rows` x (tiles_n x 128) outputs over `chunks` K
 // chunks of 128: whole waves of tiles over the SMs, each ring slot costed (in ns) as
-// the longest of its loads from L2 (128 B_d rows and half of the pair's bn A_c rows at
-// the ~82 bytes per ns a SM draws when all of them load), its MMAs (a slot of a split
-// product serves 1.5 products) and the ~1.6 us a load takes shared by the slots in
-// flight; plus 1 us a tile.  (1500 x 2048 over 81 split chunks: 176 rows, one wave.)
+// the longest of its loads from L2 (128 B_d rows and half of the pair's bn A_c rows, at
+// 1.56 ns a row of 128 bytes: a cost fitted to the times of such products, above the 0.9
+// or so that the rate in tc.cuh allows), its MMAs (a slot of a split product serves 1.5
+// products) and the ~1.6 us a load takes shared by the slots in flight; plus 1 us a tile.
+// (1500 x 2048 over 81 split chunks: 176 rows, one wave.)
 int mx_single_rows(int64_t rows, int64_t tiles_n, int64_t chunks, bool split, int sms) {
   int best = XBN;
   double best_t = 0;

@@ -35,7 +35,7 @@
 #include "tc.cuh"
 #include "tmap.hpp"
 #if PJ_CTA_PAIRS
-#include "tc_pair.cuh"   // as in every GEMM of the build with CTA pairs
+#include "tc_pair.cuh"   // (nothing here uses it: the build's multicast forms are looked for in this file)
 #endif
 
 namespace pj {
@@ -102,7 +102,6 @@ __device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, G
     t.k0 = unit * static_cast<int>(start - static_cast<int64_t>(tile) * S);
     t.k1 = unit * static_cast<int>(end - static_cast<int64_t>(tile) * S);
     t.red = (t.k0 != 0 || t.k1 != p.single.kc) ? 1 : 0;
-    t.pad0 = 0;
     return &p.single;
   }
   const int tile = blockIdx.x + n * gridDim.x;
@@ -112,7 +111,6 @@ __device__ __forceinline__ const GemmInst* tile_of(const GemmParams& p, int n, G
   t.k0 = 0;
   t.k1 = p.single.kc;
   t.red = 0;
-  t.pad0 = 0;  // no pair flags: the epilogue's stores (and its barriers) run in every warp
   return &p.single;
 }
 
