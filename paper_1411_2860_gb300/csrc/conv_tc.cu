@@ -75,7 +75,7 @@ struct ConvParams {
   int RB;                 // rows per ring half-load
   int tiles_per_sub;
   int num_tiles;
-  int nst;                // template-chunk pipeline stages (4 with one epilogue set, 3 with two)
+  int nst;                // template-chunk pipeline stages (4 with one epilogue set, 3 with four)
   int pstep;              // phases computed: every pstep-th (1 = all lags)
   int* err;
 };
@@ -255,9 +255,9 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
     // output rows of parity e = q / 2 for templates t0 .. t0+31, column = row pair;
     // with four sets, set s takes the 32-column chunks s and s + 4.
     // Full row pairs leave through the warp's own TMA bulk stores of 16 rows x
-    // 32 templates from two alternating 2 KB staging buffers, so a buffer is
-    // only waited for when the store issued two before it still reads it, and
-    // the four warps never wait for one another.  Ragged rows: direct stores.
+    // 32 templates, so the warps never wait for one another.  With one set a warp has two
+    // 2 KB staging buffers and waits for the store issued two before to be read; with four
+    // it has one, and waits for its last.
     // Template counts that are no multiple of 4 (rows TMA cannot address) and ragged
     // rows: direct stores, 32 lanes of one lag each.  Those are bound by the warp's
     // issue: with the bounds test and the 64-bit address formed per store, a tile of
@@ -356,8 +356,9 @@ __global__ void __launch_bounds__(conv_threads<NEPI>(), 1) conv_tc_kernel(const 
 // stages and one epilogue set.  Shorter ones are bound by the output write and
 // drain the accumulators with four epilogue sets (three template stages): with two
 // sets of two buffers each, R = 256 on 2^20 samples and 64 templates took 70.0 us a
-// call, with four of one buffer (the same memory) 68.0.  (Rows TMA cannot address
-// gain nothing from more sets: 37 templates at R = 1024 47.1 us with one, 49.0 with four.)
+// call, with four of one buffer (the same memory) 68.0.  (Rows TMA cannot address gain
+// nothing from more sets where the MMAs take their time, 37 templates at R = 1024 47.1 us
+// with one, 49.0 with four; shorter reductions take four whatever the template count.)
 int conv_epilogue_sets(int Kc) { return Kc >= 16 ? 1 : 4; }
 
 }  // namespace

@@ -25,10 +25,10 @@
 // PFLOP/s).
 //
 // A batch's products run here too (kGrouped): on CTAs of their own (gemm_tc.cu) they
-// drew 96 KB of operands per 64-component chunk through an SM that can take in about 74
-// bytes a clock, and the grouped launch of 40 products and 20 correlations took 818 us;
-// here it takes 64 KB and 733 us at 98 % of the tensor pipe's cycles, under the power
-// cap (1.74 GHz).
+// drew 96 KB of operands per 64-component chunk through SMs that take in about 70 bytes a
+// clock each (tc.cuh), and the grouped launch of 40 products and 20 correlations took 818
+// us; here it took 64 KB and 733 us at 98 % of the tensor pipe's cycles, under the power
+// cap (1.74 GHz).  (The correlations have since moved to a launch of their own, batch.cu.)
 #include <cuda_bf16.h>
 #include <string.h>
 

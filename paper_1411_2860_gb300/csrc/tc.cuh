@@ -140,9 +140,10 @@ __device__ __forceinline__ bool mbar_wait_first(uint64_t* bar, uint32_t parity, 
 // The copy producers and MMA issuers are warps that run their loop together and elect a
 // lane for each copy or MMA.  A loop that one lane runs inside a branch keeps its operands
 // in vector registers, and each copy or MMA first moves them to uniform ones: a ring step
-// with one TMA load took 343 clocks that way and 248 this way, whatever it loaded (a probe
-// streaming boxes of 64 to 256 rows of 128 bytes on 1 and on 152 SMs; +70 clocks for a
-// second load), against 448 to 512 clocks of MMAs per 64-deep K stage.
+// with one TMA load took 343 clocks that way and 248 this way, whatever it loaded, and 70
+// more for a second load, against 448 to 512 clocks of MMAs per 64-deep K stage.  (A probe
+// streaming boxes of 64 to 256 rows of 128 bytes from L2 into a ring; where the loads and
+// not the steps set its pace, one SM took in 126 bytes a clock and 152 SMs 70 each.)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, int code) {
   WaitClock clk;
   for (uint32_t it = 1;; ++it) {
